@@ -540,6 +540,10 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, const Batch &B = Batch{n
   CK(h->cell_cursor.ensure(g.ncell + 1), "alloc cells");
   CK(h->cell_start.ensure(g.ncell + 1), "alloc cells");
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
+  if (h->cap_r && h->cap_a) {  // capacities of an earlier, possibly smaller system: room for N atoms
+    const int rc = ensure_lists(h, N, h->cap_r, h->cap_a);
+    if (rc) return rc;
+  }
   for (int attempt = 0; attempt < 3; ++attempt) {
     const bool count_only = (h->cap_r == 0 || h->cap_a == 0);
     CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
