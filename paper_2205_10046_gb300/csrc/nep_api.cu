@@ -140,7 +140,11 @@ int build_grid(const double *box, double rl, int N, Grid &g, float4 *dtab, doubl
   g.jmask = (jb >= 32) ? 0xffffffffu : ((1u << jb) - 1u);
   g.ncode = 1 << (3 * g.obits);
   for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) g.Hc[a][b] = g.H[a][b] / g.nc[a];
+    for (int b = 0; b < 3; ++b) {
+      g.Hc[a][b] = g.H[a][b] / g.nc[a];
+      g.Hf[a][b] = (float)g.H[a][b];
+      g.Hinvf[a][b] = (float)g.Hinv[a][b];
+    }
   if (!dtab) return NEP_OK;
   for (int c = 0; c < g.ncode; ++c) dtab[c] = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int ox = -g.R[0]; ox <= g.R[0]; ++ox)
@@ -339,6 +343,7 @@ struct nep_handle {
   DevBuf<float4> pos4, posA, dtab, p_ang;
   DevBuf<float> e_rad;
   DevBuf<BuildStatus> status;
+  DevBuf<unsigned long long> stat_part;  // partial sums of a build's list statistics
   BuildStatus *h_status = nullptr;  // pinned mirror
   // md
   bool md_ready = false;
@@ -476,6 +481,7 @@ int ensure_atoms(nep_handle *h, int N, cudaStream_t s) {
     std::memset(h->h_status, 0, sizeof(BuildStatus));
   }
   CK(h->thermo_ctl.ensure(4), "alloc");
+  CK(h->stat_part.ensure(4 * kStatSlots), "alloc");
   return NEP_OK;
 }
 
@@ -524,7 +530,7 @@ ListBufs list_bufs(nep_handle *h) {
   ListBufs L;
   L.cell_count = h->cell_count.p; L.cell_cursor = h->cell_cursor.p; L.cell_start = h->cell_start.p;
   L.cell_atoms = h->cell_atoms.p; L.nl_r = h->nl_r.p; L.nn_r = h->nn_r.p; L.nl_a = h->nl_a.p; L.nn_a = h->nn_a.p;
-  L.rev_a = h->rev_a.p; L.cap_r = h->cap_r; L.cap_a = h->cap_a;
+  L.rev_a = h->rev_a.p; L.cap_r = h->cap_r; L.cap_a = h->cap_a; L.part = h->stat_part.p;
   L.stage_e = h->stage_e.p; L.stage_g = h->stage_g.p;
   return L;
 }
@@ -534,7 +540,9 @@ ListBufs list_bufs(nep_handle *h) {
 int round_cap(int m) { return std::min(kListBuf, (2 * m + 16 + 3) / 4 * 4); }
 
 // Bin, size and build the neighbour lists for the positions in h->x (forced rebuild).
-int rebuild_lists(nep_handle *h, int N, cudaStream_t s, const Batch &B = Batch{nullptr, nullptr, 0}) {
+// move: the per-atom arrays that go into the new atom order besides positions and types (bit 0
+// velocities, bit 1 forces).
+int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B = Batch{nullptr, nullptr, 0}) {
   Grid &g = h->grid;
   CK(h->cell_count.ensure(g.ncell + 1), "alloc cells");
   CK(h->cell_cursor.ensure(g.ncell + 1), "alloc cells");
@@ -553,7 +561,7 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, const Batch &B = Batch{n
     h->h_status->full = 1;
     CK(cudaMemcpyAsync(h->status.p, h->h_status, sizeof(BuildStatus), cudaMemcpyHostToDevice, s), "status");
     CK(launch_rebuild(N, h->T, g, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
-                      list_bufs(h), count_only ? 1 : 0, h->status.p, s),
+                      list_bufs(h), count_only ? 1 : 0, move, h->status.p, s),
        "launch rebuild");
     CK(cudaGetLastError(), "launch rebuild");
     int rc = read_status(h, s);
@@ -636,7 +644,8 @@ int kernel_form(const nep_handle *h) {
 }
 
 // Load positions (device, [N][3]) and types, set up the grid and build the lists.
-int load_structure(nep_handle *h, int N, const double *pos, const int *types, const double *box, cudaStream_t s) {
+int load_structure(nep_handle *h, int N, const double *pos, const int *types, const double *box, cudaStream_t s,
+                   int move = 0) {
   int rc = ensure_atoms(h, N, s);
   if (rc) return rc;
   std::vector<float4> dtab;
@@ -650,7 +659,7 @@ int load_structure(nep_handle *h, int N, const double *pos, const int *types, co
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = h->grid.nc[a];
-  return rebuild_lists(h, N, s);
+  return rebuild_lists(h, N, s, move);
 }
 
 // Outputs for the caller (nep_compute) are scattered to the caller's atom order; the MD
@@ -849,7 +858,7 @@ int capture_batch(nep_handle *h, int N, const BatchOut &o, cudaStream_t s) {
   launch_arm_rebuild(h->status.p, c);
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
   cudaError_t e = launch_rebuild(N, h->T, h->grid, batch_of(h), h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(),
-                                 h->rcA2f(), atom_state(h), list_bufs(h), 0, h->status.p, c);
+                                 h->rcA2f(), atom_state(h), list_bufs(h), 0, 0, h->status.p, c);
   int rc = e == cudaSuccess ? batch_kernels(h, N, o, c, true) : cuda_fail(h, e, "batch rebuild");
   if (!rc) cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, c);
   cudaGraph_t graph = nullptr;
@@ -1033,7 +1042,7 @@ int engine_relayout(nep_handle *h, const std::vector<int> &keep, const std::vect
   if (rc) return rc;
   // the first layout sizes the lists with a counting pass; later ones keep the capacity (an
   // iteration whose build overflows is undone and run again with grown lists)
-  if (h->cap_r == 0 || h->cap_a == 0) return rebuild_lists(h, N_new, s, batch_of(h));
+  if (h->cap_r == 0 || h->cap_a == 0) return rebuild_lists(h, N_new, s, 3, batch_of(h));
   CK(h->cell_count.ensure(h->grid.ncell + 1), "alloc cells");
   CK(h->cell_cursor.ensure(h->grid.ncell + 1), "alloc cells");
   CK(h->cell_start.ensure(h->grid.ncell + 1), "alloc cells");
@@ -1097,7 +1106,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   Batch B = batch_of(h);
   B.sflag = h->e_sflag.p;
   cudaError_t e = launch_rebuild(N, h->T, h->grid, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
-                                 atom_state(h), list_bufs(h), 0, h->status.p, s);
+                                 atom_state(h), list_bufs(h), 0, 3, h->status.p, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine rebuild");
   AtomArgs a = make_args(h, N);
   a.perm = nullptr;  // every output in the internal order
@@ -1345,7 +1354,7 @@ int nep_destroy(nep_handle *h) {
   h->e_slots.release(); h->e_slots_ck.release(); h->e_energy.release(); h->e_virial.release(); h->e_u.release();
   h->e_w.release(); h->e_xck.release(); h->e_vck.release(); h->e_table.release();
   h->stage_e.release(); h->stage_g.release();
-  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->d_tc.release(); h->d_ann.release();
+  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->d_tc.release(); h->d_ann.release();
   h->d_grids.release(); h->d_sid.release(); h->d_offsets.release(); h->b_e.release(); h->b_w.release();
   if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
   if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
@@ -1446,7 +1455,7 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = 0;
-  rc = rebuild_lists(h, N, s, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h));
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   rc = batch_kernels(h, N, o, s, false);
@@ -1497,7 +1506,7 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
   launch_iota(N, h->perm.p, s);
   h->N = N;
   h->stats_cache.n_atoms = N;
-  rc = rebuild_lists(h, N, s, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h));
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   // parameter vectors -> FP32 kernel arrays (and BF16 tiles for the tensor-core network)
@@ -1595,7 +1604,7 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   CK(cudaMemcpyAsync(h->types.p, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
   launch_iota(N, h->perm.p, s);
   h->N = N;
-  rc = rebuild_lists(h, N, s, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h));
   if (rc) return rc;
   // candidates: atoms per CTA of both kernels, then (for a population) members per launch
   const int est = ((h->KR + 2) + 3) / 4 * 4;
@@ -1800,7 +1809,7 @@ int md_init(nep_handle *h, int n_atoms, const double *pos, const int *types, con
   if (rc) return rc;
   if (vel) CK(cudaMemcpyAsync(h->v.p, vel, sizeof(double) * 3 * n_atoms, cudaMemcpyDeviceToDevice, s), "copy vel");
   else CK(cudaMemsetAsync(h->v.p, 0, sizeof(double) * 3 * n_atoms, s), "memset vel");
-  rc = load_structure(h, n_atoms, pos, types, box, s);
+  rc = load_structure(h, n_atoms, pos, types, box, s, 1);
   if (rc) return rc;
   rc = run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false);
   if (rc) return rc;
@@ -1875,7 +1884,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     CK(cudaStreamBeginCaptureToGraph(h->cap_stream2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
        "capture body");
     cudaError_t e = launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
-                                   atom_state(h), list_bufs(h), 0, h->status.p, h->cap_stream2);
+                                   atom_state(h), list_bufs(h), 0, 1, h->status.p, h->cap_stream2);
     cudaGraph_t out = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream2, &out);
     if (e != cudaSuccess) return cuda_fail(h, e, "launch rebuild");
@@ -1885,7 +1894,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     h->rebuild_kernels = (int)nn;
   } else {
     CK(launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
-                      list_bufs(h), 0, h->status.p, s),
+                      list_bufs(h), 0, 1, h->status.p, s),
        "launch rebuild");
     h->rebuild_kernels = 0;
   }
@@ -2049,7 +2058,7 @@ int run_steps(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double
            "restore");
       rc = ensure_lists(h, N, round_cap(st.max_r), round_cap(st.max_a));
       if (rc) return rc;
-      rc = rebuild_lists(h, N, s);
+      rc = rebuild_lists(h, N, s, 3);
       if (rc) return rc;
       h->h_status->md_steps = steps0;
       h->h_status->n_rebuilds = rebuilds0;

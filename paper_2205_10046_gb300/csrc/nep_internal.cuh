@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+#include <unordered_map>
 #include <vector>
 
 namespace nep {
@@ -31,6 +33,8 @@ struct Grid {
   double H[3][3];     // cell rows
   double Hinv[3][3];  // s = r . Hinv
   double Hc[3][3];    // rows of one grid cell: H[a] / nc[a]
+  float Hf[3][3], Hinvf[3][3];  // H and Hinv rounded to FP32 (candidate search: the FP64 to FP32
+                                // conversions run on the slow FP64 pipe)
   float reach[3];     // (r_c^R + skin + kReachMargin) / cell thickness per axis: a cell whose
                       // gap to an atom's cell position exceeds it along any axis holds no pair
   int cell_off;       // first global cell of this structure (batches; 0 for one structure)
@@ -72,7 +76,9 @@ struct ListBufs {
   int cap_r, cap_a;
   unsigned *stage_e;        // [cap_r][N] accepted candidates of one build, or null (second scan)
   unsigned char *stage_g;   // [cap_r][N] their groups
+  unsigned long long *part;  // [kStatSlots][4] partial sums of a build's list statistics
 };
+constexpr int kStatSlots = 64;
 
 // Device-visible status written by the builders.
 struct BuildStatus {
@@ -148,6 +154,23 @@ __device__ __forceinline__ float norm2(const float3 &d) {
 // pos4.w holds the atom type in bits 0-7 and its structure (batches) in bits 8-31.
 __device__ __forceinline__ int type_of(const float4 &p) { return __float_as_int(p.w) & 0xFF; }
 __device__ __forceinline__ int struct_of(const float4 &p) { return __float_as_int(p.w) >> 8; }
+
+// Raise a kernel's dynamic shared memory limit once, to a bound that covers every launch
+// (any type count up to kMaxTypes, the largest shift table). The attribute is per function
+// and process-wide: setting it per launch to that launch's size would race between threads
+// launching the same kernel with different sizes.
+template <class K>
+cudaError_t smem_limit_once(K kern, size_t bound) {
+  static std::mutex mu;
+  static std::unordered_map<const void *, size_t> done;
+  std::lock_guard<std::mutex> lk(mu);
+  const void *key = reinterpret_cast<const void *>(kern);
+  auto it = done.find(key);
+  if (it != done.end() && it->second >= bound) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bound);
+  if (e == cudaSuccess) done[key] = bound;
+  return e;
+}
 
 // Arguments of the per-atom and gather kernels (everything except the model weights).
 struct AtomArgs {
@@ -254,7 +277,7 @@ void model_constants(ModelF &m);
 int build_grid(const double *box, double rl, int N, Grid &g, float4 *dtab, double *volume, const char **err);
 cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
                            float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only,
-                           BuildStatus *st, cudaStream_t s);
+                           int move, BuildStatus *st, cudaStream_t s);
 void launch_iota(int N, int *perm, cudaStream_t s);
 void launch_export(int N, const AtomState &a, const Grid &g, const Batch &B, double *pos, double *vel, double *force,
                    cudaStream_t s);

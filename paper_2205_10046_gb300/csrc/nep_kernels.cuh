@@ -26,9 +26,6 @@
 #pragma once
 #include <cuda_bf16.h>
 
-#include <mutex>
-#include <unordered_map>
-
 #include "nep_internal.cuh"
 
 namespace nep {
@@ -1477,23 +1474,6 @@ __global__ void __launch_bounds__(GB, BATCH ? 1 : (S::KR <= 8 ? 1024 : 896) / GB
 }
 
 // ------------------------------------------------------------------------ launchers
-// Raise a kernel's dynamic shared memory limit once, to a bound that covers every launch
-// (any type count up to kMaxTypes, the largest shift table). The attribute is per function
-// and process-wide: setting it per launch to that launch's size would race between threads
-// launching the same kernel with different sizes.
-template <class K>
-cudaError_t smem_limit_once(K kern, size_t bound) {
-  static std::mutex mu;
-  static std::unordered_map<const void *, size_t> done;
-  std::lock_guard<std::mutex> lk(mu);
-  const void *key = reinterpret_cast<const void *>(kern);
-  auto it = done.find(key);
-  if (it != done.end() && it->second >= bound) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bound);
-  if (e == cudaSuccess) done[key] = bound;
-  return e;
-}
-
 template <class S>
 size_t atom_smem_bytes(int T, int ncode, int prec, int ab = kAtomBlock, bool tclr = false) {
   // the last region: BF16 operand tiles (tensor-core network; tclr: the per-thread S_nk blocks

@@ -96,7 +96,7 @@ int run_build(int N, int T, const Grid &g, const float4 *dtab, float rlR2, float
   std::memset(st_host, 0, sizeof(BuildStatus));
   st_host->rebuild = 1;
   SK(cudaMemcpyAsync(st_dev, st_host, sizeof(BuildStatus), cudaMemcpyHostToDevice, s), "status");
-  SK(launch_rebuild(N, T, g, Batch{}, dtab, rlR2, rlA2, rcR2, rcA2, a, L, count_only, st_dev, s), "neighbour build");
+  SK(launch_rebuild(N, T, g, Batch{}, dtab, rlR2, rlA2, rcR2, rcA2, a, L, count_only, 0, st_dev, s), "neighbour build");
   SK(cudaMemcpyAsync(st_host, st_dev, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   SK(cudaStreamSynchronize(s), "synchronise");
   if (st_host->bad_input & 1) return fail_static(NEP_ERR_ARG, "atom type out of range");
@@ -181,9 +181,10 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.cell_atoms = arena.take<int>(N);
   L.nn_r = arena.take<int>((size_t)T * N);
   L.nn_a = arena.take<int>(N);
+  L.part = arena.take<unsigned long long>(4 * kStatSlots);
   if (!st || !dtab || !dcR || !dcA || !a.x || !a.v || !a.F || !a.x_ref || !a.origin || !a.x2 || !a.v2 || !a.F2 ||
       !a.types || !a.perm || !a.cell_of || !a.types2 || !a.perm2 || !a.cell2 || !a.pos4 || !a.posA || !L.cell_count ||
-      !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a)
+      !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part)
     return fail_static(NEP_ERR_ARG, "structure too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
 
   // inputs into the arena; the arena keeps the previous call's contents, so everything the
