@@ -209,7 +209,7 @@ int n_des_of(const nep_params *p) {
 }
 
 // Run-time shape fields of the kernel arguments (read only by the run-time-shape kernels).
-void set_shape_args(AtomArgs &a, const nep_params &p, const float *ann) {
+void set_shape_args(AtomArgs &a, const nep_params &p) {
   a.gR = p.n_max_radial;
   a.gKR = p.basis_radial;
   a.gA = p.n_max_angular;
@@ -219,7 +219,47 @@ void set_shape_args(AtomArgs &a, const nep_params &p, const float *ann) {
   a.gL4 = p.l_max_4b;
   a.gL5 = p.l_max_5b;
   a.gD = n_des_of(&p);
-  a.ann = ann;
+}
+
+// BF16 (round to nearest even) of a float, as raw bits.
+static uint16_t to_bf16(float f) {
+  uint32_t u;
+  std::memcpy(&u, &f, 4);
+  u += 0x7FFFu + ((u >> 16) & 1u);
+  return (uint16_t)(u >> 16);
+}
+
+static float from_bf16(uint16_t b) {
+  const uint32_t u = (uint32_t)b << 16;
+  float f;
+  std::memcpy(&f, &u, 4);
+  return f;
+}
+
+// Fills a model table from the parameters (out: t.total floats, zeroed padding).
+void fill_table(const TableLayout &t, const nep_params &p, float *out) {
+  for (int v = 0; v < t.total; ++v) out[v] = 0.f;
+  int v = 0;
+  auto put = [&](const double *src, int n) {
+    for (int k = 0; k < n; ++k) out[table_place(t, v++)] = (float)src[k];
+  };
+  put(p.c_radial, t.T * t.T * (t.nR + 1) * (t.KR + 1));
+  put(p.c_angular, t.T * t.T * (t.nA + 1) * (t.KA + 1));
+  put(p.w0, t.H * t.D);
+  put(p.b0, t.H);
+  put(p.w1, t.H);
+  put(&p.b1, 1);
+  // BF16 (round to nearest even) of the value, then of what is left
+  uint16_t *tile = reinterpret_cast<uint16_t *>(out + t.tc);
+  for (int mu = 0; t.np1 && mu < t.H; ++mu)
+    for (int nu = 0; nu < t.D; ++nu) {
+      float x = (float)p.w0[(size_t)mu * t.D + nu];
+      for (int k = 0; k < 2; ++k) {
+        const uint16_t b = to_bf16(x);
+        tile[(size_t)k * t.np1 * t.kp1 + tile_place(t, mu, nu)] = b;
+        x -= from_bf16(b);
+      }
+    }
 }
 
 }  // namespace nep
@@ -309,7 +349,7 @@ struct Tuning {
   int last_members = 0;  // members per launch of the last population evaluation
   int n_tried = 0;       // candidates timed by the last autotune
   float best_ms = 0.f, default_ms = 0.f;  // per-evaluation times of the choice and of the defaults
-  int atom_form = 0;     // FP32 per-atom kernel of nep_compute / md_run: 0 default, 1, 3 (AtomArgs.atom_occ)
+  int atom_form = 0;     // nep_tuning.atom_form: 0 default, 1, 3
 };
 
 
@@ -317,15 +357,14 @@ struct nep_handle {
   // model
   int T = 0, nR = 0, nA = 0, KR = 0, KA = 0, L3 = 0, L4 = 0, L5 = 0, H = 0, n_des = 0;
   double rcR = 0, rcA = 0, skin = 1.0;
-  std::vector<float> w0, b0, w1, cR, cA;
-  float b1 = 0;
   std::vector<double> mass;
   ModelF mf;
   const ShapeOps *ops = nullptr;
   int device = 0;
   std::string err;
   // device model copies
-  DevBuf<float> d_cR, d_cA;
+  TableLayout tl{};
+  DevBuf<float> d_tab;  // model table
   DevBuf<double> d_inv_mk, d_mk_half;
   // workspace
   int N = 0;
@@ -370,8 +409,6 @@ struct nep_handle {
   bool graph_cond = true;   // rebuild inside a conditional node (else early-exit kernel nodes)
   int precision = 0;        // network arithmetic: 0 FP32 SIMT, 1 BF16 tensor cores
   int graph_prec = 0;
-  DevBuf<uint4> d_tc;       // BF16 W0 operand tiles for the tensor-core network
-  DevBuf<float> d_ann;      // FP32 network [w0 | b0 | w1 | b1] (run-time-shape kernels)
   bool generic = false;     // no compiled instantiation of this shape
   bool graph_cond_used = true;
   // batches of structures: layout of the last batch (reused while unchanged)
@@ -387,8 +424,7 @@ struct nep_handle {
   int b_graph_kernels = 0;
   BatchKey b_key{}, b_last{};
   // population evaluation: per-member kernel arrays and the sums of Eq. loss
-  DevBuf<float> pop_cr, pop_ca, pop_ann;
-  DevBuf<uint4> pop_tc;
+  DevBuf<float> pop_tab;
   DevBuf<double> pop_reg, pop_es, pop_ws;
   Tuning tune;
   // profiling
@@ -404,7 +440,7 @@ struct nep_handle {
     f(ck_x); f(ck_v); f(ck_F); f(ck_types); f(ck_perm); f(x2); f(v2); f(F2); f(types2); f(perm2); f(cell2);
     f(perm); f(types); f(cell_of); f(cell_count); f(cell_cursor); f(cell_start); f(cell_atoms); f(nn_r);
     f(nn_a); f(rev_a); f(thermo_ctl); f(nl_r); f(nl_a); f(pos4); f(posA); f(dtab); f(p_ang); f(e_rad); f(d_grids);
-    f(d_sid); f(d_offsets); f(b_e); f(b_w); f(pop_cr); f(pop_ca); f(pop_ann); f(pop_tc); f(pop_reg); f(pop_es);
+    f(d_sid); f(d_offsets); f(b_e); f(b_w); f(pop_tab); f(pop_reg); f(pop_es);
     f(pop_ws); f(fire); f(ck_fire); f(thermo_state); f(ck_thermo); f(stage_e); f(stage_g); f(e_slots);
     f(e_slots_ck); f(e_energy); f(e_virial); f(e_u); f(e_w); f(e_xck); f(e_vck); f(e_table);
   }
@@ -589,9 +625,8 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
   return fail(h, NEP_ERR_NEIGHBOR_OVERFLOW, "neighbour lists could not be sized");
 }
 
-// The FP32 per-atom kernel form in use: the caller's choice, else the low-register form (3)
-// where the shape has it (measured faster: 8.86 against 9.43 ms per step on 8,000,000 Si
-// atoms), else 1.
+// nep_tuning.atom_form in use: the caller's choice, else 3 where the shape has it, else 1. Both
+// run the same kernel; the autotuner tries 64-atom CTAs with form 1 only.
 int atom_form_of(const nep_handle *h) {
   const int f = h->tune.atom_form ? h->tune.atom_form : 3;
   return (f == 3 && h->ops && h->ops->lowreg) ? 3 : 1;
@@ -616,8 +651,9 @@ AtomArgs make_args(nep_handle *h, int N) {
   a.rev_a = h->rev_a.p;
   a.cap_r = h->cap_r;
   a.cap_a = h->cap_a;
-  a.c_r = h->d_cR.p;
-  a.c_a = h->d_cA.p;
+  a.tab = h->d_tab.p;
+  a.c_r = a.tab + h->tl.cr;
+  a.c_a = a.tab + h->tl.ca;
   a.e_rad = h->e_rad.p;
   a.est = ((h->KR + 2) + 3) / 4 * 4;
   a.p_ang = h->p_ang.p;
@@ -628,20 +664,14 @@ AtomArgs make_args(nep_handle *h, int N) {
   a.vel = h->v.p;
   a.perm = h->perm.p;
   a.precision = h->precision;
-  a.tc_b1 = h->d_tc.p;
-  a.tc_b2 = h->d_tc.p ? h->d_tc.p + (size_t)h->ops->np1 * h->ops->kp1 * 2 / 16 : nullptr;
   a.tc_err = h->status.p ? &h->status.p->tc_timeout : nullptr;
   a.gR = h->nR; a.gKR = h->KR; a.gA = h->nA; a.gKA = h->KA; a.gH = h->H;
   a.gL3 = h->L3; a.gL4 = h->L4; a.gL5 = h->L5; a.gD = h->n_des;
-  a.ann = h->d_ann.p;
-  a.atom_occ = atom_form_of(h);
   return a;
 }
 
-// Identity of the per-atom kernel a captured MD step uses (network form and FP32 kernel form).
-int kernel_form(const nep_handle *h) {
-  return h->precision * 16 + atom_form_of(h);
-}
+// Identity of the per-atom kernel a captured graph uses (the network).
+int kernel_form(const nep_handle *h) { return h->precision; }
 
 // Load positions (device, [N][3]) and types, set up the grid and build the lists.
 int load_structure(nep_handle *h, int N, const double *pos, const int *types, const double *box, cudaStream_t s,
@@ -675,7 +705,7 @@ int run_forces(nep_handle *h, int N, double *energy, double *force, double *viri
   a.md_kick = md_kick;
   a.half_dt = half_dt;
   ev_record(h, SLOT_ATOM, 0, s, capturing);
-  cudaError_t e = h->ops->atom(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, 0, s);
+  cudaError_t e = h->ops->atom(a, h->mf, 0, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "nep_atom kernel");
   ev_record(h, SLOT_ATOM, 1, s, capturing);
   ev_record(h, SLOT_GATHER, 0, s, capturing);
@@ -809,7 +839,7 @@ int batch_kernels(nep_handle *h, int N, const BatchOut &o, cudaStream_t s, bool 
   a.s_out = N;
   ev_record(h, SLOT_ATOM, 0, s, capturing);
   cudaError_t e =
-      h->ops->atom_batch(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, 1, atom_block(h), s);
+      h->ops->atom_batch(a, h->mf, 1, atom_block(h), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "nep_atom kernel (batch)");
   ev_record(h, SLOT_ATOM, 1, s, capturing);
   ev_record(h, SLOT_GATHER, 0, s, capturing);
@@ -1115,7 +1145,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   a.virial = h->e_w.p;
   a.s_out = N;
   a.slots = h->e_slots.p;
-  e = h->ops->atom_batch(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, 1, atom_block(h), s);
+  e = h->ops->atom_batch(a, h->mf, 1, atom_block(h), s);
   if (e == cudaSuccess) e = h->ops->gather_batch(a, 1, gather_block(h), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine kernels");
   launch_engine_fire(S, h->d_offsets.p, atom_state(h), h->e_slots.p, s);
@@ -1274,17 +1304,9 @@ int nep_create(const nep_params *p, nep_handle **out) {
   h->rcA = p->rc_angular;
   h->skin = p->skin > 0 ? p->skin : 1.0;
   const int T = h->T;
-  auto copyf = [](const double *src, size_t n, std::vector<float> &dst) {
-    dst.resize(n);
-    for (size_t k = 0; k < n; ++k) dst[k] = (float)src[k];
-  };
-  copyf(p->c_radial, (size_t)T * T * (h->nR + 1) * (h->KR + 1), h->cR);
-  copyf(p->c_angular, (size_t)T * T * (h->nA + 1) * (h->KA + 1), h->cA);
-  copyf(p->w0, (size_t)h->H * h->n_des, h->w0);
-  copyf(p->b0, h->H, h->b0);
-  copyf(p->w1, h->H, h->w1);
-  h->b1 = (float)p->b1;
-  for (float v : h->w0) if (!std::isfinite(v)) { delete h; return fail(nullptr, NEP_ERR_ARG, "non-finite weight"); }
+  for (size_t k = 0; k < (size_t)h->H * h->n_des; ++k)
+    if (!std::isfinite((float)p->w0[k])) { delete h; return fail(nullptr, NEP_ERR_ARG, "non-finite weight"); }
+  h->tl = table_layout(ops, T, h->nR, h->KR, h->nA, h->KA, h->H, h->n_des);
   if (p->mass) {
     h->mass.assign(p->mass, p->mass + T);
     for (double m : h->mass)
@@ -1295,8 +1317,7 @@ int nep_create(const nep_params *p, nep_handle **out) {
   cudaError_t e = cudaMallocHost(&h->h_status, sizeof(BuildStatus));
   if (e != cudaSuccess) { delete h; return fail(nullptr, NEP_ERR_CUDA, "pinned alloc failed"); }
   std::memset(h->h_status, 0, sizeof(BuildStatus));
-  if (h->d_cR.ensure(h->cR.size()) != cudaSuccess || h->d_cA.ensure(h->cA.size()) != cudaSuccess ||
-      h->d_inv_mk.ensure(T) != cudaSuccess || h->d_mk_half.ensure(T) != cudaSuccess) {
+  if (h->d_tab.ensure(h->tl.total) != cudaSuccess || h->d_inv_mk.ensure(T) != cudaSuccess || h->d_mk_half.ensure(T) != cudaSuccess) {
     nep_destroy(h);
     return fail(nullptr, NEP_ERR_OOM, "device alloc failed");
   }
@@ -1305,19 +1326,9 @@ int nep_create(const nep_params *p, nep_handle **out) {
     imk[t] = 1.0 / (h->mass[t] * kKappa);
     mkh[t] = 0.5 * h->mass[t] * kKappa;
   }
-  if (h->generic) {  // the run-time-shape kernels read the network from global memory
-    std::vector<float> ann(h->w0);
-    ann.insert(ann.end(), h->b0.begin(), h->b0.end());
-    ann.insert(ann.end(), h->w1.begin(), h->w1.end());
-    ann.push_back(h->b1);
-    if (h->d_ann.ensure(ann.size()) != cudaSuccess ||
-        cudaMemcpy(h->d_ann.p, ann.data(), ann.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) {
-      nep_destroy(h);
-      return fail(nullptr, NEP_ERR_OOM, "device alloc failed");
-    }
-  }
-  cudaMemcpy(h->d_cR.p, h->cR.data(), h->cR.size() * sizeof(float), cudaMemcpyHostToDevice);
-  cudaMemcpy(h->d_cA.p, h->cA.data(), h->cA.size() * sizeof(float), cudaMemcpyHostToDevice);
+  std::vector<float> tab(h->tl.total);
+  fill_table(h->tl, *p, tab.data());
+  cudaMemcpy(h->d_tab.p, tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice);
   cudaMemcpy(h->d_inv_mk.p, imk.data(), T * sizeof(double), cudaMemcpyHostToDevice);
   e = cudaMemcpy(h->d_mk_half.p, mkh.data(), T * sizeof(double), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) { nep_destroy(h); return fail(nullptr, NEP_ERR_CUDA, cudaGetErrorString(e)); }
@@ -1341,7 +1352,7 @@ int nep_destroy(nep_handle *h) {
     for (int w = 0; w < 2; ++w)
       if (h->ev[sl][w]) cudaEventDestroy(h->ev[sl][w]);
   if (h->h_status) cudaFreeHost(h->h_status);
-  h->d_cR.release(); h->d_cA.release(); h->d_inv_mk.release(); h->d_mk_half.release();
+  h->d_tab.release(); h->d_inv_mk.release(); h->d_mk_half.release();
   h->x.release(); h->v.release(); h->F.release(); h->x_ref.release(); h->origin.release();
   h->partial_atom.release(); h->partial_gather.release(); h->thermo_stage.release();
   h->ck_x.release(); h->ck_v.release(); h->ck_F.release(); h->ck_types.release(); h->ck_perm.release();
@@ -1354,11 +1365,11 @@ int nep_destroy(nep_handle *h) {
   h->e_slots.release(); h->e_slots_ck.release(); h->e_energy.release(); h->e_virial.release(); h->e_u.release();
   h->e_w.release(); h->e_xck.release(); h->e_vck.release(); h->e_table.release();
   h->stage_e.release(); h->stage_g.release();
-  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->d_tc.release(); h->d_ann.release();
+  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release();
   h->d_grids.release(); h->d_sid.release(); h->d_offsets.release(); h->b_e.release(); h->b_w.release();
   if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
   if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
-  h->pop_cr.release(); h->pop_ca.release(); h->pop_ann.release(); h->pop_tc.release(); h->pop_reg.release();
+  h->pop_tab.release(); h->pop_reg.release();
   h->pop_es.release(); h->pop_ws.release();
   delete h;
   return NEP_OK;
@@ -1509,22 +1520,14 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
   rc = rebuild_lists(h, N, s, 0, batch_of(h));
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
-  // parameter vectors -> FP32 kernel arrays (and BF16 tiles for the tensor-core network)
-  const int T2 = h->T * h->T;
-  const int n_cr = T2 * (h->nR + 1) * (h->KR + 1), n_ca = T2 * (h->nA + 1) * (h->KA + 1);
-  const int n_par = nep_n_par(h), n_ann = n_par - n_cr - n_ca;
-  CK(h->pop_cr.ensure((size_t)n_pop * n_cr), "alloc population");
-  CK(h->pop_ca.ensure((size_t)n_pop * n_ca), "alloc population");
-  CK(h->pop_ann.ensure((size_t)n_pop * n_ann), "alloc population");
+  // parameter vectors -> FP32 model tables (and BF16 tiles for the tensor-core network)
+  const int n_par = nep_n_par(h);
+  const size_t s_tab = h->tl.total;
+  CK(h->pop_tab.ensure(n_pop * s_tab), "alloc population");
   CK(h->pop_reg.ensure(2 * (size_t)n_pop), "alloc population");
-  launch_unpack_population(n_pop, z, n_par, n_cr, n_ca, h->pop_cr.p, h->pop_ca.p, h->pop_ann.p, h->pop_reg.p, s);
-  const long long s_tc = (long long)h->ops->np1 * h->ops->kp1 * 2 * 4 / 16;  // four tiles, uint4 units
-  if (h->precision >= 1) {
-    CK(h->pop_tc.ensure((size_t)n_pop * s_tc), "alloc population");
-    CK(cudaMemsetAsync(h->pop_tc.p, 0, sizeof(uint4) * (size_t)n_pop * s_tc, s), "memset tiles");
-    launch_population_tiles(n_pop, h->pop_ann.p, n_ann, h->H, h->n_des, h->ops->kp1, h->ops->np1,
-                            reinterpret_cast<unsigned short *>(h->pop_tc.p), s);
-  }
+  CK(cudaMemsetAsync(h->pop_tab.p, 0, sizeof(float) * n_pop * s_tab, s), "memset tables");
+  launch_unpack_population(n_pop, z, n_par, h->tl, h->pop_tab.p, h->pop_reg.p, s);
+  if (h->precision >= 1) launch_population_tiles(n_pop, h->pop_tab.p, h->tl, s);
   // members evaluated per launch (grid.y): the tuned value, else as many as the workspace
   // budget holds
   const int est = ((h->KR + 2) + 3) / 4 * 4;
@@ -1554,19 +1557,15 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
     a.force = nullptr;
     a.virial = w_tar ? h->b_w.p : nullptr;
     a.s_out = N;
-    a.c_r = h->pop_cr.p + (size_t)p0 * n_cr;
-    a.s_cr = n_cr;
-    a.c_a = h->pop_ca.p + (size_t)p0 * n_ca;
-    a.s_ca = n_ca;
-    a.pop_ann = h->pop_ann.p + (size_t)p0 * n_ann;
-    a.s_ann = n_ann;
-    a.pop_tc = h->precision >= 1 ? h->pop_tc.p + (size_t)p0 * s_tc : nullptr;
-    a.s_tc = s_tc;
+    a.tab = h->pop_tab.p + (size_t)p0 * s_tab;
+    a.c_r = a.tab + h->tl.cr;
+    a.c_a = a.tab + h->tl.ca;
+    a.s_tab = (long long)s_tab;
     a.s_erad = (long long)N * h->T * est;
     a.s_pang = (long long)h->cap_a * N;
     a.f_tar = f_tar;
     ev_record(h, SLOT_ATOM, 0, s, false);
-    cudaError_t e = h->ops->atom_batch(a, h->mf, nullptr, nullptr, nullptr, 0.f, m, atom_block(h), s);
+    cudaError_t e = h->ops->atom_batch(a, h->mf, m, atom_block(h), s);
     if (e != cudaSuccess) return cuda_fail(h, e, "nep_atom kernel (population)");
     ev_record(h, SLOT_ATOM, 1, s, false);
     ev_record(h, SLOT_GATHER, 0, s, false);
@@ -1632,7 +1631,7 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
     float best = 1e30f;
     for (int it = 0; it < 4; ++it) {
       cudaEventRecord(e0, s);
-      cudaError_t e = h->ops->atom_batch(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, m,
+      cudaError_t e = h->ops->atom_batch(a, h->mf, m,
                                          atom_block(h), s);
       if (e == cudaSuccess) e = h->ops->gather_batch(a, m, gather_block(h), s);
       if (e != cudaSuccess) return cuda_fail(h, e, "autotune launch");
@@ -1650,7 +1649,7 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   int best_ab = 128, best_gb = 128;
   const int abs_[2] = {64, 128}, gbs[3] = {64, 128, 256};
   for (int ia = 0; ia < 2 && !rc; ++ia) {
-    // the tensor-core forms, the run-time-shape kernels and the low-register FP32 form work on
+    // the tensor-core networks, the run-time-shape kernels and nep_tuning.atom_form 3 take
     // 128-atom CTAs only (a 64-atom CTA would change the FP32 form, hence the rounding)
     if ((h->precision >= 1 || h->generic || atom_form_of(h) == 3) && abs_[ia] != 128) continue;
     for (int ig = 0; ig < 3 && !rc; ++ig) {
@@ -1744,7 +1743,7 @@ int nep_descriptors(nep_handle *h, int n_atoms, const double *pos, const int *ty
   if (rc) return rc;
   AtomArgs a = make_args(h, n_atoms);
   a.q_out = q;
-  cudaError_t e = h->ops->atom(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, 1, s);
+  cudaError_t e = h->ops->atom(a, h->mf, 1, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "descriptor kernel");
   return NEP_OK;
 }
@@ -2146,7 +2145,7 @@ int nep_heat_current(nep_handle *h, int n_atoms, const double *pos, const int *t
   AtomArgs a = make_args(h, n_atoms);
   a.vel_in = vel;
   a.heat = heat;
-  cudaError_t e = h->ops->atom(a, h->mf, h->w0.data(), h->b0.data(), h->w1.data(), h->b1, 0, s);
+  cudaError_t e = h->ops->atom(a, h->mf, 0, s);
   if (e == cudaSuccess) e = h->ops->gather(a, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "heat current kernels");
   launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
@@ -2276,20 +2275,6 @@ int nep_set_profiling(nep_handle *h, int enable) {
   return NEP_OK;
 }
 
-// BF16 (round to nearest even) of a float, as raw bits.
-static uint16_t to_bf16(float f) {
-  uint32_t u;
-  std::memcpy(&u, &f, 4);
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  return (uint16_t)(u >> 16);
-}
-
-static float from_bf16(uint16_t b) {
-  const uint32_t u = (uint32_t)b << 16;
-  float f;
-  std::memcpy(&f, &u, 4);
-  return f;
-}
 
 int nep_set_precision(nep_handle *h, int mode) {
   if (!valid_handle(h)) return NEP_ERR_ARG;
@@ -2297,28 +2282,6 @@ int nep_set_precision(nep_handle *h, int mode) {
     return fail(h, NEP_ERR_ARG, "precision must be 0 (FP32), 1 (BF16 tensor cores) or 2 (split BF16)");
   if (mode >= 1 && h->generic)
     return fail(h, NEP_ERR_UNSUPPORTED, "the tensor-core forms need a compiled hyper-parameter shape");
-  if (mode >= 1 && !h->d_tc.p) {
-    // W0 as the two GEMM operands, K-major no-swizzle UMMA layout, zero padded:
-    //   B1 [NP1 x KP1]: (mu, nu) -> w0[mu][nu];  B2 [KP1 x NP1]: (nu, mu) -> w0[mu][nu]
-    // first rounded to BF16, then (for the split form) the BF16 of the remainder
-    const int KP1 = h->ops->kp1, NP1 = h->ops->np1, D = h->n_des, H = h->H;
-    const size_t tile = (size_t)NP1 * KP1;
-    std::vector<uint16_t> t(4 * tile, 0);
-    auto off = [](int r, int k, int KC) { return ((r / 8) * KC + k / 8) * 64 + (r % 8) * 8 + (k % 8); };
-    uint16_t *b1 = t.data(), *b2 = b1 + tile, *b1lo = b2 + tile, *b2lo = b1lo + tile;
-    for (int mu = 0; mu < H; ++mu)
-      for (int nu = 0; nu < D; ++nu) {
-        const float x = h->w0[(size_t)mu * D + nu];
-        const uint16_t v = to_bf16(x);
-        const uint16_t vl = to_bf16(x - from_bf16(v));
-        b1[off(mu, nu, KP1 / 8)] = v;
-        b2[off(nu, mu, NP1 / 8)] = v;
-        b1lo[off(mu, nu, KP1 / 8)] = vl;
-        b2lo[off(nu, mu, NP1 / 8)] = vl;
-      }
-    CK(h->d_tc.ensure(t.size() * 2 / 16), "alloc tiles");
-    CK(cudaMemcpy(h->d_tc.p, t.data(), t.size() * 2, cudaMemcpyHostToDevice), "copy tiles");
-  }
   h->precision = mode;
   return NEP_OK;
 }

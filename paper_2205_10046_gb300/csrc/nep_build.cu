@@ -972,21 +972,17 @@ __global__ void arm_rebuild_kernel(BuildStatus *st) {
 
 // ------------------------------------------------------------------ population evaluation
 // Candidate parameter vectors z [P][N_par], in the order c^R, c^A, w0, b0, w1, b1, become
-// the FP32 arrays of the batched kernels (c^R, c^A and the network [w0 | b0 | w1 | b1]);
+// the FP32 model tables of the batched kernels (TableLayout; padding zeroed before);
 // reg[m] = (sum |z|, sum z^2) for the regularisation terms of Eq. loss. One block per member.
-__global__ void unpack_population_kernel(const double *z, int n_par, int n_cr, int n_ca, float *cr, float *ca,
-                                         float *ann, double *reg) {
+__global__ void unpack_population_kernel(const double *z, int n_par, const TableLayout t, float *tab, double *reg) {
   const int m = blockIdx.x;
-  const int n_ann = n_par - n_cr - n_ca;
   const double *zm = z + (size_t)m * n_par;
   double s1 = 0.0, s2 = 0.0;
   for (int v = threadIdx.x; v < n_par; v += blockDim.x) {
     const double x = zm[v];
     s1 += fabs(x);
     s2 += x * x;
-    if (v < n_cr) cr[(size_t)m * n_cr + v] = (float)x;
-    else if (v < n_cr + n_ca) ca[(size_t)m * n_ca + (v - n_cr)] = (float)x;
-    else ann[(size_t)m * n_ann + (v - n_cr - n_ca)] = (float)x;
+    tab[(size_t)m * t.total + table_place(t, v)] = (float)x;
   }
   __shared__ double r1[256], r2[256];
   r1[threadIdx.x] = s1;
@@ -1005,28 +1001,22 @@ __global__ void unpack_population_kernel(const double *z, int n_par, int n_cr, i
   }
 }
 
-// BF16 operand tiles of every member's w0 (the layout of the single-model tiles): tile 1
-// [NP1 x KP1] holds (mu, nu) -> w0[mu][nu], tile 2 [KP1 x NP1] holds (nu, mu) -> w0[mu][nu].
-// The tiles must be zeroed before (padding).
-__global__ void population_tiles_kernel(int n_pop, const float *ann, int n_ann, int H, int D, int KP1, int NP1,
-                                        unsigned short *tiles) {
+// BF16 operand tiles of every member's w0 in its model table (TableLayout).
+__global__ void population_tiles_kernel(int n_pop, float *tab, const TableLayout t) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= (long long)n_pop * H * D) return;
-  const int m = (int)(v / ((long long)H * D));
-  const int r = (int)(v % ((long long)H * D));
-  const int mu = r / D, nu = r % D;
-  const float x = ann[(size_t)m * n_ann + r];
-  const __nv_bfloat16 bh = __float2bfloat16_rn(x);
-  const unsigned short b = __bfloat16_as_ushort(bh);
-  const unsigned short bl = __bfloat16_as_ushort(__float2bfloat16_rn(x - __bfloat162float(bh)));
-  const size_t tile = (size_t)NP1 * KP1;
-  // per member: B1, B2, then the split form's B1_lo, B2_lo
-  unsigned short *t1 = tiles + (size_t)m * 4 * tile, *t2 = t1 + tile;
-  auto off = [](int row, int k, int kc) { return ((row / 8) * kc + k / 8) * 64 + (row % 8) * 8 + (k % 8); };
-  t1[off(mu, nu, KP1 / 8)] = b;
-  t2[off(nu, mu, NP1 / 8)] = b;
-  t1[2 * tile + off(mu, nu, KP1 / 8)] = bl;
-  t2[2 * tile + off(nu, mu, NP1 / 8)] = bl;
+  if (v >= (long long)n_pop * t.H * t.D) return;
+  const int m = (int)(v / ((long long)t.H * t.D));
+  const int r = (int)(v % ((long long)t.H * t.D));
+  const int mu = r / t.D, nu = r % t.D;
+  float *tm = tab + (size_t)m * t.total;
+  float x = tm[mu * t.ndp + nu];
+  __nv_bfloat16 *tile = reinterpret_cast<__nv_bfloat16 *>(tm + t.tc) + tile_place(t, mu, nu);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const __nv_bfloat16 b = __float2bfloat16_rn(x);
+    tile[(size_t)k * t.np1 * t.kp1] = b;
+    x -= __bfloat162float(b);
+  }
 }
 
 // Eq. loss for `members` candidates (one block each, fixed-order sums): RMSE of the energy
@@ -1088,16 +1078,14 @@ __global__ void population_loss_kernel(int n_struct, const int *offsets, const d
 
 void launch_arm_rebuild(BuildStatus *st, cudaStream_t s) { arm_rebuild_kernel<<<1, 1, 0, s>>>(st); }
 
-void launch_unpack_population(int n_pop, const double *z, int n_par, int n_cr, int n_ca, float *cr, float *ca,
-                              float *ann, double *reg, cudaStream_t s) {
-  if (n_pop > 0) unpack_population_kernel<<<n_pop, 256, 0, s>>>(z, n_par, n_cr, n_ca, cr, ca, ann, reg);
+void launch_unpack_population(int n_pop, const double *z, int n_par, const TableLayout &t, float *tab, double *reg,
+                              cudaStream_t s) {
+  if (n_pop > 0) unpack_population_kernel<<<n_pop, 256, 0, s>>>(z, n_par, t, tab, reg);
 }
 
-void launch_population_tiles(int n_pop, const float *ann, int n_ann, int H, int D, int KP1, int NP1,
-                             unsigned short *tiles, cudaStream_t s) {
-  const long long n = (long long)n_pop * H * D;
-  if (n > 0)
-    population_tiles_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n_pop, ann, n_ann, H, D, KP1, NP1, tiles);
+void launch_population_tiles(int n_pop, float *tab, const TableLayout &t, cudaStream_t s) {
+  const long long n = (long long)n_pop * t.H * t.D;
+  if (n > 0 && t.np1) population_tiles_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n_pop, tab, t);
 }
 
 void launch_population_loss(int members, int n_struct, const int *offsets, const double *e_struct,

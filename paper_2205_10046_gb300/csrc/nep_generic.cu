@@ -57,10 +57,10 @@ __global__ void __launch_bounds__(128) generic_atom_kernel(const AtomArgs a, con
   const int NK = n_poly(L3, L4);
   const int off4 = (nR + 1) + (nA + 1) * L3, off5 = off4 + (L4 >= 2 ? nA + 1 : 0);
   const int mem = BATCH ? (int)blockIdx.y : 0;
-  const float *ann = (BATCH && a.pop_ann) ? a.pop_ann + mem * a.s_ann : a.ann;
+  const float *ann = a.tab + mem * a.s_tab;
   const float *w0 = ann, *b0 = ann + H * D, *w1 = b0 + H;
   const float b1 = w1[H];
-  const float *c_r = a.c_r + mem * a.s_cr, *c_a = a.c_a + mem * a.s_ca;
+  const float *c_r = a.c_r + mem * a.s_tab, *c_a = a.c_a + mem * a.s_tab;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double Ublock = 0.0;
   // (serving engine) atoms of a finished job frozen in the batch are skipped
@@ -331,8 +331,7 @@ __global__ void __launch_bounds__(128) generic_gather_kernel(const AtomArgs a) {
 }
 
 // ------------------------------------------------------------------------ launchers
-cudaError_t generic_atom(const AtomArgs &a, const ModelF &mf, const float *, const float *, const float *, float,
-                         int descriptor_only, cudaStream_t s) {
+cudaError_t generic_atom(const AtomArgs &a, const ModelF &mf, int descriptor_only, cudaStream_t s) {
   if (a.N <= 0) return cudaSuccess;
   const int blocks = (a.N + 127) / 128;
   if (descriptor_only) generic_atom_kernel<true, false><<<blocks, 128, 0, s>>>(a, mf);
@@ -347,8 +346,7 @@ cudaError_t generic_gather(const AtomArgs &a, cudaStream_t s) {
 }
 
 // batches: one block shape (128 atoms per CTA), population members along grid.y
-cudaError_t generic_atom_batch(const AtomArgs &a, const ModelF &mf, const float *, const float *, const float *,
-                               float, int members, int block, cudaStream_t s) {
+cudaError_t generic_atom_batch(const AtomArgs &a, const ModelF &mf, int members, int block, cudaStream_t s) {
   if (a.N <= 0 || members <= 0) return cudaSuccess;
   if (block != 128 || a.precision != 0) return cudaErrorInvalidValue;
   generic_atom_kernel<false, true><<<dim3((a.N + 127) / 128, members), 128, 0, s>>>(a, mf);

@@ -187,8 +187,11 @@ struct AtomArgs {
   const int *nn_a;         // [N]
   const int *rev_a;        // [cap_a][N] flat index of the reverse angular pair
   int cap_r, cap_a;        // list capacities (slots per atom), bounds of the list prefetches
-  const float *c_r;        // [T][T][nR+1][KR+1] FP32 copy
-  const float *c_a;        // [T][T][nA+1][KA+1]
+  // model table(s) in FP32 (TableLayout): network and descriptor coefficients, one per member
+  const float *tab;        // [members][s_tab]
+  long long s_tab;         // member stride in floats (0: one model)
+  const float *c_r;        // its c^R [T][T][nR+1][krp]
+  const float *c_a;        // its c^A [T][T][cap]
   float *e_rad;            // [N][T][est] radial force coefficients
   int est;
   float4 *p_ang;           // [cap_a][N] angular partial forces
@@ -206,18 +209,12 @@ struct AtomArgs {
   const double *inv_mass_kappa;  // [T] 1 / (m * 103.64...) for a = F * that
   const double *mass_kappa_half; // [T] m * 103.64... / 2 for kinetic energy
   double *vel;             // [N][3]
-  // tensor-core network (precision 1): W0 operand tiles in the UMMA layout, error flag
-  int precision;           // 0: FP32 network on the FMA pipes; 1: BF16 tensor-core network
-  const uint4 *tc_b1;      // GEMM1 operand W0 [NP1 x KP1] (bf16)
-  const uint4 *tc_b2;      // GEMM2 operand W0^T [NP2 x KP2] (bf16)
+  int precision;           // network: 0 FP32 on the FMA pipes; 1 BF16, 2 split BF16 on the tensor cores
   int *tc_err;             // set when a tensor-core wait ran out
   // Batched kernels only. dtab then holds ncode shift vectors per structure (the structure
   // index sits in pos4.w above the type bits), and blockIdx.y selects the member of a
   // population whose coefficients and network the block uses; every per-member array is
   // offset by member x its stride (in elements).
-  const float *pop_ann;    // [P][H*N_des + 2H + 1]: w0, b0, w1, b1 per member, or null
-  const uint4 *pop_tc;     // [P][2 tiles] BF16 operand tiles per member (precision 1), or null
-  long long s_cr, s_ca, s_ann, s_tc;  // strides of c_r, c_a, pop_ann, pop_tc
   long long s_erad, s_pang;           // strides of e_rad, p_ang
   long long s_out;                    // atoms per member in energy (x1), force (x3), virial (x9)
   const double *f_tar;     // [N][3] caller order, or null: sum of (F_i - F_tar,i)^2 per block
@@ -228,13 +225,9 @@ struct AtomArgs {
   double *heat;            // [N][3] caller order, or null
   // batched serving engine: per-structure kick (phase, time step, FIRE state), or null
   const EngineSlot *slots;
-  // model shape at run time and the FP32 network [w0 | b0 | w1 | b1] on the device: read only
-  // by the kernels that take the shape at run time (shapes without a compiled instantiation)
+  // model shape at run time: read only by the kernels that take the shape at run time (shapes
+  // without a compiled instantiation)
   int gR, gKR, gA, gKA, gH, gL3, gL4, gL5, gD;
-  const float *ann;
-  // FP32 per-atom kernel form: 1 the register-resident form, 3 the low-register form (three
-  // blocks per SM; shapes whose S_nk fit 128 TMEM columns)
-  int atom_occ;
 };
 
 // Model constants of one handle, FP32.
@@ -249,18 +242,17 @@ struct ShapeOps {
   int nR, KR, nA, KA, H, L3, L4, L5;
   int n_des;
   int kp1, np1;  // tensor-core network tile shapes (K of GEMM1, N of GEMM1)
-  cudaError_t (*atom)(const AtomArgs &, const ModelF &, const float *w0, const float *b0, const float *w1,
-                      float b1, int descriptor_only, cudaStream_t s);
+  int ndp, krp, cap;  // padded rows of the model table (TableLayout); 0: unpadded
+  cudaError_t (*atom)(const AtomArgs &, const ModelF &, int descriptor_only, cudaStream_t s);
   cudaError_t (*gather)(const AtomArgs &, cudaStream_t s);
   // batched kernels (per-structure shift tables; `members` population members along y;
   // `block` atoms per CTA: 64 or 128 for the atom kernel (128 with the tensor-core network),
   // 64, 128 or 256 for the gather kernel)
-  cudaError_t (*atom_batch)(const AtomArgs &, const ModelF &, const float *w0, const float *b0, const float *w1,
-                            float b1, int members, int block, cudaStream_t s);
+  cudaError_t (*atom_batch)(const AtomArgs &, const ModelF &, int members, int block, cudaStream_t s);
   cudaError_t (*gather_batch)(const AtomArgs &, int members, int block, cudaStream_t s);
   int (*atom_blocks)(int N);
   int (*gather_blocks)(int N);
-  int lowreg;  // the shape's S_nk fit 128 TMEM columns: the low-register FP32 form (3) exists
+  int lowreg;  // nep_tuning.atom_form 3 exists ((n_max^A + 1) x 24 <= 128)
 };
 
 int shape_count();
@@ -270,6 +262,43 @@ constexpr int kGenMaxN = 19;     // n_max^R, n_max^A, N_bas^R, N_bas^A
 constexpr int kGenMaxNeu = 256;  // N_neu
 constexpr int kGenMaxDes = (kGenMaxN + 1) * 7;
 const ShapeOps *shape_generic();
+
+// FP32 table of one model on the device: w0 [H][ndp], b0 [H], w1 [H], b1, c^R [T][T][n_R+1][krp],
+// c^A [T][T][cap] ([n][k] packed), and w0 as the BF16 operand tiles of the tensor-core network
+// (two terms hi + lo of every value, K-major core matrices of 8 rows x 16 bytes, zero padded
+// to [np1][kp1]); the parts at multiples of 4 floats. The compiled shapes pad
+// the rows to whole float4s, so that a block copies the table into shared memory as it stands.
+struct TableLayout {
+  int T, nR, KR, nA, KA, H, D;  // model shape
+  int ndp, krp, cap;
+  int np1, kp1;                 // W0 tile of the tensor-core network (0: none)
+  int cr, ca, tc, total;        // offsets of c^R, c^A and the two tiles, size (floats)
+};
+inline TableLayout table_layout(const ShapeOps *o, int T, int nR, int KR, int nA, int KA, int H, int D) {
+  TableLayout t{T, nR, KR, nA, KA, H, D, o->ndp ? o->ndp : D, o->krp ? o->krp : KR + 1,
+                o->cap ? o->cap : (nA + 1) * (KA + 1), o->np1, o->kp1, 0, 0, 0, 0};
+  auto r4 = [](int x) { return (x + 3) / 4 * 4; };
+  t.cr = r4(H * t.ndp + 2 * H + 1);
+  t.ca = t.cr + r4(T * T * (nR + 1) * t.krp);
+  t.tc = t.ca + r4(T * T * t.cap);
+  t.total = t.tc + t.np1 * t.kp1;  // two tiles of 2-byte values
+  return t;
+}
+// Place in the table of entry v of the parameter vector (order c^R, c^A, w0, b0, w1, b1).
+__host__ __device__ inline int table_place(const TableLayout &t, int v) {
+  const int ncr = t.T * t.T * (t.nR + 1) * (t.KR + 1);
+  if (v < ncr) return t.cr + v / (t.KR + 1) * t.krp + v % (t.KR + 1);
+  v -= ncr;
+  const int c = (t.nA + 1) * (t.KA + 1), nca = t.T * t.T * c;
+  if (v < nca) return t.ca + v / c * t.cap + v % c;
+  v -= nca;
+  return v < t.H * t.D ? v / t.D * t.ndp + v % t.D : t.H * t.ndp + (v - t.H * t.D);
+}
+
+// Element (mu, nu) of a W0 tile.
+__host__ __device__ inline int tile_place(const TableLayout &t, int mu, int nu) {
+  return ((mu / 8) * (t.kp1 / 8) + nu / 8) * 64 + (mu % 8) * 8 + (nu % 8);
+}
 
 // Host helpers shared by the handle-based and the static-scratch entry points.
 struct Grid;
@@ -304,10 +333,9 @@ void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src,
 void launch_thermostat(int N, const AtomState &a, int nb_gather, const double *partial_gather, ThermoState *ts,
                        cudaStream_t s);
 // population evaluation: parameter vectors into kernel arrays, BF16 tiles, Eq. loss
-void launch_unpack_population(int n_pop, const double *z, int n_par, int n_cr, int n_ca, float *cr, float *ca,
-                              float *ann, double *reg, cudaStream_t s);
-void launch_population_tiles(int n_pop, const float *ann, int n_ann, int H, int D, int KP1, int NP1,
-                             unsigned short *tiles, cudaStream_t s);
+void launch_unpack_population(int n_pop, const double *z, int n_par, const TableLayout &t, float *tab, double *reg,
+                              cudaStream_t s);
+void launch_population_tiles(int n_pop, float *tab, const TableLayout &t, cudaStream_t s);
 void launch_population_loss(int members, int n_struct, const int *offsets, const double *e_struct,
                             const double *w_struct, const double *e_tar, const double *w_tar,
                             const double *partial_gather, int nb_gather, int N, const double *reg, int n_par,

@@ -1,7 +1,7 @@
 // NEP3 per-atom kernels for GB300 (sm_103a), templated on the model shape.
 //
 // Two kernels replace the four of the paper's Appendix B:
-//   atom_kernel   one thread per atom: radial descriptor (Eq. qin), angular sums S_nk
+//   atom_kernel   two lanes per atom: radial descriptor (Eq. qin), angular sums S_nk
 //                 (Eq. S_nk) and the explicit 3/4/5-body components (Sec. II D), the
 //                 network U_i and dU_i/dq (Eq. Ui), then the per-type radial force
 //                 coefficients and the angular partial forces dU_i/dr_ij (the angular terms
@@ -16,13 +16,13 @@
 //     F^t_k = sum_{j of type t} f_k(r_ij), and contracts with c^{t_i t}_{nk} once per atom
 //     (the radial list is grouped by neighbour type), so a pair costs O(K) instead of
 //     O(n K); the radial partial forces likewise use e^t_k = sum_n dU/dq_n c^{t_i t}_{nk};
-//   * S_nk are evaluated from the homogeneous polynomials b_k(d) scaled by r^-l, and the
-//     angular gradient uses the tangential projection of grad b_k (no unit-vector round-off);
+//   * S_nk are evaluated from the polynomials b_k of the unit vector, factored into powers of
+//     (x + i y) and polynomials of z that the 24 of them share, and the angular gradient uses
+//     the tangential projection of grad b_k, folded factor by factor;
 //   * pair vectors come from cell-local FP32 coordinates plus an image shift table, so no
 //     FP64 arithmetic (slow on GB300) runs in the pair loops;
-//   * all S_nk of an atom are summed in one pass in registers and wait in the thread's TMEM
-//     lane while the network runs; dU/dS_nk stay in registers for the force loop (shapes
-//     that do not fit fall back to passes over chunks of n and a shared-memory block).
+//   * two lanes work on one atom and share a row of shared memory (S_nk, dU/dS_nk, q, dU/dq),
+//     so an atom's sums fit 128 registers a thread and every phase has work for both lanes.
 #pragma once
 #include <cuda_bf16.h>
 
@@ -41,58 +41,24 @@ struct Shape {
   static constexpr int OFF4 = (NR + 1) + (NA + 1) * L3;
   static constexpr int OFF5 = OFF4 + (L4 >= 2 ? NA + 1 : 0);
   static constexpr int NDP = (NDES + 3) / 4 * 4;  // padded w0 row in shared memory
-  // Shared-memory rows padded to whole float4s: c^A and c^R rows over k (KAP, KRP) and S_nk
-  // rows over k (NKP). Without TMEM each thread parks its S_nk in a block of SPT floats,
-  // n-major; SPT/4 is odd so the 16-byte accesses of 8 consecutive threads fall on 8 distinct
-  // bank groups.
-  static constexpr int KAP = (KA + 1 + 3) / 4 * 4;
+  // model table rows padded to whole float4s: c^A of a type pair (CAP), c^R rows over k (KRP)
+  static constexpr int CAP = ((NA + 1) * (KA + 1) + 3) / 4 * 4;  // c^A of one type pair, [n][k] packed
   static constexpr int KRP = (KR + 1 + 3) / 4 * 4;  // c^R rows over k, padded likewise
-  static constexpr int NKP = (NK + 3) / 4 * 4;
-  static constexpr int SPT = ((NA + 1) * NKP / 4) % 2 ? (NA + 1) * NKP : (NA + 1) * NKP + 4;
   // float offsets of the shared regions after the shift table, each a whole number of float4s
   static constexpr int r4(int x) { return (x + 3) / 4 * 4; }
+  // (the model table of TableLayout; without w0 where the network does not read it from there)
   static constexpr int off_b0(int prec) { return prec == 0 ? H * NDP : 0; }
-  static constexpr int off_cR(int prec) { return off_b0(prec) + r4(2 * H); }
+  static constexpr int off_cR(int prec) { return off_b0(prec) + r4(2 * H + 1); }
   static constexpr int off_cA(int prec, int T) { return off_cR(prec) + T * T * (NR + 1) * KRP; }
-  static constexpr int off_S(int prec, int T) { return off_cA(prec, T) + T * T * (NA + 1) * KAP; }
-  // S_nk is accumulated in NPASS passes over the angular neighbours, NCH values of n per
-  // pass, so that at most ~4 x 24 accumulators are live at once
-  static constexpr int NPASS = ((NA + 1) * NK > 144) ? ((NA + 1) + 3) / 4 : 1;
-  static constexpr int NCH = ((NA + 1) + NPASS - 1) / NPASS;
+  static constexpr int off_S(int prec, int T) { return off_cA(prec, T) + T * T * CAP; }
   // tensor-core network (BF16 operands, FP32 accumulation in TMEM), one 128-atom tile:
   //   GEMM1 z[128 x NP1] = q[128 x KP1] . W0[NP1 x KP1]^T,  GEMM2 dq[128 x NP2] = beta[128 x KP2] . W0^T
   static constexpr int KP1 = (NDES + 15) / 16 * 16;
   static constexpr int NP1 = (H + 15) / 16 * 16;
   static constexpr int KP2 = NP1, NP2 = KP1;
-  static constexpr int NS = (NA + 1) * NK;               // TMEM columns holding S_nk
-  static constexpr int DCOL = (NS + 15) / 16 * 16;       // TMEM column of the GEMM results
-  static constexpr int TMEM_COLS = 256;
-  static constexpr int TILE_A = kAtomBlock * (KP1 > KP2 ? KP1 : KP2) * 2;  // bytes
-  static constexpr int TILE_B = NP1 * KP1 * 2;                             // each of B1, B2
-  static_assert(DCOL + (NP1 > NP2 ? NP1 : NP2) <= TMEM_COLS, "S and the network results must fit 256 TMEM columns");
+  static constexpr int TILE_B = NP1 * KP1 * 2;           // bytes of a W0 tile
+  static constexpr int ACOL = NP1 > NP2 ? NP1 : NP2;     // TMEM columns of the GEMM results; A after them
   static_assert(NP1 <= 256 && NP2 <= 256, "UMMA N limit");
-  // Low-register form of the tensor-core network: S_nk waits in the thread's shared block
-  // (SPTC floats, later dU/dS_nk in place), the GEMM results take TMEM columns [0, ACOL) and
-  // the A operands (BF16 pairs, one lane per atom) columns [ACOL, ACOL + KP/2): 128 columns a
-  // block. With (SPTC/4) % 4 == 2 the rows are packed without padding and the float4 index is
-  // rotated by ((thread >> 2) & 1), which keeps 8 consecutive threads on 8 distinct bank groups.
-  // The split form keeps the A_lo operands after the A ones, at column ALO.
-  static constexpr int ACOL = NP1 > NP2 ? NP1 : NP2;
-  static constexpr int ALO = ACOL + (KP1 > KP2 ? KP1 : KP2) / 2;
-  static constexpr bool TCLR_OK = NS <= 128 && NK % 8 == 0 && ALO <= 128;
-  static constexpr bool TCLR2_OK = TCLR_OK && ALO + (KP1 > KP2 ? KP1 : KP2) / 2 <= 128;
-  static constexpr int SW = (NA + 1) * NKP / 4;  // float4s of one thread's S_nk block
-  static constexpr bool SROT = SW % 4 == 2;
-  static constexpr int SPTC = SROT ? 4 * SW : SPT;
-};
-
-template <class S>
-struct AnnConst {
-  float w0[S::H * S::NDES];
-  float b0[S::H];
-  float w1[S::H];
-  float b1;
-  ModelF m;
 };
 
 // l of polynomial k (blocks 0-2, 3-7, 8-14, 15-23)
@@ -162,6 +128,117 @@ __device__ __forceinline__ float3 poly_grad(float x, float y, float z, float s) 
   else return make_float3(4.f * y * (3.f * x * x - y * y), 4.f * x * (x * x - 3.f * y * y), 0.f);
 }
 
+// b_k of the unit vector (x, y, z) = d / r: b_k(d) r^-l of Sec. II D. Every b_k is a polynomial
+// Z(z) of degree l - m times Re or Im of (x + i y)^m, so a pair evaluates the few Z and the
+// powers once (about 45 operations for all 24, where each b_k(d) by itself and its r^-l took
+// about 100). UnitB holds the shared factors, ylm<k> combines them.
+struct UnitB {
+  float x, y, z, z2, z51, z71, z73, c2, s2, c3, s3;
+};
+
+__device__ __forceinline__ UnitB unit_b(float x, float y, float z) {
+  UnitB u;
+  u.x = x, u.y = y, u.z = z;
+  u.z2 = __fmul_rn(z, z);
+  u.z51 = __fmaf_rn(5.f, u.z2, -1.f);                  // 5 z^2 - 1
+  u.z71 = __fmaf_rn(7.f, u.z2, -1.f);                  // 7 z^2 - 1
+  u.z73 = __fmul_rn(__fmaf_rn(7.f, u.z2, -3.f), z);    // (7 z^2 - 3) z
+  u.c2 = __fmaf_rn(x, x, -__fmul_rn(y, y));            // Re, Im (x + i y)^2
+  u.s2 = __fmul_rn(__fadd_rn(x, x), y);
+  u.c3 = __fmaf_rn(x, u.c2, -__fmul_rn(y, u.s2));      // Re, Im (x + i y)^3
+  u.s3 = __fmaf_rn(x, u.s2, __fmul_rn(y, u.c2));
+  return u;
+}
+
+template <int k>
+__device__ __forceinline__ float ylm(const UnitB &u) {
+  if constexpr (k == 0) return u.z;
+  else if constexpr (k == 1) return u.x;
+  else if constexpr (k == 2) return u.y;
+  else if constexpr (k == 3) return __fmaf_rn(3.f, u.z2, -1.f);
+  else if constexpr (k == 4) return __fmul_rn(u.x, u.z);
+  else if constexpr (k == 5) return __fmul_rn(u.y, u.z);
+  else if constexpr (k == 6) return u.c2;
+  else if constexpr (k == 7) return u.s2;
+  else if constexpr (k == 8) return __fmul_rn(__fmaf_rn(5.f, u.z2, -3.f), u.z);
+  else if constexpr (k == 9) return __fmul_rn(u.z51, u.x);
+  else if constexpr (k == 10) return __fmul_rn(u.z51, u.y);
+  else if constexpr (k == 11) return __fmul_rn(u.c2, u.z);
+  else if constexpr (k == 12) return __fmul_rn(u.s2, u.z);
+  else if constexpr (k == 13) return u.c3;
+  else if constexpr (k == 14) return u.s3;
+  else if constexpr (k == 15) return __fmaf_rn(__fmaf_rn(35.f, u.z2, -30.f), u.z2, 3.f);
+  else if constexpr (k == 16) return __fmul_rn(u.z73, u.x);
+  else if constexpr (k == 17) return __fmul_rn(u.z73, u.y);
+  else if constexpr (k == 18) return __fmul_rn(u.z71, u.c2);
+  else if constexpr (k == 19) return __fmul_rn(u.z71, u.s2);
+  else if constexpr (k == 20) return __fmul_rn(u.c3, u.z);
+  else if constexpr (k == 21) return __fmul_rn(u.s3, u.z);
+  else if constexpr (k == 22) return __fmaf_rn(u.c2, u.c2, -__fmul_rn(u.s2, u.s2));
+  else return __fmul_rn(__fadd_rn(u.c2, u.c2), u.s2);
+}
+
+// Order in which the force loop takes the 24 polynomials, four at a time: the ones that share
+// Re or Im (x + i y)^m together. dU/dS_nk rows are kept in this order.
+__host__ __device__ constexpr int harm_k(int j) {
+  constexpr int o[24] = {0, 3, 8, 15, 1, 4, 9, 16, 2, 5, 10, 17, 6, 11, 18, 13, 7, 12, 19, 14, 20, 22, 21, 23};
+  return o[j];
+}
+
+// One group of four (harm_k(4 Q) ...) of one pair: with a_k = sum_n dU/dS_nk g_n and c_k =
+// sum_n dU/dS_nk g_n', adds sum_k a_k grad b_k (b_k as polynomials of the unit vector, |u|
+// held at 1: only the tangential part is used) to (gx, gy, gz) and sum_k c_k b_k to Y. The four
+// share their Re / Im factor, so their Z and Z' sums are formed first.
+template <int Q>
+__device__ __forceinline__ void harm_fold(const UnitB &u, const float *a, const float *c, float &gx, float &gy, float &gz,
+                                          float &Y) {
+  if constexpr (Q == 0) {  // m = 0
+    gz = __fadd_rn(gz, __fmaf_rn(a[3], __fmul_rn(__fmaf_rn(140.f, u.z2, -60.f), u.z),
+                                 __fmaf_rn(a[2], __fmaf_rn(15.f, u.z2, -3.f), __fmaf_rn(a[1], __fmul_rn(6.f, u.z), a[0]))));
+    Y = __fmaf_rn(c[0], u.z, Y);
+    Y = __fmaf_rn(c[1], __fmaf_rn(3.f, u.z2, -1.f), Y);
+    Y = __fmaf_rn(c[2], __fmul_rn(__fmaf_rn(5.f, u.z2, -3.f), u.z), Y);
+    Y = __fmaf_rn(c[3], __fmaf_rn(__fmaf_rn(35.f, u.z2, -30.f), u.z2, 3.f), Y);
+  } else if constexpr (Q == 1 || Q == 2) {  // m = 1: x, y
+    const float A = __fmaf_rn(a[3], u.z73, __fmaf_rn(a[2], u.z51, __fmaf_rn(a[1], u.z, a[0])));
+    const float C = __fmaf_rn(c[3], u.z73, __fmaf_rn(c[2], u.z51, __fmaf_rn(c[1], u.z, c[0])));
+    const float D = __fmaf_rn(a[3], __fmaf_rn(21.f, u.z2, -3.f), __fmaf_rn(a[2], __fmul_rn(10.f, u.z), a[1]));
+    const float w = Q == 1 ? u.x : u.y;
+    if constexpr (Q == 1) gx = __fadd_rn(gx, A);
+    else gy = __fadd_rn(gy, A);
+    gz = __fmaf_rn(D, w, gz);
+    Y = __fmaf_rn(C, w, Y);
+  } else if constexpr (Q == 3 || Q == 4) {  // m = 2 (three), and the first of m = 3
+    const float A = __fmaf_rn(a[2], u.z71, __fmaf_rn(a[1], u.z, a[0]));
+    const float C = __fmaf_rn(c[2], u.z71, __fmaf_rn(c[1], u.z, c[0]));
+    const float D = __fmaf_rn(a[2], __fmul_rn(14.f, u.z), a[1]);
+    const float A2 = __fadd_rn(A, A), A3 = __fmul_rn(3.f, a[3]);
+    if constexpr (Q == 3) {  // c2, c3: d/dx = 2x, 3 c2; d/dy = -2y, -3 s2
+      gx = __fmaf_rn(A3, u.c2, __fmaf_rn(A2, u.x, gx));
+      gy = __fmaf_rn(-A3, u.s2, __fmaf_rn(-A2, u.y, gy));
+      gz = __fmaf_rn(D, u.c2, gz);
+      Y = __fmaf_rn(c[3], u.c3, __fmaf_rn(C, u.c2, Y));
+    } else {  // s2, s3: d/dx = 2y, 3 s2; d/dy = 2x, 3 c2
+      gx = __fmaf_rn(A3, u.s2, __fmaf_rn(A2, u.y, gx));
+      gy = __fmaf_rn(A3, u.c2, __fmaf_rn(A2, u.x, gy));
+      gz = __fmaf_rn(D, u.s2, gz);
+      Y = __fmaf_rn(c[3], u.s3, __fmaf_rn(C, u.s2, Y));
+    }
+  } else {  // c3 z, c4, s3 z, s4
+    const float z3 = __fmul_rn(3.f, u.z);
+    const float A0 = __fmul_rn(a[0], z3), A1 = __fmul_rn(a[2], z3);
+    gx = __fmaf_rn(A1, u.s2, __fmaf_rn(A0, u.c2, gx));
+    gy = __fmaf_rn(A1, u.c2, __fmaf_rn(-A0, u.s2, gy));
+    gz = __fmaf_rn(a[2], u.s3, __fmaf_rn(a[0], u.c3, gz));
+    const float B0 = __fmul_rn(4.f, a[1]), B1 = __fmul_rn(4.f, a[3]);
+    gx = __fmaf_rn(B1, u.s3, __fmaf_rn(B0, u.c3, gx));
+    gy = __fmaf_rn(B1, u.c3, __fmaf_rn(-B0, u.s3, gy));
+    Y = __fmaf_rn(u.z, __fmaf_rn(c[2], u.s3, __fmul_rn(c[0], u.c3)), Y);
+    Y = __fmaf_rn(c[1], ylm<22>(u), Y);
+    Y = __fmaf_rn(c[3], ylm<23>(u), Y);
+  }
+}
+
 // Unrolled compile-time loop helper.
 template <int I, int N, class F>
 __device__ __forceinline__ void static_for(F &&f) {
@@ -195,13 +272,6 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16_bmn() {
   return umma_idesc_bf16<M, N>() | (1u << 16);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc));
-}
-
 __device__ __forceinline__ void umma_commit(uint64_t *mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(mbar))
                : "memory");
@@ -230,15 +300,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
   for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float *v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
-               "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-               "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-               "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
-               : "memory");
-}
-
-// The same MMA with the A operand read from tensor memory (lane m = row m, K packed along the
+// D (+)= A.B with the A operand read from tensor memory (lane m = row m, K packed along the
 // columns: two BF16 values per 32-bit column, the lower K index in the low half).
 __device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
                                              uint32_t acc) {
@@ -248,21 +310,10 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, u
       "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc));
 }
 
-__device__ __forceinline__ void tmem_st8u(uint32_t taddr, const uint32_t *v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
-               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+__device__ __forceinline__ void tmem_st4u(uint32_t taddr, const uint32_t *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
+               "r"(v[2]), "r"(v[3])
                : "memory");
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&b);
-}
-
-// Byte offset of element (row r, k) in a K-major no-swizzle operand tile with KC = K/8
-// 16-byte chunks per row group: core matrix (r/8, k/8) at ((r/8) KC + k/8) * 128.
-__host__ __device__ constexpr int umma_off(int r, int k, int KC) {
-  return ((r / 8) * KC + k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2;
 }
 
 // f_k(r) = (T_k(x) + 1) fc/2 with fc = (1 + cos(pi r/rc))/2 and x = 2(r/rc - 1)^2 - 1
@@ -319,31 +370,18 @@ __device__ __forceinline__ void cheb_basis_d(float r, float inv_rc, float *f, fl
   }
 }
 
-// Loop over the cnt list entries of atom i starting at slot `slot0` (slot-major lists),
-// software-pipelined: the list entry is fetched two iterations ahead and the neighbour's
-// position one iteration ahead, so the gathers overlap the arithmetic of earlier pairs.
-template <class Body>
-__device__ __forceinline__ void for_pairs(const unsigned *__restrict__ nl, int slot0, int cnt, int N, int i,
-                                          const float4 *__restrict__ pos4, unsigned jmask, Body &&body) {
-  if (cnt <= 0) return;
-  const unsigned *col = nl + (size_t)slot0 * N + i;
-  unsigned e0 = __ldg(col);
-  unsigned e1 = cnt > 1 ? __ldg(col + N) : 0u;
-  float4 p0 = __ldg(pos4 + (e0 & jmask));
-  for (int m = 0; m < cnt; ++m) {
-    const unsigned e = e0;
-    const float4 pj = p0;
-    if (m + 1 < cnt) p0 = __ldg(pos4 + (e1 & jmask));
-    e0 = e1;
-    if (m + 2 < cnt) e1 = __ldg(col + (size_t)(m + 2) * N);
-    body(m, e, pj);
-  }
-}
-
 // Request the line holding *p into L2 (no register, no wait). Callers keep p inside the
 // list allocation: slot rows below the list capacity.
 __device__ __forceinline__ void l2_prefetch(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
+// The block's copy of the model table into shared memory, from float `from` on (whole float4s).
+template <class S>
+__device__ __forceinline__ void stage_table(const float *tab, int from, int T, float *dst) {
+  const float4 *src = reinterpret_cast<const float4 *>(tab + from);
+  const int n4 = (S::off_S(0, T) - from) / 4;
+  for (int v = threadIdx.x; v < n4; v += blockDim.x) reinterpret_cast<float4 *>(dst)[v] = __ldg(src + v);
 }
 
 // Load of a list entry: read-only cached, or streaming (evict-first) for a list that the
@@ -393,204 +431,141 @@ __device__ __forceinline__ void for_pairs_batch(const unsigned *__restrict__ nl,
   }
 }
 
-// Plain loop over list entries (for pair bodies long enough to hide the gather themselves).
-template <class Body>
-__device__ __forceinline__ void for_pairs_plain(const unsigned *__restrict__ nl, int cnt, int N, int i,
-                                                const float4 *__restrict__ pos4, unsigned jmask, Body &&body) {
-  for (int m = 0; m < cnt; ++m) {
-    const unsigned e = __ldg(nl + (size_t)m * N + i);
-    body(m, e, __ldg(pos4 + (e & jmask)));
-  }
-}
-
 // ------------------------------------------------------------------------ per-atom kernel
-// OCC = 3 is the low-register form of the FP32 kernel: S_nk summed in two passes over the
-// angular neighbours, parked in 128 TMEM columns, and dU/dS_nk kept in the thread's shared
-// block instead of registers, so that three blocks (12 warps) fit an SM instead of two.
-template <class S, bool DESC_ONLY, int PREC, bool BATCH = false, int AB = kAtomBlock, int OCC = 1>
-__global__ void __launch_bounds__(AB, OCC)
-    atom_kernel(const AtomArgs a, const __grid_constant__ AnnConst<S> w) {
-  static_assert(PREC >= 0 && PREC <= 2, "network forms: 0 FP32, 1 BF16, 2 split BF16");
-  constexpr bool LOWREG = OCC > 1;
-  static_assert(!LOWREG || (!DESC_ONLY && AB == 128 && S::NS <= 128 && S::NK % 8 == 0),
-                "the low-register form: S_nk within 128 TMEM columns");
-  // TCLR: the low-register form with a tensor-core network. S_nk then waits in the thread's
-  // shared block (not in TMEM), whose 128 columns hold the GEMM operands and results.
-  constexpr bool TCLR = LOWREG && PREC >= 1;
-  static_assert(!TCLR || (PREC == 1 ? S::TCLR_OK : S::TCLR2_OK), "the tensor-core network within 128 TMEM columns");
-  constexpr uint32_t TCOLS = LOWREG ? 128u : (uint32_t)S::TMEM_COLS;
-  static_assert(PREC == 0 || !DESC_ONLY, "the descriptor-only kernel has no network");
-  static_assert(PREC == 0 || AB == 128, "the tensor-core network works on 128-atom tiles (UMMA M = 128)");
-  // S_nk waits for the network in this thread's TMEM lane (128-atom blocks, whole groups of 8
-  // columns), else in a per-thread block of shared memory
-  constexpr bool TM = !DESC_ONLY && AB == 128 && S::NK % 8 == 0;
-  static_assert(PREC == 0 || TM, "the tensor-core network works in TMEM");
-  constexpr bool STM = TM && !TCLR;  // S_nk parked in TMEM during the network
-  // With S_nk parked in TMEM the registers hold all (n_max^A + 1) x 24 sums at once: one pass
-  // over the angular neighbours (PbTe: 168 sums); otherwise NPASS passes of NCH values of n.
-  constexpr int NPASS = LOWREG ? ((S::NA + 1) >= 2 ? 2 : 1) : (TM && (S::NA + 1) * S::NK <= 192 ? 1 : S::NPASS);
-  constexpr int NCH = (S::NA + 1 + NPASS - 1) / NPASS;
-  static_assert(AB % 32 == 0 && AB <= 256, "whole warps, at most 256 atoms per block");
-  constexpr int NR = S::NR, KR = S::KR, NA = S::NA, KA = S::KA, NK = S::NK, NDES = S::NDES;
+// Two lanes per atom (h = 0, 1), AB atoms per block of 2 AB threads. The pair of lanes shares
+// one row of shared memory per atom: S_nk (later dU/dS_nk) and q (later dU/dq).
+//   radial sums      each lane takes every second neighbour of a type; the sums are added
+//                    across the pair, each lane contracts every second n with c_nk;
+//   S_nk             each lane prepares every second pair and hands it across; lane 0 sums the
+//                    polynomials with Re (x + i y)^m (and two of m = 0), lane 1 those with Im (and
+//                    the other two): the same instructions on swapped factors, 12 (n_max^A + 1)
+//                    sums a lane;
+//   components       each lane takes every second n; the row passes S_nk and q across;
+//   network          each lane holds every second float4 of q and dU/dq; see there;
+//   dU/dS_nk         every second n, in place of S_nk;
+//   partial forces   pairs 4 t + 2 h and 4 t + 2 h + 1: two pairs share every read of dU/dS_nk.
+//
+// What bounds it: instruction issue (70% of the slots busy with 16 warps per SM; FP32 arithmetic
+// is 72% of the instructions), then shared-memory bandwidth (59%). One thread per atom, with
+// all (n_max^A + 1) 24 sums in its registers or in two passes, ran 8 to 12 warps per SM and left
+// small systems to one long serial chain per atom. One thread / two lanes per atom, us: 216 Si
+// atoms 46 / 26, 13,824 Si atoms 41 / 28, 262,144 PbTe atoms 248 / 233, 8,000,000 Si atoms
+// 7787 / 7181, 4096 structures (1.05 million atoms) 1528 / 1173, 32 candidates on 256 structures
+// 3010 / 2318. Of that, reading the model table from global memory instead of copying it from
+// the kernel parameters (lane-varying constant addresses, served one by one) took 0.8 ms of the
+// 8,000,000-atom step, and the factored polynomials 0.6 ms.
+template <class S>
+struct PairRow {
+  static constexpr int Q4 = S::NDP / 4;                  // float4s of q
+  static constexpr int S4 = (S::NA + 1) * 6;             // float4s of S_nk
+  static constexpr int R4 = (Q4 + S4) | 1;               // odd: 8 consecutive rows on 8 bank groups
+  static constexpr int OCC = S::NA <= 4 ? 4 : 3;         // blocks of 128 threads per SM (shared memory)
+  // tensor-core network: BF16 terms per operand value, TMEM columns of the block
+  static constexpr int terms(int prec) { return prec; }
+  static constexpr int AC = (S::KP1 > S::KP2 ? S::KP1 : S::KP2) / 2;  // columns of one A term
+  static constexpr int cols(int) { return 128; }
+  static_assert(S::ACOL + 2 * AC <= 128, "results and both A terms within 128 TMEM columns");
+  static constexpr bool tc(int prec) { return prec > 0; }
+  // float offset of the rows in shared memory, after the table and the W0 tiles
+  static constexpr int from(int prec) { return tc(prec) ? S::off_b0(0) : 0; }
+  static constexpr int off_tiles(int prec, int T) { return S::off_S(0, T) - from(prec); }
+  static constexpr int off_rows(int prec, int T) {
+    return off_tiles(prec, T) + (tc(prec) ? terms(prec) * S::TILE_B / 4 : 0);
+  }
+};
+
+template <class S, int PREC, bool DESC, bool BATCH, int AB>
+__global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
+    atom_kernel(const AtomArgs a, const __grid_constant__ ModelF mf) {
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int NR = S::NR, KR = S::KR, NA = S::NA, KA = S::KA, NDES = S::NDES, NDP = S::NDP;
+  constexpr int CAP = S::CAP, KRP = S::KRP, NJ = (NA + 2) / 2;
+  static_assert(S::NK == 24, "harm_k lists the 24 polynomials of l <= 4");
   extern __shared__ float4 smem4[];
-  const int T = a.T;
-  const int N = a.N;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  // Threads past the last atom, and (serving engine) atoms of a finished job frozen in the
-  // batch, run the same code with no neighbours (the tensor-core steps are block- and
-  // warp-collective); they write nothing.
-  // This atom's position, list lengths and first list entries are requested before the
-  // block's setup (shared tables, TMEM), which hides their DRAM latency: the counts into
-  // registers, the first 16 radial and 2 angular slots into L2.
+  const int T = a.T, N = a.N;
+  const int h = threadIdx.x & 1, ia = threadIdx.x >> 1;
+  const int i = blockIdx.x * AB + ia;
+  // Lanes past the last atom, and (serving engine) those of a finished job frozen in the batch,
+  // run along with no neighbours (the pair exchanges are warp-collective); they write nothing.
   const float4 pi = i < N ? __ldg(a.pos4 + i) : make_float4(0.f, 0.f, 0.f, __int_as_float(0));
   const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(pi)].phase == 2);
   const int na = active ? __ldg(a.nn_a + i) : 0;
   int cnt_r = active ? __ldg(a.nn_r + i) : 0;
-  if (active) {
+  if (active) {  // the first list slots into L2 before the block's setup
 #pragma unroll
-    for (int m = 0; m < 16; ++m)
-      if (m < a.cap_r) l2_prefetch(a.nl_r + (size_t)m * N + i);
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-      if (m < a.cap_a) l2_prefetch(a.nl_a + (size_t)m * N + i);
+    for (int m = 0; m < 16; m += 2)
+      if (m + h < a.cap_r) l2_prefetch(a.nl_r + (size_t)(m + h) * N + i);
+    if (h < a.cap_a) l2_prefetch(a.nl_a + (size_t)h * N + i);
   }
-  constexpr int NDP = S::NDP;
-  // batches: the shift tables stay in global memory, one per structure, and blockIdx.y is
-  // the population member whose coefficients and network this block evaluates
   const int mem = BATCH ? (int)blockIdx.y : 0;
-  const float *pw = (BATCH && a.pop_ann) ? a.pop_ann + mem * a.s_ann : nullptr;
-  float4 *dtab_s = smem4;                                        // [ncode] (one structure)
-  constexpr int KAP = S::KAP, NKP = S::NKP, SPT = TCLR ? S::SPTC : S::SPT;
-  float *w0_s = reinterpret_cast<float *>(smem4 + (BATCH ? 0 : a.ncode));  // [H][NDP] (FP32 network)
-  float *b0_s = w0_s + S::off_b0(PREC);                          // [H]
-  float *w1_s = b0_s + S::H;                                     // [H]
-  float *cR_s = w0_s + S::off_cR(PREC);                          // [T][T][NR+1][KRP]
-  float *cA_s = w0_s + S::off_cA(PREC, T);                       // [T][T][NA+1][KAP]
-  // [block][SPT]: each thread's S_nk ([n][NKP]) while the network runs (without TMEM), or
-  // the BF16 operand tiles of the tensor-core network
-  float *S_s = w0_s + S::off_S(PREC, T);
+  using PR = PairRow<S>;
+  constexpr bool TC = PR::tc(PREC);
+  static_assert(!DESC || PREC == 0, "the descriptors need no network");
+  constexpr int NT = TC ? PR::terms(PREC) : 1;  // BF16 terms per operand value of the tensor-core network
+  // W0 tiles first (16-byte core matrices), then the shift table, the model table and the rows
+  float *tiles = reinterpret_cast<float *>(smem4);
+  float4 *dtab_s = smem4 + (TC ? NT * S::TILE_B / 16 : 0);  // [ncode] (one structure)
+  float *w0_s = reinterpret_cast<float *>(dtab_s + (BATCH ? 0 : a.ncode)) - PR::from(PREC);  // [H][NDP] (FMA network)
+  float *b0_s = w0_s + S::off_b0(0), *w1_s = b0_s + S::H;                  // [H]; [H], then b1
+  float *cR_s = w0_s + S::off_cR(0);      // [T][T][NR+1][KRP]
+  float *cA_s = w0_s + S::off_cA(0, T);   // [T][T][CAP]
+  float4 *const rows = reinterpret_cast<float4 *>(w0_s + S::off_S(0, T));
+  float4 *const row = rows + ia * PR::R4;  // [n][6], then q
+  float *const qrow = reinterpret_cast<float *>(row + PairRow<S>::S4);
   if constexpr (!BATCH)
     for (int v = threadIdx.x; v < a.ncode; v += blockDim.x) dtab_s[v] = a.dtab[v];
-  if constexpr (PREC == 0) {
-    for (int v = threadIdx.x; v < S::H * NDP; v += blockDim.x) {
-      const int mu = v / NDP, c = v - mu * NDP;
-      w0_s[v] = c < NDES ? (pw ? pw[mu * NDES + c] : w.w0[mu * NDES + c]) : 0.f;
-    }
-  }
-  for (int v = threadIdx.x; v < S::H; v += blockDim.x) {
-    b0_s[v] = pw ? pw[S::H * NDES + v] : w.b0[v];
-    w1_s[v] = pw ? pw[S::H * NDES + S::H + v] : w.w1[v];
-  }
-  __shared__ float b1_s;
-  if (threadIdx.x == 0) b1_s = pw ? pw[S::H * NDES + 2 * S::H] : w.b1;
-  const float *c_r = a.c_r + mem * a.s_cr, *c_a = a.c_a + mem * a.s_ca;
-  constexpr int KRP = S::KRP;
-  for (int v = threadIdx.x; v < T * T * (NR + 1) * KRP; v += blockDim.x) {
-    const int row = v / KRP, k = v - row * KRP;
-    cR_s[v] = k <= KR ? c_r[row * (KR + 1) + k] : 0.f;
-  }
-  for (int v = threadIdx.x; v < T * T * (NA + 1) * KAP; v += blockDim.x) {
-    const int row = v / KAP, k = v - row * KAP;
-    cA_s[v] = k <= KA ? c_a[row * (KA + 1) + k] : 0.f;
-  }
-  // tensor-core network: operand tiles (128-byte aligned) and TMEM for S_nk and the results
+  stage_table<S>(a.tab + mem * a.s_tab, PR::from(PREC), T, w0_s + PR::from(PREC));
   __shared__ __align__(8) uint64_t tc_mbar;
   __shared__ uint32_t tc_tmem;
-  // PREC 2 splits every operand value into two BF16 terms (hi + lo) and adds the products
-  // hi.hi + lo.hi + hi.lo: operand tiles A_lo, B1_lo, B2_lo follow the plain ones
-  constexpr bool SPLIT = PREC == 2;
-  unsigned char *tileA = nullptr, *tileB1 = nullptr, *tileB2 = nullptr;
-  unsigned char *tileAlo = nullptr, *tileB1lo = nullptr, *tileB2lo = nullptr;
-  if constexpr (PREC >= 1) {
-    // (TCLR: after the per-thread S_nk blocks, and no A tile: the A operands are in TMEM)
-    unsigned char *base = reinterpret_cast<unsigned char *>(S_s + (TCLR ? AB * SPT : 0));
-    base += (128u - (smem_addr(base) & 127u)) & 127u;
-    tileA = base;
-    tileB1 = tileA + (TCLR ? 0 : S::TILE_A);
-    tileB2 = tileB1 + S::TILE_B;
-    if constexpr (SPLIT) {
-      tileB1lo = tileB2 + S::TILE_B;
-      tileB2lo = tileB1lo + S::TILE_B;
-      tileAlo = tileB2lo + S::TILE_B;
-    }
-    if constexpr (TCLR) {  // one W0 tile (and its lo part) serves both GEMMs
-      tileB1lo = tileB1 + S::TILE_B;
-      tileB2 = tileB2lo = tileA = tileAlo = nullptr;
-    }
-    // W0 tiles in global memory: B1, B2, then (split form) B1_lo, B2_lo
-    const uint4 *b1t = a.tc_b1, *b2t = a.tc_b2;
-    if (BATCH && a.pop_tc) {
-      b1t = a.pop_tc + mem * a.s_tc;
-      b2t = b1t + S::TILE_B / 16;
-    }
-    for (int v = threadIdx.x; v < S::TILE_B / 16; v += blockDim.x) {
-      reinterpret_cast<uint4 *>(tileB1)[v] = b1t[v];
-      if constexpr (!TCLR) reinterpret_cast<uint4 *>(tileB2)[v] = b2t[v];
-      if constexpr (SPLIT) {
-        reinterpret_cast<uint4 *>(tileB1lo)[v] = b1t[v + 2 * (S::TILE_B / 16)];
-        if constexpr (!TCLR) reinterpret_cast<uint4 *>(tileB2lo)[v] = b2t[v + 2 * (S::TILE_B / 16)];
-      }
-    }
+  __shared__ float u_s[TC ? AB : 1];  // U of the rows
+  if constexpr (TC) {
+    const float4 *src = reinterpret_cast<const float4 *>(a.tab + mem * a.s_tab + S::off_S(0, T));
+    for (int v = threadIdx.x; v < NT * S::TILE_B / 16; v += blockDim.x) reinterpret_cast<float4 *>(tiles)[v] = __ldg(src + v);
     if (threadIdx.x == 0) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&tc_mbar)));
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-  }
-  if constexpr (TM) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tiles, before the MMAs read them
     if (threadIdx.x < 32) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tc_tmem)),
-                   "r"(TCOLS));
+                   "r"((uint32_t)PR::cols(PREC)));
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
-  uint32_t tmem_row = 0;  // TMEM address of this warp's 32 lanes, column 0
-  if constexpr (TM) {
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tmem_row = tc_tmem + ((uint32_t)((threadIdx.x >> 5) * 32) << 16);
-  }
-  // this thread's shared block of S_nk, later dU/dS_nk: float4 v of [n][NKP / 4]
-  float4 *const Sblk = reinterpret_cast<float4 *>(S_s + threadIdx.x * SPT);
-  const int srot = (TCLR && S::SROT) ? ((threadIdx.x >> 2) & 1) : 0;
-  auto sref = [&](int v) -> float4 & {
-    if constexpr (TCLR && S::SROT) return v == S::SW - 1 ? Sblk[srot ? 0 : S::SW - 1] : Sblk[v + srot];
-    else return Sblk[v];
+  const int ti = type_of(pi);
+  const float inv_rcR = 1.f / a.rcR, inv_rcA = 1.f / a.rcA;
+  const float rcR2 = a.rcR * a.rcR, rcA2 = a.rcA * a.rcA;
+  // shift vector of a list entry: from shared memory, or from the structure's own table
+  const float4 *dtab_b = BATCH ? a.dtab + (size_t)struct_of(pi) * a.ncode : dtab_s;
+  auto shift = [&](unsigned e) -> float4 {
+    if constexpr (BATCH) return __ldg(dtab_b + (e >> a.jbits));
+    else return dtab_s[e >> a.jbits];
   };
 
-  double Ublock = 0.0;
+  // ---- radial descriptor, Eq. qin: per neighbour type, sum_j T_k(x_j) fc_j/2 (k >= 1) and
+  // sum_j fc_j/2, then F_0 = 2H, F_k = sum_j T_k fc_j/2 + H, contracted with c_nk
   {
-    const int ti = type_of(pi);
-    const float inv_rcR = 1.f / a.rcR, inv_rcA = 1.f / a.rcA;
-    const float rcR2 = a.rcR * a.rcR, rcA2 = a.rcA * a.rcA;
-    // shift vector of a list entry: from shared memory, or from the structure's own table
-    const float4 *dtab_b = BATCH ? a.dtab + (size_t)struct_of(pi) * a.ncode : dtab_s;
-    auto shift = [&](unsigned e) -> float4 {
-      if constexpr (BATCH) return __ldg(dtab_b + (e >> a.jbits));
-      else return dtab_s[e >> a.jbits];
-    };
-
-    float q[NDES];
+    float qr[(NR + 2) / 2];
 #pragma unroll
-    for (int v = 0; v < NDES; ++v) q[v] = 0.f;
-
-    // ---- radial descriptor, Eq. qin: per neighbour type, F^t_k = sum_j f_k(r_ij). With
-    // f_k = (T_k(x) + 1) fc/2 the sums are kept as sum_j T_k(x_j) fc_j/2 (k >= 1) and
-    // H = sum_j fc_j/2, added once at the end: F_0 = 2H, F_k = sum_j T_k fc_j/2 + H.
+    for (int j = 0; j < (NR + 2) / 2; ++j) qr[j] = 0.f;
     int base = 0;
     for (int t = 0; t < T; ++t) {
       const int cnt = cnt_r;
-      if (t + 1 < T) {  // the next type's count, and its first 16 slots into L2
+      if (t + 1 < T) {  // the next type's count, and its first slots into L2
         cnt_r = active ? __ldg(a.nn_r + (size_t)(t + 1) * N + i) : 0;
         if (active)
 #pragma unroll
-          for (int m = 0; m < 16; ++m)
-            if (base + cnt + m < a.cap_r) l2_prefetch(a.nl_r + (size_t)(base + cnt + m) * N + i);
+          for (int m = 0; m < 16; m += 2)
+            if (base + cnt + m + h < a.cap_r) l2_prefetch(a.nl_r + (size_t)(base + cnt + m + h) * N + i);
       }
       float Fk[KR + 1];
 #pragma unroll
       for (int k = 0; k <= KR; ++k) Fk[k] = 0.f;
-      for_pairs_batch<8, true>(a.nl_r, base, cnt, N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
+      // entries h, h + 2, ... of the type's group
+      for_pairs_batch<4, true>(a.nl_r + (size_t)(base + h) * N, 0, (cnt + 1 - h) >> 1, 2 * N, i, a.pos4, a.jmask,
+                               [&](int, unsigned e, const float4 &pj) {
         const float3 d = pair_vector(pi, pj, shift(e));
         const float r2 = norm2(d);
         if (r2 < rcR2) {
@@ -612,622 +587,541 @@ __global__ void __launch_bounds__(AB, OCC)
         }
       });
 #pragma unroll
-      for (int k = 1; k <= KR; ++k) Fk[k] += Fk[0];
-      Fk[0] *= 2.f;
+      for (int k = 0; k <= KR; ++k) Fk[k] = __fadd_rn(Fk[k], __shfl_xor_sync(kAll, Fk[k], 1));
+#pragma unroll
+      for (int k = 1; k <= KR; ++k) Fk[k] = __fadd_rn(Fk[k], Fk[0]);
+      Fk[0] = __fadd_rn(Fk[0], Fk[0]);
       const float4 *c = reinterpret_cast<const float4 *>(cR_s + (ti * T + t) * (NR + 1) * KRP);
 #pragma unroll
-      for (int n = 0; n <= NR; ++n) {
-        float acc = q[n];
+      for (int j = 0; j < (NR + 2) / 2; ++j) {
+        const int n = min(2 * j + h, NR);
+        float acc = qr[j];
 #pragma unroll
         for (int k4 = 0; k4 < KRP / 4; ++k4) {
           const float4 cv = c[n * (KRP / 4) + k4];
           const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (4 * k4 + j <= KR) acc = __fmaf_rn(cw[j], Fk[4 * k4 + j], acc);
+          for (int jj = 0; jj < 4; ++jj)
+            if (4 * k4 + jj <= KR) acc = __fmaf_rn(cw[jj], Fk[4 * k4 + jj], acc);
         }
-        q[n] = acc;
+        qr[j] = acc;
       }
       base += cnt;
     }
+#pragma unroll
+    for (int j = 0; j < (NR + 2) / 2; ++j)
+      if (2 * j + h <= NR) qrow[2 * j + h] = qr[j];
+    if (h == 0)
+#pragma unroll
+      for (int v = NDES; v < NDP; ++v) qrow[v] = 0.f;
+  }
 
-    // ---- angular sums S_nk (Eq. S_nk, b_k(d) r^-l) and the angular descriptor components
-    // (Sec. II D): one pass over the angular neighbours, or one chunk of n per pass when the
-    // sums do not fit the registers (NPASS above)
-    if constexpr (LOWREG) {
-      // low-register form: two passes split over k, pass 0 the polynomials k < 16 (the 3-body
-      // blocks l = 1..3 and k = 15 of l = 4, the 4- and 5-body terms), pass 1 the rest; every
-      // pass sums all n, so each pair evaluates each b_k once
-      constexpr int KSPL = NK > 16 ? 16 : NK;
-      static_for<0, (NK > KSPL ? 2 : 1)>([&](auto pc) {
-        constexpr int k0 = decltype(pc)::value == 0 ? 0 : KSPL;
-        constexpr int k1 = decltype(pc)::value == 0 ? KSPL : NK;
-        constexpr int NKC = k1 - k0;
-        float Sv[NA + 1][NKC];
+  // ---- angular sums S_nk (Eq. S_nk, b_k of the unit vector): this lane's 12 polynomials
+  {
+    float Sv[NA + 1][12];
 #pragma unroll
-        for (int n = 0; n <= NA; ++n)
+    for (int n = 0; n <= NA; ++n)
 #pragma unroll
-          for (int k = 0; k < NKC; ++k) Sv[n][k] = 0.f;
-        for_pairs(a.nl_a, 0, na, N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
-          const float3 d = pair_vector(pi, pj, shift(e));
-          const float r2 = norm2(d);
-          if (r2 < rcA2) {
-            const int tj = type_of(pj);
-            const float rinv = rsqrtf(r2);
-            float f[KA + 1];
-            cheb_basis<KA>(r2 * rinv, inv_rcA, f);
-            const float4 *cc = reinterpret_cast<const float4 *>(cA_s + (ti * T + tj) * (NA + 1) * KAP);
-            float g[NA + 1];
+      for (int j = 0; j < 12; ++j) Sv[n][j] = 0.f;
+    // Lane h takes entries h, h + 2, ...: distance, basis and g_n of its own pair, which the other
+    // lane gets by shuffles (both lanes computing every pair took 40 instructions per atom and
+    // pair more); each lane then adds both pairs to its own sums. Entries are fetched two steps
+    // ahead, positions one.
+    const unsigned *col = a.nl_a + i;
+    unsigned e0 = h < na ? __ldg(col + (size_t)h * N) : 0u;
+    unsigned e1 = h + 2 < na ? __ldg(col + (size_t)(h + 2) * N) : 0u;
+    float4 p0 = __ldg(a.pos4 + (e0 & a.jmask));
+    const int steps = __reduce_max_sync(kAll, na);
+#pragma unroll 1
+    for (int m = h; m < steps + h; m += 2) {
+      const float3 d = pair_vector(pi, p0, shift(e0));
+      const int tj = type_of(p0);
+      const float r2 = norm2(d);
+      const bool in = m < na && r2 < rcA2;
+      e0 = e1;
+      if (m + 2 < na) p0 = __ldg(a.pos4 + (e0 & a.jmask));
+      e1 = m + 4 < na ? __ldg(col + (size_t)(m + 4) * N) : 0u;
+      float g[NA + 1], x = 0.f, y = 0.f, z = 0.f;
 #pragma unroll
-            for (int n = 0; n <= NA; ++n) {
-              float acc = 0.f;
+      for (int n = 0; n <= NA; ++n) g[n] = 0.f;
+      if (in) {
+        const float rinv = rsqrtf(r2);
+        float f[KA + 1];
+        cheb_basis<KA>(r2 * rinv, inv_rcA, f);
+        const float4 *c4 = reinterpret_cast<const float4 *>(cA_s + (ti * T + tj) * CAP);
 #pragma unroll
-              for (int k4 = 0; k4 < KAP / 4; ++k4) {
-                const float4 cv = cc[n * (KAP / 4) + k4];
-                const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
+        for (int v = 0; v < CAP / 4; ++v) {
+          const float4 cv = c4[v];
+          const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  if (4 * k4 + j <= KA) acc = __fmaf_rn(cw[j], f[4 * k4 + j], acc);
-              }
-              g[n] = acc;
+          for (int j = 0; j < 4; ++j)
+            if (4 * v + j < (NA + 1) * (KA + 1)) {
+              const int n = (4 * v + j) / (KA + 1), k = (4 * v + j) % (KA + 1);
+              g[n] = __fmaf_rn(cw[j], f[k], g[n]);
             }
-            const float rl[5] = {1.f, rinv, rinv * rinv, rinv * rinv * rinv, (rinv * rinv) * (rinv * rinv)};
-            static_for<k0, k1>([&](auto kc) {
-              constexpr int k = decltype(kc)::value;
-              const float b = poly_b<k>(d.x, d.y, d.z, r2) * rl[l_of_k(k)];
-#pragma unroll
-              for (int n = 0; n <= NA; ++n) Sv[n][k - k0] = __fmaf_rn(g[n], b, Sv[n][k - k0]);
-            });
-          }
-        });
-#pragma unroll
-        for (int n = 0; n <= NA; ++n) {
-          // 3-body components: the part of each l block inside [k0, k1)
-          static_for<0, S::L3>([&](auto lc) {
-            constexpr int l = decltype(lc)::value + 1;
-            constexpr int b0 = l == 1 ? 0 : l == 2 ? 3 : l == 3 ? 8 : 15;
-            constexpr int b1 = l == 1 ? 3 : l == 2 ? 8 : l == 3 ? 15 : 24;
-            constexpr int lo = b0 > k0 ? b0 : k0, hi = b1 < k1 ? b1 : k1;
-            if constexpr (lo < hi) {
-              float acc = q[(NR + 1) + (l - 1) * (NA + 1) + n];
-#pragma unroll
-              for (int k = lo; k < hi; ++k) acc = __fmaf_rn(w.m.c3b[k] * Sv[n][k - k0], Sv[n][k - k0], acc);
-              q[(NR + 1) + (l - 1) * (NA + 1) + n] = acc;
-            }
-          });
-          if constexpr (k0 == 0) {
-            if constexpr (S::L4 >= 2) {
-              const float s3 = Sv[n][3], s4 = Sv[n][4], s5 = Sv[n][5], s6 = Sv[n][6], s7 = Sv[n][7];
-              q[S::OFF4 + n] = w.m.c4b[0] * s3 * s3 * s3 + w.m.c4b[1] * s3 * (s4 * s4 + s5 * s5) +
-                               w.m.c4b[2] * s3 * (s6 * s6 + s7 * s7) + w.m.c4b[3] * s6 * (s5 * s5 - s4 * s4) +
-                               w.m.c4b[4] * s4 * s5 * s7;
-            }
-            if constexpr (S::L5 >= 1) {
-              const float s0 = Sv[n][0], s12 = Sv[n][1] * Sv[n][1] + Sv[n][2] * Sv[n][2];
-              q[S::OFF5 + n] = w.m.c5b[0] * s0 * s0 * s0 * s0 + w.m.c5b[1] * s0 * s0 * s12 + w.m.c5b[2] * s12 * s12;
-            }
-          }
-          if constexpr (TCLR) {
-            // park this part of S_n in the thread's shared block (TMEM serves the network)
-#pragma unroll
-            for (int k4 = 0; k4 < NKC / 4; ++k4)
-              sref(n * (NKP / 4) + k0 / 4 + k4) =
-                  make_float4(Sv[n][4 * k4], Sv[n][4 * k4 + 1], Sv[n][4 * k4 + 2], Sv[n][4 * k4 + 3]);
-          } else {
-            // park this part of S_n in TMEM, columns n NK + k0 .. n NK + k1 - 1
-            __syncwarp();
-#pragma unroll
-            for (int k8 = 0; k8 < NKC / 8; ++k8) tmem_st8(tmem_row + n * NK + k0 + 8 * k8, &Sv[n][8 * k8]);
-          }
         }
-      });
-    } else
-    static_for<0, NPASS>([&](auto pc) {
-      constexpr int n0 = decltype(pc)::value * NCH;
-      constexpr int n1 = (n0 + NCH < NA + 1) ? n0 + NCH : NA + 1;
-      constexpr int NC = n1 - n0;
-      float Sv[NC][NK];
-#pragma unroll
-      for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int k = 0; k < NK; ++k) Sv[c][k] = 0.f;
-      for_pairs(a.nl_a, 0, na, N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
-        const float3 d = pair_vector(pi, pj, shift(e));
-        const float r2 = norm2(d);
-        if (r2 < rcA2) {
-          const int tj = type_of(pj);
-          const float rinv = rsqrtf(r2);
-          float f[KA + 1];
-          cheb_basis<KA>(r2 * rinv, inv_rcA, f);
-          const float4 *cc = reinterpret_cast<const float4 *>(cA_s + ((ti * T + tj) * (NA + 1) + n0) * KAP);
-          float g[NC];
-#pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            float acc = 0.f;
-#pragma unroll
-            for (int k4 = 0; k4 < KAP / 4; ++k4) {
-              const float4 cv = cc[c * (KAP / 4) + k4];
-              const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (4 * k4 + j <= KA) acc = __fmaf_rn(cw[j], f[4 * k4 + j], acc);
-            }
-            g[c] = acc;
-          }
-          const float rl[5] = {1.f, rinv, rinv * rinv, rinv * rinv * rinv, (rinv * rinv) * (rinv * rinv)};
-          static_for<0, NK>([&](auto kc) {
-            constexpr int k = decltype(kc)::value;
-            const float b = poly_b<k>(d.x, d.y, d.z, r2) * rl[l_of_k(k)];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) Sv[c][k] = __fmaf_rn(g[c], b, Sv[c][k]);
-          });
-        }
-      });
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int n = n0 + c;
-        static_for<0, S::L3>([&](auto lc) {
-          constexpr int l = decltype(lc)::value + 1;
-          constexpr int k0 = l == 1 ? 0 : l == 2 ? 3 : l == 3 ? 8 : 15;
-          constexpr int k1 = l == 1 ? 3 : l == 2 ? 8 : l == 3 ? 15 : 24;
-          float acc = 0.f;
-#pragma unroll
-          for (int k = k0; k < k1; ++k) acc = __fmaf_rn(w.m.c3b[k] * Sv[c][k], Sv[c][k], acc);
-          q[(NR + 1) + (l - 1) * (NA + 1) + n] = acc;
-        });
-        if constexpr (S::L4 >= 2) {
-          const float s3 = Sv[c][3], s4 = Sv[c][4], s5 = Sv[c][5], s6 = Sv[c][6], s7 = Sv[c][7];
-          q[S::OFF4 + n] = w.m.c4b[0] * s3 * s3 * s3 + w.m.c4b[1] * s3 * (s4 * s4 + s5 * s5) +
-                           w.m.c4b[2] * s3 * (s6 * s6 + s7 * s7) + w.m.c4b[3] * s6 * (s5 * s5 - s4 * s4) +
-                           w.m.c4b[4] * s4 * s5 * s7;
-        }
-        if constexpr (S::L5 >= 1) {
-          const float s0 = Sv[c][0], s12 = Sv[c][1] * Sv[c][1] + Sv[c][2] * Sv[c][2];
-          q[S::OFF5 + n] = w.m.c5b[0] * s0 * s0 * s0 * s0 + w.m.c5b[1] * s0 * s0 * s12 + w.m.c5b[2] * s12 * s12;
-        }
-        if constexpr (!DESC_ONLY && !TM) {
-          // park S_n in this thread's shared block while the network runs
-          float4 *dst = reinterpret_cast<float4 *>(S_s + threadIdx.x * SPT + n * NKP);
-#pragma unroll
-          for (int k4 = 0; k4 < NKP / 4; ++k4) {
-            float v4[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v4[j] = 4 * k4 + j < NK ? Sv[c][4 * k4 + j] : 0.f;
-            dst[k4] = make_float4(v4[0], v4[1], v4[2], v4[3]);
-          }
-        }
-        if constexpr (TM) {
-          // park S_n in this thread's TMEM lane, columns n NK .. n NK + NK - 1
-          __syncwarp();
-#pragma unroll
-          for (int k8 = 0; k8 < NK / 8; ++k8) tmem_st8(tmem_row + n * NK + 8 * k8, &Sv[c][8 * k8]);
-        }
+        x = __fmul_rn(d.x, rinv), y = __fmul_rn(d.y, rinv), z = __fmul_rn(d.z, rinv);
       }
-    });
-
-    if constexpr (DESC_ONLY) {
-      if (active) {
-        const size_t io = a.perm ? (size_t)a.perm[i] : (size_t)i;
+      // a pair outside the cutoff is passed on with g = 0 (and a finite vector)
+      auto add_pair = [&](const UnitB &u, const float *gn) {
+        // lane 0: 0, 3 | 1, 4, 9, 16 | 6, 11, 18, 13 | 20, 22; lane 1: 8, 15 | 2, 5, 10, 17 |
+        // 7, 12, 19, 14 | 21, 23 (the order of harm_k, split in two)
+        const float w1 = h ? u.y : u.x, w2 = h ? u.s2 : u.c2, w3 = h ? u.s3 : u.c3;
+        const float bb[12] = {h ? ylm<8>(u) : u.z, h ? ylm<15>(u) : ylm<3>(u),
+                              w1, __fmul_rn(w1, u.z), __fmul_rn(w1, u.z51), __fmul_rn(w1, u.z73),
+                              w2, __fmul_rn(w2, u.z), __fmul_rn(w2, u.z71), w3,
+                              __fmul_rn(w3, u.z), h ? ylm<23>(u) : ylm<22>(u)};
 #pragma unroll
-        for (int v = 0; v < NDES; ++v) a.q_out[io * NDES + v] = (double)q[v];
-      }
-    } else {
-      if constexpr (TM) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-
-      // ---- network, Eq. Ui, and dU/dq
-      float U = 0.f;
-      float dq[NDES];
+        for (int j = 0; j < 12; ++j)
 #pragma unroll
-      for (int v = 0; v < NDES; ++v) dq[v] = 0.f;
-      if constexpr (PREC == 0) {
-        // FP32 on the FMA pipes, weights broadcast from shared memory
-  #pragma unroll 1
-        for (int mu = 0; mu < S::H; ++mu) {
-          const float4 *row = reinterpret_cast<const float4 *>(w0_s + mu * NDP);
-          float4 wrow[NDP / 4];  // the row serves both the forward and the backward sum
-          float zp[4] = {-b0_s[mu], 0.f, 0.f, 0.f};
-  #pragma unroll
-          for (int v4 = 0; v4 < NDP / 4; ++v4) {
-            const float4 wv = wrow[v4] = row[v4];
-            const float wc[4] = {wv.x, wv.y, wv.z, wv.w};
-  #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (4 * v4 + c < NDES) zp[c] = __fmaf_rn(wc[c], q[4 * v4 + c], zp[c]);
-          }
-          const float h = tanhf((zp[0] + zp[1]) + (zp[2] + zp[3]));
-          const float w1m = w1_s[mu];
-          U = __fmaf_rn(w1m, h, U);
-          const float beta = w1m * (1.f - h * h);
-  #pragma unroll
-          for (int v4 = 0; v4 < NDP / 4; ++v4) {
-            const float4 wv = wrow[v4];
-            const float wc[4] = {wv.x, wv.y, wv.z, wv.w};
-  #pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (4 * v4 + c < NDES) dq[4 * v4 + c] = __fmaf_rn(beta, wc[c], dq[4 * v4 + c]);
-          }
-        }
-      } else {
-        // BF16 tensor cores (tcgen05), FP32 accumulation in TMEM, one 128-atom tile per block.
-        // Every completion wait is bounded; if one runs out (all threads agree through the
-        // barrier), the block flags the error, waits once more (again bounded) so that the
-        // MMAs in flight finish before the TMEM is read or freed, and skips the rest of the
-        // network: its results are then invalid and the host reports NEP_ERR_TIMEOUT.
-        static_assert(NK % 8 == 0, "S_nk is moved in groups of 8 TMEM columns");
-        constexpr int KC1 = S::KP1 / 8, KC2 = S::KP2 / 8;
-        const int r = threadIdx.x;
-        // operand row of 8 values: BF16 (round to nearest even) and, split form, the BF16 of
-        // the remainder
-        auto put8 = [&](unsigned char *hi, unsigned char *lo, int off, const float *x) {
-          uint32_t ph[4], pl[4];
+          for (int n = 0; n <= NA; ++n) Sv[n][j] = __fmaf_rn(gn[n], bb[j], Sv[n][j]);
+      };
+      float go[NA + 1];
 #pragma unroll
-          for (int h2 = 0; h2 < 4; ++h2) {
-            const __nv_bfloat162 b = __floats2bfloat162_rn(x[2 * h2], x[2 * h2 + 1]);
-            ph[h2] = *reinterpret_cast<const uint32_t *>(&b);
-            if constexpr (SPLIT)
-              pl[h2] = pack_bf16x2(x[2 * h2] - __low2float(b), x[2 * h2 + 1] - __high2float(b));
-          }
-          *reinterpret_cast<uint4 *>(hi + off) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-          if constexpr (SPLIT) *reinterpret_cast<uint4 *>(lo + off) = make_uint4(pl[0], pl[1], pl[2], pl[3]);
-        };
-        // one GEMM over K steps of 16: D = A.B^T (+ A_lo.B^T + A.B_lo^T in the split form)
-        auto gemm = [&](const unsigned char *A, const unsigned char *Alo, const unsigned char *B,
-                        const unsigned char *Blo, int ksteps, int KC, uint32_t idesc) {
-          for (int st = 0; st < ksteps; ++st) {
-            const uint64_t da = umma_desc(smem_addr(A) + 256 * st, 128, KC * 128);
-            const uint64_t db = umma_desc(smem_addr(B) + 256 * st, 128, KC * 128);
-            umma_bf16(tc_tmem + S::DCOL, da, db, idesc, st > 0 ? 1u : 0u);
-            if constexpr (SPLIT) {
-              umma_bf16(tc_tmem + S::DCOL, umma_desc(smem_addr(Alo) + 256 * st, 128, KC * 128), db, idesc, 1u);
-              umma_bf16(tc_tmem + S::DCOL, da, umma_desc(smem_addr(Blo) + 256 * st, 128, KC * 128), idesc, 1u);
-            }
-          }
-          umma_commit(&tc_mbar);
-        };
-        // wait for the commit of phase `parity`; false (block-uniform) if the wait ran out
-        auto tc_wait = [&](uint32_t parity) -> bool {
-          const bool ok = mbar_wait(&tc_mbar, parity);
-          if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) atomicOr(a.tc_err, 1);
-            mbar_wait(&tc_mbar, parity);
-            return false;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          return true;
-        };
-        if constexpr (TCLR) {
-          // Low-register form: the A operands go to TMEM columns ACOL.. as BF16 pairs (one lane
-          // per atom, no shared-memory tile; split form: their lo parts at ALO..), the results
-          // to columns 0... GEMM2 reads the GEMM1 tile of W0 MN-major (B = W0).
-          constexpr uint32_t ACOL = S::ACOL, ALO = S::ALO;
-          // 16 values -> A (and A_lo) columns col .. col + 7
-          auto put16 = [&](uint32_t col, const float *x) {
-            uint32_t u[8], ul[8];
+      for (int n = 0; n <= NA; ++n) go[n] = __shfl_xor_sync(kAll, g[n], 1);
+      const UnitB uo = unit_b(__shfl_xor_sync(kAll, x, 1), __shfl_xor_sync(kAll, y, 1), __shfl_xor_sync(kAll, z, 1));
+      add_pair(unit_b(x, y, z), g);
+      add_pair(uo, go);
+    }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const __nv_bfloat162 bh = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-              u[j] = *reinterpret_cast<const uint32_t *>(&bh);
-              if constexpr (SPLIT)
-                ul[j] = pack_bf16x2(x[2 * j] - __low2float(bh), x[2 * j + 1] - __high2float(bh));
-            }
-            tmem_st8u(tmem_row + ACOL + col, u);
-            if constexpr (SPLIT) tmem_st8u(tmem_row + ALO + col, ul);
-          };
-          // operands written by every thread -> visible to the MMA issued by thread 0
-          auto to_mma = [&]() {
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          };
-          // D = A.B over K steps of 16 (+ A_lo.B + A.B_lo in the split form, in the order of
-          // the two-CTA form); B step st at byte offset st * bstep, descriptors (lbo, sbo)
-          auto gemm_t = [&](const unsigned char *B, const unsigned char *Blo, int ksteps, uint32_t bstep,
-                            uint32_t lbo, uint32_t sbo, uint32_t idesc) {
-            for (int st = 0; st < ksteps; ++st) {
-              const uint64_t db = umma_desc(smem_addr(B) + bstep * st, lbo, sbo);
-              umma_bf16_ts(tc_tmem, tc_tmem + ACOL + 8 * st, db, idesc, st > 0 ? 1u : 0u);
-              if constexpr (SPLIT) {
-                umma_bf16_ts(tc_tmem, tc_tmem + ALO + 8 * st, db, idesc, 1u);
-                umma_bf16_ts(tc_tmem, tc_tmem + ACOL + 8 * st, umma_desc(smem_addr(Blo) + bstep * st, lbo, sbo),
-                             idesc, 1u);
-              }
-            }
-            umma_commit(&tc_mbar);
-          };
-#pragma unroll
-          for (int c8 = 0; c8 < S::KP1 / 16; ++c8) {  // q row -> A
-            float x[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) x[j] = 16 * c8 + j < NDES ? q[16 * c8 + j] : 0.f;
-            put16(8 * c8, x);
-          }
-          to_mma();
-          if (threadIdx.x == 0)  // GEMM1: z = q . W0^T into columns 0 .. NP1 - 1
-            gemm_t(tileB1, tileB1lo, S::KP1 / 16, 256, 128, KC1 * 128, umma_idesc_bf16<kAtomBlock, S::NP1>());
-          __syncwarp();
-          if (tc_wait(0)) {
-            // tanh layer from this row of z; beta = w1 (1 - h^2) -> A (16 hidden units per store;
-            // the GEMM that read q has completed)
-#pragma unroll
-            for (int c16 = 0; c16 < S::NP1 / 16; ++c16) {
-              float z[16];
-              tmem_ld8(tmem_row + 16 * c16, z);
-              tmem_ld8(tmem_row + 16 * c16 + 8, z + 8);
-              float bt[16];
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                const int mu = 16 * c16 + j;
-                bt[j] = 0.f;
-                if (mu < S::H) {
-                  const float h = tanhf(z[j] - b0_s[mu]);
-                  U = __fmaf_rn(w1_s[mu], h, U);
-                  bt[j] = w1_s[mu] * (1.f - h * h);
-                }
-              }
-              put16(8 * c16, bt);
-            }
-            // every lane has read its z (tcgen05.ld waited) before GEMM2 overwrites the columns
-            to_mma();
-            // GEMM2: dq = beta . W0 into columns 0 .. NP2 - 1; B = W0 (K = hidden units, N =
-            // descriptor components) MN-major from the GEMM1 tile, 16 hidden units (two row
-            // groups of KC1 core matrices) per step
-            if (threadIdx.x == 0)
-              gemm_t(tileB1, tileB1lo, S::KP2 / 16, 2 * KC1 * 128, KC1 * 128, 128,
-                     umma_idesc_bf16_bmn<kAtomBlock, S::NP2>());
-            __syncwarp();
-            if (tc_wait(1)) {
-#pragma unroll
-              for (int c8 = 0; c8 < S::NP2 / 8; ++c8) {
-                float v[8];
-                tmem_ld8(tmem_row + 8 * c8, v);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                  if (8 * c8 + j < NDES) dq[8 * c8 + j] = v[j];
-              }
-            }
-          }
-        } else {
-          // q row -> operand tile A (bf16, K-major)
-#pragma unroll
-          for (int kc = 0; kc < KC1; ++kc) {
-            float x[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) x[j] = 8 * kc + j < NDES ? q[8 * kc + j] : 0.f;
-            put8(tileA, tileAlo, umma_off(r, 8 * kc, KC1), x);
-          }
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncthreads();
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          if (threadIdx.x == 0)  // GEMM1: z = q . W0^T into TMEM columns DCOL ..
-            gemm(tileA, tileAlo, tileB1, tileB1lo, S::KP1 / 16, KC1, umma_idesc_bf16<kAtomBlock, S::NP1>());
-          __syncwarp();
-          if (tc_wait(0)) {
-            // tanh layer from this row of z; beta = w1 (1 - h^2) -> operand tile A (reused)
-#pragma unroll
-            for (int c8 = 0; c8 < S::NP1 / 8; ++c8) {
-              float z[8];
-              tmem_ld8(tmem_row + S::DCOL + 8 * c8, z);
-              float bt[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const int mu = 8 * c8 + j;
-                bt[j] = 0.f;
-                if (mu < S::H) {
-                  const float h = tanhf(z[j] - b0_s[mu]);
-                  U = __fmaf_rn(w1_s[mu], h, U);
-                  bt[j] = w1_s[mu] * (1.f - h * h);
-                }
-              }
-              put8(tileA, tileAlo, umma_off(r, 8 * c8, KC2), bt);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (threadIdx.x == 0)  // GEMM2: dq = beta . W0 into the same TMEM columns
-              gemm(tileA, tileAlo, tileB2, tileB2lo, S::KP2 / 16, KC2, umma_idesc_bf16<kAtomBlock, S::NP2>());
-            __syncwarp();
-            if (tc_wait(1)) {
-#pragma unroll
-              for (int c8 = 0; c8 < S::NP2 / 8; ++c8) {
-                float v[8];
-                tmem_ld8(tmem_row + S::DCOL + 8 * c8, v);
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                  if (8 * c8 + j < NDES) dq[8 * c8 + j] = v[j];
-              }
-            }
-          }
-        }
-      }
-      if constexpr (BATCH) U -= b1_s;
-      else U -= w.b1;
-      if (active) {
-        if (a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = (double)U;
-        Ublock = (double)U;
-      }
-
-      // ---- radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_{nk} and their sum
-      for (int t = 0; t < T; ++t) {
-        const float4 *c = reinterpret_cast<const float4 *>(cR_s + (ti * T + t) * (NR + 1) * KRP);
-        float ev[S::EST > KRP ? S::EST : KRP];
-#pragma unroll
-        for (int k4 = 0; k4 < KRP / 4; ++k4) {
-          float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int n = 0; n <= NR; ++n) {
-            const float4 cv = c[n * (KRP / 4) + k4];
-            acc[0] = __fmaf_rn(dq[n], cv.x, acc[0]);
-            acc[1] = __fmaf_rn(dq[n], cv.y, acc[1]);
-            acc[2] = __fmaf_rn(dq[n], cv.z, acc[2]);
-            acc[3] = __fmaf_rn(dq[n], cv.w, acc[3]);
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) ev[4 * k4 + j] = acc[j];
-        }
-        float tot = 0.f;
-#pragma unroll
-        for (int k = 0; k <= KR; ++k) tot += ev[k];
-        ev[KR + 1] = tot;
-#pragma unroll
-        for (int k = KR + 2; k < S::EST; ++k) ev[k] = 0.f;
-        if (active) {
-          float4 *dst = reinterpret_cast<float4 *>(a.e_rad + mem * a.s_erad + ((size_t)i * T + t) * S::EST);
-#pragma unroll
-          for (int k4 = 0; k4 < S::EST / 4; ++k4)
-            dst[k4] = make_float4(ev[4 * k4], ev[4 * k4 + 1], ev[4 * k4 + 2], ev[4 * k4 + 3]);
-        }
-      }
-
-      // ---- dU/dS_nk from the explicit 3/4/5-body forms, kept in registers for the force loop
-      // (low-register form: in this thread's shared block, row n at n NKP)
-      float dSr[LOWREG ? 1 : NA + 1][NKP];
-#pragma unroll
-      for (int n = 0; n <= NA; ++n) {
-        float s[NKP];
-        float *dS = dSr[LOWREG ? 0 : n];
-        if constexpr (!STM) {
-#pragma unroll
-          for (int k4 = 0; k4 < NKP / 4; ++k4) {
-            const float4 v = sref(n * (NKP / 4) + k4);
-            s[4 * k4] = v.x, s[4 * k4 + 1] = v.y, s[4 * k4 + 2] = v.z, s[4 * k4 + 3] = v.w;
-          }
-        } else {
-          __syncwarp();
-#pragma unroll
-          for (int k8 = 0; k8 < NK / 8; ++k8) tmem_ld8(tmem_row + n * NK + 8 * k8, &s[8 * k8]);
-        }
-#pragma unroll
-        for (int k = 0; k < NKP; ++k) {
-          if (k < S::KEND3) {
-            const float d3 = dq[(NR + 1) + (l_of_k(k) - 1) * (NA + 1) + n];
-            dS[k] = 2.f * w.m.c3b[k] * s[k] * d3;
-          } else {
-            dS[k] = 0.f;
-          }
-        }
-        if constexpr (S::L4 >= 2) {
-          const float d4 = dq[S::OFF4 + n];
-          const float *C = w.m.c4b;
-          dS[3] += d4 * (3.f * C[0] * s[3] * s[3] + C[1] * (s[4] * s[4] + s[5] * s[5]) + C[2] * (s[6] * s[6] + s[7] * s[7]));
-          dS[4] += d4 * (2.f * C[1] * s[3] * s[4] - 2.f * C[3] * s[6] * s[4] + C[4] * s[5] * s[7]);
-          dS[5] += d4 * (2.f * C[1] * s[3] * s[5] + 2.f * C[3] * s[6] * s[5] + C[4] * s[4] * s[7]);
-          dS[6] += d4 * (2.f * C[2] * s[3] * s[6] + C[3] * (s[5] * s[5] - s[4] * s[4]));
-          dS[7] += d4 * (2.f * C[2] * s[3] * s[7] + C[4] * s[4] * s[5]);
-        }
-        if constexpr (S::L5 >= 1) {
-          const float d5 = dq[S::OFF5 + n];
-          const float *C = w.m.c5b;
-          const float s12 = s[1] * s[1] + s[2] * s[2];
-          dS[0] += d5 * (4.f * C[0] * s[0] * s[0] * s[0] + 2.f * C[1] * s[0] * s12);
-          const float common = 2.f * C[1] * s[0] * s[0] + 4.f * C[2] * s12;
-          dS[1] += d5 * common * s[1];
-          dS[2] += d5 * common * s[2];
-        }
-        if constexpr (LOWREG) {
-#pragma unroll
-          for (int k4 = 0; k4 < NKP / 4; ++k4)
-            sref(n * (NKP / 4) + k4) = make_float4(dS[4 * k4], dS[4 * k4 + 1], dS[4 * k4 + 2], dS[4 * k4 + 3]);
-        }
-      }
-
-      // ---- angular partial forces dU_i/dr_ij (angular terms of Eq. partial_force)
-      for_pairs(a.nl_a, 0, na, N, i, a.pos4, a.jmask, [&](int m, unsigned e, const float4 &pj) {
-        const float3 d = pair_vector(pi, pj, shift(e));
-        const float r2 = norm2(d);
-        if (r2 < rcA2) {
-          const int tj = type_of(pj);
-          const float rinv = rsqrtf(r2);
-          float f[KA + 1], fp[KA + 1];
-          cheb_basis_d<KA>(r2 * rinv, inv_rcA, f, fp);
-          const float4 *c = reinterpret_cast<const float4 *>(cA_s + (ti * T + tj) * (NA + 1) * KAP);
-          float g[NA + 1], gp[NA + 1];
-#pragma unroll
-          for (int n = 0; n <= NA; ++n) {
-            float acc = 0.f, accp = 0.f;
-#pragma unroll
-            for (int k4 = 0; k4 < KAP / 4; ++k4) {
-              const float4 cv = c[n * (KAP / 4) + k4];
-              const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (4 * k4 + j <= KA) {
-                  acc = __fmaf_rn(cw[j], f[4 * k4 + j], acc);
-                  accp = __fmaf_rn(cw[j], fp[4 * k4 + j], accp);
-                }
-            }
-            g[n] = acc;
-            gp[n] = accp;
-          }
-          // G = sum_k a_k r^-l grad b_k (tangential part used), Y = sum_k c_k r^-l b_k
-          const float rl[5] = {1.f, rinv, rinv * rinv, rinv * rinv * rinv, (rinv * rinv) * (rinv * rinv)};
-          float gx = 0.f, gy = 0.f, gz = 0.f, yy = 0.f;
-          static_for<0, NKP / 4>([&](auto kq) {
-            constexpr int k0 = 4 * decltype(kq)::value;
-            float ak[4] = {0.f, 0.f, 0.f, 0.f}, ck[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int n = 0; n <= NA; ++n) {
-              float dv[4];
-              if constexpr (LOWREG) {
-                const float4 v = sref(n * (NKP / 4) + k0 / 4);
-                dv[0] = v.x, dv[1] = v.y, dv[2] = v.z, dv[3] = v.w;
-              } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) dv[j] = k0 + j < NK ? dSr[n][k0 + j] : 0.f;
-              }
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (k0 + j < NK) {
-                  ak[j] = __fmaf_rn(dv[j], g[n], ak[j]);
-                  ck[j] = __fmaf_rn(dv[j], gp[n], ck[j]);
-                }
-            }
-            static_for<0, 4>([&](auto jc) {
-              constexpr int j = decltype(jc)::value, k = k0 + j;
-              if constexpr (k < NK) {
-                const float akr = ak[j] * rl[l_of_k(k)], ckr = ck[j] * rl[l_of_k(k)];
-                const float3 gb = poly_grad<k>(d.x, d.y, d.z, r2);
-                gx = __fmaf_rn(akr, gb.x, gx);
-                gy = __fmaf_rn(akr, gb.y, gy);
-                gz = __fmaf_rn(akr, gb.z, gz);
-                yy = __fmaf_rn(ckr, poly_b<k>(d.x, d.y, d.z, r2), yy);
-              }
-            });
-          });
-          const float ux = d.x * rinv, uy = d.y * rinv, uz = d.z * rinv;
-          const float gu = gx * ux + gy * uy + gz * uz;
-          const float px = (gx - gu * ux) + yy * ux;
-          const float py = (gy - gu * uy) + yy * uy;
-          const float pz = (gz - gu * uz) + yy * uz;
-          a.p_ang[mem * a.s_pang + (size_t)m * N + i] = make_float4(px, py, pz, 0.f);
-        }
-      });
+    for (int n = 0; n <= NA; ++n) {
+      float4 *r = row + n * 6;
+      reinterpret_cast<float2 *>(r)[h] = make_float2(Sv[n][0], Sv[n][1]);
+      r[1 + h] = make_float4(Sv[n][2], Sv[n][3], Sv[n][4], Sv[n][5]);
+      r[3 + h] = make_float4(Sv[n][6], Sv[n][7], Sv[n][8], Sv[n][9]);
+      reinterpret_cast<float2 *>(r + 5)[h] = make_float2(Sv[n][10], Sv[n][11]);
     }
   }
-  if constexpr (!DESC_ONLY) {
-    // deterministic block sum of U (fixed shuffle tree, then fixed warp order)
-    __shared__ double red[AB / 32];
-    double v = Ublock;
+  __syncwarp();
+  // S_n of one n from the row, by polynomial index
+  auto load_S = [&](int n, float *s) {
+    static_for<0, 6>([&](auto qc) {
+      constexpr int Q = decltype(qc)::value;
+      const float4 v = row[n * 6 + Q];
+      s[harm_k(4 * Q)] = v.x, s[harm_k(4 * Q + 1)] = v.y, s[harm_k(4 * Q + 2)] = v.z, s[harm_k(4 * Q + 3)] = v.w;
+    });
+  };
+
+  // ---- angular descriptor components (Sec. II D) of n = h, h + 2, ...
+#pragma unroll 1
+  for (int n = h; n <= NA; n += 2) {
+    float s[24];
+    load_S(n, s);
+    static_for<0, S::L3>([&](auto lc) {
+      constexpr int l = decltype(lc)::value + 1;
+      constexpr int k0 = l == 1 ? 0 : l == 2 ? 3 : l == 3 ? 8 : 15;
+      constexpr int k1 = l == 1 ? 3 : l == 2 ? 8 : l == 3 ? 15 : 24;
+      float acc = 0.f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      for (int k = k0; k < k1; ++k) acc = __fmaf_rn(__fmul_rn(mf.c3b[k], s[k]), s[k], acc);
+      qrow[(NR + 1) + (l - 1) * (NA + 1) + n] = acc;
+    });
+    if constexpr (S::L4 >= 2) {
+      const float s3 = s[3], s4 = s[4], s5 = s[5], s6 = s[6], s7 = s[7];
+      qrow[S::OFF4 + n] = mf.c4b[0] * s3 * s3 * s3 + mf.c4b[1] * s3 * (s4 * s4 + s5 * s5) +
+                          mf.c4b[2] * s3 * (s6 * s6 + s7 * s7) + mf.c4b[3] * s6 * (s5 * s5 - s4 * s4) +
+                          mf.c4b[4] * s4 * s5 * s7;
+    }
+    if constexpr (S::L5 >= 1) {
+      const float s0 = s[0], s12 = s[1] * s[1] + s[2] * s[2];
+      qrow[S::OFF5 + n] = mf.c5b[0] * s0 * s0 * s0 * s0 + mf.c5b[1] * s0 * s0 * s12 + mf.c5b[2] * s12 * s12;
+    }
+  }
+  __syncwarp();
+
+  if constexpr (DESC) {
+    if (active) {
+      double *out = a.q_out + (a.perm ? (size_t)a.perm[i] : (size_t)i) * NDES;
+      for (int v = h; v < NDES; v += 2) out[v] = (double)qrow[v];
+    }
+    return;
+  }
+
+  // ---- network, Eq. Ui, and dU/dq
+  float U = 0.f;
+  float dq[NR + 1];  // the radial part (the angular part is read from the row)
+  if constexpr (TC) {
+    // On the tensor cores (tcgen05, M = 128; the block's 64 atoms are rows 0 .. 63): GEMM1
+    // z = q . W0^T, GEMM2 dq = beta . W0, every operand value as NT BF16 terms (hi, or hi + lo
+    // with the products lo.hi + hi.lo + hi.hi in the same FP32 accumulator). A in TMEM (two K
+    // values per column), W0 in shared memory (one tile per term for both GEMMs: GEMM2 reads it
+    // MN-major). Every completion wait is bounded; if one runs out (all threads agree through
+    // the barrier), the block flags the error, waits once more (again bounded) so that the MMAs
+    // in flight finish before the TMEM is read or freed, and skips the rest of the network: its
+    // results are then invalid and the host reports NEP_ERR_TIMEOUT.
+    constexpr int KC1 = S::KP1 / 8, AC = PR::AC;
+    static_assert(AB == 64, "rows 0 .. 63 of the 128-row MMA: two warps of 32 TMEM lanes each");
+    const int warp = threadIdx.x >> 5;
+    const bool mine = warp < 2;  // these two warps hold one row (atom) per thread
+    const int r = mine ? threadIdx.x : 0;
+    const uint32_t tm = tc_tmem + ((uint32_t)(warp * 32) << 16);
+    float *const qr = reinterpret_cast<float *>(rows + r * PR::R4 + PR::S4);
+    // NT BF16 terms of 8 values -> 4 columns each at A column c4
+    auto put8 = [&](int c4, const float *x) {
+      uint32_t u[NT][4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        float x0 = x[2 * j], x1 = x[2 * j + 1];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          const __nv_bfloat162 bh = __floats2bfloat162_rn(x0, x1);
+          u[t][j] = *reinterpret_cast<const uint32_t *>(&bh);
+          x0 -= __low2float(bh);
+          x1 -= __high2float(bh);
+        }
+      }
+#pragma unroll
+      for (int t = 0; t < NT; ++t) tmem_st4u(tm + S::ACOL + t * AC + c4, u[t]);
+    };
+    // operands written by every thread -> visible to the MMA issued by thread 0
+    auto to_mma = [&]() {
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    };
+    auto gemm = [&](int ksteps, uint32_t bstep, uint32_t lbo, uint32_t sbo, uint32_t idesc) {
+      uint32_t acc = 0u;
+      auto terms = [&](int ta, int tb) {
+        for (int st = 0; st < ksteps; ++st) {
+          umma_bf16_ts(tc_tmem, tc_tmem + S::ACOL + ta * AC + 8 * st,
+                       umma_desc(smem_addr(tiles) + tb * S::TILE_B + bstep * st, lbo, sbo), idesc, acc);
+          acc = 1u;
+        }
+      };
+      if constexpr (NT >= 2) {
+        terms(1, 0);
+        terms(0, 1);
+      }
+      terms(0, 0);
+      umma_commit(&tc_mbar);
+    };
+    // wait for the commit of phase `parity`; false (block-uniform) if the wait ran out
+    auto tc_wait = [&](uint32_t parity) -> bool {
+      const bool ok = mbar_wait(&tc_mbar, parity);
+      if (__syncthreads_or(!ok)) {
+        if (threadIdx.x == 0) atomicOr(a.tc_err, 1);
+        mbar_wait(&tc_mbar, parity);
+        return false;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      return true;
+    };
+    __syncthreads();  // the rows of q are complete
+    if (mine) {
+#pragma unroll
+      for (int c8 = 0; c8 < S::KP1 / 8; ++c8) {  // q row -> A
+        float x[8];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const float4 v = 8 * c8 + 4 * j < NDP ? reinterpret_cast<const float4 *>(qr)[2 * c8 + j]
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+          x[4 * j] = v.x, x[4 * j + 1] = v.y, x[4 * j + 2] = v.z, x[4 * j + 3] = v.w;
+        }
+        put8(4 * c8, x);
+      }
+    }
+    to_mma();
+    if (threadIdx.x == 0)  // GEMM1: z = q . W0^T into columns 0 .. NP1 - 1
+      gemm(S::KP1 / 16, 256, 128, KC1 * 128, umma_idesc_bf16<128, S::NP1>());
+    __syncwarp();
+    if (tc_wait(0)) {
+      // tanh layer from this row of z; beta = w1 (1 - h^2) -> A (the GEMM that read q has completed)
+      if (mine) {
+        float us = 0.f;
+#pragma unroll
+        for (int c8 = 0; c8 < S::NP1 / 8; ++c8) {
+            float z[8], bt[8];
+          tmem_ld8(tm + 8 * c8, z);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int mu = 8 * c8 + j;
+            bt[j] = 0.f;
+            if (mu < S::H) {
+              const float t = tanhf(z[j] - b0_s[mu]);
+              us = __fmaf_rn(w1_s[mu], t, us);
+              bt[j] = w1_s[mu] * (1.f - t * t);
+            }
+          }
+          put8(4 * c8, bt);
+        }
+        u_s[r] = us;
+      }
+      // every lane has read its z (tcgen05.ld waited) before GEMM2 overwrites the columns
+      to_mma();
+      if (threadIdx.x == 0)  // GEMM2: dq = beta . W0 into columns 0 .. NP2 - 1 (W0 MN-major)
+        gemm(S::KP2 / 16, 2 * KC1 * 128, KC1 * 128, 128, umma_idesc_bf16_bmn<128, S::NP2>());
+      __syncwarp();
+      if (tc_wait(1) && mine) {
+#pragma unroll
+        for (int c8 = 0; c8 < (NDES + 7) / 8; ++c8) {
+            float v[8];
+          tmem_ld8(tm + 8 * c8, v);
+          reinterpret_cast<float4 *>(qr)[2 * c8] = make_float4(v[0], v[1], v[2], v[3]);
+          if (8 * c8 + 4 < NDP) reinterpret_cast<float4 *>(qr)[2 * c8 + 1] = make_float4(v[4], v[5], v[6], v[7]);
+        }
+      }
+    }
+    __syncthreads();
+    U = u_s[ia] - w1_s[S::H];
+#pragma unroll
+    for (int v = 0; v <= NR; ++v) dq[v] = qrow[v];
+  } else {
+    // On the FMA pipes: each lane holds every second float4 of q and of dU/dq; two neurons at a
+    // time, the lanes exchange their parts of z (lane h completes neuron mu + h), take one tanh
+    // each and exchange beta.
+    constexpr int V4 = NDP / 4, VJ = (V4 + 1) / 2;
+    float4 q[VJ], dv[VJ];
+#pragma unroll
+    for (int j = 0; j < VJ; ++j) {
+      q[j] = 2 * j + h < V4 ? reinterpret_cast<const float4 *>(qrow)[2 * j + h] : make_float4(0.f, 0.f, 0.f, 0.f);
+      dv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll 1
+    for (int mu = 0; mu < S::H; mu += 2) {
+      const bool two = S::H % 2 == 0 || mu + 1 < S::H;
+      const float4 *wr = reinterpret_cast<const float4 *>(w0_s + mu * NDP) + h;
+      float4 wa[VJ], wb[VJ];  // the rows serve both the forward and the backward sums
+      float za[2] = {0.f, 0.f}, zb[2] = {0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < VJ; ++j) {
+        const bool in = V4 % 2 == 0 || 2 * j + h < V4;
+        wa[j] = in ? wr[2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        wb[j] = in && two ? wr[V4 + 2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        za[0] = __fmaf_rn(wa[j].x, q[j].x, za[0]);
+        zb[0] = __fmaf_rn(wb[j].x, q[j].x, zb[0]);
+        za[1] = __fmaf_rn(wa[j].y, q[j].y, za[1]);
+        zb[1] = __fmaf_rn(wb[j].y, q[j].y, zb[1]);
+        za[0] = __fmaf_rn(wa[j].z, q[j].z, za[0]);
+        zb[0] = __fmaf_rn(wb[j].z, q[j].z, zb[0]);
+        za[1] = __fmaf_rn(wa[j].w, q[j].w, za[1]);
+        zb[1] = __fmaf_rn(wb[j].w, q[j].w, zb[1]);
+      }
+      const float pa = __fadd_rn(za[0], za[1]), pb = __fadd_rn(zb[0], zb[1]);
+      const float zo = __shfl_xor_sync(kAll, h ? pa : pb, 1);  // the other lane's part of this lane's neuron
+      const int my = two ? mu + h : mu;
+      const float w1m = h == 0 || two ? w1_s[my] : 0.f;
+      const float t = tanhf(__fadd_rn(h ? pb : pa, zo) - b0_s[my]);
+      U = __fmaf_rn(w1m, t, U);
+      const float beta = w1m * (1.f - t * t);
+      const float bo = __shfl_xor_sync(kAll, beta, 1);
+      const float ba = h ? bo : beta, bb = h ? beta : bo;
+#pragma unroll
+      for (int j = 0; j < VJ; ++j) {
+        dv[j].x = __fmaf_rn(bb, wb[j].x, __fmaf_rn(ba, wa[j].x, dv[j].x));
+        dv[j].y = __fmaf_rn(bb, wb[j].y, __fmaf_rn(ba, wa[j].y, dv[j].y));
+        dv[j].z = __fmaf_rn(bb, wb[j].z, __fmaf_rn(ba, wa[j].z, dv[j].z));
+        dv[j].w = __fmaf_rn(bb, wb[j].w, __fmaf_rn(ba, wa[j].w, dv[j].w));
+      }
+    }
+    U = __fadd_rn(U, __shfl_xor_sync(kAll, U, 1)) - w1_s[S::H];
+#pragma unroll
+    for (int j = 0; j < VJ; ++j)
+      if (2 * j + h < V4) reinterpret_cast<float4 *>(qrow)[2 * j + h] = dv[j];
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v <= NR; ++v) dq[v] = qrow[v];
+  }
+  if (active && h == 0 && a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = (double)U;
+
+  // ---- radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_{nk} and their sum: this lane's
+  // float4s of the row
+  for (int t = 0; t < T; ++t) {
+    const float4 *c = reinterpret_cast<const float4 *>(cR_s + (ti * T + t) * (NR + 1) * KRP);
+    constexpr int E4 = S::EST / 4, EJ = (E4 + 1) / 2;
+    float ev[EJ][4], tot = 0.f;
+#pragma unroll
+    for (int j = 0; j < EJ; ++j) {
+      const int k4 = 2 * j + h;
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      if (k4 < KRP / 4) {
+#pragma unroll
+        for (int n = 0; n <= NR; ++n) {
+          const float4 cv = c[n * (KRP / 4) + k4];
+          acc[0] = __fmaf_rn(dq[n], cv.x, acc[0]);
+          acc[1] = __fmaf_rn(dq[n], cv.y, acc[1]);
+          acc[2] = __fmaf_rn(dq[n], cv.z, acc[2]);
+          acc[3] = __fmaf_rn(dq[n], cv.w, acc[3]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        ev[j][k] = acc[k];
+        tot = __fadd_rn(tot, acc[k]);  // c^R rows are zero past KR
+      }
+    }
+    tot = __fadd_rn(tot, __shfl_xor_sync(kAll, tot, 1));
+    if (active) {
+      float4 *dst = reinterpret_cast<float4 *>(a.e_rad + mem * a.s_erad + ((size_t)i * T + t) * S::EST);
+#pragma unroll
+      for (int j = 0; j < EJ; ++j) {
+        const int k4 = 2 * j + h;
+        if (k4 >= E4) continue;
+        if (k4 == (KR + 1) / 4) ev[j][(KR + 1) % 4] = tot;
+        dst[k4] = make_float4(ev[j][0], ev[j][1], ev[j][2], ev[j][3]);
+      }
+    }
+  }
+  __syncwarp();
+
+  // ---- dU/dS_nk from the explicit 3/4/5-body forms, in place of S_nk: n = h, h + 2, ...
+#pragma unroll 1
+  for (int n = h; n <= NA; n += 2) {
+    float s[24], dS[24];
+    load_S(n, s);
+    static_for<0, 24>([&](auto kc) {
+      constexpr int k = decltype(kc)::value;
+      if constexpr (k < S::KEND3) dS[k] = 2.f * mf.c3b[k] * s[k] * qrow[(NR + 1) + (l_of_k(k) - 1) * (NA + 1) + n];
+      else dS[k] = 0.f;
+    });
+    if constexpr (S::L4 >= 2) {
+      const float d4 = qrow[S::OFF4 + n];
+      const float *C = mf.c4b;
+      dS[3] += d4 * (3.f * C[0] * s[3] * s[3] + C[1] * (s[4] * s[4] + s[5] * s[5]) + C[2] * (s[6] * s[6] + s[7] * s[7]));
+      dS[4] += d4 * (2.f * C[1] * s[3] * s[4] - 2.f * C[3] * s[6] * s[4] + C[4] * s[5] * s[7]);
+      dS[5] += d4 * (2.f * C[1] * s[3] * s[5] + 2.f * C[3] * s[6] * s[5] + C[4] * s[4] * s[7]);
+      dS[6] += d4 * (2.f * C[2] * s[3] * s[6] + C[3] * (s[5] * s[5] - s[4] * s[4]));
+      dS[7] += d4 * (2.f * C[2] * s[3] * s[7] + C[4] * s[4] * s[5]);
+    }
+    if constexpr (S::L5 >= 1) {
+      const float d5 = qrow[S::OFF5 + n];
+      const float *C = mf.c5b;
+      const float s12 = s[1] * s[1] + s[2] * s[2];
+      dS[0] += d5 * (4.f * C[0] * s[0] * s[0] * s[0] + 2.f * C[1] * s[0] * s12);
+      const float common = 2.f * C[1] * s[0] * s[0] + 4.f * C[2] * s12;
+      dS[1] += d5 * common * s[1];
+      dS[2] += d5 * common * s[2];
+    }
+    static_for<0, 6>([&](auto qc) {
+      constexpr int Q = decltype(qc)::value;
+      row[n * 6 + Q] = make_float4(dS[harm_k(4 * Q)], dS[harm_k(4 * Q + 1)], dS[harm_k(4 * Q + 2)], dS[harm_k(4 * Q + 3)]);
+    });
+  }
+  __syncwarp();
+
+  // ---- angular partial forces dU_i/dr_ij (angular terms of Eq. partial_force): with
+  // a_k = sum_n dU/dS_nk g_n and c_k = sum_n dU/dS_nk g_n',
+  //   dU_i/dr_ij = (G - (G.u) u) / r + Y u,  G = sum_k a_k grad b_k(u),  Y = sum_k c_k b_k(u)
+  if (2 * h < na) {
+    constexpr int PP = 2;
+    const unsigned *col = a.nl_a + i;
+    unsigned ec[PP], en[PP];
+    float4 pc[PP];
+#pragma unroll
+    for (int p = 0; p < PP; ++p) {
+      const int m = 2 * h + p;
+      ec[p] = m < na ? __ldg(col + (size_t)m * N) : 0u;
+      en[p] = m + 4 < na ? __ldg(col + (size_t)(m + 4) * N) : 0u;
+    }
+#pragma unroll
+    for (int p = 0; p < PP; ++p) pc[p] = __ldg(a.pos4 + (ec[p] & a.jmask));
+#pragma unroll 1
+    for (int m0 = 2 * h; m0 < na; m0 += 4) {
+      float3 d[PP];
+      float r2[PP];
+      bool in[PP], any = false;
+      int tj[PP];
+#pragma unroll
+      for (int p = 0; p < PP; ++p) {
+        d[p] = pair_vector(pi, pc[p], shift(ec[p]));
+        tj[p] = type_of(pc[p]);
+        r2[p] = norm2(d[p]);
+        in[p] = m0 + p < na && r2[p] < rcA2;
+        any = any || in[p];
+        ec[p] = en[p];
+        if (m0 + 4 < na) pc[p] = __ldg(a.pos4 + (en[p] & a.jmask));
+        en[p] = m0 + 8 + p < na ? __ldg(col + (size_t)(m0 + 8 + p) * N) : 0u;
+      }
+      if (!any) continue;
+      float rinv[PP], g[PP][NA + 1], gp[PP][NA + 1];
+      float gx[PP], gy[PP], gz[PP], Y[PP];
+      UnitB u[PP];
+#pragma unroll
+      for (int p = 0; p < PP; ++p) {
+        rinv[p] = rsqrtf(r2[p]);
+        float f[KA + 1], fp[KA + 1];
+        cheb_basis_d<KA>(r2[p] * rinv[p], inv_rcA, f, fp);
+        const float4 *c4 = reinterpret_cast<const float4 *>(cA_s + (ti * T + tj[p]) * CAP);
+#pragma unroll
+        for (int n = 0; n <= NA; ++n) g[p][n] = gp[p][n] = 0.f;
+#pragma unroll
+        for (int v = 0; v < CAP / 4; ++v) {
+          const float4 cv = c4[v];
+          const float cw[4] = {cv.x, cv.y, cv.z, cv.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (4 * v + j < (NA + 1) * (KA + 1)) {
+              const int n = (4 * v + j) / (KA + 1), k = (4 * v + j) % (KA + 1);
+              g[p][n] = __fmaf_rn(cw[j], f[k], g[p][n]);
+              gp[p][n] = __fmaf_rn(cw[j], fp[k], gp[p][n]);
+            }
+        }
+        u[p] = unit_b(__fmul_rn(d[p].x, rinv[p]), __fmul_rn(d[p].y, rinv[p]), __fmul_rn(d[p].z, rinv[p]));
+        gx[p] = gy[p] = gz[p] = Y[p] = 0.f;
+      }
+      static_for<0, 6>([&](auto qc) {
+        constexpr int Q = decltype(qc)::value;
+        float ak[PP][4], ck[PP][4];
+#pragma unroll
+        for (int n = 0; n <= NA; ++n) {
+          const float4 v = row[n * 6 + Q];
+          const float dv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int p = 0; p < PP; ++p)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              ak[p][j] = n == 0 ? __fmul_rn(dv[j], g[p][n]) : __fmaf_rn(dv[j], g[p][n], ak[p][j]);
+              ck[p][j] = n == 0 ? __fmul_rn(dv[j], gp[p][n]) : __fmaf_rn(dv[j], gp[p][n], ck[p][j]);
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < PP; ++p) harm_fold<Q>(u[p], ak[p], ck[p], gx[p], gy[p], gz[p], Y[p]);
+      });
+#pragma unroll
+      for (int p = 0; p < PP; ++p) {
+        const float gu = __fmaf_rn(gz[p], u[p].z, __fmaf_rn(gy[p], u[p].y, __fmul_rn(gx[p], u[p].x)));
+        const float t = __fmaf_rn(-gu, rinv[p], Y[p]);  // P = G / r + (Y - (G.u) / r) u
+        if (in[p])
+          a.p_ang[mem * a.s_pang + (size_t)(m0 + p) * N + i] =
+              make_float4(__fmaf_rn(gx[p], rinv[p], __fmul_rn(t, u[p].x)), __fmaf_rn(gy[p], rinv[p], __fmul_rn(t, u[p].y)),
+                          __fmaf_rn(gz[p], rinv[p], __fmul_rn(t, u[p].z)), 0.f);
+      }
+    }
+  }
+  if constexpr (!BATCH) {
+    // deterministic block sum of U (fixed shuffle tree, then fixed warp order); a batch sums its
+    // structures from the per-atom energies
+    __shared__ double red[2 * AB / 32];
+    double v = active && h == 0 ? (double)U : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kAll, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     if (threadIdx.x == 0) {
       double s = 0.0;
-      for (int wv = 0; wv < AB / 32; ++wv) s += red[wv];
-      a.partial_atom[(size_t)mem * gridDim.x + blockIdx.x] = s;
+      for (int wv = 0; wv < 2 * AB / 32; ++wv) s += red[wv];
+      if (AB == 64) {
+        a.partial_atom[blockIdx.x] = s;
+      } else {  // one slot per 64 atoms (atom_blocks)
+        a.partial_atom[2 * (size_t)blockIdx.x] = s;
+        a.partial_atom[2 * (size_t)blockIdx.x + 1] = 0.0;
+      }
     }
   }
-  if constexpr (TM) {
+  if constexpr (TC) {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (threadIdx.x < 32) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc_tmem), "r"(TCOLS));
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc_tmem), "r"((uint32_t)PR::cols(PREC)));
     }
   }
+}
+
+template <class S>
+size_t atom_pair_smem(int T, int ncode, int prec, int ab) {
+  return sizeof(float4) * ncode + sizeof(float) * (size_t)PairRow<S>::off_rows(prec, T) +
+         sizeof(float4) * PairRow<S>::R4 * ab;
 }
 
 // Epilogue of the gather kernels for atom i: outputs in the caller's order, the squared force
@@ -1474,94 +1368,26 @@ __global__ void __launch_bounds__(GB, BATCH ? 1 : (S::KR <= 8 ? 1024 : 896) / GB
 }
 
 // ------------------------------------------------------------------------ launchers
-template <class S>
-size_t atom_smem_bytes(int T, int ncode, int prec, int ab = kAtomBlock, bool tclr = false) {
-  // the last region: BF16 operand tiles (tensor-core network; tclr: the per-thread S_nk blocks
-  // and the B tiles), nothing (S_nk in TMEM) or the per-thread S_nk blocks
-  const bool tm = ab == 128 && S::NK % 8 == 0;
-  const size_t last = tclr        ? sizeof(float) * (size_t)S::SPTC * ab + 128 + (prec == 2 ? 2 : 1) * (size_t)S::TILE_B
-                      : prec == 1 ? (size_t)S::TILE_A + 2 * S::TILE_B + 128
-                      : prec == 2 ? 2 * (size_t)S::TILE_A + 4 * S::TILE_B + 128
-                      : tm        ? 0
-                                  : sizeof(float) * S::SPT * ab;
-  return sizeof(float4) * ncode + sizeof(float) * (size_t)S::off_S(prec, T) + last;
-}
+// block sums of U of one structure: one slot per 64 atoms, an even number of them
+template <class S> int atom_blocks(int N) { return 2 * ((N + 127) / 128); }
 
-// A block that holds TMEM takes 256 of the SM's 512 columns; a third such block on one SM
-// would wait in tcgen05.alloc until one of the others ends. When the registers alone would
-// admit three blocks, ask for more than a third of the SM's 228 KB of shared memory.
-constexpr size_t kTmemBlockSmem = 80 * 1024;
-template <class K>
-size_t tmem_block_smem(K kern, int block, size_t smem) {
-  static std::mutex mu;
-  static std::unordered_map<const void *, int> regs;  // registers per thread of each kernel
-  int nr = 0;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    const void *key = reinterpret_cast<const void *>(kern);
-    auto it = regs.find(key);
-    if (it != regs.end()) {
-      nr = it->second;
-    } else {
-      cudaFuncAttributes fa;
-      if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return smem < kTmemBlockSmem ? kTmemBlockSmem : smem;
-      nr = regs[key] = fa.numRegs;
-    }
-  }
-  const int regs_warp = (nr * 32 + 255) / 256 * 256;
-  const int by_regs = 65536 / (regs_warp * ((block + 31) / 32));
-  return by_regs > 2 && smem < kTmemBlockSmem ? kTmemBlockSmem : smem;
+template <class S, int PREC, bool DESC, bool BATCH, int AB>
+cudaError_t launch_atom_as(const AtomArgs &a, const ModelF &mf, int members, cudaStream_t st) {
+  auto kern = atom_kernel<S, PREC, DESC, BATCH, AB>;
+  const cudaError_t e = smem_limit_once(kern, atom_pair_smem<S>(kMaxTypes, BATCH ? 0 : 1 << 9, PREC, AB));
+  if (e != cudaSuccess) return e;
+  const int blocks = (!BATCH && AB == 64) ? atom_blocks<S>(a.N) : (a.N + AB - 1) / AB;
+  kern<<<dim3(blocks, members), 2 * AB, atom_pair_smem<S>(a.T, BATCH ? 0 : a.ncode, PREC, AB), st>>>(a, mf);
+  return cudaGetLastError();
 }
 
 template <class S>
-cudaError_t launch_atom(const AtomArgs &a, const ModelF &mf, const float *w0, const float *b0, const float *w1,
-                        float b1, int descriptor_only, cudaStream_t st) {
+cudaError_t launch_atom(const AtomArgs &a, const ModelF &mf, int descriptor_only, cudaStream_t st) {
   if (a.N <= 0) return cudaSuccess;
-  AnnConst<S> w;  // host staging; copied into the launch by value
-  for (int v = 0; v < S::H * S::NDES; ++v) w.w0[v] = w0[v];
-  for (int v = 0; v < S::H; ++v) {
-    w.b0[v] = b0[v];
-    w.w1[v] = w1[v];
-  }
-  w.b1 = b1;
-  w.m = mf;
-  const int blocks = (a.N + kAtomBlock - 1) / kAtomBlock;
-  const bool tm = !descriptor_only && kAtomBlock == 128 && S::NK % 8 == 0;
-  size_t smem = atom_smem_bytes<S>(a.T, a.ncode, descriptor_only ? 0 : a.precision);
-  size_t bound = atom_smem_bytes<S>(kMaxTypes, 1 << 9, descriptor_only ? 0 : a.precision);
-  if (tm && bound < kTmemBlockSmem) bound = kTmemBlockSmem;
-  auto go = [&](auto kern) -> cudaError_t {
-    cudaError_t e = smem_limit_once(kern, bound);
-    if (e != cudaSuccess) return e;
-    if (tm) smem = tmem_block_smem(kern, kAtomBlock, smem);
-    kern<<<blocks, kAtomBlock, smem, st>>>(a, w);
-    return cudaGetLastError();
-  };
-  if (descriptor_only) return go(atom_kernel<S, true, 0>);
-  // low-register form of the tensor-core networks (BF16, split BF16)
-  auto go_tclr = [&](auto kern, int prec) -> cudaError_t {
-    cudaError_t e = smem_limit_once(kern, atom_smem_bytes<S>(kMaxTypes, 1 << 9, prec, 128, true));
-    if (e != cudaSuccess) return e;
-    kern<<<blocks, kAtomBlock, atom_smem_bytes<S>(a.T, a.ncode, prec, 128, true), st>>>(a, w);
-    return cudaGetLastError();
-  };
-  if constexpr (S::TCLR_OK)
-    if (a.precision == 1 && a.atom_occ == 3) return go_tclr(atom_kernel<S, false, 1, false, 128, 3>, 1);
-  if constexpr (S::TCLR2_OK)
-    if (a.precision == 2 && a.atom_occ == 3) return go_tclr(atom_kernel<S, false, 2, false, 128, 3>, 2);
-  if (a.precision == 1) return go(atom_kernel<S, false, 1>);
-  if (a.precision == 2) return go(atom_kernel<S, false, 2>);
-  if constexpr (S::NS <= 128 && S::NK % 8 == 0) {
-    if (a.atom_occ == 3) {  // low-register form: the per-thread dU/dS_nk blocks, no TMEM-driven cap
-      auto kern = atom_kernel<S, false, 0, false, 128, 3>;
-      const size_t extra = sizeof(float) * (size_t)S::SPT * kAtomBlock;
-      cudaError_t e = smem_limit_once(kern, atom_smem_bytes<S>(kMaxTypes, 1 << 9, 0) + extra);
-      if (e != cudaSuccess) return e;
-      kern<<<blocks, kAtomBlock, atom_smem_bytes<S>(a.T, a.ncode, 0) + extra, st>>>(a, w);
-      return cudaGetLastError();
-    }
-  }
-  return go(atom_kernel<S, false, 0>);
+  if (descriptor_only) return launch_atom_as<S, 0, true, false, 64>(a, mf, 1, st);
+  if (a.precision == 1) return launch_atom_as<S, 1, false, false, 64>(a, mf, 1, st);
+  if (a.precision == 2) return launch_atom_as<S, 2, false, false, 64>(a, mf, 1, st);
+  return launch_atom_as<S, 0, false, false, 64>(a, mf, 1, st);
 }
 
 template <class S>
@@ -1574,63 +1400,20 @@ cudaError_t launch_gather(const AtomArgs &a, cudaStream_t st) {
 
 // Batched launches (grid.y = population members); instantiated in the nep_batch_*.cu units.
 template <class S>
-cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, const float *w0, const float *b0,
-                              const float *w1, float b1, int members, int block, cudaStream_t st);
+cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, int members, int block, cudaStream_t st);
 template <class S>
 cudaError_t launch_gather_batch(const AtomArgs &a, int members, int block, cudaStream_t st);
 
 #ifdef NEP_BATCH_KERNELS
 template <class S>
-cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, const float *w0, const float *b0,
-                              const float *w1, float b1, int members, int block, cudaStream_t st) {
+cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, int members, int block, cudaStream_t st) {
   if (a.N <= 0 || members <= 0) return cudaSuccess;
   if (block != 64 && block != 128) return cudaErrorInvalidValue;
   if (a.precision >= 1 && block != 128) return cudaErrorInvalidValue;
-  AnnConst<S> w;
-  for (int v = 0; v < S::H * S::NDES; ++v) w.w0[v] = w0 ? w0[v] : 0.f;
-  for (int v = 0; v < S::H; ++v) {
-    w.b0[v] = b0 ? b0[v] : 0.f;
-    w.w1[v] = w1 ? w1[v] : 0.f;
-  }
-  w.b1 = b1;
-  w.m = mf;
-  const dim3 grid((a.N + block - 1) / block, members);
-  const bool tm = block == 128 && S::NK % 8 == 0;
-  size_t smem = atom_smem_bytes<S>(a.T, 0, a.precision, block);
-  size_t bound = atom_smem_bytes<S>(kMaxTypes, 0, a.precision, block);
-  if (tm && bound < kTmemBlockSmem) bound = kTmemBlockSmem;
-  auto go = [&](auto kern) -> cudaError_t {
-    cudaError_t e = smem_limit_once(kern, bound);
-    if (e != cudaSuccess) return e;
-    if (tm) smem = tmem_block_smem(kern, block, smem);
-    kern<<<grid, block, smem, st>>>(a, w);
-    return cudaGetLastError();
-  };
-  // the low-register tensor-core forms
-  auto go_tclr = [&](auto kern, int prec) -> cudaError_t {
-    cudaError_t e = smem_limit_once(kern, atom_smem_bytes<S>(kMaxTypes, 0, prec, 128, true));
-    if (e != cudaSuccess) return e;
-    kern<<<grid, 128, atom_smem_bytes<S>(a.T, 0, prec, 128, true), st>>>(a, w);
-    return cudaGetLastError();
-  };
-  if constexpr (S::TCLR_OK)
-    if (a.precision == 1 && a.atom_occ == 3) return go_tclr(atom_kernel<S, false, 1, true, 128, 3>, 1);
-  if constexpr (S::TCLR2_OK)
-    if (a.precision == 2 && a.atom_occ == 3) return go_tclr(atom_kernel<S, false, 2, true, 128, 3>, 2);
-  if (a.precision == 1) return go(atom_kernel<S, false, 1, true, 128>);
-  if (a.precision == 2) return go(atom_kernel<S, false, 2, true, 128>);
-  if (block == 64) return go(atom_kernel<S, false, 0, true, 64>);
-  if constexpr (S::NS <= 128 && S::NK % 8 == 0) {
-    if (a.atom_occ == 3) {  // the low-register form, as in the single-structure launch
-      auto kern = atom_kernel<S, false, 0, true, 128, 3>;
-      const size_t extra = sizeof(float) * (size_t)S::SPT * 128;
-      cudaError_t e = smem_limit_once(kern, atom_smem_bytes<S>(kMaxTypes, 0, 0, 128) + extra);
-      if (e != cudaSuccess) return e;
-      kern<<<grid, 128, atom_smem_bytes<S>(a.T, 0, 0, 128) + extra, st>>>(a, w);
-      return cudaGetLastError();
-    }
-  }
-  return go(atom_kernel<S, false, 0, true, 128>);
+  if (a.precision == 1) return launch_atom_as<S, 1, false, true, 64>(a, mf, members, st);
+  if (a.precision == 2) return launch_atom_as<S, 2, false, true, 64>(a, mf, members, st);
+  return block == 64 ? launch_atom_as<S, 0, false, true, 64>(a, mf, members, st)
+                     : launch_atom_as<S, 0, false, true, 128>(a, mf, members, st);
 }
 
 template <class S>
@@ -1654,7 +1437,6 @@ template <class S>
 void attach_batch(ShapeOps &o);  // explicitly instantiated in the batch translation unit
 #endif
 
-template <class S> int atom_blocks(int N) { return (N + kAtomBlock - 1) / kAtomBlock; }
 template <class S> int gather_blocks(int N) { return (N + kGatherBlock - 1) / kGatherBlock; }
 
 template <class S>
@@ -1663,11 +1445,12 @@ ShapeOps make_ops() {
   o.nR = S::NR; o.KR = S::KR; o.nA = S::NA; o.KA = S::KA; o.H = S::H;
   o.L3 = S::L3; o.L4 = S::L4; o.L5 = S::L5; o.n_des = S::NDES;
   o.kp1 = S::KP1; o.np1 = S::NP1;
+  o.ndp = S::NDP; o.krp = S::KRP; o.cap = S::CAP;
   o.atom = &launch_atom<S>;
   o.gather = &launch_gather<S>;
   o.atom_blocks = &atom_blocks<S>;
   o.gather_blocks = &gather_blocks<S>;
-  o.lowreg = (S::NS <= 128 && S::NK % 8 == 0) ? 1 : 0;
+  o.lowreg = (S::NA + 1) * S::NK <= 128 ? 1 : 0;
   attach_batch<S>(o);
   return o;
 }

@@ -19,7 +19,8 @@
 namespace nep {
 int check_params(const nep_params *p, const ShapeOps **ops_out, const char **err);
 int n_des_of(const nep_params *p);
-void set_shape_args(AtomArgs &a, const nep_params &p, const float *ann);
+void set_shape_args(AtomArgs &a, const nep_params &p);
+void fill_table(const TableLayout &t, const nep_params &p, float *out);
 void set_create_error(const char *msg);  // read back by nep_last_error(NULL)
 }
 
@@ -125,20 +126,15 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
             KA = params->basis_angular, H = params->n_neuron, D = n_des_of(params);
   const double skin = params->skin > 0 ? params->skin : 1.0;
 
-  // host-side model tables (fixed-size, on the stack)
-  constexpr int kMaxW = 8192, kMaxC = 8192;
+  // host-side model table (fixed-size, on the stack)
+  constexpr int kMaxW = 8192, kMaxC = 8192, kMaxTab = 32768;
   static_assert(kMaxC >= kMaxTypes * kMaxTypes * 121, "radial table bound");
-  float w0[kMaxW], b0[512], w1[512], cR[kMaxC], cA[kMaxC];
   const int ncR = T * T * (nR + 1) * (KR + 1), ncA = T * T * (nA + 1) * (KA + 1);
-  if (H * D > kMaxW || H > 512 || ncR > kMaxC || ncA > kMaxC)
+  const TableLayout tl = table_layout(ops, T, nR, KR, nA, KA, H, D);
+  if (H * D > kMaxW || H > 512 || ncR > kMaxC || ncA > kMaxC || tl.total > kMaxTab)
     return fail_static(NEP_ERR_UNSUPPORTED, "model too large for the static entry point");
-  for (int v = 0; v < H * D; ++v) w0[v] = (float)params->w0[v];
-  for (int v = 0; v < H; ++v) {
-    b0[v] = (float)params->b0[v];
-    w1[v] = (float)params->w1[v];
-  }
-  for (int v = 0; v < ncR; ++v) cR[v] = (float)params->c_radial[v];
-  for (int v = 0; v < ncA; ++v) cA[v] = (float)params->c_angular[v];
+  float tab[kMaxTab];
+  fill_table(tl, *params, tab);
   ModelF mf;
   model_constants(mf);
 
@@ -155,7 +151,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   Bump arena{base, kStaticBytes};
   BuildStatus *st = arena.take<BuildStatus>(1);
   float4 *dtab = arena.take<float4>(g.ncode);
-  float *dcR = arena.take<float>(ncR), *dcA = arena.take<float>(ncA);
+  float *dtabm = arena.take<float>(tl.total);
   AtomState a;
   a.x = arena.take<double>(3 * (size_t)N);
   a.v = arena.take<double>(3 * (size_t)N);
@@ -182,7 +178,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.nn_r = arena.take<int>((size_t)T * N);
   L.nn_a = arena.take<int>(N);
   L.part = arena.take<unsigned long long>(4 * kStatSlots);
-  if (!st || !dtab || !dcR || !dcA || !a.x || !a.v || !a.F || !a.x_ref || !a.origin || !a.x2 || !a.v2 || !a.F2 ||
+  if (!st || !dtab || !dtabm || !a.x || !a.v || !a.F || !a.x_ref || !a.origin || !a.x2 || !a.v2 || !a.F2 ||
       !a.types || !a.perm || !a.cell_of || !a.types2 || !a.perm2 || !a.cell2 || !a.pos4 || !a.posA || !L.cell_count ||
       !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part)
     return fail_static(NEP_ERR_ARG, "structure too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
@@ -190,8 +186,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   // inputs into the arena; the arena keeps the previous call's contents, so everything the
   // kernels read is written here first (the builder clears the cell counters itself)
   SK(cudaMemcpyAsync(dtab, dtab_h, sizeof(float4) * g.ncode, cudaMemcpyHostToDevice, s), "copy");
-  SK(cudaMemcpyAsync(dcR, cR, sizeof(float) * ncR, cudaMemcpyHostToDevice, s), "copy");
-  SK(cudaMemcpyAsync(dcA, cA, sizeof(float) * ncA, cudaMemcpyHostToDevice, s), "copy");
+  SK(cudaMemcpyAsync(dtabm, tab, sizeof(float) * tl.total, cudaMemcpyHostToDevice, s), "copy");
   SK(cudaMemcpyAsync(a.x, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
   SK(cudaMemcpyAsync(a.types, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
   SK(cudaMemsetAsync(a.v, 0, sizeof(double) * 3 * N, s), "clear");
@@ -237,12 +232,13 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   args.rev_a = L.rev_a;
   args.cap_r = L.cap_r;
   args.cap_a = L.cap_a;
-  args.c_r = dcR;
-  args.c_a = dcA;
+  args.tab = dtabm;
+  args.c_r = dtabm + tl.cr;
+  args.c_a = dtabm + tl.ca;
   args.perm = a.perm;
   args.q_out = q;
-  set_shape_args(args, *params, nullptr);  // the descriptor pass reads no network
-  const cudaError_t e = ops->atom(args, mf, w0, b0, w1, (float)params->b1, 1, s);
+  set_shape_args(args, *params);
+  const cudaError_t e = ops->atom(args, mf, 1, s);
   if (e != cudaSuccess) return cuda_err(e, "descriptor kernel");
   return NEP_OK;
 }
