@@ -29,10 +29,12 @@ struct NvtxRange {
 namespace nep {
 void launch_rebuild_condition(cudaGraphConditionalHandle hc, const BuildStatus *st, cudaStream_t s);
 void launch_drift(int N, const AtomState &a, const double *inv_mass_kappa, double dt, double half_skin2,
-                  BuildStatus *st, cudaStream_t s, const FireState *fire);
-void launch_finalize(int nb_atom, const double *partial_atom, int nb_gather, const double *partial_gather,
+                  BuildStatus *st, cudaStream_t s, const FireState *fire, int *step_ctl);
+void launch_finalize(int nb_atom, const double *partial_atom, int nb_gather, const double *partial_gather, int sums,
                      double *energy_total, double *virial_total, double *heat_total, double *thermo_stage,
-                     int *thermo_ctl, int N, double volume, const ThermoState *ts, cudaStream_t s);
+                     int *thermo_ctl, int N, double volume, const ThermoState *ts, double *scratch, int *ticket,
+                     cudaStream_t s);
+constexpr int kFinalScratch = 64 * kReduceSlots;  // block sums of finalize_kernel
 constexpr int kThermoCols = 8;  // staged thermo row: E, KE, T, P, J[3], thermostat factor
 const ShapeOps *shape_si();
 const ShapeOps *shape_pbte();
@@ -382,6 +384,8 @@ struct nep_handle {
   DevBuf<float4> pos4, posA, dtab, p_ang;
   DevBuf<float> e_rad;
   DevBuf<BuildStatus> status;
+  DevBuf<double> fin_scratch;  // finalize_kernel: block sums
+  DevBuf<int> fin_ticket;      // and its ticket (0 between launches)
   DevBuf<unsigned long long> stat_part;  // partial sums of a build's list statistics
   BuildStatus *h_status = nullptr;  // pinned mirror
   // md
@@ -400,7 +404,8 @@ struct nep_handle {
   cudaGraphExec_t e_graph = nullptr;            // one captured iteration of the current layout
   EngineKey e_key{}, e_last{};
   bool nvt = false;                             // the MD step graph rescales velocities
-  bool graph_nvt = false;
+  bool heat_rows = false;                       // and its thermo rows hold the heat current
+  bool graph_nvt = false, graph_heat = false;
   double graph_dt = 0;
   bool graph_prof = false;
   const double *graph_thermo = nullptr;
@@ -518,6 +523,11 @@ int ensure_atoms(nep_handle *h, int N, cudaStream_t s) {
   }
   CK(h->thermo_ctl.ensure(4), "alloc");
   CK(h->stat_part.ensure(4 * kStatSlots), "alloc");
+  CK(h->fin_scratch.ensure(kFinalScratch), "alloc");
+  if (!h->fin_ticket.p) {
+    CK(h->fin_ticket.ensure(1), "alloc");
+    CK(cudaMemsetAsync(h->fin_ticket.p, 0, sizeof(int), s), "clear ticket");
+  }
   return NEP_OK;
 }
 
@@ -695,8 +705,12 @@ int load_structure(nep_handle *h, int N, const double *pos, const int *types, co
 // Outputs for the caller (nep_compute) are scattered to the caller's atom order; the MD
 // forces (force == h->F) stay in the internal order.
 int run_forces(nep_handle *h, int N, double *energy, double *force, double *virial, int md_kick, double half_dt,
-               cudaStream_t s, bool capturing, const FireState *fire = nullptr) {
+               cudaStream_t s, bool capturing, int sums, int sums_always = 0, const int *step_ctl = nullptr,
+               const FireState *fire = nullptr) {
   AtomArgs a = make_args(h, N);
+  a.sums = sums;
+  a.sums_always = sums_always;
+  a.step_ctl = step_ctl;
   a.fire = fire;
   if (force == h->F.p) a.perm = nullptr;
   a.energy = energy;
@@ -1365,7 +1379,7 @@ int nep_destroy(nep_handle *h) {
   h->e_slots.release(); h->e_slots_ck.release(); h->e_energy.release(); h->e_virial.release(); h->e_u.release();
   h->e_w.release(); h->e_xck.release(); h->e_vck.release(); h->e_table.release();
   h->stage_e.release(); h->stage_g.release();
-  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release();
+  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->fin_scratch.release(); h->fin_ticket.release();
   h->d_grids.release(); h->d_sid.release(); h->d_offsets.release(); h->b_e.release(); h->b_w.release();
   if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
   if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
@@ -1398,12 +1412,14 @@ int nep_compute(nep_handle *h, int n_atoms, const double *pos, const int *types,
   int rc = load_structure(h, n_atoms, pos, types, box, s);
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
-  rc = run_forces(h, n_atoms, energy, force, virial, 0, 0.0, s, false);
+  const int sums = (energy_total ? kSumU : 0) | (virial_total ? kSumW : 0);
+  rc = run_forces(h, n_atoms, energy, force, virial, 0, 0.0, s, false, sums);
   if (rc) return rc;
   ev_record(h, SLOT_FINAL, 0, s, false);
-  launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
-                  h->partial_gather.p, energy_total, virial_total, nullptr, nullptr, nullptr, n_atoms, h->volume,
-                  nullptr, s);
+  if (sums)
+    launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
+                    h->partial_gather.p, sums, energy_total, virial_total, nullptr, nullptr, nullptr, n_atoms,
+                    h->volume, nullptr, h->fin_scratch.p, h->fin_ticket.p, s);
   ev_record(h, SLOT_FINAL, 1, s, false);
   CK(cudaGetLastError(), "finalize");
   return NEP_OK;
@@ -1564,6 +1580,7 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
     a.s_erad = (long long)N * h->T * est;
     a.s_pang = (long long)h->cap_a * N;
     a.f_tar = f_tar;
+    a.sums = kSumFerr;
     ev_record(h, SLOT_ATOM, 0, s, false);
     cudaError_t e = h->ops->atom_batch(a, h->mf, m, atom_block(h), s);
     if (e != cudaSuccess) return cuda_fail(h, e, "nep_atom kernel (population)");
@@ -1810,7 +1827,7 @@ int md_init(nep_handle *h, int n_atoms, const double *pos, const int *types, con
   else CK(cudaMemsetAsync(h->v.p, 0, sizeof(double) * 3 * n_atoms, s), "memset vel");
   rc = load_structure(h, n_atoms, pos, types, box, s, 1);
   if (rc) return rc;
-  rc = run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false);
+  rc = run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false, 0);
   if (rc) return rc;
   CK(wait_stream(s), "md_init");
   h->h_status->n_rebuilds = 0;
@@ -1853,7 +1870,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
   const double half_skin2 = 0.25 * h->skin * h->skin;
   FireState *fs = fire ? h->fire.p : nullptr;
   ev_record(h, SLOT_DRIFT, 0, s, capturing);
-  launch_drift(N, atom_state(h), h->d_inv_mk.p, dt, half_skin2, h->status.p, s, fs);
+  launch_drift(N, atom_state(h), h->d_inv_mk.p, dt, half_skin2, h->status.p, s, fs, h->thermo_ctl.p);
   ev_record(h, SLOT_DRIFT, 1, s, capturing);
   ev_record(h, SLOT_REBUILD, 0, s, capturing);
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
@@ -1898,13 +1915,17 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     h->rebuild_kernels = 0;
   }
   ev_record(h, SLOT_REBUILD, 1, s, capturing);
-  int rc = run_forces(h, N, nullptr, h->F.p, nullptr, 1, 0.5 * dt, s, capturing, fs);
+  // totals of the steps that write a thermo row; the thermostat reads the kinetic energy of every step
+  ThermoState *ts = (!fire && h->nvt) ? h->thermo_state.p : nullptr;
+  const int sums = kSumU | kSumKE | kSumW | (h->heat_rows ? kSumJ : 0);
+  int rc = run_forces(h, N, nullptr, h->F.p, nullptr, 1, 0.5 * dt, s, capturing, sums, ts ? kSumKE : 0,
+                      h->thermo_ctl.p, fs);
   if (rc) return rc;
   ev_record(h, SLOT_FINAL, 0, s, capturing);
-  ThermoState *ts = (!fire && h->nvt) ? h->thermo_state.p : nullptr;
   if (ts) launch_thermostat(N, atom_state(h), h->ops->gather_blocks(N), h->partial_gather.p, ts, s);
-  launch_finalize(h->ops->atom_blocks(N), h->partial_atom.p, h->ops->gather_blocks(N), h->partial_gather.p, nullptr,
-                  nullptr, nullptr, h->thermo_stage.p, h->thermo_ctl.p, N, h->volume, ts, s);
+  launch_finalize(h->ops->atom_blocks(N), h->partial_atom.p, h->ops->gather_blocks(N), h->partial_gather.p, sums,
+                  nullptr, nullptr, nullptr, h->thermo_stage.p, h->thermo_ctl.p, N, h->volume, ts, h->fin_scratch.p,
+                  h->fin_ticket.p, s);
   if (fire) launch_fire_mix(N, atom_state(h), fs, 0, s);
   ev_record(h, SLOT_FINAL, 1, s, capturing);
   CK(cudaGetLastError(), "md step launch");
@@ -1920,6 +1941,7 @@ int md_queue(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double 
     return fail(h, NEP_ERR_ARG, "need n_steps >= 0, dt > 0, thermo_every >= 1");
   if (n_steps == 0) return NEP_OK;
   const bool rows_out = thermo || heat;
+  h->heat_rows = heat != nullptr;
   const int rows = rows_out ? n_steps / thermo_every : 0;
   CK(h->thermo_stage.ensure((size_t)kThermoCols * (rows + 1)), "alloc thermo");
   int ctl[4] = {0, 0, rows_out ? thermo_every : (n_steps + 1), 0};
@@ -1929,12 +1951,13 @@ int md_queue(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double 
   cudaGraphExec_t &gx = fire ? h->fire_graph : h->graph;
   if (fire && gx && (h->graph_prof != h->prof || h->graph_thermo != h->thermo_stage.p ||
                      h->graph_cond_used != h->graph_cond || h->graph_prec != kernel_form(h) ||
-                     h->graph_nvt != h->nvt)) {
+                     h->graph_nvt != h->nvt || h->graph_heat != h->heat_rows)) {
     cudaGraphExecDestroy(gx);
     gx = nullptr;
   }
   if (!gx || (!fire && h->graph_dt != dt_fs) || h->graph_prof != h->prof || h->graph_thermo != h->thermo_stage.p ||
-      h->graph_cond_used != h->graph_cond || h->graph_prec != kernel_form(h) || h->graph_nvt != h->nvt) {
+      h->graph_cond_used != h->graph_cond || h->graph_prec != kernel_form(h) || h->graph_nvt != h->nvt ||
+      h->graph_heat != h->heat_rows) {
     // the MD and FIRE graphs share the capture settings: drop both when they change
     for (cudaGraphExec_t *g : {&h->graph, &h->fire_graph})
       if (*g) {
@@ -1961,6 +1984,7 @@ int md_queue(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double 
     h->graph_cond_used = h->graph_cond;
     h->graph_prec = kernel_form(h);
     h->graph_nvt = h->nvt;
+    h->graph_heat = h->heat_rows;
   }
   for (int st = 0; st < n_steps; ++st) CK(cudaGraphLaunch(gx, s), "graph launch");
   // rows of the staging area -> the caller's [rows][4] thermo and [rows][3] heat current
@@ -2145,12 +2169,14 @@ int nep_heat_current(nep_handle *h, int n_atoms, const double *pos, const int *t
   AtomArgs a = make_args(h, n_atoms);
   a.vel_in = vel;
   a.heat = heat;
+  a.sums = heat_total ? kSumJ : 0;
   cudaError_t e = h->ops->atom(a, h->mf, 0, s);
   if (e == cudaSuccess) e = h->ops->gather(a, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "heat current kernels");
-  launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
-                  h->partial_gather.p, nullptr, nullptr, heat_total, nullptr, nullptr, n_atoms, h->volume, nullptr,
-                  s);
+  if (a.sums)
+    launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
+                    h->partial_gather.p, a.sums, nullptr, nullptr, heat_total, nullptr, nullptr, n_atoms, h->volume,
+                    nullptr, h->fin_scratch.p, h->fin_ticket.p, s);
   CK(cudaGetLastError(), "heat current");
   return NEP_OK;
 }

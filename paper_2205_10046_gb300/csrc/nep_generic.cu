@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(128) generic_atom_kernel(const AtomArgs a, con
       }
     }
   }
-  if constexpr (!DESC_ONLY) {
+  if (!DESC_ONLY && (BATCH || (sums_needed(a) & kSumU))) {
     // deterministic block sum of U (fixed shuffle tree, then fixed warp order)
     __shared__ double red[4];
     double v = Ublock;
@@ -270,17 +270,18 @@ __global__ void __launch_bounds__(128) generic_gather_kernel(const AtomArgs a) {
   const float4 *p_ang = a.p_ang + mem * a.s_pang;
   const int N = a.N, T = a.T, KR = a.gKR, est = a.est;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double part[kReduceSlots];
-  for (int s = 0; s < kReduceSlots; ++s) part[s] = 0.0;
-  if (i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2)) {
+  __shared__ float fw[128][13];
+  __shared__ unsigned char on[128];
+  float fx = 0.f, fy = 0.f, fz = 0.f;
+  float w[9];
+  for (int c = 0; c < 9; ++c) w[c] = 0.f;
+  const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2);
+  if (active) {
     const float4 pi = a.pos4[i];
     const int ti = type_of(pi);
     const float4 *tab = a.dtab + (BATCH ? (size_t)struct_of(pi) * a.ncode : 0);
     const float inv_rcR = 1.f / a.rcR;
     const float rcR2 = a.rcR * a.rcR, rcA2 = a.rcA * a.rcA;
-    float fx = 0.f, fy = 0.f, fz = 0.f;
-    float w[9];
-    for (int c = 0; c < 9; ++c) w[c] = 0.f;
     int base = 0;
     for (int t = 0; t < T; ++t) {
       const int cnt = a.nn_r[(size_t)t * N + i];
@@ -325,9 +326,12 @@ __global__ void __launch_bounds__(128) generic_gather_kernel(const AtomArgs a) {
       w[3] = fmaf(d.x, pji.y, w[3]); w[4] = fmaf(d.x, pji.z, w[4]); w[5] = fmaf(d.y, pji.z, w[5]);
       w[6] = fmaf(d.y, pji.x, w[6]); w[7] = fmaf(d.z, pji.x, w[7]); w[8] = fmaf(d.z, pji.y, w[8]);
     }
-    gather_epilogue(a, i, pi, ti, mem, fx, fy, fz, w, part);
   }
-  gather_block_sums<128>(a, mem, part);
+  float *row = fw[threadIdx.x];
+  row[0] = fx, row[1] = fy, row[2] = fz;
+  for (int c = 0; c < 9; ++c) row[3 + c] = w[c];
+  on[threadIdx.x] = active ? 1 : 0;
+  gather_finish<128, 128>(a, mem, fw, on);
 }
 
 // ------------------------------------------------------------------------ launchers

@@ -17,8 +17,9 @@ constexpr int kMaxImage = 3;    // largest cell/image offset searched per axis
 // accept is left out.
 constexpr double kReachMargin = 2e-3;
 constexpr int kAtomBlock = 128; // threads per block of the per-atom kernel
-constexpr int kGatherBlock = 128;
 constexpr int kReduceSlots = 16; // per-block partial sums: U, KE, W[9], force error, J[3], spare
+// sums over all atoms that a call or an MD step reads (AtomArgs::sums)
+enum { kSumU = 1, kSumKE = 2, kSumW = 4, kSumFerr = 8, kSumJ = 16 };
 
 // Geometry of one neighbour build: the cell grid, the packing of list entries and the
 // table of pair shift vectors indexed by the packed image code.
@@ -203,6 +204,11 @@ struct AtomArgs {
   double *force;           // [N][3] or null (md keeps FP64 forces here)
   double *virial;          // [N][9] or null
   double *partial_gather;  // [gridDim][kReduceSlots]
+  // block sums to form (kSum*): every launch the `sums_always`, and the `sums` on every launch or,
+  // with step_ctl (MD), on steps that write a thermo row: step_ctl[0] is the step's number in
+  // the call (counted by the drift kernel), step_ctl[2] the interval of the rows
+  int sums, sums_always;
+  const int *step_ctl;
   // md kick in the gather epilogue
   int md_kick;
   double half_dt;          // dt/2 in fs
@@ -228,6 +234,30 @@ struct AtomArgs {
   // model shape at run time: read only by the kernels that take the shape at run time (shapes
   // without a compiled instantiation)
   int gR, gKR, gA, gKA, gH, gL3, gL4, gL5, gD;
+};
+
+// The block sums that this launch forms.
+__device__ __forceinline__ int sums_needed(const AtomArgs &a) {
+  const bool row = !a.step_ctl || a.step_ctl[0] % a.step_ctl[2] == 0;
+  return a.sums_always | (row ? a.sums : 0);
+}
+
+// Running sum of FP32 values as an unevaluated pair hi + lo (Knuth's two-sum): the rounding error
+// of every addition goes into lo, so the pair carries about 48 bits without FP64 instructions
+// (a warp's FP64 addition takes 16 cycles of its SM).
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x, float xlo = 0.f) {
+    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
+    hi = s;
+    lo = __fadd_rn(lo, __fadd_rn(err, xlo));
+  }
+  __device__ __forceinline__ void across(int o) {  // + the lane at distance o (xor)
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+    add(h2, l2);
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
 // Model constants of one handle, FP32.

@@ -37,7 +37,9 @@ struct Shape {
   static constexpr int NDES = (NR + 1) + (NA + 1) * NB;
   static constexpr int KEND3 = L3 == 1 ? 3 : L3 == 2 ? 8 : L3 == 3 ? 15 : 24;
   static constexpr int NK = KEND3 > 8 ? KEND3 : (L4 >= 2 ? 8 : KEND3);
-  static constexpr int EST = ((KR + 2) + 3) / 4 * 4;  // KR+1 coefficients and their sum
+  // radial force coefficients e_k of an atom and type and their sum (KR + 2 values): EF4 planes of
+  // float4 over the atoms
+  static constexpr int EF4 = (KR + 2 + 3) / 4;
   static constexpr int OFF4 = (NR + 1) + (NA + 1) * L3;
   static constexpr int OFF5 = OFF4 + (L4 >= 2 ? NA + 1 : 0);
   static constexpr int NDP = (NDES + 3) / 4 * 4;  // padded w0 row in shared memory
@@ -376,6 +378,19 @@ __device__ __forceinline__ void l2_prefetch(const void *p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// The shift table of one structure in shared memory, component by component: the lanes of a
+// warp hold different image codes, and 4-byte reads of up to 64 codes meet few bank conflicts
+// (16-byte entries took 8 passes of the shared memory per read).
+__device__ __forceinline__ void stage_shifts(const AtomArgs &a, float *tab) {
+  for (int v = threadIdx.x; v < a.ncode; v += blockDim.x) {
+    const float4 d = a.dtab[v];
+    tab[v] = d.x, tab[a.ncode + v] = d.y, tab[2 * a.ncode + v] = d.z;
+  }
+}
+__device__ __forceinline__ float4 shift_at(const float *tab, int ncode, unsigned code) {
+  return make_float4(tab[code], tab[ncode + code], tab[2 * ncode + code], 0.f);
+}
+
 // The block's copy of the model table into shared memory, from float `from` on (whole float4s).
 template <class S>
 __device__ __forceinline__ void stage_table(const float *tab, int from, int T, float *dst) {
@@ -513,7 +528,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   float4 *const row = rows + ia * PR::R4;  // [n][6], then q
   float *const qrow = reinterpret_cast<float *>(row + PairRow<S>::S4);
   if constexpr (!BATCH)
-    for (int v = threadIdx.x; v < a.ncode; v += blockDim.x) dtab_s[v] = a.dtab[v];
+    stage_shifts(a, reinterpret_cast<float *>(dtab_s));
   stage_table<S>(a.tab + mem * a.s_tab, PR::from(PREC), T, w0_s + PR::from(PREC));
   __shared__ __align__(8) uint64_t tc_mbar;
   __shared__ uint32_t tc_tmem;
@@ -541,7 +556,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   const float4 *dtab_b = BATCH ? a.dtab + (size_t)struct_of(pi) * a.ncode : dtab_s;
   auto shift = [&](unsigned e) -> float4 {
     if constexpr (BATCH) return __ldg(dtab_b + (e >> a.jbits));
-    else return dtab_s[e >> a.jbits];
+    else return shift_at(reinterpret_cast<const float *>(dtab_s), a.ncode, e >> a.jbits);
   };
 
   // ---- radial descriptor, Eq. qin: per neighbour type, sum_j T_k(x_j) fc_j/2 (k >= 1) and
@@ -924,11 +939,11 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   }
   if (active && h == 0 && a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = (double)U;
 
-  // ---- radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_{nk} and their sum: this lane's
-  // float4s of the row
+  // ---- radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_{nk} and their sum: every second
+  // group of four k
   for (int t = 0; t < T; ++t) {
     const float4 *c = reinterpret_cast<const float4 *>(cR_s + (ti * T + t) * (NR + 1) * KRP);
-    constexpr int E4 = S::EST / 4, EJ = (E4 + 1) / 2;
+    constexpr int E4 = S::EF4, EJ = (E4 + 1) / 2;
     float ev[EJ][4], tot = 0.f;
 #pragma unroll
     for (int j = 0; j < EJ; ++j) {
@@ -952,13 +967,13 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
     }
     tot = __fadd_rn(tot, __shfl_xor_sync(kAll, tot, 1));
     if (active) {
-      float4 *dst = reinterpret_cast<float4 *>(a.e_rad + mem * a.s_erad + ((size_t)i * T + t) * S::EST);
+      float4 *er = reinterpret_cast<float4 *>(a.e_rad + mem * a.s_erad);
 #pragma unroll
       for (int j = 0; j < EJ; ++j) {
         const int k4 = 2 * j + h;
         if (k4 >= E4) continue;
         if (k4 == (KR + 1) / 4) ev[j][(KR + 1) % 4] = tot;
-        dst[k4] = make_float4(ev[j][0], ev[j][1], ev[j][2], ev[j][3]);
+        er[((size_t)t * E4 + k4) * N + i] = make_float4(ev[j][0], ev[j][1], ev[j][2], ev[j][3]);
       }
     }
   }
@@ -1089,22 +1104,21 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
     }
   }
   if constexpr (!BATCH) {
-    // deterministic block sum of U (fixed shuffle tree, then fixed warp order); a batch sums its
-    // structures from the per-atom energies
-    __shared__ double red[2 * AB / 32];
-    double v = active && h == 0 ? (double)U : 0.0;
+    // deterministic block sum of U where it is read (a batch sums its structures from the
+    // per-atom energies)
+    static_assert(AB == 64, "one slot per 64 atoms (atom_blocks)");
+    if (sums_needed(a) & kSumU) {
+      __shared__ double red[2 * AB / 32];
+      Sum2 su;
+      su.add(active && h == 0 ? U : 0.f);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kAll, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int wv = 0; wv < 2 * AB / 32; ++wv) s += red[wv];
-      if (AB == 64) {
-        a.partial_atom[blockIdx.x] = s;
-      } else {  // one slot per 64 atoms (atom_blocks)
-        a.partial_atom[2 * (size_t)blockIdx.x] = s;
-        a.partial_atom[2 * (size_t)blockIdx.x + 1] = 0.0;
+      for (int o = 16; o > 1; o >>= 1) su.across(o);  // lanes of one parity: h == 0 holds the sum
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = su.value();
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int wv = 0; wv < 2 * AB / 32; ++wv) t += red[wv];
+        a.partial_atom[blockIdx.x] = t;
       }
     }
   }
@@ -1126,11 +1140,14 @@ size_t atom_pair_smem(int T, int ncode, int prec, int ab) {
 
 // Epilogue of the gather kernels for atom i: outputs in the caller's order, the squared force
 // error of Eq. loss, the second velocity-Verlet half-kick with the kinetic energy, and the
-// heat current J_i = W_i . v_i (Eq. Ji); part[] collects the block sums.
-__device__ __forceinline__ void gather_epilogue(const AtomArgs &a, int i, const float4 &pi, int ti, int mem,
-                                                float fx, float fy, float fz, const float *w, double *part) {
-  const double Fx = fx, Fy = fy, Fz = fz;
-  const size_t io = mem * a.s_out + (a.perm ? (size_t)a.perm[i] : (size_t)i);
+// heat current J_i = W_i . v_i (Eq. Ji); part[] collects KE, the force error and J for the block
+// sums (need: the sums formed; the others are skipped).
+__device__ __forceinline__ void gather_epilogue(const AtomArgs &a, int i, const float4 &pi, int mem, const float *fw,
+                                                int need, double *part) {
+  const double Fx = fw[0], Fy = fw[1], Fz = fw[2];
+  const float *w = fw + 3;
+  const int ti = type_of(pi);
+  const size_t iu = a.perm ? (size_t)a.perm[i] : (size_t)i, io = mem * a.s_out + iu;
   if (a.force) {
     a.force[3 * io] = Fx;
     a.force[3 * io + 1] = Fy;
@@ -1140,18 +1157,10 @@ __device__ __forceinline__ void gather_epilogue(const AtomArgs &a, int i, const 
 #pragma unroll
     for (int c = 0; c < 9; ++c) a.virial[9 * io + c] = (double)w[c];
   }
-#pragma unroll
-  for (int c = 0; c < 9; ++c) part[2 + c] = (double)w[c];
-  // velocity of the heat current: after the kick below (MD), or given by the caller
-  double vh[3] = {0.0, 0.0, 0.0};
-  if (a.vel_in) {
-    const double *vi = a.vel_in + 3 * (a.perm ? (size_t)a.perm[i] : (size_t)i);
-    vh[0] = vi[0]; vh[1] = vi[1]; vh[2] = vi[2];
-  }
-  if (a.f_tar) {  // squared force error against target forces (the force term of Eq. loss)
-    const double *ft = a.f_tar + 3 * (a.perm ? (size_t)a.perm[i] : (size_t)i);
+  if (need & kSumFerr) {  // squared force error against target forces (the force term of Eq. loss)
+    const double *ft = a.f_tar + 3 * iu;
     const double ex = Fx - ft[0], ey = Fy - ft[1], ez = Fz - ft[2];
-    part[11] = ex * ex + ey * ey + ez * ez;
+    part[1] = ex * ex + ey * ey + ez * ez;
   }
   bool kick = a.md_kick && !(a.fire && a.fire->converged);
   double hdt = a.fire ? 0.5 * a.fire->dt : a.half_dt;
@@ -1160,113 +1169,156 @@ __device__ __forceinline__ void gather_epilogue(const AtomArgs &a, int i, const 
     kick = sl.phase == 1 && !(sl.kind == kJobFire && sl.fire.converged);
     hdt = 0.5 * (sl.kind == kJobFire ? sl.fire.dt : sl.dt);
   }
-  if (kick) {  // second half-kick of velocity Verlet, kinetic energy
+  const bool moments = (need & (kSumKE | kSumJ)) || a.heat;
+  // velocity of the kinetic energy and the heat current: after the kick (MD), or given by the caller
+  double vh[3] = {0.0, 0.0, 0.0};
+  if (kick) {  // second half-kick of velocity Verlet
     double *v = a.vel + 3 * (size_t)i;
     const double s = hdt * a.inv_mass_kappa[ti];
-    const double vx = v[0] + s * Fx, vy = v[1] + s * Fy, vz = v[2] + s * Fz;
-    v[0] = vx; v[1] = vy; v[2] = vz;
-    part[1] = a.mass_kappa_half[ti] * (vx * vx + vy * vy + vz * vz);
-    vh[0] = vx; vh[1] = vy; vh[2] = vz;
-  } else if (a.md_kick || a.slots) {  // converged FIRE or no step: velocities unchanged
-    const double *v = a.vel + 3 * (size_t)i;
-    part[1] = a.mass_kappa_half[ti] * (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-    vh[0] = v[0]; vh[1] = v[1]; vh[2] = v[2];
+    vh[0] = v[0] + s * Fx, vh[1] = v[1] + s * Fy, vh[2] = v[2] + s * Fz;
+    v[0] = vh[0], v[1] = vh[1], v[2] = vh[2];
+  } else if (moments && (a.md_kick || a.slots || a.vel_in)) {  // converged FIRE or no step: velocities unchanged
+    const double *v = a.vel_in ? a.vel_in + 3 * iu : a.vel + 3 * (size_t)i;
+    vh[0] = v[0], vh[1] = v[1], vh[2] = v[2];
   }
-  // J_i = W_i . v_i, W_i[a][b] in the order xx, yy, zz, xy, xz, yz, yx, zx, zy (Eq. Ji)
-  const double Jx = (double)w[0] * vh[0] + (double)w[3] * vh[1] + (double)w[4] * vh[2];
-  const double Jy = (double)w[6] * vh[0] + (double)w[1] * vh[1] + (double)w[5] * vh[2];
-  const double Jz = (double)w[7] * vh[0] + (double)w[8] * vh[1] + (double)w[2] * vh[2];
-  part[12] = Jx;
-  part[13] = Jy;
-  part[14] = Jz;
-  if (a.heat) {
-    a.heat[3 * io] = Jx;
-    a.heat[3 * io + 1] = Jy;
-    a.heat[3 * io + 2] = Jz;
+  if (!moments) return;
+  if (need & kSumKE) part[0] = a.mass_kappa_half[ti] * (vh[0] * vh[0] + vh[1] * vh[1] + vh[2] * vh[2]);
+  if ((need & kSumJ) || a.heat) {
+    // J_i = W_i . v_i, W_i[a][b] in the order xx, yy, zz, xy, xz, yz, yx, zx, zy (Eq. Ji)
+    part[2] = (double)w[0] * vh[0] + (double)w[3] * vh[1] + (double)w[4] * vh[2];
+    part[3] = (double)w[6] * vh[0] + (double)w[1] * vh[1] + (double)w[5] * vh[2];
+    part[4] = (double)w[7] * vh[0] + (double)w[8] * vh[1] + (double)w[2] * vh[2];
+    if (a.heat) {
+      a.heat[3 * io] = part[2];
+      a.heat[3 * io + 1] = part[3];
+      a.heat[3 * io + 2] = part[4];
+    }
   }
 }
 
-// Deterministic block sums of (KE, W[9], force error, J[3]) over a block of GB threads.
-template <int GB>
-__device__ __forceinline__ void gather_block_sums(const AtomArgs &a, int mem, const double *part) {
-  __shared__ double red[GB / 32][kReduceSlots];
+// End of a gather kernel: fw[GA][13] holds F_i and W_i (12 floats) of the block's GA atoms, zeros
+// for the inactive ones (`on` marks the others). One thread per atom runs the epilogue, then
+// the block forms the sums that are read, in a fixed order: W in FP32 pairs (Sum2) from the
+// shared rows, the rest in FP64. Without the test every MD step of every atom paid 15 FP64
+// block sums for totals that only thermo rows show (half of the gather's time).
+template <int GA, int NT>
+__device__ __forceinline__ void gather_finish(const AtomArgs &a, int mem, float (*fw)[13], const unsigned char *on) {
+  static_assert(GA % 32 == 0 && NT >= GA && NT >= 96, "whole warps of atoms; 72 threads for the virial sums");
+  __shared__ double red[GA / 32][5];
+  const int need = sums_needed(a);
+  double part[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  __syncthreads();
+  if (threadIdx.x < GA && on[threadIdx.x]) {
+    const int i = blockIdx.x * GA + threadIdx.x;
+    gather_epilogue(a, i, a.pos4[i], mem, fw[threadIdx.x], need, part);
+  }
+  if (!(need & (kSumKE | kSumW | kSumFerr | kSumJ))) return;
+  double *out = a.partial_gather + ((size_t)mem * gridDim.x + blockIdx.x) * kReduceSlots;
+  if ((need & kSumW) && threadIdx.x < 96) {  // eight threads per component (96: whole warps)
+    const int c = threadIdx.x >> 3, p = threadIdx.x & 7;
+    Sum2 s;
+    if (c < 9)
+      for (int r = p; r < GA; r += 8) s.add(fw[r][3 + c]);
 #pragma unroll
-  for (int s = 1; s < kReduceSlots; ++s) {
-    double v = part[s];
+    for (int o = 4; o > 0; o >>= 1) s.across(o);
+    if (c < 9 && p == 0) out[2 + c] = s.value();
+  }
+  if (!(need & (kSumKE | kSumFerr | kSumJ))) return;
+  if (threadIdx.x < GA) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][s] = v;
+    for (int k = 0; k < 5; ++k) {
+      if (!(need & (k == 0 ? kSumKE : k == 1 ? kSumFerr : kSumJ))) continue;
+      double v = part[k];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
+    }
   }
   __syncthreads();
-  if (threadIdx.x < kReduceSlots && threadIdx.x >= 1) {
+  if (threadIdx.x < 5 && (need & (threadIdx.x == 0 ? kSumKE : threadIdx.x == 1 ? kSumFerr : kSumJ))) {
     double s = 0.0;
-    for (int wv = 0; wv < GB / 32; ++wv) s += red[wv][threadIdx.x];
-    a.partial_gather[((size_t)mem * gridDim.x + blockIdx.x) * kReduceSlots + threadIdx.x] = s;
+    for (int wv = 0; wv < GA / 32; ++wv) s += red[wv][threadIdx.x];
+    out[threadIdx.x == 0 ? 1 : 10 + threadIdx.x] = s;  // KE 1, force error 11, J 12 .. 14
   }
 }
 
 // ------------------------------------------------------------------------ gather kernel
-// For one structure the gather is held to 64 registers for N_bas^R <= 8 (1024 threads per SM:
-// 8 CTAs of 128 instead of 7 hide more of the neighbour gathers' latency; 8,000,000 Si atoms:
-// 3.17 against 3.52 ms) and to 72 above (7 CTAs); the batched form keeps the compiler's choice.
-template <class S, bool BATCH = false, int GB = kGatherBlock>
-__global__ void __launch_bounds__(GB, BATCH ? 1 : (S::KR <= 8 ? 1024 : 896) / GB)
+// kGatherLanes lanes per atom take every kGatherLanes-th entry of its lists; their sums are
+// added across, and one thread per atom finishes (gather_finish).
+//
+// What bounds it: the L1 data stage (84% busy): the neighbours' e_k, positions and partial
+// forces are 16-byte reads at 32 scattered addresses, about 10 passes each. The e_k lie in
+// planes of float4 over the atoms and the image shifts component by component in shared memory,
+// which took a fifth of the passes out. For one structure the kernel is held to 64 registers
+// for N_bas^R <= 8 (1024 threads per SM hide more of the latency than 896: 8,000,000 Si atoms
+// 2.47 against 2.73 ms) and to 72 above. Two lanes halve the serial chain of small systems; four
+// shorten it further (216 atoms: 13.8 us) but cost large ones more than they give
+// (8,000,000 atoms: 2.98 ms). Before / after (one thread per atom, all block sums in every
+// launch), us: 216 Si atoms 32 / 18, 262,144 PbTe atoms 121 / 100, 8,000,000 Si atoms 2846 /
+// 2472, 4096 structures 681 / 550.
+constexpr int kGatherLanes = 2;
+constexpr int gather_min_blocks(int KR, int threads) {
+  return (KR <= 8 ? 1024 : 896) / threads > 0 ? (KR <= 8 ? 1024 : 896) / threads : 1;
+}
+
+template <class S, bool BATCH, int GA>
+__global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA *kGatherLanes))
     gather_kernel(const AtomArgs a) {
-  constexpr int KR = S::KR, EST = S::EST;
+  constexpr int L = kGatherLanes;
+  __shared__ float fw[GA][13];
+  __shared__ unsigned char on[GA];
+  constexpr int KR = S::KR;
   extern __shared__ float4 smem4[];
   float4 *dtab_s = smem4;
   const int mem = BATCH ? (int)blockIdx.y : 0;
   if constexpr (!BATCH) {
-    for (int v = threadIdx.x; v < a.ncode; v += blockDim.x) dtab_s[v] = a.dtab[v];
+    stage_shifts(a, reinterpret_cast<float *>(dtab_s));
     __syncthreads();
   }
   const float *e_rad = a.e_rad + mem * a.s_erad;
   const float4 *p_ang = a.p_ang + mem * a.s_pang;
   const int N = a.N, T = a.T;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double part[kReduceSlots];
+  const int ia = threadIdx.x / L, l = threadIdx.x % L;
+  const int i = blockIdx.x * GA + ia;
+  float fx = 0.f, fy = 0.f, fz = 0.f;
+  float w[9];
 #pragma unroll
-  for (int s = 0; s < kReduceSlots; ++s) part[s] = 0.0;
+  for (int c = 0; c < 9; ++c) w[c] = 0.f;
   // (serving engine) atoms of a finished job frozen in the batch are skipped
-  if (i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2)) {
+  const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2);
+  if (active) {
     const float4 pi = a.pos4[i];
     const int ti = type_of(pi);
     const float4 *dtab_b = BATCH ? a.dtab + (size_t)struct_of(pi) * a.ncode : dtab_s;
     auto shift = [&](unsigned e) -> float4 {
       if constexpr (BATCH) return __ldg(dtab_b + (e >> a.jbits));
-      else return dtab_s[e >> a.jbits];
+      else return shift_at(reinterpret_cast<const float *>(dtab_s), a.ncode, e >> a.jbits);
     };
     const float inv_rcR = 1.f / a.rcR;
     const float rcR2 = a.rcR * a.rcR, rcA2 = a.rcA * a.rcA;
-    float fx = 0.f, fy = 0.f, fz = 0.f;
-    float w[9];
+    // e_k of atom j and type t and (entry KR + 1) their sum
+    auto load_e = [&](float *e, int t, int j) {
 #pragma unroll
-    for (int c = 0; c < 9; ++c) w[c] = 0.f;
+      for (int k4 = 0; k4 < S::EF4; ++k4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(e_rad) + ((size_t)t * S::EF4 + k4) * N + j);
+        e[4 * k4] = v.x, e[4 * k4 + 1] = v.y, e[4 * k4 + 2] = v.z, e[4 * k4 + 3] = v.w;
+      }
+    };
     // ---- radial part (Algorithm 2): s_i from own e^{t_j}, s_j from neighbour's e^{t_i}
     int base = 0;
     for (int t = 0; t < T; ++t) {
       const int cnt = a.nn_r[t * N + i];
-      float eo[EST];
-      const float4 *src = reinterpret_cast<const float4 *>(e_rad + ((size_t)i * T + t) * EST);
-#pragma unroll
-      for (int k4 = 0; k4 < EST / 4; ++k4) {
-        const float4 v = src[k4];
-        eo[4 * k4] = v.x; eo[4 * k4 + 1] = v.y; eo[4 * k4 + 2] = v.z; eo[4 * k4 + 3] = v.w;
-      }
-      for_pairs_batch<2, true, 1>(a.nl_r, base, cnt, N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
+      float eo[4 * S::EF4];
+      load_e(eo, t, i);
+      for_pairs_batch<2, true, 1>(a.nl_r + (size_t)(base + l) * N, 0, (cnt + L - 1 - l) / L, L * N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
         const int j = e & a.jmask;
         const float3 d = pair_vector(pi, pj, shift(e));
         const float r2 = norm2(d);
         if (r2 < rcR2) {
           const float rinv = rsqrtf(r2);
           const float r = r2 * rinv;
-          float ej[EST];
-          const float4 *srcj = reinterpret_cast<const float4 *>(e_rad + ((size_t)j * T + ti) * EST);
-#pragma unroll
-          for (int k4 = 0; k4 < EST / 4; ++k4) {
-            const float4 v = __ldg(srcj + k4);
-            ej[4 * k4] = v.x; ej[4 * k4 + 1] = v.y; ej[4 * k4 + 2] = v.z; ej[4 * k4 + 3] = v.w;
-          }
+          float ej[4 * S::EF4];
+          load_e(ej, ti, j);
           // sum_k e_k f_k'(r) = (x' fc/2) sum_k e_k T_k'(x) + (fc'/2) (sum_k e_k T_k(x) + sum_k e_k)
           const float u = r * inv_rcR;
           float sn, cs;
@@ -1324,25 +1376,26 @@ __global__ void __launch_bounds__(GB, BATCH ? 1 : (S::KR <= 8 ? 1024 : 896) / GB
     // and a slot's partial force is used only when the pair is inside the cutoff, which is
     // exactly when the per-atom kernel wrote it).
     const int na = a.nn_a[i];
-    if (na > 0) {
+    if (l < na) {
       const unsigned *col = a.nl_a + i;
       const int *rcol = a.rev_a + i;
-      unsigned e0 = __ldcs(col), e1 = na > 1 ? __ldcs(col + N) : 0u;
-      int r1 = na > 1 ? __ldcs(rcol + N) : 0;
+      auto at = [&](int m) { return (size_t)m * N; };
+      unsigned e0 = __ldcs(col + at(l)), e1 = l + L < na ? __ldcs(col + at(l + L)) : 0u;
+      int r1 = l + L < na ? __ldcs(rcol + at(l + L)) : 0;
       float4 p0 = __ldg(a.pos4 + (e0 & a.jmask));
-      float4 pij0 = __ldcs(p_ang + i), pji0 = __ldg(p_ang + __ldcs(rcol));
-      for (int m = 0; m < na; ++m) {
+      float4 pij0 = __ldcs(p_ang + at(l) + i), pji0 = __ldg(p_ang + __ldcs(rcol + at(l)));
+      for (int m = l; m < na; m += L) {
         const unsigned e = e0;
         const float4 pj = p0, pij = pij0, pji = pji0;
-        if (m + 1 < na) {
+        if (m + L < na) {
           p0 = __ldg(a.pos4 + (e1 & a.jmask));
-          pij0 = __ldcs(p_ang + (size_t)(m + 1) * N + i);
+          pij0 = __ldcs(p_ang + at(m + L) + i);
           pji0 = __ldg(p_ang + r1);
         }
         e0 = e1;
-        if (m + 2 < na) {
-          e1 = __ldcs(col + (size_t)(m + 2) * N);
-          r1 = __ldcs(rcol + (size_t)(m + 2) * N);
+        if (m + 2 * L < na) {
+          e1 = __ldcs(col + at(m + 2 * L));
+          r1 = __ldcs(rcol + at(m + 2 * L));
         }
         const float3 d = pair_vector(pi, pj, shift(e));
         const float r2 = norm2(d);
@@ -1362,9 +1415,17 @@ __global__ void __launch_bounds__(GB, BATCH ? 1 : (S::KR <= 8 ? 1024 : 896) / GB
         }
       }
     }
-    gather_epilogue(a, i, pi, ti, mem, fx, fy, fz, w, part);
   }
-  gather_block_sums<GB>(a, mem, part);
+  // the sums of the atom's lanes; one row per atom for the epilogue
+  float v[12] = {fx, fy, fz, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7], w[8]};
+#pragma unroll
+  for (int c = 0; c < 12; ++c) {
+#pragma unroll
+    for (int o = 1; o < L; o <<= 1) v[c] = __fadd_rn(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
+    if (l == 0) fw[ia][c] = v[c];
+  }
+  if (l == 0) on[ia] = active ? 1 : 0;
+  gather_finish<GA, GA * L>(a, mem, fw, on);
 }
 
 // ------------------------------------------------------------------------ launchers
@@ -1390,11 +1451,13 @@ cudaError_t launch_atom(const AtomArgs &a, const ModelF &mf, int descriptor_only
   return launch_atom_as<S, 0, false, false, 64>(a, mf, 1, st);
 }
 
+constexpr int kGatherAtoms = 64;  // atoms per CTA of the gather of one structure
+
 template <class S>
 cudaError_t launch_gather(const AtomArgs &a, cudaStream_t st) {
   if (a.N <= 0) return cudaSuccess;
-  const int blocks = (a.N + kGatherBlock - 1) / kGatherBlock;
-  gather_kernel<S><<<blocks, kGatherBlock, sizeof(float4) * a.ncode, st>>>(a);
+  constexpr int GA = kGatherAtoms;
+  gather_kernel<S, false, GA><<<(a.N + GA - 1) / GA, GA * kGatherLanes, sizeof(float4) * a.ncode, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1420,9 +1483,10 @@ template <class S>
 cudaError_t launch_gather_batch(const AtomArgs &a, int members, int block, cudaStream_t st) {
   if (a.N <= 0 || members <= 0) return cudaSuccess;
   const dim3 grid((a.N + block - 1) / block, members);
-  if (block == 64) gather_kernel<S, true, 64><<<grid, 64, 0, st>>>(a);
-  else if (block == 128) gather_kernel<S, true, 128><<<grid, 128, 0, st>>>(a);
-  else if (block == 256) gather_kernel<S, true, 256><<<grid, 256, 0, st>>>(a);
+  constexpr int L = kGatherLanes;
+  if (block == 64) gather_kernel<S, true, 64><<<grid, 64 * L, 0, st>>>(a);
+  else if (block == 128) gather_kernel<S, true, 128><<<grid, 128 * L, 0, st>>>(a);
+  else if (block == 256) gather_kernel<S, true, 256><<<grid, 256 * L, 0, st>>>(a);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
@@ -1437,7 +1501,7 @@ template <class S>
 void attach_batch(ShapeOps &o);  // explicitly instantiated in the batch translation unit
 #endif
 
-template <class S> int gather_blocks(int N) { return (N + kGatherBlock - 1) / kGatherBlock; }
+template <class S> int gather_blocks(int N) { return (N + kGatherAtoms - 1) / kGatherAtoms; }
 
 template <class S>
 ShapeOps make_ops() {
