@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <functional>
 #include <thread>
 #include <cstdio>
 #include <cstring>
@@ -33,7 +34,7 @@ void launch_drift(int N, const AtomState &a, const double *inv_mass_kappa, doubl
 void launch_finalize(int nb_atom, const double *partial_atom, int nb_gather, const double *partial_gather, int sums,
                      double *energy_total, double *virial_total, double *heat_total, double *thermo_stage,
                      int *thermo_ctl, int N, double volume, const ThermoState *ts, double *scratch, int *ticket,
-                     cudaStream_t s);
+                     const BuildStatus *guard, cudaStream_t s);
 constexpr int kFinalScratch = 64 * kReduceSlots;  // block sums of finalize_kernel
 constexpr int kThermoCols = 8;  // staged thermo row: E, KE, T, P, J[3], thermostat factor
 const ShapeOps *shape_si();
@@ -77,10 +78,9 @@ void model_constants(ModelF &m) {
   m.c5b[2] = (float)(21.0 / (80.0 * p * p));
 }
 
-// Cell grid, image range and shift table (dtab[0..ncode), at most 512 entries; skipped when
-// dtab is null) for the cell rows `box` and the list radius rl. Returns NEP_OK or an error
-// code with *err set.
-int build_grid(const double *box, double rl, int N, Grid &g, float4 *dtab, double *volume, const char **err) {
+// Cell grid and image range (the shift table, at most 512 entries, is formed on the device) for
+// the cell rows `box` and the list radius rl. Returns NEP_OK or an error code with *err set.
+int build_grid(const double *box, double rl, int N, Grid &g, double *volume, const char **err) {
   g.cell_off = 0;
   g.dtab_off = 0;
   for (int a = 0; a < 3; ++a)
@@ -147,17 +147,6 @@ int build_grid(const double *box, double rl, int N, Grid &g, float4 *dtab, doubl
       g.Hf[a][b] = (float)g.H[a][b];
       g.Hinvf[a][b] = (float)g.Hinv[a][b];
     }
-  if (!dtab) return NEP_OK;
-  for (int c = 0; c < g.ncode; ++c) dtab[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int ox = -g.R[0]; ox <= g.R[0]; ++ox)
-    for (int oy = -g.R[1]; oy <= g.R[1]; ++oy)
-      for (int oz = -g.R[2]; oz <= g.R[2]; ++oz) {
-        const unsigned code = (unsigned)(ox + g.R[0]) | ((unsigned)(oy + g.R[1]) << g.obits) |
-                              ((unsigned)(oz + g.R[2]) << (2 * g.obits));
-        double D[3];
-        for (int b = 0; b < 3; ++b) D[b] = ox * g.Hc[0][b] + oy * g.Hc[1][b] + oz * g.Hc[2][b];
-        dtab[code] = make_float4((float)D[0], (float)D[1], (float)D[2], 0.f);
-      }
   return NEP_OK;
 }
 
@@ -289,6 +278,16 @@ cudaError_t wait_stream(cudaStream_t s) {
   if (!t_alloc_async) return cudaStreamSynchronize(s);
   for (;;) {
     const cudaError_t e = cudaStreamQuery(s);
+    if (e != cudaErrorNotReady) return e;
+    std::this_thread::sleep_for(std::chrono::microseconds(20));
+  }
+}
+
+// The same for an event recorded in a stream.
+cudaError_t wait_event(cudaEvent_t ev) {
+  if (!t_alloc_async) return cudaEventSynchronize(ev);
+  for (;;) {
+    const cudaError_t e = cudaEventQuery(ev);
     if (e != cudaErrorNotReady) return e;
     std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
@@ -434,6 +433,7 @@ struct nep_handle {
   Tuning tune;
   // profiling
   bool prof = false;
+  cudaEvent_t ev_status = nullptr;  // the status of a build has reached h_status
   cudaEvent_t ev[N_SLOTS][2] = {};
   bool slot_ran[N_SLOTS] = {};
   nep_stats stats_cache{};
@@ -481,15 +481,6 @@ void ev_record(nep_handle *h, int slot, int which, cudaStream_t s, bool capturin
   if (capturing) cudaEventRecordWithFlags(h->ev[slot][which], s, cudaEventRecordExternal);
   else cudaEventRecord(h->ev[slot][which], s);
   if (which == 1) h->slot_ran[slot] = true;
-}
-
-int setup_grid(nep_handle *h, int N, const double *box, std::vector<float4> &dtab) {
-  dtab.assign(1 << (3 * 3), make_float4(0.f, 0.f, 0.f, 0.f));
-  const char *err = nullptr;
-  const int rc = nep::build_grid(box, h->rcR + h->skin, N, h->grid, dtab.data(), &h->volume, &err);
-  if (rc) return fail(h, rc, err);
-  dtab.resize(h->grid.ncode);
-  return NEP_OK;
 }
 
 int ensure_atoms(nep_handle *h, int N, cudaStream_t s) {
@@ -550,19 +541,6 @@ int read_status(nep_handle *h, cudaStream_t s) {
   return NEP_OK;
 }
 
-void reset_status_counts(nep_handle *h) {
-  h->h_status->overflow = 0;
-  h->h_status->max_r = 0;
-  h->h_status->max_a = 0;
-  h->h_status->rev_missing = 0;
-  h->h_status->sum_r = 0;
-  h->h_status->sum_a = 0;
-  h->h_status->bad_input = 0;
-  h->h_status->in_r = 0;
-  h->h_status->in_a = 0;
-  h->h_status->tc_timeout = 0;
-}
-
 AtomState atom_state(nep_handle *h) {
   AtomState a;
   a.x = h->x.p; a.v = h->v.p; a.F = h->F.p; a.x_ref = h->x_ref.p; a.origin = h->origin.p;
@@ -585,10 +563,14 @@ ListBufs list_bufs(nep_handle *h) {
 // (random-weight models do) before a regrow is needed.
 int round_cap(int m) { return std::min(kListBuf, (2 * m + 16 + 3) / 4 * 4); }
 
-// Bin, size and build the neighbour lists for the positions in h->x (forced rebuild).
+// Bin, size and build the neighbour lists (forced rebuild) of the structure in `src`, or of the
+// positions in h->x.
 // move: the per-atom arrays that go into the new atom order besides positions and types (bit 0
-// velocities, bit 1 forces).
-int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B = Batch{nullptr, nullptr, 0}) {
+// velocities, bit 1 forces). after: queues the kernels that use the lists right behind a build
+// that may succeed, before the host looks at its status (they test it on the device); the host
+// waits for the status alone, so neither it nor the GPU idles for the other.
+int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B = Batch{nullptr, nullptr, 0},
+                  LoadSrc src = LoadSrc{}, const std::function<int()> &after = nullptr) {
   Grid &g = h->grid;
   CK(h->cell_count.ensure(g.ncell + 1), "alloc cells");
   CK(h->cell_cursor.ensure(g.ncell + 1), "alloc cells");
@@ -600,18 +582,22 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
   }
   for (int attempt = 0; attempt < 3; ++attempt) {
     const bool count_only = (h->cap_r == 0 || h->cap_a == 0);
-    CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
-    CK(wait_stream(s), "sync");
-    reset_status_counts(h);
-    h->h_status->rebuild = 1;
-    h->h_status->full = 1;
-    CK(cudaMemcpyAsync(h->status.p, h->h_status, sizeof(BuildStatus), cudaMemcpyHostToDevice, s), "status");
+    if (!src.pos) launch_arm_rebuild(h->status.p, s);  // else requested by the load
     CK(launch_rebuild(N, h->T, g, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
-                      list_bufs(h), count_only ? 1 : 0, move, h->status.p, s),
+                      list_bufs(h), count_only ? 1 : 0, move, src, h->status.p, s),
        "launch rebuild");
-    CK(cudaGetLastError(), "launch rebuild");
-    int rc = read_status(h, s);
-    if (rc) return rc;
+    src = LoadSrc{};  // the atoms are in place from here on
+    int rc = NEP_OK;
+    if (after && !count_only) {
+      CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
+      CK(cudaEventRecord(h->ev_status, s), "status");
+      rc = after();
+      if (rc) return rc;
+      CK(wait_event(h->ev_status), "sync");
+    } else {
+      rc = read_status(h, s);
+      if (rc) return rc;
+    }
     const BuildStatus &st = *h->h_status;
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
@@ -683,23 +669,20 @@ AtomArgs make_args(nep_handle *h, int N) {
 // Identity of the per-atom kernel a captured graph uses (the network).
 int kernel_form(const nep_handle *h) { return h->precision; }
 
-// Load positions (device, [N][3]) and types, set up the grid and build the lists.
+// Load positions (device, [N][3]) and types, set up the grid and build the lists; `after` as in
+// rebuild_lists.
 int load_structure(nep_handle *h, int N, const double *pos, const int *types, const double *box, cudaStream_t s,
-                   int move = 0) {
+                   int move, const std::function<int()> &after) {
   int rc = ensure_atoms(h, N, s);
   if (rc) return rc;
-  std::vector<float4> dtab;
-  rc = setup_grid(h, N, box, dtab);
-  if (rc) return rc;
-  CK(h->dtab.ensure(dtab.size()), "alloc");
-  CK(cudaMemcpyAsync(h->dtab.p, dtab.data(), dtab.size() * sizeof(float4), cudaMemcpyHostToDevice, s), "copy");
-  CK(cudaMemcpyAsync(h->x.p, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
-  CK(cudaMemcpyAsync(h->types.p, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
-  launch_iota(N, h->perm.p, s);
+  const char *err = nullptr;
+  rc = nep::build_grid(box, h->rcR + h->skin, N, h->grid, &h->volume, &err);
+  if (rc) return fail(h, rc, err);
+  CK(h->dtab.ensure(h->grid.ncode), "alloc");
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = h->grid.nc[a];
-  return rebuild_lists(h, N, s, move);
+  return rebuild_lists(h, N, s, move, Batch{nullptr, nullptr, 0}, LoadSrc{pos, types, h->dtab.p}, after);
 }
 
 // Outputs for the caller (nep_compute) are scattered to the caller's atom order; the MD
@@ -711,6 +694,7 @@ int run_forces(nep_handle *h, int N, double *energy, double *force, double *viri
   a.sums = sums;
   a.sums_always = sums_always;
   a.step_ctl = step_ctl;
+  if (!md_kick) a.guard = h->status.p;  // queued behind a build whose status is still unread
   a.fire = fire;
   if (force == h->F.p) a.perm = nullptr;
   a.energy = energy;
@@ -749,7 +733,7 @@ int setup_batch(nep_handle *h, int n_struct, const int *offsets, const double *b
       const char *err = nullptr;
       double vol = 0;
       rc = nep::build_grid(boxes + 9 * (size_t)k, h->rcR + h->skin, std::max(offsets[k + 1] - offsets[k], 1), G[k],
-                           nullptr, &vol, &err);
+                           &vol, &err);
       if (rc) return fail(h, rc, "structure " + std::to_string(k) + ": " + err);
       obits = std::max(obits, G[k].obits);
     }
@@ -785,7 +769,7 @@ int setup_batch(nep_handle *h, int n_struct, const int *offsets, const double *b
     CK(cudaMemcpyAsync(h->d_grids.p, G.data(), sizeof(Grid) * n_struct, cudaMemcpyHostToDevice, s), "copy grids");
     CK(cudaMemcpyAsync(h->d_offsets.p, h->b_offsets.data(), sizeof(int) * (n_struct + 1), cudaMemcpyHostToDevice, s),
        "copy offsets");
-    launch_shift_tables(n_struct, h->d_grids.p, ncode, obits, h->dtab.p, s);
+    launch_shift_tables(n_struct, h->d_grids.p, ncode, h->dtab.p, s);
     h->b_gen += 1;
     h->nb_struct = n_struct;
   }
@@ -896,13 +880,10 @@ int capture_batch(nep_handle *h, int N, const BatchOut &o, cudaStream_t s) {
   CK(wait_stream(s), "sync");
   cudaStream_t c = h->cap_stream;
   CK(cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal), "capture");
-  cudaMemcpyAsync(h->x.p, o.pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, c);
-  cudaMemcpyAsync(h->types.p, o.types, sizeof(int) * N, cudaMemcpyDeviceToDevice, c);
-  launch_iota(N, h->perm.p, c);
-  launch_arm_rebuild(h->status.p, c);
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
   cudaError_t e = launch_rebuild(N, h->T, h->grid, batch_of(h), h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(),
-                                 h->rcA2f(), atom_state(h), list_bufs(h), 0, 0, h->status.p, c);
+                                 h->rcA2f(), atom_state(h), list_bufs(h), 0, 0, LoadSrc{o.pos, o.types, nullptr},
+                                 h->status.p, c);
   int rc = e == cudaSuccess ? batch_kernels(h, N, o, c, true) : cuda_fail(h, e, "batch rebuild");
   if (!rc) cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, c);
   cudaGraph_t graph = nullptr;
@@ -1150,7 +1131,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   Batch B = batch_of(h);
   B.sflag = h->e_sflag.p;
   cudaError_t e = launch_rebuild(N, h->T, h->grid, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
-                                 atom_state(h), list_bufs(h), 0, 3, h->status.p, s);
+                                 atom_state(h), list_bufs(h), 0, 3, LoadSrc{}, h->status.p, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine rebuild");
   AtomArgs a = make_args(h, N);
   a.perm = nullptr;  // every output in the internal order
@@ -1348,6 +1329,7 @@ int nep_create(const nep_params *p, nep_handle **out) {
   if (e != cudaSuccess) { nep_destroy(h); return fail(nullptr, NEP_ERR_CUDA, cudaGetErrorString(e)); }
   for (int sl = 0; sl < N_SLOTS; ++sl)
     for (int w = 0; w < 2; ++w) cudaEventCreate(&h->ev[sl][w]);
+  cudaEventCreateWithFlags(&h->ev_status, cudaEventDisableTiming);
   cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking);
   cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking);
   *out = h;
@@ -1365,6 +1347,7 @@ int nep_destroy(nep_handle *h) {
   for (int sl = 0; sl < N_SLOTS; ++sl)
     for (int w = 0; w < 2; ++w)
       if (h->ev[sl][w]) cudaEventDestroy(h->ev[sl][w]);
+  if (h->ev_status) cudaEventDestroy(h->ev_status);
   if (h->h_status) cudaFreeHost(h->h_status);
   h->d_tab.release(); h->d_inv_mk.release(); h->d_mk_half.release();
   h->x.release(); h->v.release(); h->F.release(); h->x_ref.release(); h->origin.release();
@@ -1408,21 +1391,21 @@ int nep_compute(nep_handle *h, int n_atoms, const double *pos, const int *types,
     if (virial_total) CK(cudaMemsetAsync(virial_total, 0, 9 * sizeof(double), s), "memset");
     return NEP_OK;
   }
-  ev_record(h, SLOT_REBUILD, 0, s, false);
-  int rc = load_structure(h, n_atoms, pos, types, box, s);
-  if (rc) return rc;
-  ev_record(h, SLOT_REBUILD, 1, s, false);
   const int sums = (energy_total ? kSumU : 0) | (virial_total ? kSumW : 0);
-  rc = run_forces(h, n_atoms, energy, force, virial, 0, 0.0, s, false, sums);
-  if (rc) return rc;
-  ev_record(h, SLOT_FINAL, 0, s, false);
-  if (sums)
-    launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
-                    h->partial_gather.p, sums, energy_total, virial_total, nullptr, nullptr, nullptr, n_atoms,
-                    h->volume, nullptr, h->fin_scratch.p, h->fin_ticket.p, s);
-  ev_record(h, SLOT_FINAL, 1, s, false);
-  CK(cudaGetLastError(), "finalize");
-  return NEP_OK;
+  ev_record(h, SLOT_REBUILD, 0, s, false);
+  return load_structure(h, n_atoms, pos, types, box, s, 0, [&]() -> int {
+    ev_record(h, SLOT_REBUILD, 1, s, false);
+    const int rc = run_forces(h, n_atoms, energy, force, virial, 0, 0.0, s, false, sums);
+    if (rc) return rc;
+    ev_record(h, SLOT_FINAL, 0, s, false);
+    if (sums)
+      launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
+                      h->partial_gather.p, sums, energy_total, virial_total, nullptr, nullptr, nullptr, n_atoms,
+                      h->volume, nullptr, h->fin_scratch.p, h->fin_ticket.p, h->status.p, s);
+    ev_record(h, SLOT_FINAL, 1, s, false);
+    CK(cudaGetLastError(), "finalize");
+    return NEP_OK;
+  });
 }
 
 int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const double *pos, const int *types,
@@ -1476,13 +1459,10 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
     // the lists outgrew their capacity: size them again on the eager path below
   }
   ev_record(h, SLOT_REBUILD, 0, s, false);
-  CK(cudaMemcpyAsync(h->x.p, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
-  CK(cudaMemcpyAsync(h->types.p, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
-  launch_iota(N, h->perm.p, s);
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = 0;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   rc = batch_kernels(h, N, o, s, false);
@@ -1528,12 +1508,9 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
   rc = setup_batch(h, n_struct, offsets, boxes, N, s);
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 0, s, false);
-  CK(cudaMemcpyAsync(h->x.p, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
-  CK(cudaMemcpyAsync(h->types.p, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
-  launch_iota(N, h->perm.p, s);
   h->N = N;
   h->stats_cache.n_atoms = N;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   // parameter vectors -> FP32 model tables (and BF16 tiles for the tensor-core network)
@@ -1616,11 +1593,8 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   h->md_ready = false;
   rc = setup_batch(h, n_struct, offsets, boxes, N, s);
   if (rc) return rc;
-  CK(cudaMemcpyAsync(h->x.p, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
-  CK(cudaMemcpyAsync(h->types.p, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
-  launch_iota(N, h->perm.p, s);
   h->N = N;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h));
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
   if (rc) return rc;
   // candidates: atoms per CTA of both kernels, then (for a population) members per launch
   const int est = ((h->KR + 2) + 3) / 4 * 4;
@@ -1756,13 +1730,13 @@ int nep_descriptors(nep_handle *h, int n_atoms, const double *pos, const int *ty
   if (n_atoms == 0) return NEP_OK;
   if (!pos || !types || !q) return fail(h, NEP_ERR_ARG, "null pointer");
   h->md_ready = false;
-  int rc = load_structure(h, n_atoms, pos, types, box, s);
-  if (rc) return rc;
-  AtomArgs a = make_args(h, n_atoms);
-  a.q_out = q;
-  cudaError_t e = h->ops->atom(a, h->mf, 1, s);
-  if (e != cudaSuccess) return cuda_fail(h, e, "descriptor kernel");
-  return NEP_OK;
+  return load_structure(h, n_atoms, pos, types, box, s, 0, [&]() -> int {
+    AtomArgs a = make_args(h, n_atoms);
+    a.q_out = q;
+    a.guard = h->status.p;
+    const cudaError_t e = h->ops->atom(a, h->mf, 1, s);
+    return e == cudaSuccess ? NEP_OK : cuda_fail(h, e, "descriptor kernel");
+  });
 }
 
 int nep_compute_host(nep_handle *h, int n_atoms, const double *pos, const int *types, const double *box, double *energy,
@@ -1825,9 +1799,9 @@ int md_init(nep_handle *h, int n_atoms, const double *pos, const int *types, con
   if (rc) return rc;
   if (vel) CK(cudaMemcpyAsync(h->v.p, vel, sizeof(double) * 3 * n_atoms, cudaMemcpyDeviceToDevice, s), "copy vel");
   else CK(cudaMemsetAsync(h->v.p, 0, sizeof(double) * 3 * n_atoms, s), "memset vel");
-  rc = load_structure(h, n_atoms, pos, types, box, s, 1);
-  if (rc) return rc;
-  rc = run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false, 0);
+  rc = load_structure(h, n_atoms, pos, types, box, s, 1, [&]() -> int {
+    return run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false, 0);
+  });
   if (rc) return rc;
   CK(wait_stream(s), "md_init");
   h->h_status->n_rebuilds = 0;
@@ -1900,7 +1874,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     CK(cudaStreamBeginCaptureToGraph(h->cap_stream2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
        "capture body");
     cudaError_t e = launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
-                                   atom_state(h), list_bufs(h), 0, 1, h->status.p, h->cap_stream2);
+                                   atom_state(h), list_bufs(h), 0, 1, LoadSrc{}, h->status.p, h->cap_stream2);
     cudaGraph_t out = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream2, &out);
     if (e != cudaSuccess) return cuda_fail(h, e, "launch rebuild");
@@ -1910,7 +1884,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     h->rebuild_kernels = (int)nn;
   } else {
     CK(launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
-                      list_bufs(h), 0, 1, h->status.p, s),
+                      list_bufs(h), 0, 1, LoadSrc{}, h->status.p, s),
        "launch rebuild");
     h->rebuild_kernels = 0;
   }
@@ -1925,7 +1899,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
   if (ts) launch_thermostat(N, atom_state(h), h->ops->gather_blocks(N), h->partial_gather.p, ts, s);
   launch_finalize(h->ops->atom_blocks(N), h->partial_atom.p, h->ops->gather_blocks(N), h->partial_gather.p, sums,
                   nullptr, nullptr, nullptr, h->thermo_stage.p, h->thermo_ctl.p, N, h->volume, ts, h->fin_scratch.p,
-                  h->fin_ticket.p, s);
+                  h->fin_ticket.p, nullptr, s);
   if (fire) launch_fire_mix(N, atom_state(h), fs, 0, s);
   ev_record(h, SLOT_FINAL, 1, s, capturing);
   CK(cudaGetLastError(), "md step launch");
@@ -2164,21 +2138,22 @@ int nep_heat_current(nep_handle *h, int n_atoms, const double *pos, const int *t
     return fail(h, NEP_ERR_ARG, "need atoms, velocities and an output");
   cudaStream_t s = (cudaStream_t)stream;
   h->md_ready = false;
-  int rc = load_structure(h, n_atoms, pos, types, box, s);
-  if (rc) return rc;
-  AtomArgs a = make_args(h, n_atoms);
-  a.vel_in = vel;
-  a.heat = heat;
-  a.sums = heat_total ? kSumJ : 0;
-  cudaError_t e = h->ops->atom(a, h->mf, 0, s);
-  if (e == cudaSuccess) e = h->ops->gather(a, s);
-  if (e != cudaSuccess) return cuda_fail(h, e, "heat current kernels");
-  if (a.sums)
-    launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
-                    h->partial_gather.p, a.sums, nullptr, nullptr, heat_total, nullptr, nullptr, n_atoms, h->volume,
-                    nullptr, h->fin_scratch.p, h->fin_ticket.p, s);
-  CK(cudaGetLastError(), "heat current");
-  return NEP_OK;
+  return load_structure(h, n_atoms, pos, types, box, s, 0, [&]() -> int {
+    AtomArgs a = make_args(h, n_atoms);
+    a.vel_in = vel;
+    a.heat = heat;
+    a.sums = heat_total ? kSumJ : 0;
+    a.guard = h->status.p;
+    cudaError_t e = h->ops->atom(a, h->mf, 0, s);
+    if (e == cudaSuccess) e = h->ops->gather(a, s);
+    if (e != cudaSuccess) return cuda_fail(h, e, "heat current kernels");
+    if (a.sums)
+      launch_finalize(h->ops->atom_blocks(n_atoms), h->partial_atom.p, h->ops->gather_blocks(n_atoms),
+                      h->partial_gather.p, a.sums, nullptr, nullptr, heat_total, nullptr, nullptr, n_atoms, h->volume,
+                      nullptr, h->fin_scratch.p, h->fin_ticket.p, h->status.p, s);
+    CK(cudaGetLastError(), "heat current");
+    return NEP_OK;
+  });
 }
 
 int fire_run(nep_handle *h, int n_steps, double dt0_fs, double fmax, double *thermo, int *steps_taken,

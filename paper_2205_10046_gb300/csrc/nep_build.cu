@@ -53,22 +53,15 @@ __global__ void zero_cells_kernel(int ncell, int *count, int *cursor, unsigned l
   }
 }
 
-__global__ void bin_atoms_kernel(int N, int T, AtomState a, int *count, const Grid g0, const Batch B,
-                                 BuildStatus *st) {
-  if (!rebuild_pending(st)) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  if (kept_by_build(B, st, i)) {  // counted in its old cell: its structure's order stays
-    atomicAdd(count + a.cell_of[i], 1);
-    return;
-  }
-  const Grid &g = grid_of(B, g0, i);
-  double *x = a.x + 3 * (size_t)i;
-  double r[3] = {x[0], x[1], x[2]};
-  const int ti = a.types[i];
-  if (ti < 0 || ti >= T) {
+// Validates position r and type ti of an atom (flags in st; replaced by 0), wraps r into the cell
+// (FP64; only atoms outside it are moved, so a position is not re-rounded by every build) and
+// returns its cell. *moved: r or ti changed.
+__device__ __forceinline__ int bin_position(const Grid &g, int T, double *r, int *ti, bool *moved, BuildStatus *st) {
+  *moved = false;
+  if (*ti < 0 || *ti >= T) {
     atomicOr(&st->bad_input, 1);
-    a.types[i] = 0;
+    *ti = 0;
+    *moved = true;
   }
   bool inside = true;
   if (!isfinite(r[0]) || !isfinite(r[1]) || !isfinite(r[2])) {
@@ -86,10 +79,85 @@ __global__ void bin_atoms_kernel(int N, int T, AtomState a, int *count, const Gr
     const int cb = (int)(s[b] * g.nc[b]);
     c[b] = cb < 0 ? 0 : (cb >= g.nc[b] ? g.nc[b] - 1 : cb);
   }
-  // only atoms outside the cell are moved (a position is not re-rounded by every build)
-  if (!inside)
-    for (int b = 0; b < 3; ++b) x[b] = s[0] * g.H[0][b] + s[1] * g.H[1][b] + s[2] * g.H[2][b];
-  const int id = g.cell_off + (c[0] * g.nc[1] + c[1]) * g.nc[2] + c[2];
+  if (!inside) {
+    for (int b = 0; b < 3; ++b) r[b] = s[0] * g.H[0][b] + s[1] * g.H[1][b] + s[2] * g.H[2][b];
+    *moved = true;
+  }
+  return g.cell_off + (c[0] * g.nc[1] + c[1]) * g.nc[2] + c[2];
+}
+
+// Writes the coordinates of internal atom p derived from its position r and cell gid:
+// reference position, cell origin, cell-local and cell-frame FP32 coordinates.
+__device__ __forceinline__ void commit_position(const Grid &g, int gid, int tag, const double *r, size_t p,
+                                                const AtomState &a) {
+  const int id = gid - g.cell_off;
+  const int c0 = id / (g.nc[1] * g.nc[2]), c1 = (id / g.nc[2]) % g.nc[1], c2 = id % g.nc[2];
+  double o[3];
+  for (int b = 0; b < 3; ++b) {
+    o[b] = c0 * g.Hc[0][b] + c1 * g.Hc[1][b] + c2 * g.Hc[2][b];
+    a.x[3 * p + b] = r[b];
+    a.x_ref[3 * p + b] = r[b];
+    a.origin[3 * p + b] = o[b];
+  }
+  a.pos4[p] = make_float4((float)(r[0] - o[0]), (float)(r[1] - o[1]), (float)(r[2] - o[2]), __int_as_float(tag));
+  a.posA[p] = make_float4((float)r[0], (float)r[1], (float)r[2], __int_as_float(tag));
+}
+
+__device__ __forceinline__ void arm_status(BuildStatus *st) {
+  st->overflow = 0;
+  st->max_r = 0;
+  st->max_a = 0;
+  st->rev_missing = 0;
+  st->bad_input = 0;
+  st->tc_timeout = 0;
+  st->rebuild = 1;
+  st->full = 1;
+}
+
+// Shift vector of image code `code` (zero for codes outside the range); the explicitly rounded
+// FP64 operations give the same values on every path that forms the table.
+__device__ __forceinline__ float4 shift_vector(const Grid &g, int code) {
+  const int om = (1 << g.obits) - 1;
+  const int o[3] = {(code & om) - g.R[0], ((code >> g.obits) & om) - g.R[1], ((code >> (2 * g.obits)) & om) - g.R[2]};
+  if (abs(o[0]) > g.R[0] || abs(o[1]) > g.R[1] || abs(o[2]) > g.R[2]) return make_float4(0.f, 0.f, 0.f, 0.f);
+  double d[3];
+  for (int b = 0; b < 3; ++b)
+    d[b] = __dadd_rn(__dadd_rn(__dmul_rn(o[0], g.Hc[0][b]), __dmul_rn(o[1], g.Hc[1][b])), __dmul_rn(o[2], g.Hc[2][b]));
+  return make_float4((float)d[0], (float)d[1], (float)d[2], 0.f);
+}
+
+// Takes a structure over from the caller: positions, types, caller order, the shift table of a
+// single structure (src.dtab), and a forced build requested.
+__global__ void load_kernel(int N, const LoadSrc src, AtomState a, const Grid g, BuildStatus *st) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) arm_status(st);
+  if (src.dtab)
+    for (int c = i; c < g.ncode; c += gridDim.x * blockDim.x) src.dtab[c] = shift_vector(g, c);
+  for (int k = i; k < 3 * N; k += gridDim.x * blockDim.x) a.x[k] = src.pos[k];
+  for (int k = i; k < N; k += gridDim.x * blockDim.x) {
+    a.types[k] = src.types[k];
+    a.perm[k] = k;
+  }
+}
+
+__global__ void bin_atoms_kernel(int N, int T, AtomState a, int *count, const Grid g0, const Batch B,
+                                 BuildStatus *st) {
+  if (!rebuild_pending(st)) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  if (kept_by_build(B, st, i)) {  // counted in its old cell: its structure's order stays
+    atomicAdd(count + a.cell_of[i], 1);
+    return;
+  }
+  double *x = a.x + 3 * (size_t)i;
+  double r[3] = {x[0], x[1], x[2]};
+  int ti = a.types[i];
+  bool moved;
+  const int id = bin_position(grid_of(B, g0, i), T, r, &ti, &moved, st);
+  if (moved) {
+    a.types[i] = ti;
+    for (int b = 0; b < 3; ++b) x[b] = r[b];
+  }
   a.cell_of[i] = id;
   atomicAdd(count + id, 1);
 }
@@ -190,17 +258,10 @@ __global__ void reorder_commit_kernel(int N, AtomState a, int move, const Grid g
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= N || kept_by_build(B, st, p)) return;
   // cells are numbered structure by structure, so atom p stays inside its structure's range
-  const Grid &g = grid_of(B, g0, p);
   const int gid = a.cell2[p];
-  const int id = gid - g.cell_off;
-  const int c0 = id / (g.nc[1] * g.nc[2]), c1 = (id / g.nc[2]) % g.nc[1], c2 = id % g.nc[2];
-  double r[3], o[3];
+  double r[3];
   for (int b = 0; b < 3; ++b) {
     r[b] = a.x2[3 * (size_t)p + b];
-    o[b] = c0 * g.Hc[0][b] + c1 * g.Hc[1][b] + c2 * g.Hc[2][b];
-    a.x[3 * (size_t)p + b] = r[b];
-    a.x_ref[3 * (size_t)p + b] = r[b];
-    a.origin[3 * (size_t)p + b] = o[b];
     if (move & 1) a.v[3 * (size_t)p + b] = a.v2[3 * (size_t)p + b];
     if (move & 2) a.F[3 * (size_t)p + b] = a.F2[3 * (size_t)p + b];
   }
@@ -208,10 +269,116 @@ __global__ void reorder_commit_kernel(int N, AtomState a, int move, const Grid g
   a.types[p] = t;
   a.perm[p] = a.perm2[p];
   a.cell_of[p] = gid;
-  const int sidp = B.grids ? B.sid[p] : 0;
-  a.pos4[p] = make_float4((float)(r[0] - o[0]), (float)(r[1] - o[1]), (float)(r[2] - o[2]),
-                          __int_as_float(t | (sidp << 8)));
-  a.posA[p] = make_float4((float)r[0], (float)r[1], (float)r[2], __int_as_float(t | (sidp << 8)));
+  commit_position(grid_of(B, g0, p), gid, t | ((B.grids ? B.sid[p] : 0) << 8), r, p, a);
+}
+
+// The steps above (load, zero, bin, scan, scatter, reorder, commit) for a small system in one
+// block: counts, cell starts and the cells' atoms stay in shared memory, every thread keeps its
+// atoms' data in registers until all places are known. Bound by launches and latency: seven
+// launches of 2 to 6 us each become one. With the status read only once, behind the force kernels
+// (rebuild_lists), the neighbour build of a call takes 48 us instead of 97 for 216 Si atoms; the
+// general path, which shares that and the load kernel, 77 instead of 113 us for 4,999 atoms.
+// Above 2,048 atoms the one block's FP64 work (16 cycles of its SM per warp instruction) outgrows
+// the launches it saves.
+constexpr int kSmallBuild = 2048;       // atoms at most: two per thread
+constexpr int kSmallBuildCells = 8192;  // cells at most: eight per thread
+__global__ void __launch_bounds__(1024)
+    small_build_kernel(int N, int T, const LoadSrc src, AtomState a, const ListBufs L, int move, const Grid g0,
+                       const Batch B, int ncell, BuildStatus *st) {
+  if (!src.pos && !rebuild_pending(st)) return;
+  extern __shared__ int sb[];
+  int *const start = sb, *const cursor = start + ncell + 1, *const order = cursor + ncell;  // order [N]
+  __shared__ int wsum[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (src.pos) {
+    if (tid == 0) arm_status(st);
+    if (src.dtab)
+      for (int c = tid; c < g0.ncode; c += 1024) src.dtab[c] = shift_vector(g0, c);
+  }
+  for (int k = tid; k < 4 * kStatSlots; k += 1024) L.part[k] = 0ull;
+  for (int c = tid; c < ncell; c += 1024) start[c] = cursor[c] = 0;
+  __syncthreads();
+  const bool part_build = !src.pos && B.sflag && !*(volatile const int *)&st->full;
+  double r[2][3], v[2][3], F[2][3];
+  int ti[2], pm[2], gid[2];
+  bool mv[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int i = tid + 1024 * u;
+    mv[u] = false;
+    if (i >= N) continue;
+    mv[u] = !(part_build && B.sflag[B.sid[i]] == 0);
+    if (!mv[u]) {  // its structure's order stays
+      atomicAdd(start + a.cell_of[i], 1);
+      continue;
+    }
+    const double *x = src.pos ? src.pos : a.x;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      r[u][b] = x[3 * (size_t)i + b];
+      if (move & 1) v[u][b] = a.v[3 * (size_t)i + b];
+      if (move & 2) F[u][b] = a.F[3 * (size_t)i + b];
+    }
+    ti[u] = src.pos ? src.types[i] : a.types[i];
+    pm[u] = src.pos ? i : a.perm[i];
+    bool moved;
+    gid[u] = bin_position(grid_of(B, g0, i), T, r[u], &ti[u], &moved, st);
+    atomicAdd(start + gid[u], 1);
+  }
+  __syncthreads();
+  // exclusive prefix sum of the counts: eight cells per thread
+  int c8[8], tot = 0;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    c8[k] = 8 * tid + k < ncell ? start[8 * tid + k] : 0;
+    tot += c8[k];
+  }
+  int x = tot;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[wid] = x;
+  __syncthreads();
+  if (wid == 0) {
+    int y = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int z = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += z;
+    }
+    wsum[lane] = y;
+  }
+  __syncthreads();
+  int at = (wid > 0 ? wsum[wid - 1] : 0) + (x - tot);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    if (8 * tid + k < ncell) start[8 * tid + k] = L.cell_start[8 * tid + k] = at;
+    at += c8[k];
+  }
+  if (tid == 0) start[ncell] = L.cell_start[ncell] = N;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (mv[u]) order[start[gid[u]] + atomicAdd(cursor + gid[u], 1)] = tid + 1024 * u;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    if (!mv[u]) continue;
+    const int i = tid + 1024 * u, b0 = start[gid[u]], b1 = start[gid[u] + 1];
+    int p = b0;  // the cell's atoms in index order
+    for (int q = b0; q < b1; ++q) p += order[q] < i ? 1 : 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      if (move & 1) a.v[3 * (size_t)p + b] = v[u][b];
+      if (move & 2) a.F[3 * (size_t)p + b] = F[u][b];
+    }
+    a.types[p] = ti[u];
+    a.perm[p] = pm[u];
+    a.cell_of[p] = gid[u];
+    commit_position(grid_of(B, g0, p), gid[u], ti[u] | ((B.grids ? B.sid[p] : 0) << 8), r[u], p, a);
+  }
 }
 
 // floor(x / n) and the remainder, for n >= 1 and x > -n * 8
@@ -699,11 +866,6 @@ __global__ void rebuild_condition_kernel(cudaGraphConditionalHandle hc, const Bu
   cudaGraphSetConditional(hc, *(volatile const int *)&st->rebuild != 0 ? 1u : 0u);
 }
 
-__global__ void iota_kernel(int N, int *perm) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < N) perm[i] = i;
-}
-
 // Velocity Verlet, first half: v += dt/2 F/m; x += dt v; refresh cell-local coordinates;
 // request a rebuild when an atom moved more than skin/2 since the last build.
 // With a FIRE state, its time step is used and a converged relaxation stays where it is.
@@ -775,7 +937,8 @@ __global__ void __launch_bounds__(32 * kReduceSlots)
     finalize_kernel(int nb_atom, const double *partial_atom, int nb_gather, const double *partial_gather, int sums,
                     double *energy_total, double *virial_total, double *heat_total, double *thermo_stage,
                     int *thermo_ctl /* [0] step-in-call, [1] rows written, [2] every */, double t_fac, double p_fac,
-                    const ThermoState *ts, double *scratch, int *ticket) {
+                    const ThermoState *ts, double *scratch, int *ticket, const BuildStatus *guard) {
+  if (build_failed(guard)) return;
   if (thermo_ctl && thermo_ctl[0] % thermo_ctl[2] != 0) return;
   __shared__ double tot[kReduceSlots];
   __shared__ int last;
@@ -889,21 +1052,11 @@ __global__ void struct_ids_kernel(int n_struct, const int *offsets, int *sid) {
 }
 
 // Shift vector of every image code of every structure (zero for codes outside the range).
-__global__ void shift_tables_kernel(int n_struct, const Grid *grids, int ncode, int obits, float4 *dtab) {
+__global__ void shift_tables_kernel(int n_struct, const Grid *grids, int ncode, float4 *dtab) {
   const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= (long long)n_struct * ncode) return;
   const int s = (int)(v / ncode), code = (int)(v % ncode);
-  const Grid &g = grids[s];
-  const int om = (1 << obits) - 1;
-  const int o[3] = {(code & om) - g.R[0], ((code >> obits) & om) - g.R[1], ((code >> (2 * obits)) & om) - g.R[2]};
-  float4 D = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (abs(o[0]) <= g.R[0] && abs(o[1]) <= g.R[1] && abs(o[2]) <= g.R[2]) {
-    double d[3];
-    for (int b = 0; b < 3; ++b)
-      d[b] = __dadd_rn(__dadd_rn(__dmul_rn(o[0], g.Hc[0][b]), __dmul_rn(o[1], g.Hc[1][b])), __dmul_rn(o[2], g.Hc[2][b]));
-    D = make_float4((float)d[0], (float)d[1], (float)d[2], 0.f);
-  }
-  dtab[g.dtab_off + code] = D;
+  dtab[grids[s].dtab_off + code] = shift_vector(grids[s], code);
 }
 
 // Per-structure sums E_s = sum U_i and W_s = sum W_i (FP64, fixed order). A structure of at
@@ -980,16 +1133,7 @@ __global__ void struct_sums_kernel(int n_struct, int members, const int *offsets
 
 // Marks a rebuild as pending and clears the per-build flags (the device form of the host
 // reset before a forced rebuild, for captured graphs).
-__global__ void arm_rebuild_kernel(BuildStatus *st) {
-  st->overflow = 0;
-  st->max_r = 0;
-  st->max_a = 0;
-  st->rev_missing = 0;
-  st->bad_input = 0;
-  st->tc_timeout = 0;
-  st->rebuild = 1;
-  st->full = 1;
-}
+__global__ void arm_rebuild_kernel(BuildStatus *st) { arm_status(st); }
 
 // ------------------------------------------------------------------ population evaluation
 // Candidate parameter vectors z [P][N_par], in the order c^R, c^A, w0, b0, w1, b1, become
@@ -1123,9 +1267,9 @@ void launch_struct_ids(int n_struct, const int *offsets, int *sid, cudaStream_t 
   if (n_struct > 0) struct_ids_kernel<<<n_struct, 128, 0, s>>>(n_struct, offsets, sid);
 }
 
-void launch_shift_tables(int n_struct, const Grid *grids, int ncode, int obits, float4 *dtab, cudaStream_t s) {
+void launch_shift_tables(int n_struct, const Grid *grids, int ncode, float4 *dtab, cudaStream_t s) {
   const long long n = (long long)n_struct * ncode;
-  if (n > 0) shift_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n_struct, grids, ncode, obits, dtab);
+  if (n > 0) shift_tables_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n_struct, grids, ncode, dtab);
 }
 
 void launch_struct_sums(int n_struct, int members, const int *offsets, int N, const double *e_atom,
@@ -1186,16 +1330,26 @@ cudaError_t launch_lists(int N, int T, const Grid &g, const Batch &B, float rlR2
 
 cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
                            float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only, int move,
-                           BuildStatus *st, cudaStream_t s) {
+                           const LoadSrc &src, BuildStatus *st, cudaStream_t s) {
   const int tb = 256;
   const int nb = (N + tb - 1) / tb;
   const int cb = (g.ncell + tb - 1) / tb;
-  zero_cells_kernel<<<cb < 1024 ? cb : 1024, tb, 0, s>>>(g.ncell, L.cell_count, L.cell_cursor, L.part, st);
-  bin_atoms_kernel<<<nb, tb, 0, s>>>(N, T, a, L.cell_count, g, B, st);
-  scan_cells_kernel<<<1, 1024, 0, s>>>(g.ncell, L.cell_count, L.cell_start, st);
-  scatter_atoms_kernel<<<nb, tb, 0, s>>>(N, a.cell_of, L.cell_start, L.cell_cursor, L.cell_atoms, B, st);
-  reorder_gather_kernel<<<nb, tb, 0, s>>>(N, L.cell_start, L.cell_atoms, a, move, B, st);
-  reorder_commit_kernel<<<nb, tb, 0, s>>>(N, a, move, g, B, st);
+  if (N <= kSmallBuild && g.ncell <= kSmallBuildCells) {
+    const cudaError_t e = smem_limit_once(small_build_kernel, sizeof(int) * (2 * kSmallBuildCells + 1 + kSmallBuild));
+    if (e != cudaSuccess) return e;
+    small_build_kernel<<<1, 1024, sizeof(int) * (2 * g.ncell + 1 + N), s>>>(N, T, src, a, L, move, g, B, g.ncell, st);
+  } else {
+    if (src.pos) {
+      const int lb = (3LL * N + tb - 1) / tb < 8 * 152 ? (int)((3LL * N + tb - 1) / tb) : 8 * 152;
+      load_kernel<<<lb, tb, 0, s>>>(N, src, a, g, st);
+    }
+    zero_cells_kernel<<<cb < 1024 ? cb : 1024, tb, 0, s>>>(g.ncell, L.cell_count, L.cell_cursor, L.part, st);
+    bin_atoms_kernel<<<nb, tb, 0, s>>>(N, T, a, L.cell_count, g, B, st);
+    scan_cells_kernel<<<1, 1024, 0, s>>>(g.ncell, L.cell_count, L.cell_start, st);
+    scatter_atoms_kernel<<<nb, tb, 0, s>>>(N, a.cell_of, L.cell_start, L.cell_cursor, L.cell_atoms, B, st);
+    reorder_gather_kernel<<<nb, tb, 0, s>>>(N, L.cell_start, L.cell_atoms, a, move, B, st);
+    reorder_commit_kernel<<<nb, tb, 0, s>>>(N, a, move, g, B, st);
+  }
   // Warp per atom up to kWideBuildAtoms atoms, thread per atom above: a small system leaves the
   // thread form with a few long serial scans, a large one makes the warp form pay for its idle
   // lanes (ranges of ~20 candidates). Whole neighbour build, thread / warp form, us: 216 Si atoms
@@ -1214,8 +1368,6 @@ cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const fl
 void launch_rebuild_condition(cudaGraphConditionalHandle hc, const BuildStatus *st, cudaStream_t s) {
   rebuild_condition_kernel<<<1, 1, 0, s>>>(hc, st);
 }
-
-void launch_iota(int N, int *perm, cudaStream_t s) { iota_kernel<<<(N + 255) / 256, 256, 0, s>>>(N, perm); }
 
 void launch_drift(int N, const AtomState &a, const double *inv_mass_kappa, double dt, double half_skin2,
                   BuildStatus *st, cudaStream_t s, const FireState *fire, int *step_ctl) {
@@ -1510,7 +1662,7 @@ void launch_export(int N, const AtomState &a, const Grid &g, const Batch &B, dou
 void launch_finalize(int nb_atom, const double *partial_atom, int nb_gather, const double *partial_gather, int sums,
                      double *energy_total, double *virial_total, double *heat_total, double *thermo_stage,
                      int *thermo_ctl, int N, double volume, const ThermoState *ts, double *scratch, int *ticket,
-                     cudaStream_t s) {
+                     const BuildStatus *guard, cudaStream_t s) {
   const double kb = 8.617333262e-5;
   const double t_fac = N > 1 ? 2.0 / ((3.0 * N - 3.0) * kb) : 0.0;
   const double p_fac = 160.21766208 / (3.0 * volume);  // eV/A^3 -> GPa
@@ -1519,7 +1671,7 @@ void launch_finalize(int nb_atom, const double *partial_atom, int nb_gather, con
   blocks = blocks < 1 ? 1 : blocks > kFinalBlocks ? kFinalBlocks : blocks;
   finalize_kernel<<<blocks, 32 * kReduceSlots, 0, s>>>(nb_atom, partial_atom, nb_gather, partial_gather, sums,
                                                        energy_total, virial_total, heat_total, thermo_stage, thermo_ctl,
-                                                       t_fac, p_fac, ts, scratch, ticket);
+                                                       t_fac, p_fac, ts, scratch, ticket, guard);
 }
 
 }  // namespace nep

@@ -52,6 +52,7 @@ __device__ __forceinline__ int n_poly(int L3, int L4) {
 
 template <bool DESC_ONLY, bool BATCH>
 __global__ void __launch_bounds__(128) generic_atom_kernel(const AtomArgs a, const ModelF mf) {
+  if (!BATCH && build_failed(a.guard)) return;
   const int N = a.N, T = a.T;
   const int nR = a.gR, KR = a.gKR, nA = a.gA, KA = a.gKA, H = a.gH, L3 = a.gL3, L4 = a.gL4, L5 = a.gL5, D = a.gD;
   const int NK = n_poly(L3, L4);
@@ -265,6 +266,7 @@ __global__ void __launch_bounds__(128) generic_atom_kernel(const AtomArgs a, con
 // compiled gather kernel's.
 template <bool BATCH>
 __global__ void __launch_bounds__(128) generic_gather_kernel(const AtomArgs a) {
+  if (!BATCH && build_failed(a.guard)) return;
   const int mem = BATCH ? (int)blockIdx.y : 0;
   const float *e_rad = a.e_rad + mem * a.s_erad;
   const float4 *p_ang = a.p_ang + mem * a.s_pang;

@@ -66,6 +66,14 @@ struct AtomState {
   int *types2, *perm2, *cell2;         // reorder scratch [N]
 };
 
+// A structure as the caller holds it (device arrays), taken over at the start of a build; pos ==
+// nullptr: the build uses the atoms in place. dtab: shift table to fill (one structure), or null.
+struct LoadSrc {
+  const double *pos = nullptr;
+  const int *types = nullptr;
+  float4 *dtab = nullptr;
+};
+
 // Cell list and neighbour lists.
 struct ListBufs {
   int *cell_count, *cell_cursor, *cell_start, *cell_atoms;
@@ -217,6 +225,7 @@ struct AtomArgs {
   double *vel;             // [N][3]
   int precision;           // network: 0 FP32 on the FMA pipes; 1 BF16, 2 split BF16 on the tensor cores
   int *tc_err;             // set when a tensor-core wait ran out
+  const BuildStatus *guard;  // of the build queued before this launch (build_failed), or null
   // Batched kernels only. dtab then holds ncode shift vectors per structure (the structure
   // index sits in pos4.w above the type bits), and blockIdx.y selects the member of a
   // population whose coefficients and network the block uses; every per-member array is
@@ -235,6 +244,12 @@ struct AtomArgs {
   // without a compiled instantiation)
   int gR, gKR, gA, gKA, gH, gL3, gL4, gL5, gD;
 };
+
+// The build before this launch failed (the host, which has not looked yet, reports it or builds
+// again): kernels queued behind it write nothing.
+__device__ __forceinline__ bool build_failed(const BuildStatus *st) {
+  return st && (st->overflow | st->bad_input | st->rev_missing);
+}
 
 // The block sums that this launch forms.
 __device__ __forceinline__ int sums_needed(const AtomArgs &a) {
@@ -333,11 +348,10 @@ __host__ __device__ inline int tile_place(const TableLayout &t, int mu, int nu) 
 // Host helpers shared by the handle-based and the static-scratch entry points.
 struct Grid;
 void model_constants(ModelF &m);
-int build_grid(const double *box, double rl, int N, Grid &g, float4 *dtab, double *volume, const char **err);
+int build_grid(const double *box, double rl, int N, Grid &g, double *volume, const char **err);
 cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
                            float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only,
-                           int move, BuildStatus *st, cudaStream_t s);
-void launch_iota(int N, int *perm, cudaStream_t s);
+                           int move, const LoadSrc &src, BuildStatus *st, cudaStream_t s);
 void launch_export(int N, const AtomState &a, const Grid &g, const Batch &B, double *pos, double *vel, double *force,
                    cudaStream_t s);
 void launch_export_lists(int N, int T, const float4 *pos4, const int *perm, const ListBufs &L, const float4 *dtab,
@@ -346,7 +360,7 @@ void launch_export_lists(int N, int T, const float4 *pos4, const int *perm, cons
 // batches: structure index of every atom, the shift tables of all structures, and the
 // per-structure sums of per-atom energies and virials (caller order, per member)
 void launch_struct_ids(int n_struct, const int *offsets, int *sid, cudaStream_t s);
-void launch_shift_tables(int n_struct, const Grid *grids, int ncode, int obits, float4 *dtab, cudaStream_t s);
+void launch_shift_tables(int n_struct, const Grid *grids, int ncode, float4 *dtab, cudaStream_t s);
 // max_atoms: the largest structure (structures above kWideSum atoms are summed by a block)
 void launch_struct_sums(int n_struct, int members, const int *offsets, int N, const double *e_atom,
                         const double *w_atom, double *e_struct, double *w_struct, int max_atoms, cudaStream_t s);

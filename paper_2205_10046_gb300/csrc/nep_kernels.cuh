@@ -513,6 +513,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
     if (h < a.cap_a) l2_prefetch(a.nl_a + (size_t)h * N + i);
   }
   const int mem = BATCH ? (int)blockIdx.y : 0;
+  if (!BATCH && build_failed(a.guard)) return;
   using PR = PairRow<S>;
   constexpr bool TC = PR::tc(PREC);
   static_assert(!DESC || PREC == 0, "the descriptors need no network");
@@ -1264,6 +1265,7 @@ constexpr int gather_min_blocks(int KR, int threads) {
 template <class S, bool BATCH, int GA>
 __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA *kGatherLanes))
     gather_kernel(const AtomArgs a) {
+  if (!BATCH && build_failed(a.guard)) return;
   constexpr int L = kGatherLanes;
   __shared__ float fw[GA][13];
   __shared__ unsigned char on[GA];

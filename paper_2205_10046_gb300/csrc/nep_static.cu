@@ -92,12 +92,13 @@ int cuda_err(cudaError_t e, const char *where) {
   } while (0)
 
 int run_build(int N, int T, const Grid &g, const float4 *dtab, float rlR2, float rlA2, float rcR2, float rcA2,
-              const AtomState &a, const ListBufs &L, int count_only, BuildStatus *st_dev, BuildStatus *st_host,
-              cudaStream_t s) {
+              const AtomState &a, const ListBufs &L, int count_only, const LoadSrc &src, BuildStatus *st_dev,
+              BuildStatus *st_host, cudaStream_t s) {
   std::memset(st_host, 0, sizeof(BuildStatus));
   st_host->rebuild = 1;
   SK(cudaMemcpyAsync(st_dev, st_host, sizeof(BuildStatus), cudaMemcpyHostToDevice, s), "status");
-  SK(launch_rebuild(N, T, g, Batch{}, dtab, rlR2, rlA2, rcR2, rcA2, a, L, count_only, 0, st_dev, s), "neighbour build");
+  SK(launch_rebuild(N, T, g, Batch{}, dtab, rlR2, rlA2, rcR2, rcA2, a, L, count_only, 0, src, st_dev, s),
+     "neighbour build");
   SK(cudaMemcpyAsync(st_host, st_dev, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   SK(cudaStreamSynchronize(s), "synchronise");
   if (st_host->bad_input & 1) return fail_static(NEP_ERR_ARG, "atom type out of range");
@@ -139,10 +140,9 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   model_constants(mf);
 
   Grid g;
-  float4 dtab_h[512];
   double volume = 0;
   const char *gerr = nullptr;
-  rc = build_grid(box, params->rc_radial + skin, N, g, dtab_h, &volume, &gerr);
+  rc = build_grid(box, params->rc_radial + skin, N, g, &volume, &gerr);
   if (rc) return fail_static(rc, gerr);
 
   unsigned char *base = nullptr;
@@ -184,21 +184,18 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
     return fail_static(NEP_ERR_ARG, "structure too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
 
   // inputs into the arena; the arena keeps the previous call's contents, so everything the
-  // kernels read is written here first (the builder clears the cell counters itself)
-  SK(cudaMemcpyAsync(dtab, dtab_h, sizeof(float4) * g.ncode, cudaMemcpyHostToDevice, s), "copy");
+  // kernels read is written first, here or by the build (positions, types, order, shift table,
+  // cell counters)
   SK(cudaMemcpyAsync(dtabm, tab, sizeof(float) * tl.total, cudaMemcpyHostToDevice, s), "copy");
-  SK(cudaMemcpyAsync(a.x, pos, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "copy pos");
-  SK(cudaMemcpyAsync(a.types, types, sizeof(int) * N, cudaMemcpyDeviceToDevice, s), "copy types");
   SK(cudaMemsetAsync(a.v, 0, sizeof(double) * 3 * N, s), "clear");
   SK(cudaMemsetAsync(a.F, 0, sizeof(double) * 3 * N, s), "clear");
-  launch_iota(N, a.perm, s);
-  SK(cudaGetLastError(), "iota");
 
   const float rlR = (float)(params->rc_radial + skin), rlA = (float)(params->rc_angular + skin);
   const float rcR = (float)params->rc_radial, rcA = (float)params->rc_angular;
   BuildStatus host_st;
   // sizing pass, then the lists
-  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, st, &host_st, s);
+  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, LoadSrc{pos, types, dtab}, st,
+                 &host_st, s);
   if (rc) return rc;
   // the same per-atom list limit, with the same error, as the handle-based entry points
   if (host_st.max_r > kListBuf || host_st.max_a > kListBuf)
@@ -210,7 +207,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.rev_a = arena.take<int>((size_t)L.cap_a * N);
   if (!L.nl_r || !L.nl_a || !L.rev_a)
     return fail_static(NEP_ERR_ARG, "neighbour lists too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
-  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 0, st, &host_st, s);
+  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 0, LoadSrc{}, st, &host_st, s);
   if (rc) return rc;
   if (host_st.overflow || host_st.rev_missing) return fail_static(NEP_ERR_NEIGHBOR_OVERFLOW, "neighbour build failed");
 
