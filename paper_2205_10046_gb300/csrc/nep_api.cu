@@ -1143,8 +1143,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   e = h->ops->atom_batch(a, h->mf, 1, atom_block(h), s);
   if (e == cudaSuccess) e = h->ops->gather_batch(a, 1, gather_block(h), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine kernels");
-  launch_engine_fire(S, h->d_offsets.p, atom_state(h), h->e_slots.p, s);
-  launch_engine_advance(S, h->e_slots.p, s);
+  launch_engine_advance(S, h->d_offsets.p, atom_state(h), h->e_slots.p, s);
   CK(cudaGetLastError(), "engine step");
   return NEP_OK;
 }

@@ -23,6 +23,8 @@
 // far (per-structure flags); the others keep their cells, atom order, lists and x_ref.
 #include <cuda_bf16.h>
 
+#include <cooperative_groups.h>
+
 #include "nep_internal.cuh"
 
 namespace nep {
@@ -1374,78 +1376,110 @@ void launch_drift(int N, const AtomState &a, const double *inv_mass_kappa, doubl
   md_drift_kernel<<<(N + 255) / 256, 256, 0, s>>>(N, a, inv_mass_kappa, dt, half_skin2, st, fire, step_ctl);
 }
 
-// FIRE velocity mixing after a velocity-Verlet step (Bitzek et al. 2006), one block, FP64
-// sums in a fixed order: P = F . v, |F|, |v| over all atoms and max_i |F_i|^2. Converged
-// when max_i |F_i| < fmax (then nothing moves again). Otherwise, for P > 0:
-// v <- (1 - alpha) v + alpha |v| F / |F|, and after more than N_min such steps in a row the
-// step grows (dt <- min(f_inc dt, dt_max)) and alpha shrinks (alpha <- f_alpha alpha); for
-// P <= 0: v <- 0, dt <- f_dec dt, alpha <- alpha_start. check_only: only the convergence test
-// (for the starting forces).
+// FIRE velocity mixing after a velocity-Verlet step (Bitzek et al. 2006), FP64 sums in a fixed
+// order: P = F . v, |F|, |v| over all atoms and max_i |F_i|^2. Converged when max_i |F_i| < fmax
+// (then nothing moves again). Otherwise, for P > 0: v <- (1 - alpha) v + alpha |v| F / |F|, and
+// after more than N_min such steps in a row the step grows (dt <- min(f_inc dt, dt_max)) and
+// alpha shrinks (alpha <- f_alpha alpha); for P <= 0: v <- 0, dt <- f_dec dt, alpha <-
+// alpha_start. check_only: only the convergence test (for the starting forces).
+//
+// One cluster of 8 CTAs takes the atoms [b0, b1) of one relaxation; the CTAs read each other's
+// four sums from shared memory. Bound by the FP64 pipe (16 cycles of its SM per warp
+// instruction), which is why one CTA is not enough: 1,001 atoms 17.5 us in one CTA of 1024 threads,
+// now 5; the serving engine's jobs (up to 4,000 atoms) 21 us in one CTA each.
 constexpr int kFireNmin = 5;
 constexpr double kFireFinc = 1.1, kFireFdec = 0.5, kFireAlphaStart = 0.1, kFireFalpha = 0.99;
+constexpr int kFireCluster = 8;
 
-__global__ void fire_mix_kernel(int N, AtomState a, FireState *fire, int check_only) {
-  __shared__ double red[4][1024];
-  __shared__ int decision;
-  if (fire->converged) return;
-  double p = 0.0, ff = 0.0, vv = 0.0, fm = 0.0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const double *F = a.F + 3 * (size_t)i, *v = a.v + 3 * (size_t)i;
+// Returns on thread 0 of the cluster's first CTA, and only there, the state after the step in
+// `next` (the caller writes it, now that every CTA has read the old one); converged in *done.
+__device__ __forceinline__ void fire_mix(int b0, int b1, const AtomState &a, const FireState &old, bool check_only,
+                                         FireState *next) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double red[32][4], tot[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int first = b0 + (int)cl.block_rank() * blockDim.x + tid, step = kFireCluster * blockDim.x;
+  double sum[4] = {0.0, 0.0, 0.0, 0.0};  // P, |F|^2, |v|^2, max |F_i|^2
+  double F0[3] = {0.0, 0.0, 0.0}, v0[3] = {0.0, 0.0, 0.0};  // of the thread's first atom, kept
+  for (int i = first; i < b1; i += step) {
+    double F[3], v[3];
+    for (int b = 0; b < 3; ++b) F[b] = a.F[3 * (size_t)i + b], v[b] = a.v[3 * (size_t)i + b];
     const double f2 = F[0] * F[0] + F[1] * F[1] + F[2] * F[2];
-    p += F[0] * v[0] + F[1] * v[1] + F[2] * v[2];
-    ff += f2;
-    vv += v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    fm = fmax(fm, f2);
+    sum[0] += F[0] * v[0] + F[1] * v[1] + F[2] * v[2];
+    sum[1] += f2;
+    sum[2] += v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    sum[3] = fmax(sum[3], f2);
+    if (i == first)
+      for (int b = 0; b < 3; ++b) F0[b] = F[b], v0[b] = v[b];
   }
-  red[0][threadIdx.x] = p;
-  red[1][threadIdx.x] = ff;
-  red[2][threadIdx.x] = vv;
-  red[3][threadIdx.x] = fm;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + o];
-      red[1][threadIdx.x] += red[1][threadIdx.x + o];
-      red[2][threadIdx.x] += red[2][threadIdx.x + o];
-      red[3][threadIdx.x] = fmax(red[3][threadIdx.x], red[3][threadIdx.x + o]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double y = __shfl_xor_sync(0xffffffffu, sum[k], o);
+      sum[k] = k == 3 ? fmax(sum[k], y) : sum[k] + y;
     }
-    __syncthreads();
-  }
-  const double P = red[0][0], FF = red[1][0], VV = red[2][0], FM = red[3][0];
-  if (threadIdx.x == 0) {
-    decision = 0;
-    if (!check_only) fire->steps += 1;  // velocity-Verlet steps taken
-    if (FM < fire->fmax2) fire->converged = 1;
-    else if (!check_only) decision = P > 0.0 ? 1 : 2;
+    if (lane == 0) red[warp][k] = sum[k];
   }
   __syncthreads();
-  if (decision == 0) return;
-  const double alpha = fire->alpha;
-  const double c1 = decision == 1 ? 1.0 - alpha : 0.0;
-  const double c2 = (decision == 1 && FF > 0.0) ? alpha * sqrt(VV / FF) : 0.0;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    double *v = a.v + 3 * (size_t)i;
-    const double *F = a.F + 3 * (size_t)i;
-    for (int b = 0; b < 3; ++b) v[b] = c1 * v[b] + c2 * F[b];
+  if (tid < 4) {
+    double t = red[0][tid];
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) t = tid == 3 ? fmax(t, red[w][tid]) : t + red[w][tid];
+    tot[tid] = t;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (decision == 1) {
-      if (fire->n_pos > kFireNmin) {
-        fire->dt = fmin(fire->dt * kFireFinc, fire->dt_max);
-        fire->alpha = alpha * kFireFalpha;
+  cl.sync();
+  double all[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    all[k] = *cl.map_shared_rank(&tot[k], 0);
+    for (int c = 1; c < kFireCluster; ++c) {
+      const double t = *cl.map_shared_rank(&tot[k], c);
+      all[k] = k == 3 ? fmax(all[k], t) : all[k] + t;
+    }
+  }
+  cl.sync();  // every CTA has read the others' sums (and the old state)
+  const double P = all[0], FF = all[1], VV = all[2];
+  const bool converged = all[3] < old.fmax2, mix = !converged && !check_only, up = P > 0.0;
+  const double c1 = up ? 1.0 - old.alpha : 0.0;
+  const double c2 = (up && FF > 0.0) ? old.alpha * sqrt(VV / FF) : 0.0;
+  if (mix)
+    for (int i = first; i < b1; i += step)
+      for (int b = 0; b < 3; ++b) {
+        const double v = i == first ? v0[b] : a.v[3 * (size_t)i + b], F = i == first ? F0[b] : a.F[3 * (size_t)i + b];
+        a.v[3 * (size_t)i + b] = c1 * v + c2 * F;
       }
-      fire->n_pos += 1;
-    } else {
-      fire->dt *= kFireFdec;
-      fire->alpha = kFireAlphaStart;
-      fire->n_pos = 0;
+  if (cl.block_rank() != 0 || tid != 0) return;
+  *next = old;
+  if (converged) next->converged = 1;
+  if (!mix) return;
+  if (up) {
+    if (old.n_pos > kFireNmin) {
+      next->dt = fmin(old.dt * kFireFinc, old.dt_max);
+      next->alpha = old.alpha * kFireFalpha;
     }
+    next->n_pos = old.n_pos + 1;
+  } else {
+    next->dt = old.dt * kFireFdec;
+    next->alpha = kFireAlphaStart;
+    next->n_pos = 0;
+  }
+}
+
+__global__ void __cluster_dims__(kFireCluster, 1, 1) __launch_bounds__(512)
+    fire_mix_kernel(int N, AtomState a, FireState *fire, int check_only) {
+  const FireState old = *fire;  // read before the cluster's barriers, written after them
+  if (old.converged) return;
+  FireState next;
+  fire_mix(0, N, a, old, check_only != 0, &next);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (!check_only) next.steps = old.steps + 1;  // velocity-Verlet steps taken
+    *fire = next;
   }
 }
 
 void launch_fire_mix(int N, const AtomState &a, FireState *fire, int check_only, cudaStream_t s) {
-  fire_mix_kernel<<<1, 1024, 0, s>>>(N, a, fire, check_only);
+  fire_mix_kernel<<<kFireCluster, N > kFireCluster * 128 ? 512 : 128, 0, s>>>(N, a, fire, check_only);
 }
 
 // ------------------------------------------------------------------ batched serving engine
@@ -1496,83 +1530,27 @@ __global__ void clear_flags_kernel(BuildStatus *st) {
 
 void launch_clear_flags(BuildStatus *st, cudaStream_t s) { clear_flags_kernel<<<1, 1, 0, s>>>(st); }
 
-// FIRE update of every FIRE job after its step (the FIRE definition of fire_mix_kernel, one
-// block per job over the job's own atoms [offsets[s], offsets[s+1])); at the job's first
-// iteration only the convergence test on the starting forces.
-__global__ void engine_fire_kernel(const int *offsets, AtomState a, EngineSlot *slots) {
-  const int s = blockIdx.x;
-  EngineSlot &sl = slots[s];
-  if (sl.kind != kJobFire || sl.phase == 2 || sl.fire.converged) return;
-  const bool check_only = sl.phase == 0;
-  __shared__ double red[4][256];
-  __shared__ int decision;
-  const int b0 = offsets[s], b1 = offsets[s + 1];
-  double p = 0.0, ff = 0.0, vv = 0.0, fm = 0.0;
-  for (int i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-    const double *F = a.F + 3 * (size_t)i, *v = a.v + 3 * (size_t)i;
-    const double f2 = F[0] * F[0] + F[1] * F[1] + F[2] * F[2];
-    p += F[0] * v[0] + F[1] * v[1] + F[2] * v[2];
-    ff += f2;
-    vv += v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-    fm = fmax(fm, f2);
-  }
-  red[0][threadIdx.x] = p;
-  red[1][threadIdx.x] = ff;
-  red[2][threadIdx.x] = vv;
-  red[3][threadIdx.x] = fm;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      red[0][threadIdx.x] += red[0][threadIdx.x + o];
-      red[1][threadIdx.x] += red[1][threadIdx.x + o];
-      red[2][threadIdx.x] += red[2][threadIdx.x + o];
-      red[3][threadIdx.x] = fmax(red[3][threadIdx.x], red[3][threadIdx.x + o]);
-    }
-    __syncthreads();
-  }
-  const double P = red[0][0], FF = red[1][0], VV = red[2][0], FM = red[3][0];
-  if (threadIdx.x == 0) {
-    decision = 0;
-    if (FM < sl.fire.fmax2) sl.fire.converged = 1;
-    else if (!check_only) decision = P > 0.0 ? 1 : 2;
-  }
-  __syncthreads();
-  if (decision == 0) return;
-  const double alpha = sl.fire.alpha;
-  const double c1 = decision == 1 ? 1.0 - alpha : 0.0;
-  const double c2 = (decision == 1 && FF > 0.0) ? alpha * sqrt(VV / FF) : 0.0;
-  for (int i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-    double *v = a.v + 3 * (size_t)i;
-    const double *F = a.F + 3 * (size_t)i;
-    for (int b = 0; b < 3; ++b) v[b] = c1 * v[b] + c2 * F[b];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    if (decision == 1) {
-      if (sl.fire.n_pos > kFireNmin) {
-        sl.fire.dt = fmin(sl.fire.dt * kFireFinc, sl.fire.dt_max);
-        sl.fire.alpha = alpha * kFireFalpha;
-      }
-      sl.fire.n_pos += 1;
-    } else {
-      sl.fire.dt *= kFireFdec;
-      sl.fire.alpha = kFireAlphaStart;
-      sl.fire.n_pos = 0;
-    }
-  }
-}
-
-// Phase and step bookkeeping of every job after an iteration.
-__global__ void engine_advance_kernel(int n_struct, EngineSlot *slots) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n_struct) return;
-  EngineSlot &sl = slots[s];
-  const bool converged = sl.kind == kJobFire && sl.fire.converged;
-  if (sl.phase == 0) {
-    sl.phase = (sl.kind == kJobSingle || sl.n_steps <= 0 || converged) ? 2 : 1;
-  } else if (sl.phase == 1) {
-    sl.steps_done += 1;
-    if (sl.steps_done >= sl.n_steps || converged) sl.phase = 2;
+// End of an engine iteration, one cluster per job: the FIRE update of a FIRE job after its step,
+// then the phase and step bookkeeping.
+__global__ void __cluster_dims__(kFireCluster, 1, 1) __launch_bounds__(128)
+    engine_advance_kernel(const int *offsets, AtomState a, EngineSlot *slots) {
+  EngineSlot &sl = slots[blockIdx.x / kFireCluster];
+  const EngineSlot old = sl;  // read before the cluster's barriers, written after them
+  if (old.phase == 2) return;
+  const int s = blockIdx.x / kFireCluster;
+  bool converged = old.kind == kJobFire && old.fire.converged;
+  if (old.kind == kJobFire && !converged) {
+    FireState next;
+    fire_mix(offsets[s], offsets[s + 1], a, old.fire, old.phase == 0, &next);
+    if (blockIdx.x % kFireCluster != 0 || threadIdx.x != 0) return;
+    sl.fire = next;
+    converged = next.converged;
+  } else if (blockIdx.x % kFireCluster != 0 || threadIdx.x != 0) return;
+  if (old.phase == 0) {
+    sl.phase = (old.kind == kJobSingle || old.n_steps <= 0 || converged) ? 2 : 1;
+  } else {
+    sl.steps_done = old.steps_done + 1;
+    if (sl.steps_done >= old.n_steps || converged) sl.phase = 2;
   }
 }
 
@@ -1599,12 +1577,8 @@ void launch_engine_drift(int N, const AtomState &a, const int *sid, const Engine
     engine_drift_kernel<<<(N + 255) / 256, 256, 0, s>>>(N, a, sid, slots, inv_mass_kappa, half_skin2, sflag, st);
 }
 
-void launch_engine_fire(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s) {
-  if (n_struct > 0) engine_fire_kernel<<<n_struct, 256, 0, s>>>(offsets, a, slots);
-}
-
-void launch_engine_advance(int n_struct, EngineSlot *slots, cudaStream_t s) {
-  if (n_struct > 0) engine_advance_kernel<<<(n_struct + 127) / 128, 128, 0, s>>>(n_struct, slots);
+void launch_engine_advance(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s) {
+  if (n_struct > 0) engine_advance_kernel<<<n_struct * kFireCluster, 128, 0, s>>>(offsets, a, slots);
 }
 
 void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src, AtomState dst, cudaStream_t s) {

@@ -371,8 +371,7 @@ void launch_engine_drift(int N, const AtomState &a, const int *sid, const Engine
                          const double *inv_mass_kappa, double half_skin2, int *sflag, BuildStatus *st,
                          cudaStream_t s);
 void launch_clear_flags(BuildStatus *st, cudaStream_t s);
-void launch_engine_fire(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s);
-void launch_engine_advance(int n_struct, EngineSlot *slots, cudaStream_t s);
+void launch_engine_advance(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s);
 void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src, AtomState dst, cudaStream_t s);
 void launch_thermostat(int N, const AtomState &a, int nb_gather, const double *partial_gather, ThermoState *ts,
                        cudaStream_t s);
