@@ -418,7 +418,8 @@ int nep_set_precision(nep_handle *h, int mode);
 /* How md_run captures the neighbour rebuild in its step graph: 1 (default) = inside a
  * conditional graph node that runs only when a rebuild is due; 0 = as ordinary kernel
  * nodes that return at once when no rebuild is due (for profilers that cannot look inside
- * graphs with conditional nodes). Results are identical. */
+ * graphs with conditional nodes). Up to 131,072 atoms the rebuild is one kernel that returns at
+ * once in either mode (a conditional node costs more). Results are identical. */
 int nep_set_graph_conditional(nep_handle *h, int enable);
 int nep_kernel_slots(void);
 const char *nep_kernel_name(int slot);

@@ -384,6 +384,7 @@ struct nep_handle {
   DevBuf<float> e_rad;
   DevBuf<BuildStatus> status;
   DevBuf<double> fin_scratch;  // finalize_kernel: block sums
+  DevBuf<unsigned> bar;        // grid barrier of the one-kernel build (0 between launches), block sums
   DevBuf<int> fin_ticket;      // and its ticket (0 between launches)
   DevBuf<unsigned long long> stat_part;  // partial sums of a build's list statistics
   BuildStatus *h_status = nullptr;  // pinned mirror
@@ -515,6 +516,10 @@ int ensure_atoms(nep_handle *h, int N, cudaStream_t s) {
   CK(h->thermo_ctl.ensure(4), "alloc");
   CK(h->stat_part.ensure(4 * kStatSlots), "alloc");
   CK(h->fin_scratch.ensure(kFinalScratch), "alloc");
+  if (!h->bar.p) {
+    CK(h->bar.ensure(1 + kBuildSums), "alloc");
+    CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
+  }
   if (!h->fin_ticket.p) {
     CK(h->fin_ticket.ensure(1), "alloc");
     CK(cudaMemsetAsync(h->fin_ticket.p, 0, sizeof(int), s), "clear ticket");
@@ -555,6 +560,7 @@ ListBufs list_bufs(nep_handle *h) {
   L.cell_count = h->cell_count.p; L.cell_cursor = h->cell_cursor.p; L.cell_start = h->cell_start.p;
   L.cell_atoms = h->cell_atoms.p; L.nl_r = h->nl_r.p; L.nn_r = h->nn_r.p; L.nl_a = h->nl_a.p; L.nn_a = h->nn_a.p;
   L.rev_a = h->rev_a.p; L.cap_r = h->cap_r; L.cap_a = h->cap_a; L.part = h->stat_part.p;
+  L.bar = h->bar.p;
   L.stage_e = h->stage_e.p; L.stage_g = h->stage_g.p;
   return L;
 }
@@ -582,7 +588,9 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
   }
   for (int attempt = 0; attempt < 3; ++attempt) {
     const bool count_only = (h->cap_r == 0 || h->cap_a == 0);
-    if (!src.pos) launch_arm_rebuild(h->status.p, s);  // else requested by the load
+    if (h->h_status->tc_timeout)  // the barrier may have been left in mid-count
+      CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
+    if (!src.pos) launch_arm_rebuild(h->status.p, h->bar.p, s);  // else requested by the load
     CK(launch_rebuild(N, h->T, g, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
                       list_bufs(h), count_only ? 1 : 0, move, src, h->status.p, s),
        "launch rebuild");
@@ -599,6 +607,7 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
       if (rc) return rc;
     }
     const BuildStatus &st = *h->h_status;
+    if (st.bad_input & 4) return fail(h, NEP_ERR_TIMEOUT, "the barrier of the neighbour build ran out");
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
     if (st.max_r > kListBuf || st.max_a > kListBuf)
@@ -1174,7 +1183,7 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
        "checkpoint");
     const bool forced = force_rebuild || attempt > 0;
     // the flags of this chunk start cleared; a forced build is requested before the first step
-    if (forced) launch_arm_rebuild(h->status.p, s);
+    if (forced) launch_arm_rebuild(h->status.p, h->bar.p, s);
     else launch_clear_flags(h->status.p, s);
     const EngineKey key = engine_key(h);
     for (int it = 0; it < n_iter; ++it) {
@@ -1361,7 +1370,7 @@ int nep_destroy(nep_handle *h) {
   h->e_slots.release(); h->e_slots_ck.release(); h->e_energy.release(); h->e_virial.release(); h->e_u.release();
   h->e_w.release(); h->e_xck.release(); h->e_vck.release(); h->e_table.release();
   h->stage_e.release(); h->stage_g.release();
-  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->fin_scratch.release(); h->fin_ticket.release();
+  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->bar.release(); h->fin_scratch.release(); h->fin_ticket.release();
   h->d_grids.release(); h->d_sid.release(); h->d_offsets.release(); h->b_e.release(); h->b_w.release();
   if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
   if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
@@ -1448,6 +1457,8 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
   // copy-in, neighbour build, both kernels and the structure sums, then one status read
   BatchKey key = batch_key(h, N, o);
   if (!h->prof && h->b_graph && std::memcmp(&key, &h->b_key, sizeof(key)) == 0) {
+    if (h->h_status->tc_timeout)  // the barrier may have been left in mid-count
+      CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
     CK(cudaGraphLaunch(h->b_graph, s), "batch graph launch");
     CK(wait_stream(s), "batch graph");
     const BuildStatus &st = *h->h_status;
@@ -1847,7 +1858,8 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
   ev_record(h, SLOT_DRIFT, 1, s, capturing);
   ev_record(h, SLOT_REBUILD, 0, s, capturing);
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
-  if (capturing && h->graph_cond) {
+  // (up to kWideBuildAtoms atoms the build is one kernel that returns at once)
+  if (capturing && h->graph_cond && N > kWideBuildAtoms) {
     // the rebuild kernels sit in the body of a conditional (IF) node; a one-thread kernel sets
     // its condition from the drift kernel's request, so steps without a rebuild launch none
     cudaStreamCaptureStatus cs;

@@ -17,13 +17,16 @@
 //   build_rev      for every angular pair (i, j, image), the slot of (j, i, -image) in the list
 //                  of j, so forces are gathered without atomics (Algorithm 4's "index
 //                  manipulations").
-// Every builder returns early unless a rebuild is pending, so the whole sequence sits in the
+// Up to kWideBuildAtoms atoms one cooperative kernel (build_kernel) runs all steps, above they are
+// kernels of their own. Every builder returns early unless a rebuild is pending, so the whole sequence sits in the
 // captured MD step graph and only works when an atom moved more than skin/2. In the serving
 // engine's batch a build that was not forced covers only the structures whose atoms moved that
 // far (per-structure flags); the others keep their cells, atom order, lists and x_ref.
 #include <cuda_bf16.h>
 
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "nep_internal.cuh"
 
@@ -272,115 +275,6 @@ __global__ void reorder_commit_kernel(int N, AtomState a, int move, const Grid g
   a.perm[p] = a.perm2[p];
   a.cell_of[p] = gid;
   commit_position(grid_of(B, g0, p), gid, t | ((B.grids ? B.sid[p] : 0) << 8), r, p, a);
-}
-
-// The steps above (load, zero, bin, scan, scatter, reorder, commit) for a small system in one
-// block: counts, cell starts and the cells' atoms stay in shared memory, every thread keeps its
-// atoms' data in registers until all places are known. Bound by launches and latency: seven
-// launches of 2 to 6 us each become one. With the status read only once, behind the force kernels
-// (rebuild_lists), the neighbour build of a call takes 48 us instead of 97 for 216 Si atoms; the
-// general path, which shares that and the load kernel, 77 instead of 113 us for 4,999 atoms.
-// Above 2,048 atoms the one block's FP64 work (16 cycles of its SM per warp instruction) outgrows
-// the launches it saves.
-constexpr int kSmallBuild = 2048;       // atoms at most: two per thread
-constexpr int kSmallBuildCells = 8192;  // cells at most: eight per thread
-__global__ void __launch_bounds__(1024)
-    small_build_kernel(int N, int T, const LoadSrc src, AtomState a, const ListBufs L, int move, const Grid g0,
-                       const Batch B, int ncell, BuildStatus *st) {
-  if (!src.pos && !rebuild_pending(st)) return;
-  extern __shared__ int sb[];
-  int *const start = sb, *const cursor = start + ncell + 1, *const order = cursor + ncell;  // order [N]
-  __shared__ int wsum[32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (src.pos) {
-    if (tid == 0) arm_status(st);
-    if (src.dtab)
-      for (int c = tid; c < g0.ncode; c += 1024) src.dtab[c] = shift_vector(g0, c);
-  }
-  for (int k = tid; k < 4 * kStatSlots; k += 1024) L.part[k] = 0ull;
-  for (int c = tid; c < ncell; c += 1024) start[c] = cursor[c] = 0;
-  __syncthreads();
-  const bool part_build = !src.pos && B.sflag && !*(volatile const int *)&st->full;
-  double r[2][3], v[2][3], F[2][3];
-  int ti[2], pm[2], gid[2];
-  bool mv[2];
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int i = tid + 1024 * u;
-    mv[u] = false;
-    if (i >= N) continue;
-    mv[u] = !(part_build && B.sflag[B.sid[i]] == 0);
-    if (!mv[u]) {  // its structure's order stays
-      atomicAdd(start + a.cell_of[i], 1);
-      continue;
-    }
-    const double *x = src.pos ? src.pos : a.x;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      r[u][b] = x[3 * (size_t)i + b];
-      if (move & 1) v[u][b] = a.v[3 * (size_t)i + b];
-      if (move & 2) F[u][b] = a.F[3 * (size_t)i + b];
-    }
-    ti[u] = src.pos ? src.types[i] : a.types[i];
-    pm[u] = src.pos ? i : a.perm[i];
-    bool moved;
-    gid[u] = bin_position(grid_of(B, g0, i), T, r[u], &ti[u], &moved, st);
-    atomicAdd(start + gid[u], 1);
-  }
-  __syncthreads();
-  // exclusive prefix sum of the counts: eight cells per thread
-  int c8[8], tot = 0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    c8[k] = 8 * tid + k < ncell ? start[8 * tid + k] : 0;
-    tot += c8[k];
-  }
-  int x = tot;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[wid] = x;
-  __syncthreads();
-  if (wid == 0) {
-    int y = wsum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int z = __shfl_up_sync(0xffffffffu, y, o);
-      if (lane >= o) y += z;
-    }
-    wsum[lane] = y;
-  }
-  __syncthreads();
-  int at = (wid > 0 ? wsum[wid - 1] : 0) + (x - tot);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    if (8 * tid + k < ncell) start[8 * tid + k] = L.cell_start[8 * tid + k] = at;
-    at += c8[k];
-  }
-  if (tid == 0) start[ncell] = L.cell_start[ncell] = N;
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 2; ++u)
-    if (mv[u]) order[start[gid[u]] + atomicAdd(cursor + gid[u], 1)] = tid + 1024 * u;
-  __syncthreads();
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    if (!mv[u]) continue;
-    const int i = tid + 1024 * u, b0 = start[gid[u]], b1 = start[gid[u] + 1];
-    int p = b0;  // the cell's atoms in index order
-    for (int q = b0; q < b1; ++q) p += order[q] < i ? 1 : 0;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      if (move & 1) a.v[3 * (size_t)p + b] = v[u][b];
-      if (move & 2) a.F[3 * (size_t)p + b] = F[u][b];
-    }
-    a.types[p] = ti[u];
-    a.perm[p] = pm[u];
-    a.cell_of[p] = gid[u];
-    commit_position(grid_of(B, g0, p), gid[u], ti[u] | ((B.grids ? B.sid[p] : 0) << 8), r[u], p, a);
-  }
 }
 
 // floor(x / n) and the remainder, for n >= 1 and x > -n * 8
@@ -636,25 +530,16 @@ __global__ void build_lists_kernel(int N, const float4 *posA, const float4 *pos4
 // What bounds it: latency (start offsets, then positions, then the class ballots): a few atoms
 // occupy few warps. 216 Si atoms (skin 1 A): 10 us against 118 us of the thread form; 4999
 // atoms of a three-species cell: 17 us.
-constexpr int kWideWarps = 4;             // warps (atoms) per block
-constexpr int kWideBuildAtoms = 131072;   // largest system of this form (the rule is in launch_rebuild)
-
+// List of atom i by a whole warp; se: cap_r entries of shared memory of the warp. The positions
+// and cells were written by other blocks of the running kernel: no read-only (ld.global.nc) loads.
 template <int TT, bool COUNT>
-__global__ void __launch_bounds__(32 * kWideWarps)
-    build_lists_wide_kernel(int N, const float4 *__restrict__ posA, const float4 *__restrict__ pos4,
-                            const int *__restrict__ cell_of, const int *__restrict__ start, const Grid g0,
-                            const Batch B, float rlR2, float rlA2, float rcR2, float rcA2, ListBufs L,
-                            BuildStatus *st) {
-  if (!rebuild_pending(st)) return;
+__device__ __forceinline__ void list_of_atom(int i, int N, const float4 *posA, const float4 *pos4, const int *cell_of,
+                                             const int *start, const Grid &g, float rlR2, float rlA2, float rcR2,
+                                             float rcA2, const ListBufs &L, uint2 *se, BuildStatus *st) {
   constexpr unsigned kAll = 0xffffffffu;
-  extern __shared__ uint2 bl_stage[];  // [kWideWarps][cap_r] (entry, r^2), later (entry, class)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const int i = blockIdx.x * kWideWarps + warp;
-  if (i >= N || kept_by_build(B, st, i)) return;  // uniform over the warp
   const int cap = COUNT ? 0 : L.cap_r;
-  uint2 *const se = bl_stage + (size_t)warp * cap;
-  const Grid &g = grid_of(B, g0, i);
   const int nc1 = g.nc[1], nc2 = g.nc[2];
   const int id = cell_of[i] - g.cell_off;
   const int cx = id / (nc1 * nc2), cy = (id / nc2) % nc1, cz = id % nc2;
@@ -711,7 +596,7 @@ __global__ void __launch_bounds__(32 * kWideWarps)
         bool ok = false;
         float r2 = 0.f;
         if (j < e0) {
-          r2 = norm2(pair_vector(pi, __ldg(posA + j), S));
+          r2 = norm2(pair_vector(pi, posA[j], S));
           ok = r2 < rlR2 && j != self;
         }
         const unsigned m = __ballot_sync(kAll, ok);
@@ -801,15 +686,11 @@ __global__ void __launch_bounds__(32 * kWideWarps)
 // side and every search keeps four list entries in flight (a thread per atom searched its
 // pairs one after the other: 50 us for 216 atoms, 253 us for a 4096-structure batch; now 10 and
 // 222 us).
-__global__ void __launch_bounds__(256) build_rev_kernel(int N, const ListBufs L, const Grid g0, const Batch B,
-                                                        BuildStatus *st) {
-  if (!rebuild_pending(st)) return;
-  const int i = blockIdx.x * 32 + (threadIdx.x & 31);
-  if (i >= N || kept_by_build(B, st, i)) return;
-  const Grid &g = grid_of(B, g0, i);
+__device__ __forceinline__ void reverse_pairs(int i, int first, int N, const ListBufs &L, const Grid &g,
+                                              BuildStatus *st) {
   const unsigned om = (1u << g.obits) - 1u;
   const int na = L.nn_a[i];
-  for (int m = threadIdx.x >> 5; m < na; m += 8) {
+  for (int m = first; m < na; m += 8) {
     const size_t slot = (size_t)m * N + i;
     const unsigned e = L.nl_a[slot];
     const int j = e & g.jmask;
@@ -823,7 +704,7 @@ __global__ void __launch_bounds__(256) build_rev_kernel(int N, const ListBufs L,
     for (int q = 0; q < nj && found < 0; q += 4) {
       unsigned v[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = q + k < nj ? __ldg(col + (size_t)(q + k) * N) : ~target;
+      for (int k = 0; k < 4; ++k) v[k] = q + k < nj ? col[(size_t)(q + k) * N] : ~target;
 #pragma unroll
       for (int k = 3; k >= 0; --k)
         if (v[k] == target) found = q + k;
@@ -837,15 +718,22 @@ __global__ void __launch_bounds__(256) build_rev_kernel(int N, const ListBufs L,
   }
 }
 
+__global__ void __launch_bounds__(256) build_rev_kernel(int N, const ListBufs L, const Grid g0, const Batch B,
+                                                        BuildStatus *st) {
+  if (!rebuild_pending(st)) return;
+  const int i = blockIdx.x * 32 + (threadIdx.x & 31);
+  if (i >= N || kept_by_build(B, st, i)) return;
+  reverse_pairs(i, threadIdx.x >> 5, N, L, grid_of(B, g0, i), st);
+}
+
 // The pending build is done, and the per-structure requests (sflag) are served; its list
 // statistics are summed. One block of 256 threads.
-__global__ void finish_build_kernel(int n_struct, int *sflag, const unsigned long long *part, BuildStatus *st) {
-  if (!rebuild_pending(st)) return;  // read before thread 0 clears it
-  __syncthreads();
+__device__ __forceinline__ void finish_build(int n_struct, int *sflag, const unsigned long long *part,
+                                             BuildStatus *st) {
   for (int s = threadIdx.x; s < n_struct; s += blockDim.x) sflag[s] = 0;
   static_assert(4 * kStatSlots == 256, "one partial sum per thread");
   __shared__ unsigned long long red[8][4];
-  unsigned long long v = part[threadIdx.x];  // statistic threadIdx.x % 4
+  unsigned long long v = __ldcg(part + threadIdx.x);  // statistic threadIdx.x % 4
 #pragma unroll
   for (int o = 16; o >= 4; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) < 4) red[threadIdx.x >> 5][threadIdx.x & 3] = v;
@@ -861,6 +749,225 @@ __global__ void finish_build_kernel(int n_struct, int *sflag, const unsigned lon
     st->full = 0;
     st->n_rebuilds += 1;
   }
+}
+
+__global__ void finish_build_kernel(int n_struct, int *sflag, const unsigned long long *part, BuildStatus *st) {
+  if (!rebuild_pending(st)) return;  // read before thread 0 clears it
+  __syncthreads();
+  finish_build(n_struct, sflag, part, st);
+}
+
+// The whole build of up to kWideBuildAtoms atoms in one cooperative launch: the steps above with
+// barriers over the grid in place of kernel boundaries, and a warp per atom for the lists. Ten
+// launches become one, and a step of a dynamics run that needs no build pays for one kernel that
+// returns at once instead of a conditional graph node, which costs about 10 us. Bound by latency:
+// six to eight phases of a few us. A dynamics step of 216 Si atoms 50 -> 44 us, of 13,824 atoms
+// 69 -> 62 us; a serving iteration 153 -> 135 us; a build by itself about as before (20,000 atoms
+// 102 us, with two blocks per SM 121, with one 163).
+//
+// Blocks that run at the same time by the cooperative launch wait at `bar` (L.bar[0], zero
+// between launches). The wait is bounded: one that runs out sets tc_timeout and bit 2 of bad_input
+// and ends the block; later builds return at once until the host has cleared both.
+constexpr int kBuildBlock = 256;
+constexpr int kBuildWarps = kBuildBlock / 32;
+constexpr int kBuildPerSM = 3;           // blocks per SM at most (registers and shared memory hold that many)
+constexpr unsigned kBarrierSpins = 1u << 22;  // seconds
+
+struct GridBarrier {
+  unsigned *bar;
+  unsigned target = 0;
+  BuildStatus *st;
+  __device__ __forceinline__ bool wait() {
+    __shared__ int ok;
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      atomicAdd(bar, 1u);
+      unsigned seen, spins = 0;
+      do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      } while (seen < target && ++spins < kBarrierSpins);
+      ok = seen >= target;
+      if (!ok) {
+        st->tc_timeout = 1;
+        atomicOr(&st->bad_input, 4);
+      }
+      __threadfence();
+    }
+    __syncthreads();
+    return ok != 0;
+  }
+};
+
+struct BuildArgs {
+  int N, T, ncell, move;
+  LoadSrc src;
+  AtomState a;
+  ListBufs L;
+  Grid g;
+  Batch B;
+  float rlR2, rlA2, rcR2, rcA2;
+  BuildStatus *st;
+};
+
+template <int TT, bool COUNT>
+__global__ void __launch_bounds__(kBuildBlock, kBuildPerSM) build_kernel(const BuildArgs p) {
+  BuildStatus *const st = p.st;
+  const bool load = p.src.pos != nullptr;
+  if (!load && (!rebuild_pending(st) || *(volatile const int *)&st->tc_timeout)) return;
+  const int N = p.N, G = gridDim.x, tid = threadIdx.x, t0 = blockIdx.x * kBuildBlock + tid, nt = G * kBuildBlock;
+  const AtomState &a = p.a;
+  const ListBufs &L = p.L;
+  const Batch &B = p.B;
+  GridBarrier grid{L.bar, 0u, st};
+  extern __shared__ uint2 bl_stage[];  // [kBuildWarps][cap_r]
+  __shared__ int wsum[kBuildWarps], carry_s;
+
+  // a barrier that ran out: empty lists, whatever is queued behind
+  auto give_up = [&]() {
+    if (COUNT) return;
+    for (int i = t0; i < N; i += nt) {
+      for (int t = 0; t < p.T; ++t) L.nn_r[(size_t)t * N + i] = 0;
+      L.nn_a[i] = 0;
+    }
+  };
+  // the caller's shift table, cell counts and list statistics cleared
+  if (load) {
+    if (t0 == 0) arm_status(st);
+    if (p.src.dtab)
+      for (int c = t0; c < p.g.ncode; c += nt) p.src.dtab[c] = shift_vector(p.g, c);
+  }
+  for (int c = t0; c < p.ncell; c += nt) L.cell_count[c] = 0;
+  for (int k = t0; k < 4 * kStatSlots; k += nt) L.part[k] = 0ull;
+  if (!grid.wait()) return give_up();
+
+  // bin: wrapped positions and everything that moves into the scratch arrays, atoms counted
+  for (int i = t0; i < N; i += nt) {
+    if (kept_by_build(B, st, i)) {  // counted in its old cell: its structure's order stays
+      atomicAdd(L.cell_count + a.cell_of[i], 1);
+      continue;
+    }
+    const size_t k = 3 * (size_t)i;
+    const double *x = (load ? p.src.pos : a.x) + k;
+    double r[3] = {x[0], x[1], x[2]};
+    int ti = load ? p.src.types[i] : a.types[i];
+    bool moved;
+    const int id = bin_position(grid_of(B, p.g, i), p.T, r, &ti, &moved, st);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      a.x2[k + b] = r[b];
+      if (p.move & 1) a.v2[k + b] = a.v[k + b];
+      if (p.move & 2) a.F2[k + b] = a.F[k + b];
+    }
+    a.types2[i] = ti;
+    a.perm2[i] = load ? i : a.perm[i];
+    a.cell2[i] = id;
+    atomicAdd(L.cell_count + id, 1);
+  }
+  if (!grid.wait()) return give_up();
+
+  // cell starts: block b scans the b-th part of the cells from the sum of the parts before
+  const int part = (p.ncell + G - 1) / G, c0 = blockIdx.x * part, c1 = min(p.ncell, c0 + part);
+  auto block_sum = [&](int v) {  // over the block, on every thread
+    v = __reduce_add_sync(0xffffffffu, v);
+    __syncthreads();
+    if ((tid & 31) == 0) wsum[tid >> 5] = v;
+    __syncthreads();
+    v = 0;
+#pragma unroll
+    for (int w = 0; w < kBuildWarps; ++w) v += wsum[w];
+    return v;
+  };
+  int before = 0;
+  if (p.ncell > 8192) {  // the parts' sums by one block each
+    int v = 0;
+    for (int c = c0 + tid; c < c1; c += kBuildBlock) v += L.cell_count[c];
+    v = block_sum(v);
+    if (tid == 0) L.bar[1 + blockIdx.x] = (unsigned)v;
+    if (!grid.wait()) return give_up();
+    for (int b = tid; b < (int)blockIdx.x; b += kBuildBlock) before += (int)L.bar[1 + b];
+  } else {  // every block adds the counts before its own part
+    for (int c = tid; c < min(c0, p.ncell); c += kBuildBlock) before += L.cell_count[c];
+  }
+  before = block_sum(before);
+  for (int cb = c0; cb < c1; cb += kBuildBlock) {
+    const int c = cb + tid, v = c < c1 ? L.cell_count[c] : 0;
+    int x = v;  // inclusive scan over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((tid & 31) >= o) x += y;
+    }
+    __syncthreads();
+    if ((tid & 31) == 31) wsum[tid >> 5] = x;
+    __syncthreads();
+    int off = before;
+    for (int w = 0; w < (tid >> 5); ++w) off += wsum[w];
+    if (c < c1) L.cell_start[c] = off + x - v;
+    if (tid == kBuildBlock - 1) carry_s = off + x;
+    __syncthreads();
+    before = carry_s;
+  }
+  if (t0 == 0) L.cell_start[p.ncell] = N;
+  if (!grid.wait()) return give_up();
+
+  // the atoms of every cell, in any order (the counts run down to zero)
+  for (int i = t0; i < N; i += nt) {
+    if (kept_by_build(B, st, i)) continue;
+    const int c = a.cell2[i];
+    L.cell_atoms[L.cell_start[c] + atomicSub(L.cell_count + c, 1) - 1] = i;
+  }
+  if (!grid.wait()) return give_up();
+
+  // into their places: the cell's atoms in index order
+  for (int q = t0; q < N; q += nt) {
+    if (kept_by_build(B, st, q)) continue;
+    const int o = L.cell_atoms[q], c = a.cell2[o], b0 = L.cell_start[c], b1 = L.cell_start[c + 1];
+    int d = b0;
+    for (int k = b0; k < b1; ++k) d += L.cell_atoms[k] < o ? 1 : 0;
+    const size_t f = 3 * (size_t)o, k = 3 * (size_t)d;
+    double r[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      r[b] = a.x2[f + b];
+      if (p.move & 1) a.v[k + b] = a.v2[f + b];
+      if (p.move & 2) a.F[k + b] = a.F2[f + b];
+    }
+    const int ti = a.types2[o];
+    a.types[d] = ti;
+    a.perm[d] = a.perm2[o];
+    a.cell_of[d] = c;
+    commit_position(grid_of(B, p.g, d), c, ti | ((B.grids ? B.sid[d] : 0) << 8), r, d, a);
+  }
+  if (!grid.wait()) return give_up();
+
+  // lists: a warp per atom
+  for (int i = blockIdx.x * kBuildWarps + (tid >> 5); i < N; i += G * kBuildWarps) {
+    if (kept_by_build(B, st, i)) continue;  // uniform over the warp
+    list_of_atom<TT, COUNT>(i, N, a.posA, a.pos4, a.cell_of, L.cell_start, grid_of(B, p.g, i), p.rlR2, p.rlA2, p.rcR2,
+                            p.rcA2, L, bl_stage + (size_t)(tid >> 5) * (COUNT ? 0 : L.cap_r), st);
+    __syncwarp();
+  }
+  if constexpr (!COUNT) {
+    if (!grid.wait()) return give_up();
+    for (int b = blockIdx.x * 32; b < N; b += G * 32) {
+      const int i = b + (tid & 31);
+      if (i < N && !kept_by_build(B, st, i)) reverse_pairs(i, tid >> 5, N, L, grid_of(B, p.g, i), st);
+    }
+  }
+  // the last block to get here ends the build and leaves the barrier at zero
+  __shared__ int last;
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    last = atomicAdd(L.bar, 1u) == grid.target + G - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  finish_build(B.sflag ? B.n : 0, B.sflag, L.part, st);
+  if (tid == 0) L.bar[0] = 0u;
 }
 
 // Sets the condition of the graph's rebuild node from the drift kernel's request.
@@ -1135,7 +1242,10 @@ __global__ void struct_sums_kernel(int n_struct, int members, const int *offsets
 
 // Marks a rebuild as pending and clears the per-build flags (the device form of the host
 // reset before a forced rebuild, for captured graphs).
-__global__ void arm_rebuild_kernel(BuildStatus *st) { arm_status(st); }
+__global__ void arm_rebuild_kernel(BuildStatus *st, unsigned *bar) {
+  arm_status(st);
+  bar[0] = 0u;
+}
 
 // ------------------------------------------------------------------ population evaluation
 // Candidate parameter vectors z [P][N_par], in the order c^R, c^A, w0, b0, w1, b1, become
@@ -1243,7 +1353,7 @@ __global__ void population_loss_kernel(int n_struct, const int *offsets, const d
   }
 }
 
-void launch_arm_rebuild(BuildStatus *st, cudaStream_t s) { arm_rebuild_kernel<<<1, 1, 0, s>>>(st); }
+void launch_arm_rebuild(BuildStatus *st, unsigned *bar, cudaStream_t s) { arm_rebuild_kernel<<<1, 1, 0, s>>>(st, bar); }
 
 void launch_unpack_population(int n_pop, const double *z, int n_par, const TableLayout &t, float *tab, double *reg,
                               cudaStream_t s) {
@@ -1288,26 +1398,31 @@ void launch_struct_sums(int n_struct, int members, const int *offsets, int N, co
 
 // ------------------------------------------------------------------ host launchers
 template <bool COUNT>
-cudaError_t launch_lists_wide(int N, int T, const Grid &g, const Batch &B, float rlR2, float rlA2, float rcR2,
-                              float rcA2, const AtomState &a, const ListBufs &L, BuildStatus *st, cudaStream_t s) {
-  const size_t smem = COUNT ? 0 : sizeof(uint2) * kWideWarps * (size_t)L.cap_r;
-  static_assert(sizeof(uint2) * kWideWarps * kListBuf <= 48 * 1024, "within the default shared memory limit");
+cudaError_t launch_build(const BuildArgs &p, cudaStream_t s) {
+  const size_t smem = COUNT ? 0 : sizeof(uint2) * kBuildWarps * (size_t)p.L.cap_r;
+  static_assert(sizeof(uint2) * kBuildWarps * kListBuf <= 48 * 1024, "within the default shared memory limit");
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int want = (p.N + kBuildWarps - 1) / kBuildWarps, most = std::min(kBuildPerSM * sms, kBuildSums);
   auto go = [&](auto kern) -> cudaError_t {
-    kern<<<(N + kWideWarps - 1) / kWideWarps, 32 * kWideWarps, smem, s>>>(N, a.posA, a.pos4, a.cell_of, L.cell_start, g, B,
-                                                                         rlR2, rlA2, rcR2, rcA2, L, st);
-    return cudaGetLastError();
+    BuildArgs args = p;
+    void *av[] = {&args};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(std::max(1, std::min(want, most))),
+                                       dim3(kBuildBlock), av, smem, s);
   };
-  if constexpr (COUNT) return go(build_lists_wide_kernel<1, true>);
+  if constexpr (COUNT) return go(build_kernel<1, true>);
   else
-    switch (T) {
-      case 1: return go(build_lists_wide_kernel<1, false>);
-      case 2: return go(build_lists_wide_kernel<2, false>);
-      case 3: return go(build_lists_wide_kernel<3, false>);
-      case 4: return go(build_lists_wide_kernel<4, false>);
-      case 5: return go(build_lists_wide_kernel<5, false>);
-      case 6: return go(build_lists_wide_kernel<6, false>);
-      case 7: return go(build_lists_wide_kernel<7, false>);
-      default: return go(build_lists_wide_kernel<8, false>);
+    switch (p.T) {
+      case 1: return go(build_kernel<1, false>);
+      case 2: return go(build_kernel<2, false>);
+      case 3: return go(build_kernel<3, false>);
+      case 4: return go(build_kernel<4, false>);
+      case 5: return go(build_kernel<5, false>);
+      case 6: return go(build_kernel<6, false>);
+      case 7: return go(build_kernel<7, false>);
+      default: return go(build_kernel<8, false>);
     }
 }
 
@@ -1336,31 +1451,26 @@ cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const fl
   const int tb = 256;
   const int nb = (N + tb - 1) / tb;
   const int cb = (g.ncell + tb - 1) / tb;
-  if (N <= kSmallBuild && g.ncell <= kSmallBuildCells) {
-    const cudaError_t e = smem_limit_once(small_build_kernel, sizeof(int) * (2 * kSmallBuildCells + 1 + kSmallBuild));
-    if (e != cudaSuccess) return e;
-    small_build_kernel<<<1, 1024, sizeof(int) * (2 * g.ncell + 1 + N), s>>>(N, T, src, a, L, move, g, B, g.ncell, st);
-  } else {
-    if (src.pos) {
-      const int lb = (3LL * N + tb - 1) / tb < 8 * 152 ? (int)((3LL * N + tb - 1) / tb) : 8 * 152;
-      load_kernel<<<lb, tb, 0, s>>>(N, src, a, g, st);
-    }
-    zero_cells_kernel<<<cb < 1024 ? cb : 1024, tb, 0, s>>>(g.ncell, L.cell_count, L.cell_cursor, L.part, st);
-    bin_atoms_kernel<<<nb, tb, 0, s>>>(N, T, a, L.cell_count, g, B, st);
-    scan_cells_kernel<<<1, 1024, 0, s>>>(g.ncell, L.cell_count, L.cell_start, st);
-    scatter_atoms_kernel<<<nb, tb, 0, s>>>(N, a.cell_of, L.cell_start, L.cell_cursor, L.cell_atoms, B, st);
-    reorder_gather_kernel<<<nb, tb, 0, s>>>(N, L.cell_start, L.cell_atoms, a, move, B, st);
-    reorder_commit_kernel<<<nb, tb, 0, s>>>(N, a, move, g, B, st);
-  }
-  // Warp per atom up to kWideBuildAtoms atoms, thread per atom above: a small system leaves the
-  // thread form with a few long serial scans, a large one makes the warp form pay for its idle
-  // lanes (ranges of ~20 candidates). Whole neighbour build, thread / warp form, us: 216 Si atoms
+  // One cooperative kernel with a warp per atom up to kWideBuildAtoms atoms, separate kernels with a
+  // thread per atom above: a small system leaves the thread form with a few long serial scans, a
+  // large one makes the warp form pay for its idle lanes (ranges of ~20 candidates). Whole neighbour build, thread / warp form, us: 216 Si atoms
   // 198 / 98, 13,824 172 / 111, 20,000 (three species, r_c 6 A) 258 / 139, 262,144 PbTe atoms
   // 404 / 482, a batch of 1.05 million atoms 2056 / 2371, 8,000,000 Si atoms 7444 / 13,803.
-  const cudaError_t e =
-      N > kWideBuildAtoms ? launch_lists(N, T, g, B, rlR2, rlA2, rcR2, rcA2, a, L, count_only, st, s)
-      : count_only        ? launch_lists_wide<true>(N, T, g, B, rlR2, rlA2, rcR2, rcA2, a, L, st, s)
-                          : launch_lists_wide<false>(N, T, g, B, rlR2, rlA2, rcR2, rcA2, a, L, st, s);
+  if (N <= kWideBuildAtoms) {
+    const BuildArgs p{N, T, g.ncell, move, src, a, L, g, B, rlR2, rlA2, rcR2, rcA2, st};
+    return count_only ? launch_build<true>(p, s) : launch_build<false>(p, s);
+  }
+  if (src.pos) {
+    const int lb = (3LL * N + tb - 1) / tb < 8 * 152 ? (int)((3LL * N + tb - 1) / tb) : 8 * 152;
+    load_kernel<<<lb, tb, 0, s>>>(N, src, a, g, st);
+  }
+  zero_cells_kernel<<<cb < 1024 ? cb : 1024, tb, 0, s>>>(g.ncell, L.cell_count, L.cell_cursor, L.part, st);
+  bin_atoms_kernel<<<nb, tb, 0, s>>>(N, T, a, L.cell_count, g, B, st);
+  scan_cells_kernel<<<1, 1024, 0, s>>>(g.ncell, L.cell_count, L.cell_start, st);
+  scatter_atoms_kernel<<<nb, tb, 0, s>>>(N, a.cell_of, L.cell_start, L.cell_cursor, L.cell_atoms, B, st);
+  reorder_gather_kernel<<<nb, tb, 0, s>>>(N, L.cell_start, L.cell_atoms, a, move, B, st);
+  reorder_commit_kernel<<<nb, tb, 0, s>>>(N, a, move, g, B, st);
+  const cudaError_t e = launch_lists(N, T, g, B, rlR2, rlA2, rcR2, rcA2, a, L, count_only, st, s);
   if (e != cudaSuccess) return e;
   if (!count_only) build_rev_kernel<<<(N + 31) / 32, 256, 0, s>>>(N, L, g, B, st);
   finish_build_kernel<<<1, 256, 0, s>>>(B.sflag ? B.n : 0, B.sflag, L.part, st);

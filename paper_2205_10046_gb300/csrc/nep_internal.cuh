@@ -10,6 +10,7 @@
 namespace nep {
 
 constexpr int kMaxTypes = 8;
+constexpr int kWideBuildAtoms = 131072;  // most atoms of the one-kernel neighbour build
 constexpr int kListBuf = 512;   // largest neighbour-list capacity per atom
 constexpr int kMaxImage = 3;    // largest cell/image offset searched per axis
 // Distance (A) added to r_c^R + skin before a cell is left out of the neighbour search: far
@@ -86,8 +87,10 @@ struct ListBufs {
   unsigned *stage_e;        // [cap_r][N] accepted candidates of one build, or null (second scan)
   unsigned char *stage_g;   // [cap_r][N] their groups
   unsigned long long *part;  // [kStatSlots][4] partial sums of a build's list statistics
+  unsigned *bar;             // [1 + kBuildSums] barrier of the one-kernel build (zero between launches), block sums
 };
 constexpr int kStatSlots = 64;
+constexpr int kBuildSums = 1023;  // blocks of the one-kernel build at most
 
 // Device-visible status written by the builders.
 struct BuildStatus {
@@ -99,8 +102,9 @@ struct BuildStatus {
   int rebuild;         // a rebuild is pending (set by the drift kernel or the host)
   int full;            // the pending build covers every structure (forced); else, with
                        // per-structure flags, only the flagged ones
-  int bad_input;       // bit 0: type out of range, bit 1: non-finite position
-  int tc_timeout;      // a tensor-core completion wait ran out (results invalid)
+  int bad_input;       // bit 0: type out of range, bit 1: non-finite position, bit 2: the build's
+                       // grid barrier ran out
+  int tc_timeout;      // a tensor-core completion wait or a grid barrier ran out (results invalid)
   long long n_rebuilds;
   long long md_steps;
 };
@@ -364,7 +368,7 @@ void launch_shift_tables(int n_struct, const Grid *grids, int ncode, float4 *dta
 // max_atoms: the largest structure (structures above kWideSum atoms are summed by a block)
 void launch_struct_sums(int n_struct, int members, const int *offsets, int N, const double *e_atom,
                         const double *w_atom, double *e_struct, double *w_struct, int max_atoms, cudaStream_t s);
-void launch_arm_rebuild(BuildStatus *st, cudaStream_t s);
+void launch_arm_rebuild(BuildStatus *st, unsigned *bar, cudaStream_t s);
 void launch_fire_mix(int N, const AtomState &a, FireState *fire, int check_only, cudaStream_t s);
 // batched serving engine
 void launch_engine_drift(int N, const AtomState &a, const int *sid, const EngineSlot *slots,

@@ -101,6 +101,7 @@ int run_build(int N, int T, const Grid &g, const float4 *dtab, float rlR2, float
      "neighbour build");
   SK(cudaMemcpyAsync(st_host, st_dev, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   SK(cudaStreamSynchronize(s), "synchronise");
+  if (st_host->bad_input & 4) return fail_static(NEP_ERR_TIMEOUT, "the barrier of the neighbour build ran out");
   if (st_host->bad_input & 1) return fail_static(NEP_ERR_ARG, "atom type out of range");
   if (st_host->bad_input & 2) return fail_static(NEP_ERR_NONFINITE, "non-finite position");
   return NEP_OK;
@@ -178,15 +179,18 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.nn_r = arena.take<int>((size_t)T * N);
   L.nn_a = arena.take<int>(N);
   L.part = arena.take<unsigned long long>(4 * kStatSlots);
+  L.bar = arena.take<unsigned>(1 + kBuildSums);
   if (!st || !dtab || !dtabm || !a.x || !a.v || !a.F || !a.x_ref || !a.origin || !a.x2 || !a.v2 || !a.F2 ||
       !a.types || !a.perm || !a.cell_of || !a.types2 || !a.perm2 || !a.cell2 || !a.pos4 || !a.posA || !L.cell_count ||
-      !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part)
+      !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part ||
+      !L.bar)
     return fail_static(NEP_ERR_ARG, "structure too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
 
   // inputs into the arena; the arena keeps the previous call's contents, so everything the
   // kernels read is written first, here or by the build (positions, types, order, shift table,
   // cell counters)
   SK(cudaMemcpyAsync(dtabm, tab, sizeof(float) * tl.total, cudaMemcpyHostToDevice, s), "copy");
+  SK(cudaMemsetAsync(L.bar, 0, sizeof(unsigned), s), "clear");
   SK(cudaMemsetAsync(a.v, 0, sizeof(double) * 3 * N, s), "clear");
   SK(cudaMemsetAsync(a.F, 0, sizeof(double) * 3 * N, s), "clear");
 

@@ -1,6 +1,6 @@
-"""The one-block neighbour build (at most 2,048 atoms and 8,192 cells) against the FP64 oracle,
-on both sides of its limits: sizes around one and two atoms per thread, a grid with more cells
-than atoms, atoms outside the cell, batches, and inputs it has to refuse."""
+"""The one-kernel neighbour build alone and over batches: sizes around its blocks, a grid with more
+cells than atoms on both sides of the 8,192 cells where its prefix sum changes, atoms outside the
+cell, batches, and inputs it has to refuse."""
 import numpy as np
 import pytest
 
@@ -34,9 +34,9 @@ def _outside(pos, box, seed):
 
 
 @pytest.mark.parametrize("sizes", [[1, 2, 1023, 1024, 1025], [2047, 2048, 2049], [7] * 290, "dilute"])
-def test_small_build_equals_general_build(torch_cuda, sizes):
-    """A structure alone (one-block build up to 2,048 atoms) and in a batch above the limits
-    (general build): the same atom order, lists and sums, hence the same bits."""
+def test_structure_alone_equals_batch(torch_cuda, sizes):
+    """A structure alone and in a batch, split over the blocks in other places: the same atom order,
+    lists and sums, hence the same bits."""
     from paper_2205_10046_gb300 import nep
     torch = torch_cuda
     if sizes == "dilute":  # more cells than atoms: 4 per atom at most, 8,192 and more in all
