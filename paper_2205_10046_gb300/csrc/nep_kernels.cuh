@@ -469,6 +469,16 @@ __device__ __forceinline__ void for_pairs_batch(const unsigned *__restrict__ nl,
 // 3010 / 2318. Of that, reading the model table from global memory instead of copying it from
 // the kernel parameters (lane-varying constant addresses, served one by one) took 0.8 ms of the
 // 8,000,000-atom step, and the factored polynomials 0.6 ms.
+// Small systems: up to kSplitAtoms atoms of one structure, four groups of lanes work on an atom (16
+// atoms per block of 128 threads), up to kSplitAtoms2 two (32 atoms per block). The sums over
+// neighbours stay with the first group, whose lanes add in the same order as ever (the same bits);
+// the network, the components, dU/dS_nk and the partial forces, which are independent term by term,
+// are shared. The limits are one wave of such blocks, three per SM: beyond it the groups that wait
+// cost more than the shorter chain gives. A dynamics step without / with, us (the gather kernel
+// split in both): 216 Si atoms 40 / 36, 5,832 46 / 43, 8,000 46.4 / 45.8, 13,824 57.4 / 55.4, past the
+// limits with four groups 13,824 Si atoms 63 / 71, 8,000 PbTe atoms 41 / 50.
+constexpr int kSplitAtoms = 152 * 3 * 16;
+constexpr int kSplitAtoms2 = 152 * 3 * 32;
 template <class S>
 struct PairRow {
   static constexpr int Q4 = S::NDP / 4;                  // float4s of q
@@ -489,8 +499,8 @@ struct PairRow {
   }
 };
 
-template <class S, int PREC, bool DESC, bool BATCH, int AB>
-__global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
+template <class S, int PREC, bool DESC, bool BATCH, int AB, int SUB>
+__global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB))
     atom_kernel(const AtomArgs a, const __grid_constant__ ModelF mf) {
   constexpr unsigned kAll = 0xffffffffu;
   constexpr int NR = S::NR, KR = S::KR, NA = S::NA, KA = S::KA, NDES = S::NDES, NDP = S::NDP;
@@ -498,7 +508,15 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   static_assert(S::NK == 24, "harm_k lists the 24 polynomials of l <= 4");
   extern __shared__ float4 smem4[];
   const int T = a.T, N = a.N;
-  const int h = threadIdx.x & 1, ia = threadIdx.x >> 1;
+  static_assert(SUB == 1 || (PREC == 0 && !DESC && AB % 16 == 0), "forces with the FP32 network");
+  // SUB > 1: SUB groups of 2 AB threads, lanes of the same atoms
+  const int sub = SUB > 1 ? threadIdx.x / (2 * AB) : 0, tl = SUB > 1 ? threadIdx.x % (2 * AB) : threadIdx.x;
+  const int h = tl & 1, ia = tl >> 1;
+  // rows written by an atom's lanes, read by its other lanes
+  auto sync_rows = [&]() {
+    if constexpr (SUB > 1) __syncthreads();
+    else __syncwarp();
+  };
   const int i = blockIdx.x * AB + ia;
   // Lanes past the last atom, and (serving engine) those of a finished job frozen in the batch,
   // run along with no neighbours (the pair exchanges are warp-collective); they write nothing.
@@ -562,7 +580,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
 
   // ---- radial descriptor, Eq. qin: per neighbour type, sum_j T_k(x_j) fc_j/2 (k >= 1) and
   // sum_j fc_j/2, then F_0 = 2H, F_k = sum_j T_k fc_j/2 + H, contracted with c_nk
-  {
+  if (sub == 0) {
     float qr[(NR + 2) / 2];
 #pragma unroll
     for (int j = 0; j < (NR + 2) / 2; ++j) qr[j] = 0.f;
@@ -633,7 +651,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   }
 
   // ---- angular sums S_nk (Eq. S_nk, b_k of the unit vector): this lane's 12 polynomials
-  {
+  if (sub == 0) {
     float Sv[NA + 1][12];
 #pragma unroll
     for (int n = 0; n <= NA; ++n)
@@ -708,7 +726,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
       reinterpret_cast<float2 *>(r + 5)[h] = make_float2(Sv[n][10], Sv[n][11]);
     }
   }
-  __syncwarp();
+  sync_rows();
   // S_n of one n from the row, by polynomial index
   auto load_S = [&](int n, float *s) {
     static_for<0, 6>([&](auto qc) {
@@ -720,7 +738,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
 
   // ---- angular descriptor components (Sec. II D) of n = h, h + 2, ...
 #pragma unroll 1
-  for (int n = h; n <= NA; n += 2) {
+  for (int n = h + 2 * sub; n <= NA; n += 2 * SUB) {
     float s[24];
     load_S(n, s);
     static_for<0, S::L3>([&](auto lc) {
@@ -743,7 +761,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
       qrow[S::OFF5 + n] = mf.c5b[0] * s0 * s0 * s0 * s0 + mf.c5b[1] * s0 * s0 * s12 + mf.c5b[2] * s12 * s12;
     }
   }
-  __syncwarp();
+  sync_rows();
 
   if constexpr (DESC) {
     if (active) {
@@ -882,6 +900,79 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
     U = u_s[ia] - w1_s[S::H];
 #pragma unroll
     for (int v = 0; v <= NR; ++v) dq[v] = qrow[v];
+  } else if constexpr (SUB > 1) {
+    // As below, term by term: the groups share the neuron pairs of the forward sums, pass t = tanh
+    // and beta on, and share the float4s of dU/dq, each adding all neurons in order.
+    constexpr int V4 = NDP / 4, VJ = (V4 + 1) / 2;
+    float2 *const tb = reinterpret_cast<float2 *>(rows + AB * PR::R4);  // [H][AB] (w1 t's t, beta)
+    float4 q[VJ];
+#pragma unroll
+    for (int j = 0; j < VJ; ++j)
+      q[j] = 2 * j + h < V4 ? reinterpret_cast<const float4 *>(qrow)[2 * j + h] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int mu = 2 * sub; mu < S::H; mu += 2 * SUB) {
+      const bool two = S::H % 2 == 0 || mu + 1 < S::H;
+      const float4 *wr = reinterpret_cast<const float4 *>(w0_s + mu * NDP) + h;
+      float za[2] = {0.f, 0.f}, zb[2] = {0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < VJ; ++j) {
+        const bool in = V4 % 2 == 0 || 2 * j + h < V4;
+        const float4 wa = in ? wr[2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 wb = in && two ? wr[V4 + 2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        za[0] = __fmaf_rn(wa.x, q[j].x, za[0]);
+        zb[0] = __fmaf_rn(wb.x, q[j].x, zb[0]);
+        za[1] = __fmaf_rn(wa.y, q[j].y, za[1]);
+        zb[1] = __fmaf_rn(wb.y, q[j].y, zb[1]);
+        za[0] = __fmaf_rn(wa.z, q[j].z, za[0]);
+        zb[0] = __fmaf_rn(wb.z, q[j].z, zb[0]);
+        za[1] = __fmaf_rn(wa.w, q[j].w, za[1]);
+        zb[1] = __fmaf_rn(wb.w, q[j].w, zb[1]);
+      }
+      const float pa = __fadd_rn(za[0], za[1]), pb = __fadd_rn(zb[0], zb[1]);
+      const float zo = __shfl_xor_sync(kAll, h ? pa : pb, 1);
+      const int my = two ? mu + h : mu;
+      const float w1m = h == 0 || two ? w1_s[my] : 0.f;
+      const float t = tanhf(__fadd_rn(h ? pb : pa, zo) - b0_s[my]);
+      if (h == 0 || two) tb[my * AB + ia] = make_float2(t, w1m * (1.f - t * t));
+    }
+    __syncthreads();  // t and beta; every q is read
+    if (sub == 0) {
+#pragma unroll 2
+      for (int mu = 0; mu < S::H; mu += 2) {
+        const bool mine = h == 0 || S::H % 2 == 0 || mu + 1 < S::H;
+        if (mine) U = __fmaf_rn(w1_s[mu + h], tb[(mu + h) * AB + ia].x, U);
+      }
+      U = __fadd_rn(U, __shfl_xor_sync(kAll, U, 1)) - w1_s[S::H];
+    }
+    constexpr int WJ = (VJ + SUB - 1) / SUB;  // this group's float4s: sub, sub + SUB, ...
+    float4 dv[WJ];
+#pragma unroll
+    for (int w = 0; w < WJ; ++w) dv[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int mu = 0; mu < S::H; mu += 2) {
+      const bool two = S::H % 2 == 0 || mu + 1 < S::H;
+      const float ba = tb[mu * AB + ia].y, bb = two ? tb[(mu + 1) * AB + ia].y : 0.f;
+      const float4 *wr = reinterpret_cast<const float4 *>(w0_s + mu * NDP) + h;
+#pragma unroll
+      for (int w = 0; w < WJ; ++w) {
+        const int j = sub + w * SUB;
+        const bool in = 2 * j + h < V4;
+        const float4 wa = in ? wr[2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 wb = in && two ? wr[V4 + 2 * j] : make_float4(0.f, 0.f, 0.f, 0.f);
+        dv[w].x = __fmaf_rn(bb, wb.x, __fmaf_rn(ba, wa.x, dv[w].x));
+        dv[w].y = __fmaf_rn(bb, wb.y, __fmaf_rn(ba, wa.y, dv[w].y));
+        dv[w].z = __fmaf_rn(bb, wb.z, __fmaf_rn(ba, wa.z, dv[w].z));
+        dv[w].w = __fmaf_rn(bb, wb.w, __fmaf_rn(ba, wa.w, dv[w].w));
+      }
+    }
+#pragma unroll
+    for (int w = 0; w < WJ; ++w) {
+      const int j = sub + w * SUB;
+      if (2 * j + h < V4) reinterpret_cast<float4 *>(qrow)[2 * j + h] = dv[w];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v <= NR; ++v) dq[v] = qrow[v];
   } else {
     // On the FMA pipes: each lane holds every second float4 of q and of dU/dq; two neurons at a
     // time, the lanes exchange their parts of z (lane h completes neuron mu + h), take one tanh
@@ -938,11 +1029,11 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
 #pragma unroll
     for (int v = 0; v <= NR; ++v) dq[v] = qrow[v];
   }
-  if (active && h == 0 && a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = (double)U;
+  if (active && h == 0 && sub == 0 && a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = (double)U;
 
   // ---- radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_{nk} and their sum: every second
   // group of four k
-  for (int t = 0; t < T; ++t) {
+  for (int t = SUB - 1 - sub; t < T; t += SUB) {  // (the last group first: it has the fewest n below)
     const float4 *c = reinterpret_cast<const float4 *>(cR_s + (ti * T + t) * (NR + 1) * KRP);
     constexpr int E4 = S::EF4, EJ = (E4 + 1) / 2;
     float ev[EJ][4], tot = 0.f;
@@ -982,7 +1073,7 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
 
   // ---- dU/dS_nk from the explicit 3/4/5-body forms, in place of S_nk: n = h, h + 2, ...
 #pragma unroll 1
-  for (int n = h; n <= NA; n += 2) {
+  for (int n = h + 2 * sub; n <= NA; n += 2 * SUB) {
     float s[24], dS[24];
     load_S(n, s);
     static_for<0, 24>([&](auto kc) {
@@ -1013,26 +1104,27 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
       row[n * 6 + Q] = make_float4(dS[harm_k(4 * Q)], dS[harm_k(4 * Q + 1)], dS[harm_k(4 * Q + 2)], dS[harm_k(4 * Q + 3)]);
     });
   }
-  __syncwarp();
+  sync_rows();
 
   // ---- angular partial forces dU_i/dr_ij (angular terms of Eq. partial_force): with
   // a_k = sum_n dU/dS_nk g_n and c_k = sum_n dU/dS_nk g_n',
   //   dU_i/dr_ij = (G - (G.u) u) / r + Y u,  G = sum_k a_k grad b_k(u),  Y = sum_k c_k b_k(u)
-  if (2 * h < na) {
-    constexpr int PP = 2;
+  if (4 * sub + 2 * h < na) {
+    constexpr int PP = 2, STEP = 4 * SUB;
+    const int first = 4 * sub + 2 * h;
     const unsigned *col = a.nl_a + i;
     unsigned ec[PP], en[PP];
     float4 pc[PP];
 #pragma unroll
     for (int p = 0; p < PP; ++p) {
-      const int m = 2 * h + p;
+      const int m = first + p;
       ec[p] = m < na ? __ldg(col + (size_t)m * N) : 0u;
-      en[p] = m + 4 < na ? __ldg(col + (size_t)(m + 4) * N) : 0u;
+      en[p] = m + STEP < na ? __ldg(col + (size_t)(m + STEP) * N) : 0u;
     }
 #pragma unroll
     for (int p = 0; p < PP; ++p) pc[p] = __ldg(a.pos4 + (ec[p] & a.jmask));
 #pragma unroll 1
-    for (int m0 = 2 * h; m0 < na; m0 += 4) {
+    for (int m0 = first; m0 < na; m0 += STEP) {
       float3 d[PP];
       float r2[PP];
       bool in[PP], any = false;
@@ -1045,8 +1137,8 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
         in[p] = m0 + p < na && r2[p] < rcA2;
         any = any || in[p];
         ec[p] = en[p];
-        if (m0 + 4 < na) pc[p] = __ldg(a.pos4 + (en[p] & a.jmask));
-        en[p] = m0 + 8 + p < na ? __ldg(col + (size_t)(m0 + 8 + p) * N) : 0u;
+        if (m0 + STEP < na) pc[p] = __ldg(a.pos4 + (en[p] & a.jmask));
+        en[p] = m0 + 2 * STEP + p < na ? __ldg(col + (size_t)(m0 + 2 * STEP + p) * N) : 0u;
       }
       if (!any) continue;
       float rinv[PP], g[PP][NA + 1], gp[PP][NA + 1];
@@ -1107,19 +1199,29 @@ __global__ void __launch_bounds__(2 * AB, PairRow<S>::OCC * 64 / AB)
   if constexpr (!BATCH) {
     // deterministic block sum of U where it is read (a batch sums its structures from the
     // per-atom energies)
-    static_assert(AB == 64, "one slot per 64 atoms (atom_blocks)");
+    // (up to kSplitAtoms2 atoms a slot per warp's 16 atoms, so that all forms agree on atom_blocks)
+    static_assert(AB == 64 || SUB > 1, "slots of 64 or of 16 atoms");
     if (sums_needed(a) & kSumU) {
       __shared__ double red[2 * AB / 32];
-      Sum2 su;
-      su.add(active && h == 0 ? U : 0.f);
+      const int warp = threadIdx.x >> 5;
+      if (sub == 0) {
+        Sum2 su;
+        su.add(active && h == 0 ? U : 0.f);
 #pragma unroll
-      for (int o = 16; o > 1; o >>= 1) su.across(o);  // lanes of one parity: h == 0 holds the sum
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = su.value();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int wv = 0; wv < 2 * AB / 32; ++wv) t += red[wv];
-        a.partial_atom[blockIdx.x] = t;
+        for (int o = 16; o > 1; o >>= 1) su.across(o);  // lanes of one parity: h == 0 holds the sum
+        if ((threadIdx.x & 31) == 0) {
+          if (N > kSplitAtoms2) red[warp] = su.value();
+          else if (blockIdx.x * (AB / 16) + warp < (N + 15) / 16)
+            a.partial_atom[blockIdx.x * (AB / 16) + warp] = su.value();
+        }
+      }
+      if (N > kSplitAtoms2) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          double t = 0.0;
+          for (int wv = 0; wv < 2 * AB / 32; ++wv) t += red[wv];
+          a.partial_atom[blockIdx.x] = t;
+        }
       }
     }
   }
@@ -1256,14 +1358,15 @@ __device__ __forceinline__ void gather_finish(const AtomArgs &a, int mem, float 
 // shorten it further (216 atoms: 13.8 us) but cost large ones more than they give
 // (8,000,000 atoms: 2.98 ms). Before / after (one thread per atom, all block sums in every
 // launch), us: 216 Si atoms 32 / 18, 262,144 PbTe atoms 121 / 100, 8,000,000 Si atoms 2846 /
-// 2472, 4096 structures 681 / 550.
+// 2472, 4096 structures 681 / 550. Up to kSplitGather2 atoms SUB groups of lanes work out an atom's
+// pairs side by side, and the pair sums are added in the order of the plain form (the same bits).
 constexpr int kGatherLanes = 2;
 constexpr int gather_min_blocks(int KR, int threads) {
   return (KR <= 8 ? 1024 : 896) / threads > 0 ? (KR <= 8 ? 1024 : 896) / threads : 1;
 }
 
-template <class S, bool BATCH, int GA>
-__global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA *kGatherLanes))
+template <class S, bool BATCH, int GA, int SUB>
+__global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_min_blocks(S::KR, GA *kGatherLanes))
     gather_kernel(const AtomArgs a) {
   if (!BATCH && build_failed(a.guard)) return;
   constexpr int L = kGatherLanes;
@@ -1280,7 +1383,7 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
   const float *e_rad = a.e_rad + mem * a.s_erad;
   const float4 *p_ang = a.p_ang + mem * a.s_pang;
   const int N = a.N, T = a.T;
-  const int ia = threadIdx.x / L, l = threadIdx.x % L;
+  const int ia = threadIdx.x / (L * SUB), l = threadIdx.x % L, sub = threadIdx.x % (L * SUB) / L;
   const int i = blockIdx.x * GA + ia;
   float fx = 0.f, fy = 0.f, fz = 0.f;
   float w[9];
@@ -1288,8 +1391,8 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
   for (int c = 0; c < 9; ++c) w[c] = 0.f;
   // (serving engine) atoms of a finished job frozen in the batch are skipped
   const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2);
-  if (active) {
-    const float4 pi = a.pos4[i];
+  if (active || SUB > 1) {  // (the lanes of a split atom exchange their pairs: whole warps)
+    const float4 pi = a.pos4[active ? i : 0];
     const int ti = type_of(pi);
     const float4 *dtab_b = BATCH ? a.dtab + (size_t)struct_of(pi) * a.ncode : dtab_s;
     auto shift = [&](unsigned e) -> float4 {
@@ -1306,6 +1409,142 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
         e[4 * k4] = v.x, e[4 * k4 + 1] = v.y, e[4 * k4 + 2] = v.z, e[4 * k4 + 3] = v.w;
       }
     };
+    // s_i and s_j of a pair at distance r from the atom's own and the neighbour's coefficients
+    auto radial_terms = [&](const float *eo, const float *ej, float r, float &si, float &sj) {
+      // sum_k e_k f_k'(r) = (x' fc/2) sum_k e_k T_k'(x) + (fc'/2) (sum_k e_k T_k(x) + sum_k e_k)
+      const float u = r * inv_rcR;
+      float sn, cs;
+      __sincosf(3.14159265358979f * u, &sn, &cs);
+      const float hfc = 0.25f * (1.f + cs);
+      const float hfcp = -0.25f * 3.14159265358979f * inv_rcR * sn;
+      const float t1 = u - 1.f;
+      const float x = 2.f * t1 * t1 - 1.f;
+      const float xp = 4.f * t1 * inv_rcR;
+      const float x2 = 2.f * x;
+      float tkm1 = 1.f, tk = x, dkm1 = 0.f, dk = 1.f;
+      float oT = eo[0], oD = 0.f, jT = ej[0], jD = 0.f;
+      if (KR >= 1) {
+        oT = __fmaf_rn(eo[1], x, oT);
+        jT = __fmaf_rn(ej[1], x, jT);
+        oD = eo[1];
+        jD = ej[1];
+      }
+#pragma unroll
+      for (int k = 2; k <= KR; ++k) {
+        const float tn = __fmaf_rn(x2, tk, -tkm1);
+        const float dn = __fmaf_rn(x2, dk, __fmaf_rn(2.f, tk, -dkm1));
+        tkm1 = tk; tk = tn; dkm1 = dk; dk = dn;
+        oT = __fmaf_rn(eo[k], tn, oT);
+        jT = __fmaf_rn(ej[k], tn, jT);
+        oD = __fmaf_rn(eo[k], dn, oD);
+        jD = __fmaf_rn(ej[k], dn, jD);
+      }
+      const float a1 = xp * hfc;
+      si = __fmaf_rn(a1, oD, hfcp * (oT + eo[KR + 1]));
+      sj = __fmaf_rn(a1, jD, hfcp * (jT + ej[KR + 1]));
+    };
+    auto add_radial = [&](const float3 &d, float fs, float ws) {
+      fx = __fmaf_rn(fs, d.x, fx);
+      fy = __fmaf_rn(fs, d.y, fy);
+      fz = __fmaf_rn(fs, d.z, fz);
+      // W_i += r_ij (x) dU_j/dr_ji with dU_j/dr_ji = -s_j d / r
+      const float px = ws * d.x, py = ws * d.y, pz = ws * d.z;
+      w[0] = __fmaf_rn(d.x, px, w[0]);
+      w[1] = __fmaf_rn(d.y, py, w[1]);
+      w[2] = __fmaf_rn(d.z, pz, w[2]);
+      w[3] = __fmaf_rn(d.x, py, w[3]);
+      w[4] = __fmaf_rn(d.x, pz, w[4]);
+      w[5] = __fmaf_rn(d.y, pz, w[5]);
+      w[6] = __fmaf_rn(d.y, px, w[6]);
+      w[7] = __fmaf_rn(d.z, px, w[7]);
+      w[8] = __fmaf_rn(d.z, py, w[8]);
+    };
+    auto add_angular = [&](const float3 &d, const float3 &df, const float3 &p) {
+      fx += df.x;
+      fy += df.y;
+      fz += df.z;
+      w[0] = __fmaf_rn(d.x, p.x, w[0]);
+      w[1] = __fmaf_rn(d.y, p.y, w[1]);
+      w[2] = __fmaf_rn(d.z, p.z, w[2]);
+      w[3] = __fmaf_rn(d.x, p.y, w[3]);
+      w[4] = __fmaf_rn(d.x, p.z, w[4]);
+      w[5] = __fmaf_rn(d.y, p.z, w[5]);
+      w[6] = __fmaf_rn(d.y, p.x, w[6]);
+      w[7] = __fmaf_rn(d.z, p.x, w[7]);
+      w[8] = __fmaf_rn(d.z, p.y, w[8]);
+    };
+    if constexpr (SUB > 1) {
+      // Lane (l, sub) works out the pairs l + 2 (sub + SUB r) of its list; then every lane of parity l
+      // adds the SUB pairs of the round in list order, as the one lane of the form below does.
+      constexpr unsigned kAll = 0xffffffffu;
+      const int lane = threadIdx.x & 31, first = (lane & ~(L * SUB - 1)) | l;
+      int base = 0;
+      for (int t = 0; t < T; ++t) {
+        const int cnt = active ? a.nn_r[(size_t)t * N + i] : 0;
+        const int nl = (cnt + L - 1 - l) / L;
+        float eo[4 * S::EF4];
+        load_e(eo, t, active ? i : 0);
+        const unsigned *col = a.nl_r + (size_t)(base + l) * N + i;
+        const int rounds = __reduce_max_sync(kAll, (nl + SUB - 1) / SUB);
+        unsigned e1 = sub < nl ? __ldg(col + (size_t)L * sub * N) : 0u;
+#pragma unroll 1
+        for (int r = 0; r < rounds; ++r) {
+          const int q = SUB * r + sub;
+          const unsigned e = e1;
+          e1 = q + SUB < nl ? __ldg(col + (size_t)L * (q + SUB) * N) : 0u;
+          const int j = e & a.jmask;
+          const float3 d = pair_vector(pi, __ldg(a.pos4 + j), shift(e));
+          const float r2 = norm2(d);
+          const bool in = q < nl && r2 < rcR2;
+          float fs = 0.f, ws = 0.f;
+          if (in) {
+            const float rinv = rsqrtf(r2);
+            float ej[4 * S::EF4], si, sj;
+            load_e(ej, ti, j);
+            radial_terms(eo, ej, r2 * rinv, si, sj);
+            fs = (si + sj) * rinv;
+            ws = -sj * rinv;
+          }
+          const unsigned mask = __ballot_sync(kAll, in);
+#pragma unroll
+          for (int s = 0; s < SUB; ++s) {
+            const int src = first + L * s;
+            const float3 ds = make_float3(__shfl_sync(kAll, d.x, src), __shfl_sync(kAll, d.y, src),
+                                          __shfl_sync(kAll, d.z, src));
+            const float f1 = __shfl_sync(kAll, fs, src), w1 = __shfl_sync(kAll, ws, src);
+            if ((mask >> src) & 1u) add_radial(ds, f1, w1);
+          }
+        }
+        base += cnt;
+      }
+      const int na = active ? a.nn_a[i] : 0, nl = (na + L - 1 - l) / L;
+      const int rounds = __reduce_max_sync(kAll, (nl + SUB - 1) / SUB);
+#pragma unroll 1
+      for (int r = 0; r < rounds; ++r) {
+        const int q = SUB * r + sub;
+        float3 d = make_float3(0.f, 0.f, 0.f), df = d, p = d;
+        bool in = false;
+        if (q < nl) {
+          const size_t slot = (size_t)(L * q + l) * N + i;
+          const unsigned e = __ldg(a.nl_a + slot);
+          const float4 pij = p_ang[slot], pji = __ldg(p_ang + __ldg(a.rev_a + slot));
+          d = pair_vector(pi, __ldg(a.pos4 + (e & a.jmask)), shift(e));
+          in = norm2(d) < rcA2;
+          df = make_float3(pij.x - pji.x, pij.y - pji.y, pij.z - pji.z);
+          p = make_float3(pji.x, pji.y, pji.z);
+        }
+        const unsigned mask = __ballot_sync(kAll, in);
+#pragma unroll
+        for (int s = 0; s < SUB; ++s) {
+          const int src = first + L * s;
+          float v[9] = {d.x, d.y, d.z, df.x, df.y, df.z, p.x, p.y, p.z};
+#pragma unroll
+          for (int c = 0; c < 9; ++c) v[c] = __shfl_sync(kAll, v[c], src);
+          if ((mask >> src) & 1u)
+            add_angular(make_float3(v[0], v[1], v[2]), make_float3(v[3], v[4], v[5]), make_float3(v[6], v[7], v[8]));
+        }
+      }
+    } else {
     // ---- radial part (Algorithm 2): s_i from own e^{t_j}, s_j from neighbour's e^{t_i}
     int base = 0;
     for (int t = 0; t < T; ++t) {
@@ -1321,53 +1560,9 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
           const float r = r2 * rinv;
           float ej[4 * S::EF4];
           load_e(ej, ti, j);
-          // sum_k e_k f_k'(r) = (x' fc/2) sum_k e_k T_k'(x) + (fc'/2) (sum_k e_k T_k(x) + sum_k e_k)
-          const float u = r * inv_rcR;
-          float sn, cs;
-          __sincosf(3.14159265358979f * u, &sn, &cs);
-          const float hfc = 0.25f * (1.f + cs);
-          const float hfcp = -0.25f * 3.14159265358979f * inv_rcR * sn;
-          const float t1 = u - 1.f;
-          const float x = 2.f * t1 * t1 - 1.f;
-          const float xp = 4.f * t1 * inv_rcR;
-          const float x2 = 2.f * x;
-          float tkm1 = 1.f, tk = x, dkm1 = 0.f, dk = 1.f;
-          float oT = eo[0], oD = 0.f, jT = ej[0], jD = 0.f;
-          if (KR >= 1) {
-            oT = __fmaf_rn(eo[1], x, oT);
-            jT = __fmaf_rn(ej[1], x, jT);
-            oD = eo[1];
-            jD = ej[1];
-          }
-#pragma unroll
-          for (int k = 2; k <= KR; ++k) {
-            const float tn = __fmaf_rn(x2, tk, -tkm1);
-            const float dn = __fmaf_rn(x2, dk, __fmaf_rn(2.f, tk, -dkm1));
-            tkm1 = tk; tk = tn; dkm1 = dk; dk = dn;
-            oT = __fmaf_rn(eo[k], tn, oT);
-            jT = __fmaf_rn(ej[k], tn, jT);
-            oD = __fmaf_rn(eo[k], dn, oD);
-            jD = __fmaf_rn(ej[k], dn, jD);
-          }
-          const float a1 = xp * hfc;
-          const float si = __fmaf_rn(a1, oD, hfcp * (oT + eo[KR + 1]));
-          const float sj = __fmaf_rn(a1, jD, hfcp * (jT + ej[KR + 1]));
-          const float fs = (si + sj) * rinv;
-          fx = __fmaf_rn(fs, d.x, fx);
-          fy = __fmaf_rn(fs, d.y, fy);
-          fz = __fmaf_rn(fs, d.z, fz);
-          // W_i += r_ij (x) dU_j/dr_ji with dU_j/dr_ji = -s_j d / r
-          const float ws = -sj * rinv;
-          const float px = ws * d.x, py = ws * d.y, pz = ws * d.z;
-          w[0] = __fmaf_rn(d.x, px, w[0]);
-          w[1] = __fmaf_rn(d.y, py, w[1]);
-          w[2] = __fmaf_rn(d.z, pz, w[2]);
-          w[3] = __fmaf_rn(d.x, py, w[3]);
-          w[4] = __fmaf_rn(d.x, pz, w[4]);
-          w[5] = __fmaf_rn(d.y, pz, w[5]);
-          w[6] = __fmaf_rn(d.y, px, w[6]);
-          w[7] = __fmaf_rn(d.z, px, w[7]);
-          w[8] = __fmaf_rn(d.z, py, w[8]);
+          float si, sj;
+          radial_terms(eo, ej, r, si, sj);
+          add_radial(d, (si + sj) * rinv, -sj * rinv);
         }
       });
       base += cnt;
@@ -1402,20 +1597,10 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
         const float3 d = pair_vector(pi, pj, shift(e));
         const float r2 = norm2(d);
         if (r2 < rcA2) {
-          fx += pij.x - pji.x;
-          fy += pij.y - pji.y;
-          fz += pij.z - pji.z;
-          w[0] = __fmaf_rn(d.x, pji.x, w[0]);
-          w[1] = __fmaf_rn(d.y, pji.y, w[1]);
-          w[2] = __fmaf_rn(d.z, pji.z, w[2]);
-          w[3] = __fmaf_rn(d.x, pji.y, w[3]);
-          w[4] = __fmaf_rn(d.x, pji.z, w[4]);
-          w[5] = __fmaf_rn(d.y, pji.z, w[5]);
-          w[6] = __fmaf_rn(d.y, pji.x, w[6]);
-          w[7] = __fmaf_rn(d.z, pji.x, w[7]);
-          w[8] = __fmaf_rn(d.z, pji.y, w[8]);
+          add_angular(d, make_float3(pij.x - pji.x, pij.y - pji.y, pij.z - pji.z), make_float3(pji.x, pji.y, pji.z));
         }
       }
+    }
     }
   }
   // the sums of the atom's lanes; one row per atom for the epilogue
@@ -1424,23 +1609,24 @@ __global__ void __launch_bounds__(GA *kGatherLanes, gather_min_blocks(S::KR, GA 
   for (int c = 0; c < 12; ++c) {
 #pragma unroll
     for (int o = 1; o < L; o <<= 1) v[c] = __fadd_rn(v[c], __shfl_xor_sync(0xffffffffu, v[c], o));
-    if (l == 0) fw[ia][c] = v[c];
+    if (l == 0 && sub == 0) fw[ia][c] = v[c];
   }
-  if (l == 0) on[ia] = active ? 1 : 0;
-  gather_finish<GA, GA * L>(a, mem, fw, on);
+  if (l == 0 && sub == 0) on[ia] = active ? 1 : 0;
+  gather_finish<GA, GA * L * SUB>(a, mem, fw, on);
 }
 
 // ------------------------------------------------------------------------ launchers
 // block sums of U of one structure: one slot per 64 atoms, an even number of them
-template <class S> int atom_blocks(int N) { return 2 * ((N + 127) / 128); }
+template <class S> int atom_blocks(int N) { return N <= kSplitAtoms2 ? (N + 15) / 16 : 2 * ((N + 127) / 128); }
 
-template <class S, int PREC, bool DESC, bool BATCH, int AB>
+template <class S, int PREC, bool DESC, bool BATCH, int AB, int SUB = 1>
 cudaError_t launch_atom_as(const AtomArgs &a, const ModelF &mf, int members, cudaStream_t st) {
-  auto kern = atom_kernel<S, PREC, DESC, BATCH, AB>;
-  const cudaError_t e = smem_limit_once(kern, atom_pair_smem<S>(kMaxTypes, BATCH ? 0 : 1 << 9, PREC, AB));
+  auto kern = atom_kernel<S, PREC, DESC, BATCH, AB, SUB>;
+  constexpr size_t tb = SUB > 1 ? sizeof(float2) * S::H * AB : 0;
+  const cudaError_t e = smem_limit_once(kern, tb + atom_pair_smem<S>(kMaxTypes, BATCH ? 0 : 1 << 9, PREC, AB));
   if (e != cudaSuccess) return e;
-  const int blocks = (!BATCH && AB == 64) ? atom_blocks<S>(a.N) : (a.N + AB - 1) / AB;
-  kern<<<dim3(blocks, members), 2 * AB, atom_pair_smem<S>(a.T, BATCH ? 0 : a.ncode, PREC, AB), st>>>(a, mf);
+  const int blocks = (!BATCH && AB == 64) ? 2 * ((a.N + 127) / 128) : (a.N + AB - 1) / AB;
+  kern<<<dim3(blocks, members), 2 * AB * SUB, tb + atom_pair_smem<S>(a.T, BATCH ? 0 : a.ncode, PREC, AB), st>>>(a, mf);
   return cudaGetLastError();
 }
 
@@ -1450,17 +1636,30 @@ cudaError_t launch_atom(const AtomArgs &a, const ModelF &mf, int descriptor_only
   if (descriptor_only) return launch_atom_as<S, 0, true, false, 64>(a, mf, 1, st);
   if (a.precision == 1) return launch_atom_as<S, 1, false, false, 64>(a, mf, 1, st);
   if (a.precision == 2) return launch_atom_as<S, 2, false, false, 64>(a, mf, 1, st);
+  if (a.N <= kSplitAtoms) return launch_atom_as<S, 0, false, false, 16, 4>(a, mf, 1, st);
+  if (a.N <= kSplitAtoms2) return launch_atom_as<S, 0, false, false, 32, 2>(a, mf, 1, st);
   return launch_atom_as<S, 0, false, false, 64>(a, mf, 1, st);
 }
 
 constexpr int kGatherAtoms = 64;  // atoms per CTA of the gather of one structure
+// Small systems: four groups of lanes per atom (half as many atoms per CTA), then two, up to one wave
+// of two CTAs per SM. A dynamics step with one / four / two groups, us: 1,000 Si atoms 43 / 36 / -,
+// 8,000 53 / 46 / -, 13,824 60.4 / 62.8 / 57.4, 13,824 PbTe atoms 54.0 / 53.7 / 48.8, 21,952 Si atoms
+// 71 / 79 / -.
+constexpr int kSplitGather = 152 * 2 * 32, kSplitGather2 = 152 * 2 * 64;
 
 template <class S>
 cudaError_t launch_gather(const AtomArgs &a, cudaStream_t st) {
   if (a.N <= 0) return cudaSuccess;
-  constexpr int GA = kGatherAtoms;
-  gather_kernel<S, false, GA><<<(a.N + GA - 1) / GA, GA * kGatherLanes, sizeof(float4) * a.ncode, st>>>(a);
-  return cudaGetLastError();
+  auto go = [&](auto ga, auto sub) {
+    constexpr int GA = decltype(ga)::value, SUB = decltype(sub)::value;
+    gather_kernel<S, false, GA, SUB><<<(a.N + GA - 1) / GA, GA * kGatherLanes * SUB, sizeof(float4) * a.ncode, st>>>(a);
+    return cudaGetLastError();
+  };
+  using std::integral_constant;
+  if (a.N <= kSplitGather) return go(integral_constant<int, kGatherAtoms / 2>{}, integral_constant<int, 4>{});
+  if (a.N <= kSplitGather2) return go(integral_constant<int, kGatherAtoms>{}, integral_constant<int, 2>{});
+  return go(integral_constant<int, kGatherAtoms>{}, integral_constant<int, 1>{});
 }
 
 // Batched launches (grid.y = population members); instantiated in the nep_batch_*.cu units.
@@ -1477,6 +1676,8 @@ cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, int members, 
   if (a.precision >= 1 && block != 128) return cudaErrorInvalidValue;
   if (a.precision == 1) return launch_atom_as<S, 1, false, true, 64>(a, mf, members, st);
   if (a.precision == 2) return launch_atom_as<S, 2, false, true, 64>(a, mf, members, st);
+  if (members == 1 && a.N <= kSplitAtoms) return launch_atom_as<S, 0, false, true, 16, 4>(a, mf, 1, st);
+  if (members == 1 && a.N <= kSplitAtoms2) return launch_atom_as<S, 0, false, true, 32, 2>(a, mf, 1, st);
   return block == 64 ? launch_atom_as<S, 0, false, true, 64>(a, mf, members, st)
                      : launch_atom_as<S, 0, false, true, 128>(a, mf, members, st);
 }
@@ -1484,13 +1685,22 @@ cudaError_t launch_atom_batch(const AtomArgs &a, const ModelF &mf, int members, 
 template <class S>
 cudaError_t launch_gather_batch(const AtomArgs &a, int members, int block, cudaStream_t st) {
   if (a.N <= 0 || members <= 0) return cudaSuccess;
-  const dim3 grid((a.N + block - 1) / block, members);
   constexpr int L = kGatherLanes;
-  if (block == 64) gather_kernel<S, true, 64><<<grid, 64 * L, 0, st>>>(a);
-  else if (block == 128) gather_kernel<S, true, 128><<<grid, 128 * L, 0, st>>>(a);
-  else if (block == 256) gather_kernel<S, true, 256><<<grid, 256 * L, 0, st>>>(a);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  auto go = [&](auto ga, auto sub) {
+    constexpr int GA = decltype(ga)::value, SUB = decltype(sub)::value;
+    gather_kernel<S, true, GA, SUB><<<dim3((a.N + GA - 1) / GA, members), GA * L * SUB, 0, st>>>(a);
+    return cudaGetLastError();
+  };
+  using std::integral_constant;
+  if (block != 64 && block != 128 && block != 256) return cudaErrorInvalidValue;
+  if (members == 1 && !a.sums && !a.sums_always) {  // no block sums, whose reader counts on `block`
+    if (a.N <= kSplitGather) return go(integral_constant<int, kGatherAtoms / 2>{}, integral_constant<int, 4>{});
+    if (a.N <= kSplitGather2) return go(integral_constant<int, kGatherAtoms>{}, integral_constant<int, 2>{});
+  }
+  const integral_constant<int, 1> one;
+  if (block == 64) return go(integral_constant<int, 64>{}, one);
+  if (block == 128) return go(integral_constant<int, 128>{}, one);
+  return go(integral_constant<int, 256>{}, one);
 }
 
 template <class S>
@@ -1503,7 +1713,10 @@ template <class S>
 void attach_batch(ShapeOps &o);  // explicitly instantiated in the batch translation unit
 #endif
 
-template <class S> int gather_blocks(int N) { return (N + kGatherAtoms - 1) / kGatherAtoms; }
+template <class S> int gather_blocks(int N) {
+  const int ga = N <= kSplitGather ? kGatherAtoms / 2 : kGatherAtoms;
+  return (N + ga - 1) / ga;
+}
 
 template <class S>
 ShapeOps make_ops() {

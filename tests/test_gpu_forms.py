@@ -81,3 +81,32 @@ def test_large_batch_equals_its_structures_alone(torch_cuda):
             np.testing.assert_array_equal(lists["d_" + r][a:e][m], l1["d_" + r][m])
     h.close()
     h1.close()
+
+
+@pytest.mark.parametrize("name", ["si", "pbte", "mixed"])
+def test_split_forms_equal_the_plain_ones(torch_cuda, name):
+    """Small systems share an atom's work among four or two groups of lanes (kernel limits 7,296,
+    9,728, 14,592 and 19,456 atoms); a batch of all of them together does not. The same bits per
+    atom, and totals that are their sums (pairs of FP32 words, about 48 bits: 1e-9 is ample)."""
+    from paper_2205_10046_gb300 import nep
+    torch = torch_cuda
+    model = {"si": lambda: W.random_model(W.SI_MODEL, 0, [W.MASS_SI]),
+             "pbte": lambda: W.random_model(W.PBTE_MODEL, 1, [W.MASS_PB, W.MASS_TE]),
+             "mixed": lambda: W.mixed_model(0)}[name]()
+    sizes = [1, 16, 33, 7296, 7297, 9729, 14592, 14593, 19457]
+    parts = [W.random_structure(700 + k, n, n_types_model=model.n_types) for k, n in enumerate(sizes)]
+    b = W.concat_structures(parts)
+    h = nep.NEP(model, skin=0.4)
+    g = _np(h.compute_batch(b.offsets, *_dev(torch, b.pos, b.types), b.boxes, per_atom=True))
+    for s in range(b.n_struct):
+        pos, types, box = b.structure(s)
+        a, e = int(b.offsets[s]), int(b.offsets[s + 1])
+        dev = _dev(torch, pos, types)
+        one = _np(h.compute(*dev, box, per_atom_virial=True))
+        few = _np(h.compute_batch(np.array([0, e - a]), *dev, np.asarray(box).reshape(1, 9), per_atom=True))
+        for k in ("U", "F", "W"):
+            np.testing.assert_array_equal(g[k][a:e], one[k], err_msg=f"{k} of {e - a} atoms")
+            np.testing.assert_array_equal(g[k][a:e], few[k], err_msg=f"{k} of {e - a} atoms, batch of one")
+        assert abs(one["E"][0] - one["U"].sum()) <= 1e-9 * np.abs(one["U"]).sum()
+        assert np.abs(one["W_total"].reshape(9) - one["W"].sum(0)).max() <= 1e-9 * np.abs(one["W"]).sum()
+    h.close()
