@@ -272,26 +272,45 @@ thread_local std::string g_create_error;  // per calling thread (serving workers
 thread_local cudaStream_t t_alloc_stream = nullptr;
 thread_local bool t_alloc_async = false;
 
-// Wait for a stream. Threads in the stream-ordered mode (the serving workers, many per CPU
-// core) poll with short sleeps instead of spinning in cudaStreamSynchronize.
-cudaError_t wait_stream(cudaStream_t s) {
-  if (!t_alloc_async) return cudaStreamSynchronize(s);
+// Wait until query() is no longer "not ready". Threads in the stream-ordered mode (the serving
+// workers) poll for a short while, as most of their waits end within it, and then with sleeps: a
+// sleep of 20 us returns after about 70, which every chunk of iterations and every finished job
+// paid.
+template <class Query>
+cudaError_t poll(Query &&query) {
+  const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
-    const cudaError_t e = cudaStreamQuery(s);
+    const cudaError_t e = query();
     if (e != cudaErrorNotReady) return e;
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
+    if (std::chrono::steady_clock::now() - t0 < std::chrono::microseconds(200)) std::this_thread::yield();
+    else std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
+}
+cudaError_t wait_stream(cudaStream_t s) {
+  return t_alloc_async ? poll([&] { return cudaStreamQuery(s); }) : cudaStreamSynchronize(s);
+}
+cudaError_t wait_event(cudaEvent_t ev) {
+  return t_alloc_async ? poll([&] { return cudaEventQuery(ev); }) : cudaEventSynchronize(ev);
 }
 
-// The same for an event recorded in a stream.
-cudaError_t wait_event(cudaEvent_t ev) {
-  if (!t_alloc_async) return cudaEventSynchronize(ev);
-  for (;;) {
-    const cudaError_t e = cudaEventQuery(ev);
-    if (e != cudaErrorNotReady) return e;
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
+// Page-locked host buffer that only grows (device accessible at the same address).
+struct PinnedBuf {
+  unsigned char *p = nullptr;
+  size_t n = 0;
+  cudaError_t ensure(size_t want) {
+    if (want <= n) return cudaSuccess;
+    release();
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&p), want + want / 2, cudaHostAllocDefault);
+    if (e == cudaSuccess) n = want + want / 2;
+    else p = nullptr;
+    return e;
   }
-}
+  void release() {
+    if (p) cudaFreeHost(p);
+    p = nullptr;
+    n = 0;
+  }
+};
 
 template <class Tp>
 struct DevBuf {
@@ -397,6 +416,8 @@ struct nep_handle {
   // batched serving engine: one structure per job, all advanced by one iteration
   std::vector<EngineSlot> e_slots_h;            // host mirror (after the last iteration)
   std::vector<double> e_energy_h, e_virial_h;   // per job, after the last iteration
+  PinnedBuf e_read, e_out;                      // job states read back; arrays of finished jobs
+  std::vector<size_t> e_out_at;                 // their offsets in e_out (doubles)
   DevBuf<EngineSlot> e_slots, e_slots_ck;
   DevBuf<int> e_sflag;  // per-job build requests of the drift kernel (partial builds)
   DevBuf<double> e_energy, e_virial, e_u, e_w, e_xck, e_vck;
@@ -1171,6 +1192,10 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
   CK(h->ck_x.ensure(3 * (size_t)N), "alloc checkpoint");
   int rc = ensure_partials(h, N, 1);
   if (rc) return rc;
+  static_assert(alignof(EngineSlot) <= alignof(double), "the job states follow 10 doubles per job");
+  CK(h->e_read.ensure((sizeof(EngineSlot) + 10 * sizeof(double)) * (size_t)S), "alloc read back");
+  double *const r_energy = reinterpret_cast<double *>(h->e_read.p), *const r_virial = r_energy + S;
+  EngineSlot *const r_slots = reinterpret_cast<EngineSlot *>(r_virial + 9 * (size_t)S);
   for (int attempt = 0;; ++attempt) {
     // a build re-sorts the atoms: the checkpoint holds every per-atom array (x_ref too)
     CK(cudaMemcpyAsync(h->e_xck.p, h->x.p, sizeof(double) * 3 * N, cudaMemcpyDeviceToDevice, s), "checkpoint");
@@ -1207,7 +1232,11 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     // its per-atom values unchanged) or the chunk's last state is ever read
     launch_struct_sums(S, 1, h->d_offsets.p, N, h->e_u.p, h->e_w.p, h->e_energy.p, h->e_virial.p,
                        max_struct_atoms(h), s);
+    // everything the host looks at in one go (job states of an undone chunk are not used)
     CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
+    CK(cudaMemcpyAsync(r_slots, h->e_slots.p, sizeof(EngineSlot) * S, cudaMemcpyDeviceToHost, s), "read back");
+    CK(cudaMemcpyAsync(r_energy, h->e_energy.p, sizeof(double) * S, cudaMemcpyDeviceToHost, s), "read back");
+    CK(cudaMemcpyAsync(r_virial, h->e_virial.p, sizeof(double) * 9 * S, cudaMemcpyDeviceToHost, s), "read back");
     CK(wait_stream(s), "sync");
     const BuildStatus st = *h->h_status;
     if (st.tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
@@ -1228,46 +1257,41 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     int rc2 = ensure_lists(h, N, round_cap(st.max_r), round_cap(st.max_a));
     if (rc2) return rc2;
   }
-  std::vector<EngineSlot> sl(S);
-  CK(cudaMemcpyAsync(sl.data(), h->e_slots.p, sizeof(EngineSlot) * S, cudaMemcpyDeviceToHost, s), "read back");
-  CK(cudaMemcpyAsync(h->e_energy_h.data(), h->e_energy.p, sizeof(double) * S, cudaMemcpyDeviceToHost, s), "read back");
-  CK(cudaMemcpyAsync(h->e_virial_h.data(), h->e_virial.p, sizeof(double) * 9 * S, cudaMemcpyDeviceToHost, s),
-     "read back");
-  CK(wait_stream(s), "sync");
-  h->e_slots_h = sl;
+  h->e_slots_h.assign(r_slots, r_slots + S);
+  h->e_energy_h.assign(r_energy, r_energy + S);
+  h->e_virial_h.assign(r_virial, r_virial + 9 * (size_t)S);
   return NEP_OK;
 }
 
 long long engine_builds(const nep_handle *h) { return h->h_status ? h->h_status->n_rebuilds : 0; }
 
-// Final arrays of job k in its own atom order: positions wrapped into its cell, forces,
-// velocities (HOST buffers [n][3], any may be null).
-int engine_fetch(nep_handle *h, int k, double *pos, double *force, double *vel, cudaStream_t s) {
-  if (k < 0 || k >= h->nb_struct) return fail(h, NEP_ERR_ARG, "engine: bad job index");
-  const int o = h->b_offsets[k], n = h->b_offsets[k + 1] - o;
-  std::vector<double> x(3 * (size_t)n), f(3 * (size_t)n), v(3 * (size_t)n);
-  std::vector<int> perm(n);
-  CK(cudaMemcpyAsync(x.data(), h->x.p + 3 * (size_t)o, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s), "read");
-  CK(cudaMemcpyAsync(f.data(), h->F.p + 3 * (size_t)o, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s), "read");
-  CK(cudaMemcpyAsync(v.data(), h->v.p + 3 * (size_t)o, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s), "read");
-  CK(cudaMemcpyAsync(perm.data(), h->perm.p + o, sizeof(int) * n, cudaMemcpyDeviceToHost, s), "read");
-  CK(wait_stream(s), "sync");
-  const Grid &g = h->b_grids[k];
-  for (int i = 0; i < n; ++i) {
-    const int t = perm[i] - o;
-    if (t < 0 || t >= n) return fail(h, NEP_ERR_CUDA, "engine: inconsistent atom order");
-    double sf[3];
-    for (int b = 0; b < 3; ++b) {
-      sf[b] = x[3 * i] * g.Hinv[0][b] + x[3 * i + 1] * g.Hinv[1][b] + x[3 * i + 2] * g.Hinv[2][b];
-      sf[b] -= std::floor(sf[b]);
-    }
-    for (int b = 0; b < 3; ++b) {
-      if (pos) pos[3 * t + b] = sf[0] * g.H[0][b] + sf[1] * g.H[1][b] + sf[2] * g.H[2][b];
-      if (force) force[3 * t + b] = f[3 * i + b];
-      if (vel) vel[3 * t + b] = v[3 * i + b];
-    }
+// Final arrays of the given jobs, each in its own atom order: positions wrapped into its cell, forces,
+// velocities. A kernel per job writes them into page-locked host memory, and the host waits once
+// for all of them (four copies from pageable memory and a wait per job took 48 us a job); read
+// them with engine_arrays, in the order of `jobs`, before the next call.
+int engine_fetch(nep_handle *h, const std::vector<int> &jobs, cudaStream_t s) {
+  h->e_out_at.assign(1, 1);  // the first double: error flag
+  for (int k : jobs) {
+    if (k < 0 || k >= h->nb_struct) return fail(h, NEP_ERR_ARG, "engine: bad job index");
+    h->e_out_at.push_back(h->e_out_at.back() + 9 * (size_t)(h->b_offsets[k + 1] - h->b_offsets[k]));
   }
+  CK(h->e_out.ensure(sizeof(double) * h->e_out_at.back()), "alloc results");
+  double *const out = reinterpret_cast<double *>(h->e_out.p);
+  volatile int *const bad = reinterpret_cast<volatile int *>(h->e_out.p);
+  *bad = 0;
+  for (size_t q = 0; q < jobs.size(); ++q) {
+    const int o = h->b_offsets[jobs[q]], n = h->b_offsets[jobs[q] + 1] - o;
+    launch_engine_export(o, n, atom_state(h), h->b_grids[jobs[q]], out + h->e_out_at[q], const_cast<int *>(bad), s);
+  }
+  CK(cudaGetLastError(), "engine export");
+  CK(wait_stream(s), "sync");
+  if (*bad) return fail(h, NEP_ERR_CUDA, "engine: inconsistent atom order");
   return NEP_OK;
+}
+
+// [3][n][3]: positions, forces, velocities of the q-th job of the last engine_fetch.
+const double *engine_arrays(const nep_handle *h, size_t q) {
+  return reinterpret_cast<const double *>(h->e_out.p) + h->e_out_at[q];
 }
 
 size_t workspace_bytes(nep_handle *h) {
@@ -1356,6 +1380,8 @@ int nep_destroy(nep_handle *h) {
     for (int w = 0; w < 2; ++w)
       if (h->ev[sl][w]) cudaEventDestroy(h->ev[sl][w]);
   if (h->ev_status) cudaEventDestroy(h->ev_status);
+  h->e_read.release();
+  h->e_out.release();
   if (h->h_status) cudaFreeHost(h->h_status);
   h->d_tab.release(); h->d_inv_mk.release(); h->d_mk_half.release();
   h->x.release(); h->v.release(); h->F.release(); h->x_ref.release(); h->origin.release();

@@ -1691,6 +1691,34 @@ void launch_engine_advance(int n_struct, const int *offsets, const AtomState &a,
   if (n_struct > 0) engine_advance_kernel<<<n_struct * kFireCluster, 128, 0, s>>>(offsets, a, slots);
 }
 
+// Arrays of a finished job (internal atoms o .. o + n - 1) in its own atom order, [3][n][3]: wrapped
+// positions, forces, velocities. out may be host memory.
+__global__ void engine_export_kernel(int o, int n, const AtomState a, const Grid g, double *out, int *bad) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int t = a.perm[o + i] - o;
+  if (t < 0 || t >= n) {
+    *bad = 1;
+    return;
+  }
+  const size_t k = 3 * (size_t)(o + i), u = 3 * (size_t)t, m = 3 * (size_t)n;
+  const double r[3] = {a.x[k], a.x[k + 1], a.x[k + 2]};
+  double s[3];
+  for (int b = 0; b < 3; ++b) {
+    s[b] = r[0] * g.Hinv[0][b] + r[1] * g.Hinv[1][b] + r[2] * g.Hinv[2][b];
+    s[b] -= floor(s[b]);
+  }
+  for (int b = 0; b < 3; ++b) {
+    out[u + b] = s[0] * g.H[0][b] + s[1] * g.H[1][b] + s[2] * g.H[2][b];
+    out[m + u + b] = a.F[k + b];
+    out[2 * m + u + b] = a.v[k + b];
+  }
+}
+
+void launch_engine_export(int o, int n, const AtomState &a, const Grid &g, double *out, int *bad, cudaStream_t s) {
+  if (n > 0) engine_export_kernel<<<(n + 127) / 128, 128, 0, s>>>(o, n, a, g, out, bad);
+}
+
 void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src, AtomState dst, cudaStream_t s) {
   if (n_keep > 0) engine_relayout_kernel<<<n_keep, 256, 0, s>>>(table, src, dst);
 }

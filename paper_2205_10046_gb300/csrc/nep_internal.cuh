@@ -376,6 +376,7 @@ void launch_engine_drift(int N, const AtomState &a, const int *sid, const Engine
                          cudaStream_t s);
 void launch_clear_flags(BuildStatus *st, cudaStream_t s);
 void launch_engine_advance(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s);
+void launch_engine_export(int o, int n, const AtomState &a, const Grid &g, double *out, int *bad, cudaStream_t s);
 void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src, AtomState dst, cudaStream_t s);
 void launch_thermostat(int N, const AtomState &a, int nb_gather, const double *partial_gather, ThermoState *ts,
                        cudaStream_t s);
@@ -398,7 +399,8 @@ int engine_relayout(nep_handle *h, const std::vector<int> &keep, const std::vect
 int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild);
 // neighbour builds of the engine's batch so far (read with the status after every chunk)
 long long engine_builds(const nep_handle *h);
-int engine_fetch(nep_handle *h, int k, double *pos, double *force, double *vel, cudaStream_t s);
+int engine_fetch(nep_handle *h, const std::vector<int> &jobs, cudaStream_t s);
+const double *engine_arrays(const nep_handle *h, size_t q);
 int engine_jobs(const nep_handle *h);
 int engine_atoms(const nep_handle *h);
 const EngineSlot &engine_slot(const nep_handle *h, int k);

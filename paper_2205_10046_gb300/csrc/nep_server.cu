@@ -308,6 +308,11 @@ void nep_server::scheduler_main() {
     std::vector<std::pair<long long, Arrays>> outa;
     double evals = 0;
     int n_finished = 0;
+    std::vector<int> ended;
+    for (size_t k = 0; k < active.size(); ++k)
+      if (!active[k].finished && nep::engine_slot(h, (int)k).phase == 2) ended.push_back((int)k);
+    const int fetched = ended.empty() ? NEP_OK : nep::engine_fetch(h, ended, s);
+    size_t q_ended = 0;
     for (size_t k = 0; k < active.size(); ++k) {
       Job &j = active[k];
       if (j.finished) {
@@ -328,11 +333,16 @@ void nep_server::scheduler_main() {
       res.workspace_est = j.est;
       const size_t n3 = 3 * (size_t)j.spec.n_atoms;
       Arrays a;
-      a.pos.resize(n3);
-      a.force.resize(n3);
-      if (j.spec.kind == NEP_JOB_NVE) a.vel.resize(n3);
-      res.status = nep::engine_fetch(h, (int)k, a.pos.data(), a.force.data(), a.vel.empty() ? nullptr : a.vel.data(), s);
-      if (res.status != NEP_OK) std::snprintf(res.message, sizeof(res.message), "%s", nep_last_error(h));
+      res.status = fetched;
+      if (fetched == NEP_OK) {
+        const double *x = nep::engine_arrays(h, q_ended);
+        a.pos.assign(x, x + n3);
+        a.force.assign(x + n3, x + 2 * n3);
+        if (j.spec.kind == NEP_JOB_NVE) a.vel.assign(x + 2 * n3, x + 3 * n3);
+      } else {
+        std::snprintf(res.message, sizeof(res.message), "%s", nep_last_error(h));
+      }
+      ++q_ended;
       res.workspace_used = nep::workspace_bytes(h);
       res.t_done = now_since(t0);
       evals += (double)j.spec.n_atoms * (1 + sl.steps_done);
