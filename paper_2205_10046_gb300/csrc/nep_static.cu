@@ -155,13 +155,10 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   float *dtabm = arena.take<float>(tl.total);
   AtomState a;
   a.x = arena.take<double>(3 * (size_t)N);
-  a.v = arena.take<double>(3 * (size_t)N);
-  a.F = arena.take<double>(3 * (size_t)N);
+  a.v = a.F = a.v2 = a.F2 = nullptr;  // the build moves neither velocities nor forces here
   a.x_ref = arena.take<double>(3 * (size_t)N);
   a.origin = arena.take<double>(3 * (size_t)N);
   a.x2 = arena.take<double>(3 * (size_t)N);
-  a.v2 = arena.take<double>(3 * (size_t)N);
-  a.F2 = arena.take<double>(3 * (size_t)N);
   a.types = arena.take<int>(N);
   a.perm = arena.take<int>(N);
   a.cell_of = arena.take<int>(N);
@@ -180,7 +177,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.nn_a = arena.take<int>(N);
   L.part = arena.take<unsigned long long>(4 * kStatSlots);
   L.bar = arena.take<unsigned>(1 + kBuildSums);
-  if (!st || !dtab || !dtabm || !a.x || !a.v || !a.F || !a.x_ref || !a.origin || !a.x2 || !a.v2 || !a.F2 ||
+  if (!st || !dtab || !dtabm || !a.x || !a.x_ref || !a.origin || !a.x2 ||
       !a.types || !a.perm || !a.cell_of || !a.types2 || !a.perm2 || !a.cell2 || !a.pos4 || !a.posA || !L.cell_count ||
       !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part ||
       !L.bar)
@@ -191,8 +188,6 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   // cell counters)
   SK(cudaMemcpyAsync(dtabm, tab, sizeof(float) * tl.total, cudaMemcpyHostToDevice, s), "copy");
   SK(cudaMemsetAsync(L.bar, 0, sizeof(unsigned), s), "clear");
-  SK(cudaMemsetAsync(a.v, 0, sizeof(double) * 3 * N, s), "clear");
-  SK(cudaMemsetAsync(a.F, 0, sizeof(double) * 3 * N, s), "clear");
 
   const float rlR = (float)(params->rc_radial + skin), rlA = (float)(params->rc_angular + skin);
   const float rcR = (float)params->rc_radial, rcA = (float)params->rc_angular;
