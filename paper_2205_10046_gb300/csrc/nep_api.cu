@@ -1676,8 +1676,8 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   int best_ab = 128, best_gb = 128;
   const int abs_[2] = {64, 128}, gbs[3] = {64, 128, 256};
   for (int ia = 0; ia < 2 && !rc; ++ia) {
-    // the tensor-core networks, the run-time-shape kernels and nep_tuning.atom_form 3 take
-    // 128-atom CTAs only (a 64-atom CTA would change the FP32 form, hence the rounding)
+    // one size for the tensor-core networks (64 atoms whatever it says), the run-time-shape kernels
+    // (16) and, by the caller's choice, nep_tuning.atom_form 3; the results do not depend on it
     if ((h->precision >= 1 || h->generic || atom_form_of(h) == 3) && abs_[ia] != 128) continue;
     for (int ig = 0; ig < 3 && !rc; ++ig) {
       if (h->generic && gbs[ig] != 128) continue;  // one block shape for the run-time-shape kernels

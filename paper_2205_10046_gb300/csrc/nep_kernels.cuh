@@ -6,7 +6,7 @@
 //                 network U_i and dU_i/dq (Eq. Ui), then the per-type radial force
 //                 coefficients and the angular partial forces dU_i/dr_ij (the angular terms
 //                 of Eq. partial_force), stored per angular pair (Algorithms 1 and 3 fused).
-//   gather_kernel one thread per atom: F_i = sum_j [dU_i/dr_ij - dU_j/dr_ji] (Eqs. F_ij,
+//   gather_kernel two lanes per atom: F_i = sum_j [dU_i/dr_ij - dU_j/dr_ji] (Eqs. F_ij,
 //                 F_i) and W_i = sum_j r_ij (x) dU_j/dr_ji (Eq. virial) for the radial
 //                 part from both atoms' force coefficients and for the angular part from
 //                 the stored partial forces of both atoms, with no atomics (Algorithms 2, 4).
@@ -22,7 +22,8 @@
 //   * pair vectors come from cell-local FP32 coordinates plus an image shift table, so no
 //     FP64 arithmetic (slow on GB300) runs in the pair loops;
 //   * two lanes work on one atom and share a row of shared memory (S_nk, dU/dS_nk, q, dU/dq),
-//     so an atom's sums fit 128 registers a thread and every phase has work for both lanes.
+//     so an atom's sums fit 128 registers a thread and every phase has work for both lanes;
+//     in small systems up to four groups of such lanes share an atom (kSplitAtoms).
 #pragma once
 #include <cuda_bf16.h>
 
