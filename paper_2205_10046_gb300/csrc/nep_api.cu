@@ -2074,6 +2074,10 @@ int run_steps(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double
       rc = read_status(h, s);
       if (rc) return rc;
       const BuildStatus st = *h->h_status;
+      if (st.tc_timeout) {
+        h->md_ready = false;
+        return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait or the barrier of a neighbour build ran out");
+      }
       if (!st.overflow && !st.rev_missing) break;
       if (attempt >= 2 || st.max_r > kListBuf || st.max_a > kListBuf) {
         h->md_ready = false;

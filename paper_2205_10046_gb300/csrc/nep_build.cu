@@ -1397,8 +1397,13 @@ cudaError_t launch_build(const BuildArgs &p, cudaStream_t s) {
   auto go = [&](auto kern) -> cudaError_t {
     BuildArgs args = p;
     void *av[] = {&args};
-    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(std::max(1, std::min(want, most))),
-                                       dim3(kBuildBlock), av, smem, s);
+    for (int grid = std::max(1, std::min(want, most));; grid = (grid + 1) / 2) {
+      const cudaError_t r = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(grid),
+                                                        dim3(kBuildBlock), av, smem, s);
+      // a stream that may use only part of the SMs holds fewer blocks at a time; any number works
+      if (r != cudaErrorCooperativeLaunchTooLarge || grid == 1) return r;
+      cudaGetLastError();
+    }
   };
   if constexpr (COUNT) return go(build_kernel<1, true>);
   else
