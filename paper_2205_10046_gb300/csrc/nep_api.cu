@@ -705,6 +705,9 @@ int load_structure(nep_handle *h, int N, const double *pos, const int *types, co
                    int move, const std::function<int()> &after) {
   int rc = ensure_atoms(h, N, s);
   if (rc) return rc;
+  // the grid and the shift table below are those of the last batch too: its layout (and with it the
+  // captured batch graph, by b_gen) is set up again by the next batch call
+  h->nb_struct = 0;
   const char *err = nullptr;
   rc = nep::build_grid(box, h->rcR + h->skin, N, h->grid, &h->volume, &err);
   if (rc) return fail(h, rc, err);
