@@ -314,7 +314,8 @@ int md_init_host(nep_handle *h, int n_atoms, const double *pos, const int *types
  * state after that step (row r = step (r+1)*thermo_every of this call); thermo must hold
  * n_steps / thermo_every rows of 4 doubles. Each step replays one captured CUDA graph.
  * Returns NEP_ERR_NEIGHBOR_OVERFLOW if a rebuild found more neighbours than the lists
- * hold (the state is then unusable; call md_init again). */
+ * hold, and NEP_ERR_NONFINITE if a position became infinite or NaN (the state is then
+ * unusable; call md_init again). */
 int md_run(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double *thermo, nep_stream_t stream);
 
 /* Options of md_run_ex. */
@@ -367,8 +368,8 @@ int md_run_async(nep_handle *h, int n_steps, double dt_fs, int thermo_every, dou
                  nep_stream_t stream);
 
 /* Synchronise `stream` and report the MD health: NEP_OK, or NEP_ERR_NEIGHBOR_OVERFLOW if a
- * rebuild since md_init found more neighbours than the lists hold (the state is then
- * unusable; call md_init again). */
+ * rebuild since md_init found more neighbours than the lists hold, or NEP_ERR_NONFINITE if it
+ * met a position that is not finite (the state is then unusable; call md_init again). */
 int md_status(nep_handle *h, nep_stream_t stream);
 
 /* Copy the MD state out (DEVICE pointers; any may be NULL): positions wrapped into the

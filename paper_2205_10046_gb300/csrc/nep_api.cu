@@ -1948,6 +1948,15 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
 }  // namespace
 
 namespace {
+// The steps so far met a position that is not finite (the build that met it put the atom at the
+// origin), by the status last read: the state is then unusable.
+int md_bad_input(nep_handle *h) {
+  if (!h->h_status->bad_input) return NEP_OK;
+  h->md_ready = false;
+  return fail(h, (h->h_status->bad_input & 2) ? NEP_ERR_NONFINITE : NEP_ERR_ARG,
+              (h->h_status->bad_input & 2) ? "non-finite position; call md_init again" : "atom type out of range");
+}
+
 int md_queue(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double *thermo, cudaStream_t s,
              bool fire = false, double *heat = nullptr) {
   if (!h->md_ready) return fail(h, NEP_ERR_STATE, "md_run before md_init");
@@ -2018,6 +2027,8 @@ int md_status(nep_handle *h, nep_stream_t stream) {
   int rc = read_status(h, (cudaStream_t)stream);
   if (rc) return rc;
   if (h->h_status->tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+  rc = md_bad_input(h);
+  if (rc) return rc;
   if (h->h_status->overflow || h->h_status->rev_missing) {
     h->md_ready = false;
     return fail(h, NEP_ERR_NEIGHBOR_OVERFLOW, "neighbour list overflow during md_run; call md_init again");
@@ -2081,6 +2092,8 @@ int run_steps(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double
         h->md_ready = false;
         return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait or the barrier of a neighbour build ran out");
       }
+      rc = md_bad_input(h);
+      if (rc) return rc;
       if (!st.overflow && !st.rev_missing) break;
       if (attempt >= 2 || st.max_r > kListBuf || st.max_a > kListBuf) {
         h->md_ready = false;

@@ -992,7 +992,7 @@ __global__ void md_drift_kernel(int N, AtomState a, const double *inv_mass_kappa
   p.y = (float)(r[1] - a.origin[3 * (size_t)i + 1]);
   p.z = (float)(r[2] - a.origin[3 * (size_t)i + 2]);
   a.pos4[i] = p;
-  if (d2 > half_skin2) st->rebuild = 1;
+  if (!(d2 <= half_skin2)) st->rebuild = 1;  // also for a non-finite displacement, which the build reports
 }
 
 // Caller-order copies of the MD state: positions wrapped into the cell, velocities, forces.
