@@ -56,7 +56,7 @@ extern "C" {
 #define NEP_ERR_UNSUPPORTED (-6)       /* hyper-parameters without a compiled kernel, or a cell
                                           thinner than a third of the list radius */
 #define NEP_ERR_STATE (-7)             /* call out of order (e.g. md_run before md_init) */
-#define NEP_ERR_TIMEOUT (-8)           /* a device-side wait ran out (tensor-core completion) */
+#define NEP_ERR_TIMEOUT (-8)           /* a device-side wait ran out (tensor-core completion, neighbour build) */
 
 #define NEP_MAX_TYPES 8
 
@@ -422,6 +422,11 @@ int nep_set_precision(nep_handle *h, int mode);
  * graphs with conditional nodes). Up to 131,072 atoms the rebuild is one kernel that returns at
  * once in either mode (a conditional node costs more). Results are identical. */
 int nep_set_graph_conditional(nep_handle *h, int enable);
+
+/* Most polls of a wait between the thread blocks of the neighbour build (0: the default, some
+ * seconds). A wait that runs out ends the call, or the MD run, with NEP_ERR_TIMEOUT; the outputs
+ * stay as they were. A small limit is for tests. */
+int nep_set_wait_limit(nep_handle *h, int polls);
 int nep_kernel_slots(void);
 const char *nep_kernel_name(int slot);
 int nep_kernel_times(nep_handle *h, float *ms_out, int n_slots);

@@ -405,6 +405,7 @@ struct nep_handle {
   DevBuf<double> fin_scratch;  // finalize_kernel: block sums
   DevBuf<unsigned> bar;        // grid barrier of the one-kernel build (0 between launches), block sums
   DevBuf<int> fin_ticket;      // and its ticket (0 between launches)
+  unsigned barrier_polls = kBarrierPolls;
   DevBuf<unsigned long long> stat_part;  // partial sums of a build's list statistics
   BuildStatus *h_status = nullptr;  // pinned mirror
   // md
@@ -582,6 +583,7 @@ ListBufs list_bufs(nep_handle *h) {
   L.cell_atoms = h->cell_atoms.p; L.nl_r = h->nl_r.p; L.nn_r = h->nn_r.p; L.nl_a = h->nl_a.p; L.nn_a = h->nn_a.p;
   L.rev_a = h->rev_a.p; L.cap_r = h->cap_r; L.cap_a = h->cap_a; L.part = h->stat_part.p;
   L.bar = h->bar.p;
+  L.polls = h->barrier_polls;
   L.stage_e = h->stage_e.p; L.stage_g = h->stage_g.p;
   return L;
 }
@@ -628,7 +630,10 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
       if (rc) return rc;
     }
     const BuildStatus &st = *h->h_status;
-    if (st.bad_input & 4) return fail(h, NEP_ERR_TIMEOUT, "the barrier of the neighbour build ran out");
+    if (st.bad_input & 4) {
+      h->N = 0;  // no lists
+      return fail(h, NEP_ERR_TIMEOUT, "the barrier of the neighbour build ran out");
+    }
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
     if (st.max_r > kListBuf || st.max_a > kListBuf)
@@ -727,7 +732,7 @@ int run_forces(nep_handle *h, int N, double *energy, double *force, double *viri
   a.sums = sums;
   a.sums_always = sums_always;
   a.step_ctl = step_ctl;
-  if (!md_kick) a.guard = h->status.p;  // queued behind a build whose status is still unread
+  a.guard = h->status.p;  // queued behind a build whose status is still unread
   a.fire = fire;
   if (force == h->F.p) a.perm = nullptr;
   a.energy = energy;
@@ -868,6 +873,7 @@ int batch_kernels(nep_handle *h, int N, const BatchOut &o, cudaStream_t s, bool 
   a.force = o.force;
   a.virial = o.w_atom;
   a.s_out = N;
+  a.guard = h->status.p;
   ev_record(h, SLOT_ATOM, 0, s, capturing);
   cudaError_t e =
       h->ops->atom_batch(a, h->mf, 1, atom_block(h), s);
@@ -880,7 +886,7 @@ int batch_kernels(nep_handle *h, int N, const BatchOut &o, cudaStream_t s, bool 
   ev_record(h, SLOT_FINAL, 0, s, capturing);
   if (o.e_struct || o.w_struct)
     launch_struct_sums(h->nb_struct, 1, h->d_offsets.p, N, o.e_struct ? o.e_atom : nullptr,
-                       o.w_struct ? o.w_atom : nullptr, o.e_struct, o.w_struct, max_struct_atoms(h), s);
+                       o.w_struct ? o.w_atom : nullptr, o.e_struct, o.w_struct, max_struct_atoms(h), h->status.p, s);
   ev_record(h, SLOT_FINAL, 1, s, capturing);
   CK(cudaGetLastError(), "structure sums");
   return NEP_OK;
@@ -1173,6 +1179,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   a.virial = h->e_w.p;
   a.s_out = N;
   a.slots = h->e_slots.p;
+  a.guard = h->status.p;
   e = h->ops->atom_batch(a, h->mf, 1, atom_block(h), s);
   if (e == cudaSuccess) e = h->ops->gather_batch(a, 1, gather_block(h), s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine kernels");
@@ -1234,7 +1241,7 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     // the jobs' energies and virials, once per chunk: only a job that finished (frozen since,
     // its per-atom values unchanged) or the chunk's last state is ever read
     launch_struct_sums(S, 1, h->d_offsets.p, N, h->e_u.p, h->e_w.p, h->e_energy.p, h->e_virial.p,
-                       max_struct_atoms(h), s);
+                       max_struct_atoms(h), nullptr, s);
     // everything the host looks at in one go (job states of an undone chunk are not used)
     CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
     CK(cudaMemcpyAsync(r_slots, h->e_slots.p, sizeof(EngineSlot) * S, cudaMemcpyDeviceToHost, s), "read back");
@@ -1607,7 +1614,7 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
     ev_record(h, SLOT_GATHER, 1, s, false);
     ev_record(h, SLOT_FINAL, 0, s, false);
     launch_struct_sums(n_struct, m, h->d_offsets.p, N, h->b_e.p, w_tar ? h->b_w.p : nullptr, h->pop_es.p,
-                       w_tar ? h->pop_ws.p : nullptr, max_struct_atoms(h), s);
+                       w_tar ? h->pop_ws.p : nullptr, max_struct_atoms(h), nullptr, s);
     launch_population_loss(m, n_struct, h->d_offsets.p, h->pop_es.p, w_tar ? h->pop_ws.p : nullptr, e_tar, w_tar,
                            h->partial_gather.p, nb_g, N, h->pop_reg.p + 2 * (size_t)p0, n_par, lambda,
                            loss + 6 * (size_t)p0, s);
@@ -2026,7 +2033,10 @@ int md_status(nep_handle *h, nep_stream_t stream) {
   if (!h->md_ready) return fail(h, NEP_ERR_STATE, "no MD state");
   int rc = read_status(h, (cudaStream_t)stream);
   if (rc) return rc;
-  if (h->h_status->tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+  if (h->h_status->tc_timeout) {
+    h->md_ready = false;
+    return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+  }
   rc = md_bad_input(h);
   if (rc) return rc;
   if (h->h_status->overflow || h->h_status->rev_missing) {
@@ -2347,6 +2357,18 @@ int nep_set_precision(nep_handle *h, int mode) {
 int nep_set_graph_conditional(nep_handle *h, int enable) {
   if (!valid_handle(h)) return NEP_ERR_ARG;
   h->graph_cond = enable != 0;
+  return NEP_OK;
+}
+
+int nep_set_wait_limit(nep_handle *h, int polls) {
+  if (!valid_handle(h)) return NEP_ERR_ARG;
+  if (polls < 0) return fail(h, NEP_ERR_ARG, "polls must not be negative");
+  h->barrier_polls = polls ? (unsigned)polls : kBarrierPolls;
+  for (cudaGraphExec_t *g : {&h->graph, &h->fire_graph, &h->b_graph})  // they hold the limit
+    if (*g) {
+      cudaGraphExecDestroy(*g);
+      *g = nullptr;
+    }
   return NEP_OK;
 }
 

@@ -786,11 +786,10 @@ __global__ void finish_build_kernel(int n_struct, int *sflag, const unsigned lon
 constexpr int kBuildBlock = kScanBlock;
 constexpr int kBuildWarps = kBuildBlock / 32;
 constexpr int kBuildPerSM = 3;           // blocks per SM at most (registers and shared memory hold that many)
-constexpr unsigned kBarrierSpins = 1u << 22;  // seconds
 
 struct GridBarrier {
   unsigned *bar;
-  unsigned target = 0;
+  unsigned target = 0, polls;
   BuildStatus *st;
   __device__ __forceinline__ bool wait() {
     __shared__ int ok;
@@ -799,10 +798,10 @@ struct GridBarrier {
     if (threadIdx.x == 0) {
       __threadfence();
       atomicAdd(bar, 1u);
-      unsigned seen, spins = 0;
+      unsigned seen, n = 0;
       do {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-      } while (seen < target && ++spins < kBarrierSpins);
+      } while (seen < target && ++n < polls);
       ok = seen >= target;
       if (!ok) {
         st->tc_timeout = 1;
@@ -830,12 +829,13 @@ template <int TT, bool COUNT>
 __global__ void __launch_bounds__(kBuildBlock, kBuildPerSM) build_kernel(const BuildArgs p) {
   BuildStatus *const st = p.st;
   const bool load = p.src.pos != nullptr;
-  if (!load && (!rebuild_pending(st) || *(volatile const int *)&st->tc_timeout)) return;
+  // the whole block alike: a block of this launch may already have given up
+  if (!load && __syncthreads_or(!rebuild_pending(st) || *(volatile const int *)&st->tc_timeout)) return;
   const int N = p.N, G = gridDim.x, tid = threadIdx.x, t0 = blockIdx.x * kBuildBlock + tid, nt = G * kBuildBlock;
   const AtomState &a = p.a;
   const ListBufs &L = p.L;
   const Batch &B = p.B;
-  GridBarrier grid{L.bar, 0u, st};
+  GridBarrier grid{L.bar, 0u, L.polls, st};
   extern __shared__ uint2 bl_stage[];  // [kBuildWarps][cap_r]
   __shared__ int wsum[kBuildWarps], carry_s;
 
@@ -1166,7 +1166,9 @@ constexpr int kWideSum = 2048;
 constexpr int kSumThreads = 256;
 template <bool WIDE>
 __global__ void struct_sums_kernel(int n_struct, int members, const int *offsets, int N, const double *e_atom,
-                                   const double *w_atom, double *e_struct, double *w_struct) {
+                                   const double *w_atom, double *e_struct, double *w_struct,
+                                   const BuildStatus *guard) {
+  if (build_failed(guard)) return;
   const int lane = threadIdx.x & 31;
   const long long unit = WIDE ? (long long)blockIdx.x : ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (unit >= (long long)n_struct * members) return;  // uniform over the warp (block, WIDE)
@@ -1373,14 +1375,16 @@ void launch_shift_tables(int n_struct, const Grid *grids, int ncode, float4 *dta
 }
 
 void launch_struct_sums(int n_struct, int members, const int *offsets, int N, const double *e_atom,
-                        const double *w_atom, double *e_struct, double *w_struct, int max_atoms, cudaStream_t s) {
+                        const double *w_atom, double *e_struct, double *w_struct, int max_atoms,
+                        const BuildStatus *guard, cudaStream_t s) {
   const long long units = (long long)n_struct * members;
   if (units > 0) {
     struct_sums_kernel<false><<<(unsigned)((units * 32 + 255) / 256), 256, 0, s>>>(n_struct, members, offsets, N,
-                                                                                    e_atom, w_atom, e_struct, w_struct);
+                                                                                    e_atom, w_atom, e_struct, w_struct,
+                                                                                    guard);
     if (max_atoms > kWideSum)
       struct_sums_kernel<true><<<(unsigned)units, kSumThreads, 0, s>>>(n_struct, members, offsets, N, e_atom, w_atom,
-                                                                      e_struct, w_struct);
+                                                                      e_struct, w_struct, guard);
   }
 }
 

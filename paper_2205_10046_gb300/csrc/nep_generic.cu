@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(32 * kGenWarps, 3) generic_atom_kernel(const A
 // 20,000 MgAlCu atoms: 34 us, 120 with a thread per atom and the f_k' in local memory.
 template <bool BATCH, int GA, int NT>
 __global__ void __launch_bounds__(NT) generic_gather_kernel(const AtomArgs a) {
-  if (!BATCH && build_failed(a.guard)) return;
+  if (build_failed(a.guard)) return;
   constexpr int L = kGenGatherLanes;
   const int mem = BATCH ? (int)blockIdx.y : 0;
   const float *e_rad = a.e_rad + mem * a.s_erad;

@@ -88,9 +88,11 @@ struct ListBufs {
   unsigned char *stage_g;   // [cap_r][N] their groups
   unsigned long long *part;  // [kStatSlots][4] partial sums of a build's list statistics
   unsigned *bar;             // [1 + kBuildSums] barrier of the one-kernel build (zero between launches), block sums
+  unsigned polls;            // most polls of a wait at the barrier (kBarrierPolls, or fewer for tests)
 };
 constexpr int kStatSlots = 64;
 constexpr int kBuildSums = 1023;  // blocks of the one-kernel build at most
+constexpr unsigned kBarrierPolls = 1u << 22;  // seconds
 
 // Device-visible status written by the builders.
 struct BuildStatus {
@@ -250,7 +252,8 @@ struct AtomArgs {
 };
 
 // The build before this launch failed (the host, which has not looked yet, reports it or builds
-// again): kernels queued behind it write nothing.
+// again): kernels queued behind it write nothing, and follow no list entry or reverse slot, which a
+// build whose barrier ran out may not have written.
 __device__ __forceinline__ bool build_failed(const BuildStatus *st) {
   return st && (st->overflow | st->bad_input | st->rev_missing);
 }
@@ -367,7 +370,8 @@ void launch_struct_ids(int n_struct, const int *offsets, int *sid, cudaStream_t 
 void launch_shift_tables(int n_struct, const Grid *grids, int ncode, float4 *dtab, cudaStream_t s);
 // max_atoms: the largest structure (structures above kWideSum atoms are summed by a block)
 void launch_struct_sums(int n_struct, int members, const int *offsets, int N, const double *e_atom,
-                        const double *w_atom, double *e_struct, double *w_struct, int max_atoms, cudaStream_t s);
+                        const double *w_atom, double *e_struct, double *w_struct, int max_atoms,
+                        const BuildStatus *guard, cudaStream_t s);
 void launch_arm_rebuild(BuildStatus *st, unsigned *bar, cudaStream_t s);
 void launch_fire_mix(int N, const AtomState &a, FireState *fire, int check_only, cudaStream_t s);
 // batched serving engine

@@ -522,7 +522,8 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
   // Lanes past the last atom, and (serving engine) those of a finished job frozen in the batch,
   // run along with no neighbours (the pair exchanges are warp-collective); they write nothing.
   const float4 pi = i < N ? __ldg(a.pos4 + i) : make_float4(0.f, 0.f, 0.f, __int_as_float(0));
-  const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(pi)].phase == 2);
+  const bool failed = build_failed(a.guard);  // tested once the block's setup is under way
+  const bool active = i < N && !(BATCH && a.slots && (failed || a.slots[struct_of(pi)].phase == 2));
   const int na = active ? __ldg(a.nn_a + i) : 0;
   int cnt_r = active ? __ldg(a.nn_r + i) : 0;
   if (active) {  // the first list slots into L2 before the block's setup
@@ -532,7 +533,6 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
     if (h < a.cap_a) l2_prefetch(a.nl_a + (size_t)h * N + i);
   }
   const int mem = BATCH ? (int)blockIdx.y : 0;
-  if (!BATCH && build_failed(a.guard)) return;
   using PR = PairRow<S>;
   constexpr bool TC = PR::tc(PREC);
   static_assert(!DESC || PREC == 0, "the descriptors need no network");
@@ -550,6 +550,7 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
   if constexpr (!BATCH)
     stage_shifts(a, reinterpret_cast<float *>(dtab_s));
   stage_table<S>(a.tab + mem * a.s_tab, PR::from(PREC), T, w0_s + PR::from(PREC));
+  if (failed) return;
   __shared__ __align__(8) uint64_t tc_mbar;
   __shared__ uint32_t tc_tmem;
   __shared__ float u_s[TC ? AB : 1];  // U of the rows
@@ -1369,7 +1370,7 @@ constexpr int gather_min_blocks(int KR, int threads) {
 template <class S, bool BATCH, int GA, int SUB>
 __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_min_blocks(S::KR, GA *kGatherLanes))
     gather_kernel(const AtomArgs a) {
-  if (!BATCH && build_failed(a.guard)) return;
+  const bool failed = build_failed(a.guard);  // tested once the first loads are under way
   constexpr int L = kGatherLanes;
   __shared__ float fw[GA][13];
   __shared__ unsigned char on[GA];
@@ -1391,7 +1392,7 @@ __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_mi
 #pragma unroll
   for (int c = 0; c < 9; ++c) w[c] = 0.f;
   // (serving engine) atoms of a finished job frozen in the batch are skipped
-  const bool active = i < N && !(BATCH && a.slots && a.slots[struct_of(a.pos4[i])].phase == 2);
+  const bool active = i < N && !(BATCH && a.slots && (failed || a.slots[struct_of(a.pos4[i])].phase == 2));
   if (active || SUB > 1) {  // (the lanes of a split atom exchange their pairs: whole warps)
     const float4 pi = a.pos4[active ? i : 0];
     const int ti = type_of(pi);
@@ -1485,6 +1486,7 @@ __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_mi
         const int nl = (cnt + L - 1 - l) / L;
         float eo[4 * S::EF4];
         load_e(eo, t, active ? i : 0);
+        if (failed) return;
         const unsigned *col = a.nl_r + (size_t)(base + l) * N + i;
         const int rounds = __reduce_max_sync(kAll, (nl + SUB - 1) / SUB);
         unsigned e1 = sub < nl ? __ldg(col + (size_t)L * sub * N) : 0u;
@@ -1552,6 +1554,7 @@ __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_mi
       const int cnt = a.nn_r[t * N + i];
       float eo[4 * S::EF4];
       load_e(eo, t, i);
+      if (failed) return;
       for_pairs_batch<2, true, 1>(a.nl_r + (size_t)(base + l) * N, 0, (cnt + L - 1 - l) / L, L * N, i, a.pos4, a.jmask, [&](int, unsigned e, const float4 &pj) {
         const int j = e & a.jmask;
         const float3 d = pair_vector(pi, pj, shift(e));
@@ -1604,6 +1607,7 @@ __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_mi
     }
     }
   }
+  if (failed) return;  // the threads without an atom too
   // the sums of the atom's lanes; one row per atom for the epilogue
   float v[12] = {fx, fy, fz, w[0], w[1], w[2], w[3], w[4], w[5], w[6], w[7], w[8]};
 #pragma unroll

@@ -177,6 +177,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.nn_a = arena.take<int>(N);
   L.part = arena.take<unsigned long long>(4 * kStatSlots);
   L.bar = arena.take<unsigned>(1 + kBuildSums);
+  L.polls = kBarrierPolls;
   if (!st || !dtab || !dtabm || !a.x || !a.x_ref || !a.origin || !a.x2 ||
       !a.types || !a.perm || !a.cell_of || !a.types2 || !a.perm2 || !a.cell2 || !a.pos4 || !a.posA || !L.cell_count ||
       !L.cell_cursor || !L.cell_start || !L.cell_atoms || !L.nn_r || !L.nn_a || !L.part ||

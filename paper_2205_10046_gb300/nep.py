@@ -115,6 +115,7 @@ _SIGS = {
     "nep_get_stats": (C.c_int, [_P, C.POINTER(nep_stats)]),
     "nep_set_profiling": (C.c_int, [_P, C.c_int]),
     "nep_set_graph_conditional": (C.c_int, [_P, C.c_int]),
+    "nep_set_wait_limit": (C.c_int, [_P, C.c_int]),
     "nep_set_precision": (C.c_int, [_P, C.c_int]),
     "nep_kernel_slots": (C.c_int, []),
     "nep_kernel_name": (C.c_char_p, [C.c_int]),
@@ -490,6 +491,11 @@ def nep_set_precision(h, mode: int):
 
 def nep_set_graph_conditional(h, enable: bool):
     _check(load().nep_set_graph_conditional(h, 1 if enable else 0), h)
+
+
+def nep_set_wait_limit(h, polls: int):
+    """Most polls of a wait between the blocks of the neighbour build (0: the default)."""
+    _check(load().nep_set_wait_limit(h, int(polls)), h)
 
 
 def nep_kernel_times(h) -> dict:
