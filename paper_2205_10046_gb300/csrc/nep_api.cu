@@ -406,6 +406,7 @@ struct nep_handle {
   DevBuf<unsigned> bar;        // grid barrier of the one-kernel build (0 between launches), block sums
   DevBuf<int> fin_ticket;      // and its ticket (0 between launches)
   unsigned barrier_polls = kBarrierPolls;
+  bool build_unread = false;   // a build was queued since the host last read a status
   DevBuf<unsigned long long> stat_part;  // partial sums of a build's list statistics
   BuildStatus *h_status = nullptr;  // pinned mirror
   // md
@@ -565,6 +566,17 @@ int ensure_lists(nep_handle *h, int N, int cap_r, int cap_a) {
 int read_status(nep_handle *h, cudaStream_t s) {
   CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   CK(wait_stream(s), "sync");
+  h->build_unread = false;
+  return NEP_OK;
+}
+
+// Before a build is queued that does not clear the barrier itself: the last one may have left it in
+// mid-count, by its status or because the host has not seen its status (md_run_async, a call that
+// failed half way). A build that finds it so would let blocks through too early.
+int queue_build(nep_handle *h, cudaStream_t s) {
+  if (h->build_unread || h->h_status->tc_timeout)
+    CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
+  h->build_unread = true;
   return NEP_OK;
 }
 
@@ -611,20 +623,20 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
   }
   for (int attempt = 0; attempt < 3; ++attempt) {
     const bool count_only = (h->cap_r == 0 || h->cap_a == 0);
-    if (h->h_status->tc_timeout)  // the barrier may have been left in mid-count
-      CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
+    int rc = queue_build(h, s);
+    if (rc) return rc;
     if (!src.pos) launch_arm_rebuild(h->status.p, h->bar.p, s);  // else requested by the load
     CK(launch_rebuild(N, h->T, g, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
                       list_bufs(h), count_only ? 1 : 0, move, src, h->status.p, s),
        "launch rebuild");
     src = LoadSrc{};  // the atoms are in place from here on
-    int rc = NEP_OK;
     if (after && !count_only) {
       CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
       CK(cudaEventRecord(h->ev_status, s), "status");
       rc = after();
       if (rc) return rc;
       CK(wait_event(h->ev_status), "sync");
+      h->build_unread = false;
     } else {
       rc = read_status(h, s);
       if (rc) return rc;
@@ -1219,7 +1231,8 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     const bool forced = force_rebuild || attempt > 0;
     // the flags of this chunk start cleared; a forced build is requested before the first step
     if (forced) launch_arm_rebuild(h->status.p, h->bar.p, s);
-    else launch_clear_flags(h->status.p, s);
+    else launch_clear_flags(h->status.p, h->bar.p, s);
+    h->build_unread = true;
     const EngineKey key = engine_key(h);
     for (int it = 0; it < n_iter; ++it) {
       if (!h->prof && h->e_graph && std::memcmp(&key, &h->e_key, sizeof(key)) == 0) {
@@ -1248,6 +1261,7 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     CK(cudaMemcpyAsync(r_energy, h->e_energy.p, sizeof(double) * S, cudaMemcpyDeviceToHost, s), "read back");
     CK(cudaMemcpyAsync(r_virial, h->e_virial.p, sizeof(double) * 9 * S, cudaMemcpyDeviceToHost, s), "read back");
     CK(wait_stream(s), "sync");
+    h->build_unread = false;
     const BuildStatus st = *h->h_status;
     if (st.tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
@@ -1493,10 +1507,11 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
   // copy-in, neighbour build, both kernels and the structure sums, then one status read
   BatchKey key = batch_key(h, N, o);
   if (!h->prof && h->b_graph && std::memcmp(&key, &h->b_key, sizeof(key)) == 0) {
-    if (h->h_status->tc_timeout)  // the barrier may have been left in mid-count
-      CK(cudaMemsetAsync(h->bar.p, 0, sizeof(unsigned), s), "clear barrier");
+    rc = queue_build(h, s);
+    if (rc) return rc;
     CK(cudaGraphLaunch(h->b_graph, s), "batch graph launch");
     CK(wait_stream(s), "batch graph");
+    h->build_unread = false;
     const BuildStatus &st = *h->h_status;
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
@@ -2016,6 +2031,8 @@ int md_queue(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double 
     h->graph_nvt = h->nvt;
     h->graph_heat = h->heat_rows;
   }
+  // (the steps' builds return at once after one that ran out, until the host has cleared its flag)
+  h->build_unread = true;
   for (int st = 0; st < n_steps; ++st) CK(cudaGraphLaunch(gx, s), "graph launch");
   // rows of the staging area -> the caller's [rows][4] thermo and [rows][3] heat current
   if (thermo && rows > 0)

@@ -1629,15 +1629,17 @@ __global__ void engine_drift_kernel(int N, AtomState a, const int *sid, const En
   }
 }
 
-// Clears the error flags of a chunk of iterations (a build is not requested).
-__global__ void clear_flags_kernel(BuildStatus *st) {
+// Clears the error flags of a chunk of iterations and the barrier that a build which ran out may
+// have left in mid-count (a build is not requested).
+__global__ void clear_flags_kernel(BuildStatus *st, unsigned *bar) {
+  bar[0] = 0u;
   st->overflow = 0;
   st->rev_missing = 0;
   st->bad_input = 0;
   st->tc_timeout = 0;
 }
 
-void launch_clear_flags(BuildStatus *st, cudaStream_t s) { clear_flags_kernel<<<1, 1, 0, s>>>(st); }
+void launch_clear_flags(BuildStatus *st, unsigned *bar, cudaStream_t s) { clear_flags_kernel<<<1, 1, 0, s>>>(st, bar); }
 
 // End of an engine iteration, one cluster per job: the FIRE update of a FIRE job after its step,
 // then the phase and step bookkeeping.

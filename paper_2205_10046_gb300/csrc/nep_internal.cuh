@@ -378,7 +378,7 @@ void launch_fire_mix(int N, const AtomState &a, FireState *fire, int check_only,
 void launch_engine_drift(int N, const AtomState &a, const int *sid, const EngineSlot *slots,
                          const double *inv_mass_kappa, double half_skin2, int *sflag, BuildStatus *st,
                          cudaStream_t s);
-void launch_clear_flags(BuildStatus *st, cudaStream_t s);
+void launch_clear_flags(BuildStatus *st, unsigned *bar, cudaStream_t s);
 void launch_engine_advance(int n_struct, const int *offsets, const AtomState &a, EngineSlot *slots, cudaStream_t s);
 void launch_engine_export(int o, int n, const AtomState &a, const Grid &g, double *out, int *bad, cudaStream_t s);
 void launch_engine_relayout(int n_keep, const int4 *table, const AtomState &src, AtomState dst, cudaStream_t s);

@@ -96,3 +96,42 @@ def test_md_ends_with_the_wait(torch_cuda, reps):
         np.testing.assert_array_equal(x.cpu().numpy(), xr.cpu().numpy())
     ref.close()
     h.close()
+
+
+@pytest.mark.parametrize("reps", [3, 12])
+@pytest.mark.parametrize("next_call", ["compute", "md", "batch", "stats"])
+def test_calls_after_an_unseen_time_out(torch_cuda, reps, next_call):
+    """The build of a step queued by md_run_async runs out and no call asks for it: the next one
+    starts from a cleared barrier all the same."""
+    torch = torch_cuda
+    from paper_2205_10046_gb300 import nep
+    w = W.si_diamond(reps, seed=6)
+    pos, types, vel = torch.tensor(w.pos, device="cuda"), torch.tensor(w.types, device="cuda"), _hot(torch, w)
+    off, boxes = np.array([0, w.n_atoms], np.int32), np.asarray(w.box)[None]
+    h, ref = nep.NEP(w.model, skin=0.4), nep.NEP(w.model, skin=0.4)
+
+    def call(hh):
+        if next_call == "md":
+            x = torch.empty_like(pos)
+            nep.md_init(hh.h, pos, types, w.box, vel)
+            nep.md_run(hh.h, 4, 1.0)
+            nep.md_get_state(hh.h, pos=x)
+            out = [x]
+        elif next_call == "batch":
+            out = list(hh.compute_batch(off, pos, types, boxes, per_atom=True).values())
+        else:
+            if next_call == "stats":
+                nep.nep_get_stats(hh.h)
+            out = list(hh.compute(pos, types, w.box, per_atom_virial=True).values())
+        return [o.cpu().numpy() for o in out]
+
+    expect = call(ref)
+    for _ in range(2):
+        nep.md_init(h.h, pos, types, w.box, vel)
+        nep.nep_set_wait_limit(h.h, 1)
+        nep.md_run_async(h.h, 3, 1.0)
+        nep.nep_set_wait_limit(h.h, 0)
+        for a, b in zip(call(h), expect):
+            np.testing.assert_array_equal(a, b)
+    ref.close()
+    h.close()
