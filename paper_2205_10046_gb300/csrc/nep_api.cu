@@ -563,6 +563,12 @@ int ensure_lists(nep_handle *h, int N, int cap_r, int cap_a) {
   return NEP_OK;
 }
 
+// Fails with the wait that ran out, by the status last read.
+int timed_out(nep_handle *h) {
+  return fail(h, NEP_ERR_TIMEOUT, (h->h_status->bad_input & 4) ? "a barrier of the neighbour build ran out"
+                                                               : "a tensor-core completion wait ran out");
+}
+
 int read_status(nep_handle *h, cudaStream_t s) {
   CK(cudaMemcpyAsync(h->h_status, h->status.p, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   CK(wait_stream(s), "sync");
@@ -644,7 +650,7 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
     const BuildStatus &st = *h->h_status;
     if (st.bad_input & 4) {
       h->N = 0;  // no lists
-      return fail(h, NEP_ERR_TIMEOUT, "the barrier of the neighbour build ran out");
+      return timed_out(h);
     }
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
@@ -1263,7 +1269,7 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
     CK(wait_stream(s), "sync");
     h->build_unread = false;
     const BuildStatus st = *h->h_status;
-    if (st.tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+    if (st.tc_timeout) return timed_out(h);
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (!st.overflow && !st.rev_missing) break;
@@ -1515,7 +1521,7 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
     const BuildStatus &st = *h->h_status;
     if (st.bad_input & 1) return fail(h, NEP_ERR_ARG, "atom type out of range");
     if (st.bad_input & 2) return fail(h, NEP_ERR_NONFINITE, "non-finite position");
-    if (st.tc_timeout) return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+    if (st.tc_timeout) return timed_out(h);
     if (!st.overflow && !st.rev_missing) return NEP_OK;
     // the lists outgrew their capacity: size them again on the eager path below
   }
@@ -2052,7 +2058,7 @@ int md_status(nep_handle *h, nep_stream_t stream) {
   if (rc) return rc;
   if (h->h_status->tc_timeout) {
     h->md_ready = false;
-    return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait ran out");
+    return timed_out(h);
   }
   rc = md_bad_input(h);
   if (rc) return rc;
@@ -2117,7 +2123,7 @@ int run_steps(nep_handle *h, int n_steps, double dt_fs, int thermo_every, double
       const BuildStatus st = *h->h_status;
       if (st.tc_timeout) {
         h->md_ready = false;
-        return fail(h, NEP_ERR_TIMEOUT, "a tensor-core completion wait or the barrier of a neighbour build ran out");
+        return timed_out(h);
       }
       rc = md_bad_input(h);
       if (rc) return rc;

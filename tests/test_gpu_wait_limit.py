@@ -25,6 +25,8 @@ def _raises(code, f):
     with pytest.raises(nep.NepError) as e:
         f()
     assert e.value.code == code
+    if code == TIMEOUT:
+        assert "barrier of the neighbour build" in str(e.value)
 
 
 @pytest.mark.parametrize("n", [300, 20000])
