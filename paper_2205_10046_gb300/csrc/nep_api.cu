@@ -1870,7 +1870,13 @@ int md_init(nep_handle *h, int n_atoms, const double *pos, const int *types, con
     return run_forces(h, n_atoms, nullptr, h->F.p, nullptr, 0, 0.0, s, false, 0);
   });
   if (rc) return rc;
-  CK(wait_stream(s), "md_init");
+  if (h->precision) {  // the status that the build left was read before the network ran
+    rc = read_status(h, s);
+    if (rc) return rc;
+    if (h->h_status->tc_timeout) return timed_out(h);
+  } else {
+    CK(wait_stream(s), "md_init");
+  }
   h->h_status->n_rebuilds = 0;
   h->h_status->md_steps = 0;
   h->h_status->rebuild = 0;
