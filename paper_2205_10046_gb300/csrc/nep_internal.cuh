@@ -264,24 +264,6 @@ __device__ __forceinline__ int sums_needed(const AtomArgs &a) {
   return a.sums_always | (row ? a.sums : 0);
 }
 
-// Running sum of FP32 values as an unevaluated pair hi + lo (Knuth's two-sum): the rounding error
-// of every addition goes into lo, so the pair carries about 48 bits without FP64 instructions
-// (a warp's FP64 addition takes 16 cycles of its SM).
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
-  __device__ __forceinline__ void add(float x, float xlo = 0.f) {
-    const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b));
-    hi = s;
-    lo = __fadd_rn(lo, __fadd_rn(err, xlo));
-  }
-  __device__ __forceinline__ void across(int o) {  // + the lane at distance o (xor)
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    add(h2, l2);
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Model constants of one handle, FP32.
 struct ModelF {
   float c3b[24];

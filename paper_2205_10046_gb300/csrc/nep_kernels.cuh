@@ -1207,14 +1207,13 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
       __shared__ double red[2 * AB / 32];
       const int warp = threadIdx.x >> 5;
       if (sub == 0) {
-        Sum2 su;
-        su.add(active && h == 0 ? U : 0.f);
+        double su = active && h == 0 ? (double)U : 0.0;
 #pragma unroll
-        for (int o = 16; o > 1; o >>= 1) su.across(o);  // lanes of one parity: h == 0 holds the sum
+        for (int o = 16; o > 1; o >>= 1) su += __shfl_xor_sync(kAll, su, o);  // lanes of one parity
         if ((threadIdx.x & 31) == 0) {
-          if (N > kSplitAtoms2) red[warp] = su.value();
+          if (N > kSplitAtoms2) red[warp] = su;
           else if (blockIdx.x * (AB / 16) + warp < (N + 15) / 16)
-            a.partial_atom[blockIdx.x * (AB / 16) + warp] = su.value();
+            a.partial_atom[blockIdx.x * (AB / 16) + warp] = su;
         }
       }
       if (N > kSplitAtoms2) {
@@ -1303,9 +1302,9 @@ __device__ __forceinline__ void gather_epilogue(const AtomArgs &a, int i, const 
 
 // End of a gather kernel: fw[GA][13] holds F_i and W_i (12 floats) of the block's GA atoms, zeros
 // for the inactive ones (`on` marks the others). One thread per atom runs the epilogue, then
-// the block forms the sums that are read, in a fixed order: W in FP32 pairs (Sum2) from the
-// shared rows, the rest in FP64. Without the test every MD step of every atom paid 15 FP64
-// block sums for totals that only thermo rows show (half of the gather's time).
+// the block forms the sums that are read, in FP64 and a fixed order. Without the test every MD step
+// of every atom paid 15 FP64 block sums for totals that only thermo rows show (half of the
+// gather's time).
 template <int GA, int NT>
 __device__ __forceinline__ void gather_finish(const AtomArgs &a, int mem, float (*fw)[13], const unsigned char *on) {
   static_assert(GA % 32 == 0 && NT >= GA && NT >= 96, "whole warps of atoms; 72 threads for the virial sums");
@@ -1321,12 +1320,12 @@ __device__ __forceinline__ void gather_finish(const AtomArgs &a, int mem, float 
   double *out = a.partial_gather + ((size_t)mem * gridDim.x + blockIdx.x) * kReduceSlots;
   if ((need & kSumW) && threadIdx.x < 96) {  // eight threads per component (96: whole warps)
     const int c = threadIdx.x >> 3, p = threadIdx.x & 7;
-    Sum2 s;
+    double s = 0.0;
     if (c < 9)
-      for (int r = p; r < GA; r += 8) s.add(fw[r][3 + c]);
+      for (int r = p; r < GA; r += 8) s += (double)fw[r][3 + c];
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) s.across(o);
-    if (c < 9 && p == 0) out[2 + c] = s.value();
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (c < 9 && p == 0) out[2 + c] = s;
   }
   if (!(need & (kSumKE | kSumFerr | kSumJ))) return;
   if (threadIdx.x < GA) {
