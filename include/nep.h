@@ -191,9 +191,11 @@ int nep_get_tuning(const nep_handle *h, nep_tuning *t);
 
 /* Autotuner: builds the neighbour lists of the structure set (arguments as
  * nep_compute_batch), times the atom and gather kernels for every atoms-per-CTA pair (best of
- * three launches after a warm-up, CUDA events on `stream`) and, when n_pop > 0, members per
+ * three launches after a warm-up, CUDA events on `stream`; for a population, n_pop > 0, with its
+ * force-error sums and as many members as fit) and, when n_pop > 0, members per
  * launch 1, 2, 4, ... up to n_pop (or the workspace budget) with the best pair; keeps the
- * fastest shapes in the handle and returns them in *out (may be NULL). Synchronous. */
+ * fastest shapes in the handle and returns them in *out (may be NULL). Sizes that a small set's
+ * kernels do not read stay at the default. Synchronous. */
 int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *pos, const int *types,
                  const double *boxes, int n_pop, nep_tuning *out, nep_stream_t stream);
 

@@ -1677,7 +1677,9 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  // time one batched evaluation (atom + gather kernels) of `m` members; best of 3 after a warm-up
+  // time one batched evaluation (atom + gather kernels) of `m` members; best of 3 after a warm-up. A
+  // population forms the force error (against any FP64 values here), a batch no block sums: both
+  // kernels depend on it.
   auto time_eval = [&](int m, float *ms) -> int {
     int r = ensure_partials(h, N, m);
     if (r) return r;
@@ -1686,6 +1688,10 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
     a.s_out = N;
     a.s_erad = (long long)N * h->T * est;
     a.s_pang = (long long)h->cap_a * N;
+    if (n_pop > 0) {
+      a.sums = kSumFerr;
+      a.f_tar = h->F.p;
+    }
     float best = 1e30f;
     for (int it = 0; it < 4; ++it) {
       cudaEventRecord(e0, s);
@@ -1705,6 +1711,10 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   int n_tried = 0;
   float best_ms = 1e30f, default_ms = 0.f;
   int best_ab = 128, best_gb = 128;
+  // block sizes: with the members that a population call evaluates per launch. Small systems run split
+  // kernels, which take no block size; the default stays there.
+  const int m0 = n_pop > 0 ? max_members : 1;
+  const bool atoms_by_block = m0 > 1 || N > kSplitAtoms2, gather_by_block = n_pop > 0 || N > kSplitGather2;
   const int abs_[2] = {64, 128}, gbs[3] = {64, 128, 256};
   for (int ia = 0; ia < 2 && !rc; ++ia) {
     // one size for the tensor-core networks (64 atoms whatever it says), the run-time-shape kernels
@@ -1715,32 +1725,36 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
       h->tune.atom_block = abs_[ia];
       h->tune.gather_block = gbs[ig];
       float t = 0.f;
-      rc = time_eval(1, &t);
+      rc = time_eval(m0, &t);
       ++n_tried;
-      if (abs_[ia] == 128 && gbs[ig] == 128) default_ms = t;
-      if (!rc && t < best_ms) {
+      const bool counts = (abs_[ia] == 128 || atoms_by_block) && (gbs[ig] == 128 || gather_by_block);
+      if (m0 == 1 && abs_[ia] == 128 && gbs[ig] == 128) default_ms = t;
+      if (!rc && counts && t < best_ms) {
         best_ms = t;
         best_ab = abs_[ia];
         best_gb = gbs[ig];
       }
     }
   }
+  if (!rc && m0 > 1) {
+    h->tune.atom_block = h->tune.gather_block = 128;
+    rc = time_eval(1, &default_ms);
+    ++n_tried;
+  }
   h->tune.atom_block = best_ab;
   h->tune.gather_block = best_gb;
   int best_m = 0;
   if (!rc && n_pop > 0) {
-    float best_per = best_ms;
-    best_m = 1;
-    for (int m = 2; m <= max_members && !rc; m *= 2) {
+    best_ms = 1e30f;
+    for (int m = 1; m <= max_members && !rc; m *= 2) {
       float t = 0.f;
       rc = time_eval(m, &t);
       ++n_tried;
-      if (!rc && t / m < best_per) {
-        best_per = t / m;
+      if (!rc && t / m < best_ms) {
+        best_ms = t / m;
         best_m = m;
       }
     }
-    best_ms = best_per;
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

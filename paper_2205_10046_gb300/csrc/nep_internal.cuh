@@ -18,6 +18,10 @@ constexpr int kMaxImage = 3;    // largest cell/image offset searched per axis
 // accept is left out.
 constexpr double kReachMargin = 2e-3;
 constexpr int kAtomBlock = 128; // threads per block of the per-atom kernel
+// most atoms of the per-atom and gather kernels with four and with two groups of lanes per atom; the
+// reasons stand at the kernels
+constexpr int kSplitAtoms = 152 * 3 * 16, kSplitAtoms2 = 152 * 3 * 32;
+constexpr int kSplitGather = 152 * 2 * 32, kSplitGather2 = 152 * 2 * 64;
 constexpr int kReduceSlots = 16; // per-block partial sums: U, KE, W[9], force error, J[3], spare
 // sums over all atoms that a call or an MD step reads (AtomArgs::sums)
 enum { kSumU = 1, kSumKE = 2, kSumW = 4, kSumFerr = 8, kSumJ = 16 };

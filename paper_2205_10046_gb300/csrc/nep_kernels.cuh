@@ -478,8 +478,6 @@ __device__ __forceinline__ void for_pairs_batch(const unsigned *__restrict__ nl,
 // cost more than the shorter chain gives. A dynamics step without / with, us (the gather kernel
 // split in both): 216 Si atoms 40 / 36, 5,832 46 / 43, 8,000 46.4 / 45.8, 13,824 57.4 / 55.4, past the
 // limits with four groups 13,824 Si atoms 63 / 71, 8,000 PbTe atoms 41 / 50.
-constexpr int kSplitAtoms = 152 * 3 * 16;
-constexpr int kSplitAtoms2 = 152 * 3 * 32;
 template <class S>
 struct PairRow {
   static constexpr int Q4 = S::NDP / 4;                  // float4s of q
@@ -1650,8 +1648,6 @@ constexpr int kGatherAtoms = 64;  // atoms per CTA of the gather of one structur
 // of two CTAs per SM. A dynamics step with one / four / two groups, us: 1,000 Si atoms 43 / 36 / -,
 // 8,000 53 / 46 / -, 13,824 60.4 / 62.8 / 57.4, 13,824 PbTe atoms 54.0 / 53.7 / 48.8, 21,952 Si atoms
 // 71 / 79 / -.
-constexpr int kSplitGather = 152 * 2 * 32, kSplitGather2 = 152 * 2 * 64;
-
 template <class S>
 cudaError_t launch_gather(const AtomArgs &a, cudaStream_t st) {
   if (a.N <= 0) return cudaSuccess;
