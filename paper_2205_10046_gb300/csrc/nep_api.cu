@@ -210,6 +210,7 @@ void set_shape_args(AtomArgs &a, const nep_params &p) {
   a.gL4 = p.l_max_4b;
   a.gL5 = p.l_max_5b;
   a.gD = n_des_of(&p);
+  a.pop = 1;
 }
 
 // BF16 (round to nearest even) of a float, as raw bits.
@@ -716,6 +717,7 @@ AtomArgs make_args(nep_handle *h, int N) {
   a.tc_err = h->status.p ? &h->status.p->tc_timeout : nullptr;
   a.gR = h->nR; a.gKR = h->KR; a.gA = h->nA; a.gKA = h->KA; a.gH = h->H;
   a.gL3 = h->L3; a.gL4 = h->L4; a.gL5 = h->L5; a.gD = h->n_des;
+  a.pop = 1;
   return a;
 }
 
@@ -1625,6 +1627,7 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
     a.s_pang = (long long)h->cap_a * N;
     a.f_tar = f_tar;
     a.sums = kSumFerr;
+    a.pop = n_pop;
     ev_record(h, SLOT_ATOM, 0, s, false);
     cudaError_t e = h->ops->atom_batch(a, h->mf, m, atom_block(h), s);
     if (e != cudaSuccess) return cuda_fail(h, e, "nep_atom kernel (population)");
@@ -1691,6 +1694,7 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
     if (n_pop > 0) {
       a.sums = kSumFerr;
       a.f_tar = h->F.p;
+      a.pop = n_pop;
     }
     float best = 1e30f;
     for (int it = 0; it < 4; ++it) {

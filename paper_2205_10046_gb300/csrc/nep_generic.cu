@@ -23,6 +23,11 @@ constexpr int kSRow = 25;   // S_nk row of one n (24 used)
 constexpr int kNeu = 32;    // neurons of the network at a time: one per lane
 constexpr int kGenGatherLanes = 8;
 constexpr int kBRow = 20;   // row of dU/dz of one neuron (16 atoms used)
+// limits of the thread-per-atom kernel
+constexpr int kThinSums = 72;            // S_nk of an atom
+constexpr int kThinDes = kGenK + 40;     // descriptor components: l_max^3b = 1 with n_max^A = 19 has the most
+constexpr int kThinWeights = 4096;       // N_neu x N_des
+constexpr long long kThinEvals = 49152;  // least atoms x members
 
 // f_k(r), k = 0..K (Eq. f_n with the cosine cutoff), and f_k'(r) (0 without FP), given to out(k, f, fp)
 // one after the other. Every multiply-add is spelled out, so that all kernels round alike.
@@ -103,13 +108,214 @@ __host__ __device__ inline GenSmem gen_smem(int nA, int KA, int D) {
 }
 
 // last polynomial index + 1 used by the 3-body terms and the 4-body term
-__device__ __forceinline__ int n_poly(int L3, int L4) {
+__host__ __device__ inline int n_poly(int L3, int L4) {
   const int k3 = L3 == 1 ? 3 : L3 == 2 ? 8 : L3 == 3 ? 15 : 24;
   return (L4 >= 2 && k3 < 8) ? 8 : k3;
 }
 
-// One kernel for one structure and for batches (grid.y: members of a population), so that both give
-// the same bits. 16 atoms per block. Descriptor and forces: a warp per atom (two atoms in turn). Radial pairs:
+// Thin shapes (l <= 2, few S_nk and weights) in large calls: a thread per atom, S_nk, descriptor and dU/dq in
+// local memory. What bounds it: latency of the scattered reads and of the L1 lines behind the local
+// arrays. A warp per atom has little to spread over its lanes there and pays for its reductions and the
+// block's phases; a small call of threads is one long serial chain instead. Whole calls, warp / thread
+// per atom, us, of n_max 2/1, N_bas 3/2, l 2, 5 neurons: 1,000 atoms 103 / 123, 32,000 252 / 191, 64,000
+// 454 / 262, 8 candidates on 67,259 atoms 2607 / 1208; of n_max 8/4, N_bas 8/4, l 2, 30 neurons: 1,000
+// atoms 111 / 228, 32,000 321 / 330, 64,000 585 / 530, 8 candidates 3701 / 2387. Past the limits the warp
+// wins: l 4 with 48 sums, 67,259 atoms (this kernel alone) 372 / 440, 104 sums 849 / 1008, 256 neurons with
+// 28 components 788 / 931.
+// (The two forms round alike only up to the order of their sums.)
+template <bool DESC_ONLY>
+__global__ void __launch_bounds__(128) thin_atom_kernel(const AtomArgs a, const ModelF mf) {
+  if (build_failed(a.guard)) return;
+  const int N = a.N, T = a.T;
+  const int nR = a.gR, KR = a.gKR, nA = a.gA, KA = a.gKA, H = a.gH, L3 = a.gL3, L4 = a.gL4, L5 = a.gL5, D = a.gD;
+  const int NK = n_poly(L3, L4);
+  const int off4 = (nR + 1) + (nA + 1) * L3, off5 = off4 + (L4 >= 2 ? nA + 1 : 0);
+  const int mem = blockIdx.y;  // 0 for one structure, whose atoms carry structure 0
+  const float *w0 = a.tab + mem * a.s_tab, *b0 = w0 + H * D, *w1 = b0 + H;
+  const float *c_r = a.c_r + mem * a.s_tab, *c_a = a.c_a + mem * a.s_tab;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double U = 0.0;
+  // (serving engine) atoms of a finished job frozen in the batch are skipped
+  if (i < N && !(a.slots && a.slots[struct_of(a.pos4[i])].phase == 2)) {
+    const float4 pi = a.pos4[i];
+    const int ti = type_of(pi);
+    const float4 *tab = a.dtab + (size_t)struct_of(pi) * a.ncode;
+    const float inv_rcR = 1.f / a.rcR, inv_rcA = 1.f / a.rcA;
+    const float rcR2 = a.rcR * a.rcR, rcA2 = a.rcA * a.rcA;
+    float q[kThinDes], dq[kThinDes];  // descriptor, dU/dq
+    float S[kThinSums];               // S_nk, then dU/dS_nk, row n at n * NK
+    float f[kGenK], fp[kGenK], g[kGenK], gp[kGenK];
+    for (int v = 0; v < D; ++v) q[v] = dq[v] = 0.f;
+    for (int v = 0; v < (nA + 1) * NK; ++v) S[v] = 0.f;
+    // radial descriptor (Eq. qin): the f_k summed over each neighbour type, then contracted with c_nk
+    int base = 0;
+    for (int t = 0; t < T; ++t) {
+      const int cnt = a.nn_r[(size_t)t * N + i];
+      for (int k = 0; k <= KR; ++k) f[k] = 0.f;
+      for (int m = base; m < base + cnt; ++m) {
+        const unsigned e = a.nl_r[(size_t)m * N + i];
+        const float3 d = pair_vector(pi, a.pos4[e & a.jmask], tab[e >> a.jbits]);
+        const float r2 = norm2(d);
+        if (r2 < rcR2) basis_rt<false>(sqrtf(r2), inv_rcR, KR, [&](int k, float fk, float) { f[k] += fk; });
+      }
+      base += cnt;
+      const float *c = c_r + (size_t)(ti * T + t) * (nR + 1) * (KR + 1);
+      for (int n = 0; n <= nR; ++n)
+        for (int k = 0; k <= KR; ++k) q[n] = fmaf(__ldg(c + n * (KR + 1) + k), f[k], q[n]);
+    }
+    // angular pairs inside the cutoff: body(m, d, r2, 1 / r) with g_n, and g_n' with FP
+    const int na = a.nn_a[i];
+    auto angular = [&](auto fpc, auto body) {
+      constexpr bool FP = decltype(fpc)::value;
+      for (int m = 0; m < na; ++m) {
+        const unsigned e = a.nl_a[(size_t)m * N + i];
+        const float4 pj = a.pos4[e & a.jmask];
+        const float3 d = pair_vector(pi, pj, tab[e >> a.jbits]);
+        const float r2 = norm2(d);
+        if (!(r2 < rcA2)) continue;
+        const float rinv = rsqrtf(r2);
+        basis_rt<FP>(r2 * rinv, inv_rcA, KA, [&](int k, float fk, float fpk) {
+          f[k] = fk;
+          fp[k] = fpk;
+        });
+        const float *c = c_a + (size_t)(ti * T + type_of(pj)) * (nA + 1) * (KA + 1);
+        for (int n = 0; n <= nA; ++n) {
+          float x = 0.f, xp = 0.f;
+          for (int k = 0; k <= KA; ++k) {
+            const float ck = __ldg(c + n * (KA + 1) + k);
+            x = fmaf(ck, f[k], x);
+            if (FP) xp = fmaf(ck, fp[k], xp);
+          }
+          g[n] = x;
+          gp[n] = xp;
+        }
+        body(m, d, r2, rinv);
+      }
+    };
+    // angular sums S_nk (Eq. S_nk, b_k(d) r^-l)
+    angular(std::false_type{}, [&](int, const float3 &d, float r2, float rinv) {
+      const float rl[5] = {1.f, rinv, rinv * rinv, rinv * rinv * rinv, (rinv * rinv) * (rinv * rinv)};
+      static_for<0, 24>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        if (k < NK) {
+          const float b = poly_b<k>(d.x, d.y, d.z, r2) * rl[l_of_k(k)];
+          for (int n = 0; n <= nA; ++n) S[n * NK + k] = fmaf(g[n], b, S[n * NK + k]);
+        }
+      });
+    });
+    // angular descriptor components (Sec. II D)
+    for (int n = 0; n <= nA; ++n) {
+      const float *s = S + n * NK;
+      for (int l = 1; l <= L3; ++l) {
+        float x = 0.f;
+        for (int k = l * l - 1; k < l * (l + 2); ++k) x = fmaf(mf.c3b[k] * s[k], s[k], x);
+        q[(nR + 1) + (l - 1) * (nA + 1) + n] = x;
+      }
+      if (L4 >= 2)
+        q[off4 + n] = mf.c4b[0] * s[3] * s[3] * s[3] + mf.c4b[1] * s[3] * (s[4] * s[4] + s[5] * s[5]) +
+                      mf.c4b[2] * s[3] * (s[6] * s[6] + s[7] * s[7]) + mf.c4b[3] * s[6] * (s[5] * s[5] - s[4] * s[4]) +
+                      mf.c4b[4] * s[4] * s[5] * s[7];
+      if (L5 >= 1) {
+        const float s12 = s[1] * s[1] + s[2] * s[2];
+        q[off5 + n] = mf.c5b[0] * s[0] * s[0] * s[0] * s[0] + mf.c5b[1] * s[0] * s[0] * s12 + mf.c5b[2] * s12 * s12;
+      }
+    }
+    if constexpr (DESC_ONLY) {
+      const size_t io = a.perm ? (size_t)a.perm[i] : (size_t)i;
+      for (int v = 0; v < D; ++v) a.q_out[io * D + v] = (double)q[v];
+      return;
+    }
+    // network (Eq. Ui) and dU/dq
+    float u = 0.f;
+    for (int mu = 0; mu < H; ++mu) {
+      const float *w = w0 + mu * D;
+      float z = -__ldg(b0 + mu);
+      for (int v = 0; v < D; ++v) z = fmaf(__ldg(w + v), q[v], z);
+      const float wo = __ldg(w1 + mu), h = tanhf(z), beta = wo * (1.f - h * h);
+      u = fmaf(wo, h, u);
+      for (int v = 0; v < D; ++v) dq[v] = fmaf(beta, __ldg(w + v), dq[v]);
+    }
+    u -= __ldg(w1 + H);
+    U = (double)u;
+    if (a.energy) a.energy[mem * a.s_out + (a.perm ? a.perm[i] : i)] = U;
+    // radial force coefficients e^t_k = sum_n dU/dq_n c^{t_i t}_nk, rows padded with zeros
+    float *const erow = a.e_rad + mem * a.s_erad + (size_t)i * T * a.est;
+    for (int t = 0; t < T; ++t) {
+      const float *c = c_r + (size_t)(ti * T + t) * (nR + 1) * (KR + 1);
+      for (int k = 0; k < a.est; ++k) {
+        float e = 0.f;
+        if (k <= KR)
+          for (int n = 0; n <= nR; ++n) e = fmaf(dq[n], __ldg(c + n * (KR + 1) + k), e);
+        erow[t * a.est + k] = e;
+      }
+    }
+    // dU/dS_nk from the explicit 3/4/5-body forms, in place
+    for (int n = 0; n <= nA; ++n) {
+      float s[8];
+      float *const dS = S + n * NK;
+      for (int k = 0; k < 8; ++k) s[k] = k < NK ? dS[k] : 0.f;
+      for (int k = 0; k < NK; ++k) {
+        const int l = k < 3 ? 1 : k < 8 ? 2 : k < 15 ? 3 : 4;
+        dS[k] = l <= L3 ? 2.f * mf.c3b[k] * dS[k] * dq[(nR + 1) + (l - 1) * (nA + 1) + n] : 0.f;
+      }
+      if (L4 >= 2) {
+        const float d4 = dq[off4 + n];
+        const float *C = mf.c4b;
+        dS[3] += d4 * (3.f * C[0] * s[3] * s[3] + C[1] * (s[4] * s[4] + s[5] * s[5]) + C[2] * (s[6] * s[6] + s[7] * s[7]));
+        dS[4] += d4 * (2.f * C[1] * s[3] * s[4] - 2.f * C[3] * s[6] * s[4] + C[4] * s[5] * s[7]);
+        dS[5] += d4 * (2.f * C[1] * s[3] * s[5] + 2.f * C[3] * s[6] * s[5] + C[4] * s[4] * s[7]);
+        dS[6] += d4 * (2.f * C[2] * s[3] * s[6] + C[3] * (s[5] * s[5] - s[4] * s[4]));
+        dS[7] += d4 * (2.f * C[2] * s[3] * s[7] + C[4] * s[4] * s[5]);
+      }
+      if (L5 >= 1) {
+        const float d5 = dq[off5 + n];
+        const float *C = mf.c5b;
+        const float s12 = s[1] * s[1] + s[2] * s[2];
+        dS[0] += d5 * (4.f * C[0] * s[0] * s[0] * s[0] + 2.f * C[1] * s[0] * s12);
+        const float common = 2.f * C[1] * s[0] * s[0] + 4.f * C[2] * s12;
+        dS[1] += d5 * common * s[1];
+        dS[2] += d5 * common * s[2];
+      }
+    }
+    // angular partial forces dU_i/dr_ij (angular terms of Eq. partial_force)
+    float4 *const pang = a.p_ang + mem * a.s_pang;
+    angular(std::true_type{}, [&](int m, const float3 &d, float r2, float rinv) {
+      const float rl[5] = {1.f, rinv, rinv * rinv, rinv * rinv * rinv, (rinv * rinv) * (rinv * rinv)};
+      float gx = 0.f, gy = 0.f, gz = 0.f, yy = 0.f;
+      static_for<0, 24>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        if (k < NK) {
+          float ak = 0.f, ck = 0.f;
+          for (int n = 0; n <= nA; ++n) {
+            ak = fmaf(S[n * NK + k], g[n], ak);
+            ck = fmaf(S[n * NK + k], gp[n], ck);
+          }
+          ak *= rl[l_of_k(k)];
+          ck *= rl[l_of_k(k)];
+          const float3 gb = poly_grad<k>(d.x, d.y, d.z, r2);
+          gx = fmaf(ak, gb.x, gx);
+          gy = fmaf(ak, gb.y, gy);
+          gz = fmaf(ak, gb.z, gz);
+          yy = fmaf(ck, poly_b<k>(d.x, d.y, d.z, r2), yy);
+        }
+      });
+      const float ux = d.x * rinv, uy = d.y * rinv, uz = d.z * rinv;
+      const float gu = gx * ux + gy * uy + gz * uz;
+      pang[(size_t)m * N + i] =
+          make_float4((gx - gu * ux) + yy * ux, (gy - gu * uy) + yy * uy, (gz - gu * uz) + yy * uz, 0.f);
+    });
+  }
+  if constexpr (!DESC_ONLY) {
+    if (sums_needed(a) & kSumU) {  // a slot per kGenAtoms atoms, as the other form
+#pragma unroll
+      for (int o = kGenAtoms / 2; o > 0; o >>= 1) U += __shfl_xor_sync(0xffffffffu, U, o);
+      if (i % kGenAtoms == 0 && i < N) a.partial_atom[i / kGenAtoms] = U;
+    }
+  }
+}
+
+// The other shapes and calls: one kernel for one structure and for batches (grid.y: members of a
+// population), so that both give the same bits. 16 atoms per block. Descriptor and forces: a warp per atom (two atoms in turn). Radial pairs:
 // a lane per pair, the f_k summed over each neighbour type before the contraction with c_nk.
 // Angular pairs: those inside the cutoff go through shared memory in groups of 16, so that the
 // contractions over n and k spread over all lanes however few pairs there are. Network: the block
@@ -598,6 +804,11 @@ constexpr int kGenGatherAtoms = 32;  // one structure; batches: 128 (the caller'
 
 template <bool DESC_ONLY>
 cudaError_t launch_generic_atom(const AtomArgs &a, const ModelF &mf, int members, cudaStream_t s) {
+  const int nk = n_poly(a.gL3, a.gL4);
+  if (nk <= 8 && (a.gA + 1) * nk <= kThinSums && a.gH * a.gD <= kThinWeights && (long long)a.N * a.pop >= kThinEvals) {
+    thin_atom_kernel<DESC_ONLY><<<dim3((a.N + 127) / 128, members), 128, 0, s>>>(a, mf);
+    return cudaGetLastError();
+  }
   auto *kern = &generic_atom_kernel<DESC_ONLY>;
   const cudaError_t e = smem_limit_once(kern, sizeof(float) * gen_smem(kGenMaxN, kGenMaxN, kGenMaxDes).total);
   if (e != cudaSuccess) return e;

@@ -253,6 +253,7 @@ struct AtomArgs {
   // model shape at run time: read only by the kernels that take the shape at run time (shapes
   // without a compiled instantiation)
   int gR, gKR, gA, gKA, gH, gL3, gL4, gL5, gD;
+  int pop;  // members of the whole call (however many a launch holds): 1, or the population's
 };
 
 // The build before this launch failed (the host, which has not looked yet, reports it or builds
