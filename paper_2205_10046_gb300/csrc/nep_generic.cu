@@ -27,7 +27,8 @@ constexpr int kBRow = 20;   // row of dU/dz of one neuron (16 atoms used)
 constexpr int kThinSums = 72;            // S_nk of an atom
 constexpr int kThinDes = kGenK + 40;     // descriptor components: l_max^3b = 1 with n_max^A = 19 has the most
 constexpr int kThinWeights = 4096;       // N_neu x N_des
-constexpr long long kThinEvals = 49152;  // least atoms x members
+constexpr long long kThinEvals = 49152;  // least atoms x members of a call
+constexpr long long kThinEvals4 = 131072;  // with l > 2 and more than 30 sums
 
 // f_k(r), k = 0..K (Eq. f_n with the cosine cutoff), and f_k'(r) (0 without FP), given to out(k, f, fp)
 // one after the other. Every multiply-add is spelled out, so that all kernels round alike.
@@ -113,15 +114,16 @@ __host__ __device__ inline int n_poly(int L3, int L4) {
   return (L4 >= 2 && k3 < 8) ? 8 : k3;
 }
 
-// Thin shapes (l <= 2, few S_nk and weights) in large calls: a thread per atom, S_nk, descriptor and dU/dq in
+// Thin shapes (few S_nk and weights) in large calls: a thread per atom, S_nk, descriptor and dU/dq in
 // local memory. What bounds it: latency of the scattered reads and of the L1 lines behind the local
 // arrays. A warp per atom has little to spread over its lanes there and pays for its reductions and the
 // block's phases; a small call of threads is one long serial chain instead. Whole calls, warp / thread
 // per atom, us, of n_max 2/1, N_bas 3/2, l 2, 5 neurons: 1,000 atoms 103 / 123, 32,000 252 / 191, 64,000
 // 454 / 262, 8 candidates on 67,259 atoms 2607 / 1208; of n_max 8/4, N_bas 8/4, l 2, 30 neurons: 1,000
-// atoms 111 / 228, 32,000 321 / 330, 64,000 585 / 530, 8 candidates 3701 / 2387. Past the limits the warp
-// wins: l 4 with 48 sums, 67,259 atoms (this kernel alone) 372 / 440, 104 sums 849 / 1008, 256 neurons with
-// 28 components 788 / 931.
+// atoms 111 / 228, 32,000 321 / 330, 64,000 585 / 530, 8 candidates 3701 / 2387; of n_max 4/2, N_bas 4/4, l 4
+// with 30 neurons (72 sums): 131,072 atoms 1142 / 1009, 200,000 1617 / 1619, 8 candidates 3802 / 3445. Past the
+// limits the warp wins: l 4 with 48 sums, 67,259 atoms (this kernel alone) 372 / 440, 104 sums 849 / 1008,
+// 256 neurons with 28 components 788 / 931.
 // (The two forms round alike only up to the order of their sums.)
 template <bool DESC_ONLY>
 __global__ void __launch_bounds__(128) thin_atom_kernel(const AtomArgs a, const ModelF mf) {
@@ -805,7 +807,9 @@ constexpr int kGenGatherAtoms = 32;  // one structure; batches: 128 (the caller'
 template <bool DESC_ONLY>
 cudaError_t launch_generic_atom(const AtomArgs &a, const ModelF &mf, int members, cudaStream_t s) {
   const int nk = n_poly(a.gL3, a.gL4);
-  if (nk <= 8 && (a.gA + 1) * nk <= kThinSums && a.gH * a.gD <= kThinWeights && (long long)a.N * a.pop >= kThinEvals) {
+  const int sums = (a.gA + 1) * nk;
+  if (sums <= kThinSums && a.gH * a.gD <= kThinWeights &&
+      (long long)a.N * a.pop >= (nk <= 8 || sums <= 30 ? kThinEvals : kThinEvals4)) {
     thin_atom_kernel<DESC_ONLY><<<dim3((a.N + 127) / 128, members), 128, 0, s>>>(a, mf);
     return cudaGetLastError();
   }

@@ -9,7 +9,7 @@ from paper_2205_10046_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-THREADS = 49152  # atoms from which a thread per atom works
+THREADS = 49152  # atoms from which a thread per atom works; "wide" shapes: 131072
 
 # n_max^R, N_bas^R, n_max^A, N_bas^A, N_neu, l_max^3b, 4b, 5b, types
 SHAPES = {
@@ -18,6 +18,9 @@ SHAPES = {
     "most_sums": (19, 19, 8, 19, 33, 2, 2, 1, 2),
     "most_n": (4, 7, 19, 3, 50, 1, 0, 1, 2),
     "l2_only": (8, 8, 1, 4, 40, 2, 0, 0, 2),
+    "l3": (5, 4, 1, 4, 30, 3, 2, 1, 2),
+    "l4": (6, 5, 0, 4, 20, 4, 2, 1, 3),
+    "wide_l4": (4, 4, 2, 4, 20, 4, 2, 1, 2),
 }
 
 
@@ -48,10 +51,11 @@ def test_thread_and_warp_forms_agree(torch_cuda, name):
     from paper_2205_10046_gb300 import nep
     model = _model(name)
     T = model.n_types
+    threads = 131072 if name.startswith("wide") else THREADS
     parts = [W.random_structure(30 + n, n, n_types_model=T) for n in (33, 500, 127, 257)]
     few = W.concat_structures(parts)
-    many = W.concat_structures(parts * (THREADS // few.n_atoms + 1))  # and an odd count of atoms
-    assert few.n_atoms < THREADS <= many.n_atoms
+    many = W.concat_structures(parts * (threads // few.n_atoms + 1))  # and an odd count of atoms
+    assert few.n_atoms < threads <= many.n_atoms
     dev = lambda a, dt=torch.float64: torch.tensor(a, dtype=dt, device="cuda")  # noqa: E731
     h = nep.NEP(model, skin=0.4)
     batch = lambda b: {k: v.cpu().numpy() for k, v in h.compute_batch(  # noqa: E731
@@ -67,7 +71,7 @@ def test_thread_and_warp_forms_agree(torch_cuda, name):
         _close(t["E_struct"][s:s + few.n_struct], w["E_struct"])
         _close(t["W_struct"][s:s + few.n_struct], w["W_struct"])
     # one large structure: the sum of its atoms, its descriptors and a few steps
-    pos, types, box = W.random_structure(3, THREADS + 5, n_types_model=T)
+    pos, types, box = W.random_structure(3, threads + 5, n_types_model=T)
     p, ty = dev(pos), dev(types, torch.int32)
     o = {k: v.cpu().numpy() for k, v in h.compute(p, ty, box, per_atom_virial=True).items()}
     assert abs(o["E"][0] - o["U"].sum()) <= 1e-10 * np.abs(o["U"]).sum()
