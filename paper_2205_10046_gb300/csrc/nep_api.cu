@@ -301,8 +301,9 @@ struct PinnedBuf {
   cudaError_t ensure(size_t want) {
     if (want <= n) return cudaSuccess;
     release();
-    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&p), want + want / 2, cudaHostAllocDefault);
-    if (e == cudaSuccess) n = want + want / 2;
+    const size_t get = want + std::min<size_t>(want / 2, 32u << 20);
+    const cudaError_t e = cudaHostAlloc(reinterpret_cast<void **>(&p), get, cudaHostAllocDefault);
+    if (e == cudaSuccess) n = get;
     else p = nullptr;
     return e;
   }
@@ -1297,33 +1298,47 @@ int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild) {
 
 long long engine_builds(const nep_handle *h) { return h->h_status ? h->h_status->n_rebuilds : 0; }
 
-// Final arrays of the given jobs, each in its own atom order: positions wrapped into its cell, forces,
-// velocities. A kernel per job writes them into page-locked host memory, and the host waits once
-// for all of them (four copies from pageable memory and a wait per job took 48 us a job); read
-// them with engine_arrays, in the order of `jobs`, before the next call.
-int engine_fetch(nep_handle *h, const std::vector<int> &jobs, cudaStream_t s) {
-  h->e_out_at.assign(1, 1);  // the first double: error flag
-  for (int k : jobs) {
+// Final arrays of jobs[first .. *end), each in its own atom order: positions wrapped into its cell,
+// forces, velocities. A kernel per job writes them into page-locked host memory, and the host waits
+// once for all of them (four copies from pageable memory and a wait per job took 48 us a job). *end is
+// set to as many jobs as fit kFetchBytes, one at least, so that the memory stays bounded however many
+// end at once; read them with engine_arrays before the next call.
+constexpr size_t kFetchBytes = 64u << 20;
+
+int engine_fetch(nep_handle *h, const std::vector<int> &jobs, size_t first, size_t *end, cudaStream_t s) {
+  *end = first + 1;  // (a failure is this job's)
+  h->e_out_at.assign(1, 0);
+  size_t e = first;
+  for (; e < jobs.size(); ++e) {
+    const int k = jobs[e];
     if (k < 0 || k >= h->nb_struct) return fail(h, NEP_ERR_ARG, "engine: bad job index");
-    h->e_out_at.push_back(h->e_out_at.back() + 9 * (size_t)(h->b_offsets[k + 1] - h->b_offsets[k]));
+    const size_t at = h->e_out_at.back() + 1 + 9 * (size_t)(h->b_offsets[k + 1] - h->b_offsets[k]);  // flag, arrays
+    if (e > first && at * sizeof(double) > kFetchBytes) break;
+    h->e_out_at.push_back(at);
   }
-  CK(h->e_out.ensure(sizeof(double) * h->e_out_at.back()), "alloc results");
+  const size_t bytes = sizeof(double) * h->e_out_at.back();
+  if (h->e_out.n > 2 * kFetchBytes && bytes <= kFetchBytes) h->e_out.release();  // of a single large job
+  CK(h->e_out.ensure(bytes), "alloc results");
   double *const out = reinterpret_cast<double *>(h->e_out.p);
-  volatile int *const bad = reinterpret_cast<volatile int *>(h->e_out.p);
-  *bad = 0;
-  for (size_t q = 0; q < jobs.size(); ++q) {
-    const int o = h->b_offsets[jobs[q]], n = h->b_offsets[jobs[q] + 1] - o;
-    launch_engine_export(o, n, atom_state(h), h->b_grids[jobs[q]], out + h->e_out_at[q], const_cast<int *>(bad), s);
+  for (size_t q = 0; q < e - first; ++q) {
+    const int k = jobs[first + q], o = h->b_offsets[k], n = h->b_offsets[k + 1] - o;
+    int *const bad = reinterpret_cast<int *>(out + h->e_out_at[q]);
+    *bad = 0;
+    launch_engine_export(o, n, atom_state(h), h->b_grids[k], out + h->e_out_at[q] + 1, bad, s);
   }
   CK(cudaGetLastError(), "engine export");
   CK(wait_stream(s), "sync");
-  if (*bad) return fail(h, NEP_ERR_CUDA, "engine: inconsistent atom order");
+  *end = e;
   return NEP_OK;
 }
 
-// [3][n][3]: positions, forces, velocities of the q-th job of the last engine_fetch.
-const double *engine_arrays(const nep_handle *h, size_t q) {
-  return reinterpret_cast<const double *>(h->e_out.p) + h->e_out_at[q];
+// [3][n][3] (positions, forces, velocities) of the q-th job of the last engine_fetch, or null with the
+// handle's error set: its atom order is inconsistent.
+const double *engine_arrays(nep_handle *h, size_t q) {
+  const double *p = reinterpret_cast<const double *>(h->e_out.p) + h->e_out_at[q];
+  if (*reinterpret_cast<const volatile int *>(p) == 0) return p + 1;
+  fail(h, NEP_ERR_CUDA, "engine: inconsistent atom order");
+  return nullptr;
 }
 
 size_t workspace_bytes(nep_handle *h) {

@@ -390,8 +390,8 @@ int engine_relayout(nep_handle *h, const std::vector<int> &keep, const std::vect
 int engine_step(nep_handle *h, cudaStream_t s, int n_iter, bool force_rebuild);
 // neighbour builds of the engine's batch so far (read with the status after every chunk)
 long long engine_builds(const nep_handle *h);
-int engine_fetch(nep_handle *h, const std::vector<int> &jobs, cudaStream_t s);
-const double *engine_arrays(const nep_handle *h, size_t q);
+int engine_fetch(nep_handle *h, const std::vector<int> &jobs, size_t first, size_t *end, cudaStream_t s);
+const double *engine_arrays(nep_handle *h, size_t q);
 int engine_jobs(const nep_handle *h);
 int engine_atoms(const nep_handle *h);
 const EngineSlot &engine_slot(const nep_handle *h, int k);

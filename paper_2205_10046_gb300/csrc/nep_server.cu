@@ -311,8 +311,9 @@ void nep_server::scheduler_main() {
     std::vector<int> ended;
     for (size_t k = 0; k < active.size(); ++k)
       if (!active[k].finished && nep::engine_slot(h, (int)k).phase == 2) ended.push_back((int)k);
-    const int fetched = ended.empty() ? NEP_OK : nep::engine_fetch(h, ended, s);
-    size_t q_ended = 0;
+    // their arrays come over in groups: ended[q_first .. q_end) are here now
+    int fetched = NEP_OK;
+    size_t q_ended = 0, q_first = 0, q_end = 0;
     for (size_t k = 0; k < active.size(); ++k) {
       Job &j = active[k];
       if (j.finished) {
@@ -333,9 +334,13 @@ void nep_server::scheduler_main() {
       res.workspace_est = j.est;
       const size_t n3 = 3 * (size_t)j.spec.n_atoms;
       Arrays a;
-      res.status = fetched;
-      if (fetched == NEP_OK) {
-        const double *x = nep::engine_arrays(h, q_ended);
+      if (q_ended == q_end) {
+        q_first = q_ended;
+        fetched = nep::engine_fetch(h, ended, q_first, &q_end, s);
+      }
+      const double *x = fetched == NEP_OK ? nep::engine_arrays(h, q_ended - q_first) : nullptr;
+      res.status = x ? NEP_OK : fetched != NEP_OK ? fetched : NEP_ERR_CUDA;
+      if (x) {
         a.pos.assign(x, x + n3);
         a.force.assign(x + n3, x + 2 * n3);
         if (j.spec.kind == NEP_JOB_NVE) a.vel.assign(x + 2 * n3, x + 3 * n3);
