@@ -254,6 +254,34 @@ void fill_table(const TableLayout &t, const nep_params &p, float *out) {
     }
 }
 
+// Memory that a kernel on `device` may read: its own, or managed. Another GPU's may need peer access
+// that nobody has enabled, and a kernel that reads it without faults.
+bool readable_in_place(const void *p, int device) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
+}
+
+// The caller's positions and types as the build's kernels read them: in place, or copied by the
+// runtime (which reaches them wherever they lie) into a.x2 and a.types2, which a build overwrites.
+cudaError_t load_source(int N, const double *pos, const int *types, float4 *dtab, const AtomState &a, int device,
+                        cudaStream_t s, LoadSrc *out) {
+  *out = LoadSrc{pos, types, dtab};
+  cudaError_t e = cudaSuccess;
+  if (!readable_in_place(pos, device)) {
+    e = cudaMemcpyAsync(a.x2, pos, sizeof(double) * 3 * (size_t)N, cudaMemcpyDefault, s);
+    out->pos = a.x2;
+  }
+  if (e == cudaSuccess && !readable_in_place(types, device)) {
+    e = cudaMemcpyAsync(a.types2, types, sizeof(int) * (size_t)N, cudaMemcpyDefault, s);
+    out->types = a.types2;
+  }
+  return e;
+}
+
 }  // namespace nep
 
 namespace {
@@ -741,7 +769,9 @@ int load_structure(nep_handle *h, int N, const double *pos, const int *types, co
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = h->grid.nc[a];
-  return rebuild_lists(h, N, s, move, Batch{nullptr, nullptr, 0}, LoadSrc{pos, types, h->dtab.p}, after);
+  LoadSrc src;
+  CK(load_source(N, pos, types, h->dtab.p, atom_state(h), h->device, s, &src), "copy in");
+  return rebuild_lists(h, N, s, move, Batch{nullptr, nullptr, 0}, src, after);
 }
 
 // Outputs for the caller (nep_compute) are scattered to the caller's atom order; the MD
@@ -1510,9 +1540,11 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
   }
   rc = setup_batch(h, n_struct, offsets, boxes, N, s);
   if (rc) return rc;
+  LoadSrc src;
+  CK(load_source(N, pos, types, nullptr, atom_state(h), h->device, s, &src), "copy in");
   BatchOut o;
-  o.pos = pos;
-  o.types = types;
+  o.pos = src.pos;
+  o.types = src.types;
   o.e_atom = energy;
   o.w_atom = virial;
   o.force = force;
@@ -1541,12 +1573,13 @@ int nep_compute_batch(nep_handle *h, int n_struct, const int *offsets, const dou
     if (st.tc_timeout) return timed_out(h);
     if (!st.overflow && !st.rev_missing) return NEP_OK;
     // the lists outgrew their capacity: size them again on the eager path below
+    CK(load_source(N, pos, types, nullptr, atom_state(h), h->device, s, &src), "copy in");
   }
   ev_record(h, SLOT_REBUILD, 0, s, false);
   h->N = N;
   h->stats_cache.n_atoms = N;
   for (int a = 0; a < 3; ++a) h->stats_cache.cells[a] = 0;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), src);
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   rc = batch_kernels(h, N, o, s, false);
@@ -1594,7 +1627,9 @@ int nep_eval_population(nep_handle *h, int n_pop, const double *z, int n_struct,
   ev_record(h, SLOT_REBUILD, 0, s, false);
   h->N = N;
   h->stats_cache.n_atoms = N;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
+  LoadSrc src;
+  CK(load_source(N, pos, types, nullptr, atom_state(h), h->device, s, &src), "copy in");
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), src);
   if (rc) return rc;
   ev_record(h, SLOT_REBUILD, 1, s, false);
   // parameter vectors -> FP32 model tables (and BF16 tiles for the tensor-core network)
@@ -1679,7 +1714,9 @@ int nep_autotune(nep_handle *h, int n_struct, const int *offsets, const double *
   rc = setup_batch(h, n_struct, offsets, boxes, N, s);
   if (rc) return rc;
   h->N = N;
-  rc = rebuild_lists(h, N, s, 0, batch_of(h), LoadSrc{pos, types, nullptr});
+  LoadSrc src;
+  CK(load_source(N, pos, types, nullptr, atom_state(h), h->device, s, &src), "copy in");
+  rc = rebuild_lists(h, N, s, 0, batch_of(h), src);
   if (rc) return rc;
   // candidates: atoms per CTA of both kernels, then (for a population) members per launch
   const int est = ((h->KR + 2) + 3) / 4 * 4;

@@ -343,6 +343,8 @@ __host__ __device__ inline int tile_place(const TableLayout &t, int mu, int nu) 
 struct Grid;
 void model_constants(ModelF &m);
 int build_grid(const double *box, double rl, int N, Grid &g, double *volume, const char **err);
+cudaError_t load_source(int N, const double *pos, const int *types, float4 *dtab, const AtomState &a, int device,
+                        cudaStream_t s, LoadSrc *out);
 cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
                            float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only,
                            int move, const LoadSrc &src, BuildStatus *st, cudaStream_t s);

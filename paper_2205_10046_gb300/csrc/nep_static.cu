@@ -194,8 +194,11 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   const float rcR = (float)params->rc_radial, rcA = (float)params->rc_angular;
   BuildStatus host_st;
   // sizing pass, then the lists
-  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, LoadSrc{pos, types, dtab}, st,
-                 &host_st, s);
+  int dev = 0;
+  SK(cudaGetDevice(&dev), "device");
+  LoadSrc src;
+  SK(load_source(N, pos, types, dtab, a, dev, s, &src), "copy in");
+  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, src, st, &host_st, s);
   if (rc) return rc;
   // the same per-atom list limit, with the same error, as the handle-based entry points
   if (host_st.max_r > kListBuf || host_st.max_a > kListBuf)
