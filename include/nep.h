@@ -173,7 +173,7 @@ typedef struct {
   int members_per_launch; /* population members per launch (grid.y); 0: as many as a workspace
                              budget of min(half the free memory, 32 GiB) holds */
   int atom_block;         /* atoms per CTA of the batched per-atom kernel: 64 or 128 (0: 128;
-                             the BF16 tensor-core network always uses 128-atom tiles) */
+                             the BF16 tensor-core networks run 64 and take no other) */
   int gather_block;       /* atoms per CTA of the batched gather kernel: 64, 128, 256 (0: 128) */
   int last_members;       /* out: members per launch used by the last nep_eval_population */
   int n_tried;            /* out: candidates timed by the last nep_autotune */
@@ -408,7 +408,7 @@ int nep_set_profiling(nep_handle *h, int enable);
 /* Arithmetic of the network (Eq. Ui) and its gradient dU/dq:
  *   0 (default) FP32 on the FMA pipes;
  *   1 BF16 operands on the tensor cores (tcgen05.mma, FP32 accumulation in tensor memory):
- *     descriptor -> hidden and hidden -> dU/dq as two GEMMs per 128-atom tile. Descriptors,
+ *     descriptor -> hidden and hidden -> dU/dq as two GEMMs per 64 atoms. Descriptors,
  *     partial forces and all accumulations stay FP32; integration and totals FP64.
  *     Operand rounding (2^-9 relative) gives forces about 1e-2 relative error.
  *   2 split BF16: as 1, but every operand value x is carried as two BF16 terms

@@ -662,7 +662,7 @@ int rebuild_lists(nep_handle *h, int N, cudaStream_t s, int move, const Batch &B
     int rc = queue_build(h, s);
     if (rc) return rc;
     if (!src.pos) launch_arm_rebuild(h->status.p, h->bar.p, s);  // else requested by the load
-    CK(launch_rebuild(N, h->T, g, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
+    CK(launch_rebuild(N, h->T, g, B, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
                       list_bufs(h), count_only ? 1 : 0, move, src, h->status.p, s),
        "launch rebuild");
     src = LoadSrc{};  // the atoms are in place from here on
@@ -971,7 +971,7 @@ int capture_batch(nep_handle *h, int N, const BatchOut &o, cudaStream_t s) {
   cudaStream_t c = h->cap_stream;
   CK(cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal), "capture");
   const float rlR = (float)(h->rcR + h->skin), rlA = (float)(h->rcA + h->skin);
-  cudaError_t e = launch_rebuild(N, h->T, h->grid, batch_of(h), h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(),
+  cudaError_t e = launch_rebuild(N, h->T, h->grid, batch_of(h), rlR * rlR, rlA * rlA, h->rcR2f(),
                                  h->rcA2f(), atom_state(h), list_bufs(h), 0, 0, LoadSrc{o.pos, o.types, nullptr},
                                  h->status.p, c);
   int rc = e == cudaSuccess ? batch_kernels(h, N, o, c, true) : cuda_fail(h, e, "batch rebuild");
@@ -1220,7 +1220,7 @@ int engine_queue_iteration(nep_handle *h, cudaStream_t s) {
   // a build requested by the drift re-lists only the flagged jobs; a forced one every job
   Batch B = batch_of(h);
   B.sflag = h->e_sflag.p;
-  cudaError_t e = launch_rebuild(N, h->T, h->grid, B, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
+  cudaError_t e = launch_rebuild(N, h->T, h->grid, B, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
                                  atom_state(h), list_bufs(h), 0, 3, LoadSrc{}, h->status.p, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "engine rebuild");
   AtomArgs a = make_args(h, N);
@@ -1449,8 +1449,8 @@ int nep_destroy(nep_handle *h) {
   if (!h) return NEP_OK;
   if (h->graph) cudaGraphExecDestroy(h->graph);
   if (h->fire_graph) cudaGraphExecDestroy(h->fire_graph);
-  h->fire.release();
-  h->ck_fire.release();
+  if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
+  if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->cap_stream2) cudaStreamDestroy(h->cap_stream2);
   for (int sl = 0; sl < N_SLOTS; ++sl)
@@ -1461,24 +1461,9 @@ int nep_destroy(nep_handle *h) {
   h->e_out.release();
   if (h->h_status) cudaFreeHost(h->h_status);
   h->d_tab.release(); h->d_inv_mk.release(); h->d_mk_half.release();
-  h->x.release(); h->v.release(); h->F.release(); h->x_ref.release(); h->origin.release();
-  h->partial_atom.release(); h->partial_gather.release(); h->thermo_stage.release();
-  h->ck_x.release(); h->ck_v.release(); h->ck_F.release(); h->ck_types.release(); h->ck_perm.release();
-  h->x2.release(); h->v2.release(); h->F2.release(); h->types2.release(); h->perm2.release(); h->cell2.release();
-  h->perm.release();
-  h->types.release(); h->cell_of.release(); h->cell_count.release(); h->cell_cursor.release();
-  h->cell_start.release(); h->cell_atoms.release(); h->nn_r.release(); h->nn_a.release(); h->rev_a.release();
-  h->thermo_ctl.release(); h->nl_r.release(); h->nl_a.release(); h->pos4.release(); h->dtab.release();
-  h->posA.release();
-  h->e_slots.release(); h->e_slots_ck.release(); h->e_energy.release(); h->e_virial.release(); h->e_u.release();
-  h->e_w.release(); h->e_xck.release(); h->e_vck.release(); h->e_table.release();
-  h->stage_e.release(); h->stage_g.release();
-  h->p_ang.release(); h->e_rad.release(); h->status.release(); h->stat_part.release(); h->bar.release(); h->fin_scratch.release(); h->fin_ticket.release();
-  h->d_grids.release(); h->d_sid.release(); h->d_offsets.release(); h->b_e.release(); h->b_w.release();
-  if (h->b_graph) cudaGraphExecDestroy(h->b_graph);
-  if (h->e_graph) cudaGraphExecDestroy(h->e_graph);
-  h->pop_tab.release(); h->pop_reg.release();
-  h->pop_es.release(); h->pop_ws.release();
+  h->for_workspace([](auto &b) { b.release(); });
+  h->e_sflag.release(); h->status.release(); h->stat_part.release(); h->bar.release();
+  h->fin_scratch.release(); h->fin_ticket.release();
   delete h;
   return NEP_OK;
 }
@@ -2017,7 +2002,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     CK(cudaStreamUpdateCaptureDependencies(s, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies), "capture deps");
     CK(cudaStreamBeginCaptureToGraph(h->cap_stream2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed),
        "capture body");
-    cudaError_t e = launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
+    cudaError_t e = launch_rebuild(N, h->T, h->grid, Batch{}, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(),
                                    atom_state(h), list_bufs(h), 0, 1, LoadSrc{}, h->status.p, h->cap_stream2);
     cudaGraph_t out = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(h->cap_stream2, &out);
@@ -2027,7 +2012,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
     cudaGraphGetNodes(body, nullptr, &nn);
     h->rebuild_kernels = (int)nn;
   } else {
-    CK(launch_rebuild(N, h->T, h->grid, Batch{}, h->dtab.p, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
+    CK(launch_rebuild(N, h->T, h->grid, Batch{}, rlR * rlR, rlA * rlA, h->rcR2f(), h->rcA2f(), atom_state(h),
                       list_bufs(h), 0, 1, LoadSrc{}, h->status.p, s),
        "launch rebuild");
     h->rebuild_kernels = 0;

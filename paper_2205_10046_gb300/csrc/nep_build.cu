@@ -1442,17 +1442,22 @@ cudaError_t launch_lists(int N, int T, const Grid &g, const Batch &B, float rlR2
   }
 }
 
-cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
-                           float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only, int move,
+cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, float rlR2, float rlA2, float rcR2, float rcA2,
+                           const AtomState &a, const ListBufs &L, int count_only, int move,
                            const LoadSrc &src, BuildStatus *st, cudaStream_t s) {
   const int tb = 256;
   const int nb = (N + tb - 1) / tb;
   const int cb = (g.ncell + tb - 1) / tb;
   // One cooperative kernel with a warp per atom up to kWideBuildAtoms atoms, separate kernels with a
   // thread per atom above: a small system leaves the thread form with a few long serial scans, a
-  // large one makes the warp form pay for its idle lanes (ranges of ~20 candidates). Whole neighbour build, thread / warp form, us: 216 Si atoms
-  // 198 / 98, 13,824 172 / 111, 20,000 (three species, r_c 6 A) 258 / 139, 262,144 PbTe atoms
-  // 404 / 482, a batch of 1.05 million atoms 2056 / 2371, 8,000,000 Si atoms 7444 / 13,803.
+  // large one makes the warp form pay for its idle lanes (ranges of ~20 candidates). Whole build of a
+  // call, thread / warp form, us: 20,000 Si atoms 150 / 99, 66,000 182 / 184, 100,000 212 / 245, 131,072
+  // 238 / 311, 262,144 PbTe atoms 404 / 482; batches of 15,384 atoms of three species 232 / 94, 67,259
+  // 294 / 241, 128,755 378 / 402, 1.05 million 2056 / 2371. A single call would have the line at 66,000, a batch at
+  // 120,000. It lies at 131,072 for dynamics, where the separate kernels need a conditional graph node
+  // of about 10 us in every step: 20 steps with a build at the start, 30,000 Si atoms 2123 / 1860,
+  // 100,000 4453 / 4401, 131,072 5424 / 5456; PbTe 100,000 3911 / 3775. (A run that builds in nearly
+  // every step is better off with the threads from about 60,000 on: 120,000 atoms 12,131 / 15,268.)
   if (N <= kWideBuildAtoms) {
     const BuildArgs p{N, T, g.ncell, move, src, a, L, g, B, rlR2, rlA2, rcR2, rcA2, st};
     return count_only ? launch_build<true>(p, s) : launch_build<false>(p, s);

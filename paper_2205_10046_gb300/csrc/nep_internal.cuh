@@ -17,7 +17,6 @@ constexpr int kMaxImage = 3;    // largest cell/image offset searched per axis
 // above the FP32 rounding of a pair distance, so no candidate that the distance test would
 // accept is left out.
 constexpr double kReachMargin = 2e-3;
-constexpr int kAtomBlock = 128; // threads per block of the per-atom kernel
 // most atoms of the per-atom and gather kernels with four and with two groups of lanes per atom; the
 // reasons stand at the kernels
 constexpr int kSplitAtoms = 152 * 3 * 16, kSplitAtoms2 = 152 * 3 * 32;
@@ -285,7 +284,7 @@ struct ShapeOps {
   cudaError_t (*atom)(const AtomArgs &, const ModelF &, int descriptor_only, cudaStream_t s);
   cudaError_t (*gather)(const AtomArgs &, cudaStream_t s);
   // batched kernels (per-structure shift tables; `members` population members along y;
-  // `block` atoms per CTA: 64 or 128 for the atom kernel (128 with the tensor-core network),
+  // `block` atoms per CTA: 64 or 128 for the atom kernel (128 names the 64 of the tensor-core network),
   // 64, 128 or 256 for the gather kernel)
   cudaError_t (*atom_batch)(const AtomArgs &, const ModelF &, int members, int block, cudaStream_t s);
   cudaError_t (*gather_batch)(const AtomArgs &, int members, int block, cudaStream_t s);
@@ -345,8 +344,8 @@ void model_constants(ModelF &m);
 int build_grid(const double *box, double rl, int N, Grid &g, double *volume, const char **err);
 cudaError_t load_source(int N, const double *pos, const int *types, float4 *dtab, const AtomState &a, int device,
                         cudaStream_t s, LoadSrc *out);
-cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, const float4 *dtab, float rlR2, float rlA2,
-                           float rcR2, float rcA2, const AtomState &a, const ListBufs &L, int count_only,
+cudaError_t launch_rebuild(int N, int T, const Grid &g, const Batch &B, float rlR2, float rlA2, float rcR2, float rcA2,
+                           const AtomState &a, const ListBufs &L, int count_only,
                            int move, const LoadSrc &src, BuildStatus *st, cudaStream_t s);
 void launch_export(int N, const AtomState &a, const Grid &g, const Batch &B, double *pos, double *vel, double *force,
                    cudaStream_t s);

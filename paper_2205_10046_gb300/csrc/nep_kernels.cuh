@@ -54,7 +54,8 @@ struct Shape {
   static constexpr int off_cR(int prec) { return off_b0(prec) + r4(2 * H + 1); }
   static constexpr int off_cA(int prec, int T) { return off_cR(prec) + T * T * (NR + 1) * KRP; }
   static constexpr int off_S(int prec, int T) { return off_cA(prec, T) + T * T * CAP; }
-  // tensor-core network (BF16 operands, FP32 accumulation in TMEM), one 128-atom tile:
+  // tensor-core network (BF16 operands, FP32 accumulation in TMEM), one 128-row tile (64 atoms and 64
+  // unused rows):
   //   GEMM1 z[128 x NP1] = q[128 x KP1] . W0[NP1 x KP1]^T,  GEMM2 dq[128 x NP2] = beta[128 x KP2] . W0^T
   static constexpr int KP1 = (NDES + 15) / 16 * 16;
   static constexpr int NP1 = (H + 15) / 16 * 16;
@@ -474,8 +475,9 @@ __device__ __forceinline__ void for_pairs_batch(const unsigned *__restrict__ nl,
 // atoms per block of 128 threads), up to kSplitAtoms2 two (32 atoms per block). The sums over
 // neighbours stay with the first group, whose lanes add in the same order as ever (the same bits);
 // the network, the components, dU/dS_nk and the partial forces, which are independent term by term,
-// are shared. The limits are one wave of such blocks, three per SM: beyond it the groups that wait
-// cost more than the shorter chain gives. A dynamics step without / with, us (the gather kernel
+// are shared. The limits are three such blocks on each of the 152 SMs (one wave of the shapes that hold
+// three, less of those that hold four): beyond it the groups that wait cost more than the shorter
+// chain gives. A dynamics step without / with, us (the gather kernel
 // split in both): 216 Si atoms 40 / 36, 5,832 46 / 43, 8,000 46.4 / 45.8, 13,824 57.4 / 55.4, past the
 // limits with four groups 13,824 Si atoms 63 / 71, 8,000 PbTe atoms 41 / 50.
 template <class S>
@@ -484,17 +486,16 @@ struct PairRow {
   static constexpr int S4 = (S::NA + 1) * 6;             // float4s of S_nk
   static constexpr int R4 = (Q4 + S4) | 1;               // odd: 8 consecutive rows on 8 bank groups
   static constexpr int OCC = S::NA <= 4 ? 4 : 3;         // blocks of 128 threads per SM (shared memory)
-  // tensor-core network: BF16 terms per operand value, TMEM columns of the block
-  static constexpr int terms(int prec) { return prec; }
+  // tensor-core network (prec: BF16 terms per operand value): TMEM columns of the block
   static constexpr int AC = (S::KP1 > S::KP2 ? S::KP1 : S::KP2) / 2;  // columns of one A term
-  static constexpr int cols(int) { return 128; }
-  static_assert(S::ACOL + 2 * AC <= 128, "results and both A terms within 128 TMEM columns");
+  static constexpr int COLS = 128;
+  static_assert(S::ACOL + 2 * AC <= COLS, "results and both A terms within the block's TMEM columns");
   static constexpr bool tc(int prec) { return prec > 0; }
   // float offset of the rows in shared memory, after the table and the W0 tiles
   static constexpr int from(int prec) { return tc(prec) ? S::off_b0(0) : 0; }
   static constexpr int off_tiles(int prec, int T) { return S::off_S(0, T) - from(prec); }
   static constexpr int off_rows(int prec, int T) {
-    return off_tiles(prec, T) + (tc(prec) ? terms(prec) * S::TILE_B / 4 : 0);
+    return off_tiles(prec, T) + (tc(prec) ? prec * S::TILE_B / 4 : 0);
   }
 };
 
@@ -534,7 +535,7 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
   using PR = PairRow<S>;
   constexpr bool TC = PR::tc(PREC);
   static_assert(!DESC || PREC == 0, "the descriptors need no network");
-  constexpr int NT = TC ? PR::terms(PREC) : 1;  // BF16 terms per operand value of the tensor-core network
+  constexpr int NT = TC ? PREC : 1;  // BF16 terms per operand value of the tensor-core network
   // W0 tiles first (16-byte core matrices), then the shift table, the model table and the rows
   float *tiles = reinterpret_cast<float *>(smem4);
   float4 *dtab_s = smem4 + (TC ? NT * S::TILE_B / 16 : 0);  // [ncode] (one structure)
@@ -562,7 +563,7 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tiles, before the MMAs read them
     if (threadIdx.x < 32) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tc_tmem)),
-                   "r"((uint32_t)PR::cols(PREC)));
+                   "r"((uint32_t)PR::COLS));
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1229,7 +1230,7 @@ __global__ void __launch_bounds__(2 * AB *SUB, PairRow<S>::OCC * 64 / (AB * SUB)
     __syncthreads();
     if (threadIdx.x < 32) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc_tmem), "r"((uint32_t)PR::cols(PREC)));
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc_tmem), "r"((uint32_t)PR::COLS));
     }
   }
 }
@@ -1618,7 +1619,8 @@ __global__ void __launch_bounds__(GA *kGatherLanes *SUB, SUB > 1 ? 2 : gather_mi
 }
 
 // ------------------------------------------------------------------------ launchers
-// block sums of U of one structure: one slot per 64 atoms, an even number of them
+// block sums of U of one structure: a slot per 16 atoms up to kSplitAtoms2, above a slot per 64 atoms, an even
+// number of them
 template <class S> int atom_blocks(int N) { return N <= kSplitAtoms2 ? (N + 15) / 16 : 2 * ((N + 127) / 128); }
 
 template <class S, int PREC, bool DESC, bool BATCH, int AB, int SUB = 1>

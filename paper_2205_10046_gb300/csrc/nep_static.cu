@@ -91,13 +91,13 @@ int cuda_err(cudaError_t e, const char *where) {
     if (e_ != cudaSuccess) return cuda_err(e_, where); \
   } while (0)
 
-int run_build(int N, int T, const Grid &g, const float4 *dtab, float rlR2, float rlA2, float rcR2, float rcA2,
-              const AtomState &a, const ListBufs &L, int count_only, const LoadSrc &src, BuildStatus *st_dev,
+int run_build(int N, int T, const Grid &g, float rlR2, float rlA2, float rcR2, float rcA2, const AtomState &a,
+              const ListBufs &L, int count_only, const LoadSrc &src, BuildStatus *st_dev,
               BuildStatus *st_host, cudaStream_t s) {
   std::memset(st_host, 0, sizeof(BuildStatus));
   st_host->rebuild = 1;
   SK(cudaMemcpyAsync(st_dev, st_host, sizeof(BuildStatus), cudaMemcpyHostToDevice, s), "status");
-  SK(launch_rebuild(N, T, g, Batch{}, dtab, rlR2, rlA2, rcR2, rcA2, a, L, count_only, 0, src, st_dev, s),
+  SK(launch_rebuild(N, T, g, Batch{}, rlR2, rlA2, rcR2, rcA2, a, L, count_only, 0, src, st_dev, s),
      "neighbour build");
   SK(cudaMemcpyAsync(st_host, st_dev, sizeof(BuildStatus), cudaMemcpyDeviceToHost, s), "status");
   SK(cudaStreamSynchronize(s), "synchronise");
@@ -198,7 +198,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   SK(cudaGetDevice(&dev), "device");
   LoadSrc src;
   SK(load_source(N, pos, types, dtab, a, dev, s, &src), "copy in");
-  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, src, st, &host_st, s);
+  rc = run_build(N, T, g, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 1, src, st, &host_st, s);
   if (rc) return rc;
   // the same per-atom list limit, with the same error, as the handle-based entry points
   if (host_st.max_r > kListBuf || host_st.max_a > kListBuf)
@@ -210,7 +210,7 @@ int nep_descriptors_static(const nep_params *params, int n_atoms, const double *
   L.rev_a = arena.take<int>((size_t)L.cap_a * N);
   if (!L.nl_r || !L.nl_a || !L.rev_a)
     return fail_static(NEP_ERR_ARG, "neighbour lists too large for the static scratch (NEP_STATIC_SCRATCH_BYTES)");
-  rc = run_build(N, T, g, dtab, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 0, LoadSrc{}, st, &host_st, s);
+  rc = run_build(N, T, g, rlR * rlR, rlA * rlA, rcR * rcR, rcA * rcA, a, L, 0, LoadSrc{}, st, &host_st, s);
   if (rc) return rc;
   if (host_st.overflow || host_st.rev_missing) return fail_static(NEP_ERR_NEIGHBOR_OVERFLOW, "neighbour build failed");
 
