@@ -426,8 +426,8 @@ int nep_set_precision(nep_handle *h, int mode);
 int nep_set_graph_conditional(nep_handle *h, int enable);
 
 /* Most polls of a wait between the thread blocks of the neighbour build (0: the default, some
- * seconds). A wait that runs out ends the call, or the MD run, with NEP_ERR_TIMEOUT; the outputs
- * stay as they were. A small limit is for tests. */
+ * seconds). A wait that runs out ends the call with NEP_ERR_TIMEOUT: the outputs of an evaluation
+ * stay as they were, a dynamics state is unusable (call md_init again). A small limit is for tests. */
 int nep_set_wait_limit(nep_handle *h, int polls);
 int nep_kernel_slots(void);
 const char *nep_kernel_name(int slot);
