@@ -31,16 +31,6 @@ def _model(name, seed=7):
     return W.random_model(hyper, seed, [W.MASS_C, W.MASS_SI, W.MASS_GE][:T])
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 def _close(a, b):
     assert np.linalg.norm(a - b) <= 1e-5 * max(np.linalg.norm(b), 1e-30)
 

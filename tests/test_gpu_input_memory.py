@@ -10,16 +10,6 @@ from paper_2205_10046_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 @pytest.mark.parametrize("n", [300, 140000])  # the one-kernel build and the separate kernels
 def test_inputs_in_host_memory(torch_cuda, n):
     torch = torch_cuda

@@ -9,16 +9,6 @@ from paper_2205_10046_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 @pytest.mark.parametrize("between", ["compute", "descriptors", "md_init", "heat_current", "refused_box"])
 @pytest.mark.parametrize("calls_before", [1, 3])  # 3: the batch graph is captured
 @pytest.mark.parametrize("sizes", [[40, 8, 300, 77], [9]])

@@ -8,16 +8,6 @@ from paper_2205_10046_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 @pytest.mark.parametrize("reps", [3, 26])  # 216 and 140,608 atoms: both forms of the rebuild
 def test_nonfinite_positions_end_the_run(torch_cuda, reps):
     torch = torch_cuda

@@ -8,16 +8,6 @@ from paper_2205_10046_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 def test_groups_of_results(torch_cuda):
     torch = torch_cuda
     from paper_2205_10046_gb300 import nep

@@ -9,16 +9,6 @@ from paper_2205_10046_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 def _huge(hyper):
     """Only f_0 enters, every neuron alike: U_i = n w1 tanh(0.1 q_0), W_i,xx = sum of positive terms, each
     below the FP32 range and their sum above it."""

@@ -10,16 +10,6 @@ pytestmark = pytest.mark.gpu
 TIMEOUT, STATE = -8, -7
 
 
-@pytest.fixture(scope="module")
-def torch_cuda():
-    torch = pytest.importorskip("torch")
-    if not torch.cuda.is_available():
-        pytest.skip("no CUDA device")
-    from paper_2205_10046_gb300 import build
-    build.build()
-    return torch
-
-
 def _raises(code, f):
     from paper_2205_10046_gb300 import nep
     with pytest.raises(nep.NepError) as e:
