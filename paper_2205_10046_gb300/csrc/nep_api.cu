@@ -2020,7 +2020,7 @@ int md_step_launch(nep_handle *h, double dt, cudaStream_t s, bool capturing, boo
   ev_record(h, SLOT_REBUILD, 1, s, capturing);
   // totals of the steps that write a thermo row; the thermostat reads the kinetic energy of every step
   ThermoState *ts = (!fire && h->nvt) ? h->thermo_state.p : nullptr;
-  const int sums = kSumU | kSumKE | kSumW | (h->heat_rows ? kSumJ : 0);
+  const int sums = kSumU | kSumKE | kSumP | (h->heat_rows ? kSumJ : 0);
   int rc = run_forces(h, N, nullptr, h->F.p, nullptr, 1, 0.5 * dt, s, capturing, sums, ts ? kSumKE : 0,
                       h->thermo_ctl.p, fs);
   if (rc) return rc;

@@ -1040,7 +1040,8 @@ __global__ void __launch_bounds__(32 * kReduceSlots)
   __shared__ double tot[kReduceSlots];
   __shared__ int last;
   const int s = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool mine = s == 0 ? (sums & kSumU) : s == 1 ? (sums & kSumKE) : s <= 10 ? (sums & kSumW)
+  const bool mine = s == 0 ? (sums & kSumU) : s == 1 ? (sums & kSumKE)
+                    : s <= 10 ? (sums & kSumW) || (s <= 4 && (sums & kSumP))
                     : s >= 12 && s <= 14 ? (sums & kSumJ) : 0;
   auto warp_sum = [&](const double *p, int stride, int n) -> double {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};

@@ -23,7 +23,7 @@ constexpr int kSplitAtoms = 152 * 3 * 16, kSplitAtoms2 = 152 * 3 * 32;
 constexpr int kSplitGather = 152 * 2 * 32, kSplitGather2 = 152 * 2 * 64;
 constexpr int kReduceSlots = 16; // per-block partial sums: U, KE, W[9], force error, J[3], spare
 // sums over all atoms that a call or an MD step reads (AtomArgs::sums)
-enum { kSumU = 1, kSumKE = 2, kSumW = 4, kSumFerr = 8, kSumJ = 16 };
+enum { kSumU = 1, kSumKE = 2, kSumW = 4, kSumFerr = 8, kSumJ = 16, kSumP = 32 };  // kSumP: W's diagonal alone
 
 // Geometry of one neighbour build: the cell grid, the packing of list entries and the
 // table of pair shift vectors indexed by the packed image code.

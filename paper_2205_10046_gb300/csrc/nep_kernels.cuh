@@ -1315,16 +1315,18 @@ __device__ __forceinline__ void gather_finish(const AtomArgs &a, int mem, float 
     const int i = blockIdx.x * GA + threadIdx.x;
     gather_epilogue(a, i, a.pos4[i], mem, fw[threadIdx.x], need, part);
   }
-  if (!(need & (kSumKE | kSumW | kSumFerr | kSumJ))) return;
+  if (!(need & (kSumKE | kSumW | kSumP | kSumFerr | kSumJ))) return;
   double *out = a.partial_gather + ((size_t)mem * gridDim.x + blockIdx.x) * kReduceSlots;
-  if ((need & kSumW) && threadIdx.x < 96) {  // eight threads per component (96: whole warps)
+  // eight threads per component: nine in 96 threads (whole warps), the diagonal in 32
+  const int nw = (need & kSumW) ? 9 : (need & kSumP) ? 3 : 0;
+  if (threadIdx.x < 32 * ((nw + 3) / 4)) {
     const int c = threadIdx.x >> 3, p = threadIdx.x & 7;
     double s = 0.0;
-    if (c < 9)
+    if (c < nw)
       for (int r = p; r < GA; r += 8) s += (double)fw[r][3 + c];
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (c < 9 && p == 0) out[2 + c] = s;
+    if (c < nw && p == 0) out[2 + c] = s;
   }
   if (!(need & (kSumKE | kSumFerr | kSumJ))) return;
   if (threadIdx.x < GA) {
